@@ -36,6 +36,9 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
     // 16 bytes global -> shared without a register in between; an invalid piece is zero-filled (source size 0)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, bool valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(valid ? 4 : 0) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 template <int C> struct Stages { static constexpr int N = C <= 64 ? 3 : 2; };   // tiles resident per block (one worked on, the rest in flight)

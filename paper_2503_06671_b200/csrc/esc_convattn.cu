@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -23,6 +24,7 @@
 #include "backward_toeplitz_nchw.cuh"
 #include "stencil_dense.cuh"
 #include "stencil_dense_umma.cuh"
+#include "stencil_dense_fp32.cuh"
 #include <type_traits>
 #include "backward.cuh"
 #include "backward_pw.cuh"
@@ -443,8 +445,58 @@ int launch_dense_generic_t(const Problem& p, const void* x, const void* w_dense,
     return ESC_OK;
 }
 
-// Dense large kernel: tensor-core kernel where it applies, one thread per output elsewhere; the identity
-// channels go through the copy kernel either way.
+// Dense large kernel with 16 attention channels on the FP32 pipe; the identity channels go along as copy blocks.
+template <typename T, int LAYOUT, int K>
+int launch_dense_fp32_k(const Problem& p, const void* x, const void* w_dense, const float* dk, void* out, cudaStream_t st,
+                        bool dependent) {
+    namespace D = esc::dense32;
+    const int tiles_x = (p.W + D::TX - 1) / D::TX, tiles_y = (p.H + D::TY - 1) / D::TY;
+    const long long tiles = (long long)p.B * tiles_x * tiles_y;
+    const int split = D::choose_split(tiles, sms_or_nominal());
+    if (tiles * split > 0x3fffffffLL) return ESC_ERR_UNSUPPORTED;
+    esc::CopyJob job = make_copy_job(p, x, out, tiles * split, D::kThreads);
+    job.blocks = (job.blocks + split - 1) / split * split;               // whole clusters
+    static bool attr_set[esc::tma::kMaxDevices] = {};
+    const int dev = esc::tma::current_device();
+    if (dev < 0) return ESC_ERR_UNSUPPORTED;
+    if (!attr_set[dev]) {
+        ESC_CUDA(cudaFuncSetAttribute(D::stencil_dense_fp32<T, LAYOUT, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)std::max(D::Geo<K>::smem_bytes(1), D::Geo<K>::smem_bytes(8))));
+        attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * split + job.blocks));
+    cfg.blockDim = dim3(D::kThreads);
+    cfg.dynamicSmemBytes = D::Geo<K>::smem_bytes(split);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (dependent) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (split > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)split; attr[n].val.clusterDim.y = 1; attr[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    ESC_CUDA(cudaLaunchKernelEx(&cfg, D::stencil_dense_fp32<T, LAYOUT, K>, static_cast<const T*>(x), static_cast<T*>(out), p.C, p.H, p.W,
+                                p.K, static_cast<const T*>(w_dense), dk, p.bias, tiles_x, tiles_y, split, job));
+    ++g_last_launches;
+    return ESC_OK;
+}
+// Compiled for the sizes the paper compares (9, 13, 17); any other odd K is the next larger one with zeros around it.
+template <typename T, int LAYOUT>
+int launch_dense_fp32_t(const Problem& p, const void* x, const void* w_dense, const float* dk, void* out, cudaStream_t st, bool dependent) {
+    if (p.K <= 9) return launch_dense_fp32_k<T, LAYOUT, 9>(p, x, w_dense, dk, out, st, dependent);
+    if (p.K <= 13) return launch_dense_fp32_k<T, LAYOUT, 13>(p, x, w_dense, dk, out, st, dependent);
+    return launch_dense_fp32_k<T, LAYOUT, 17>(p, x, w_dense, dk, out, st, dependent);
+}
+
+// Dense large kernel: a tensor-core kernel where one applies, else the FP32-pipe kernel (16 attention channels) or one thread
+// per output (any other channel count).
 int launch_stencil_dense(const Problem& p, const void* x, const void* w_dense, const float* dk, void* out,
                          unsigned* ctrl, cudaStream_t st, bool dependent) {
     g_last_tile_w = 0;
@@ -464,6 +516,13 @@ int launch_stencil_dense(const Problem& p, const void* x, const void* w_dense, c
         return ESC_OK;                                     // the identity channels went along as copy blocks
     } else if (rc == esc::tma::kNotApplicable) {
         g_last_path = 1;
+        if (p.Ca == esc::dense32::CA) {
+            if (p.dtype == ESC_F32)
+                return p.layout == ESC_NCHW ? launch_dense_fp32_t<float, esc::kNCHW>(p, x, w_dense, dk, out, st, dependent)
+                                            : launch_dense_fp32_t<float, esc::kNHWC>(p, x, w_dense, dk, out, st, dependent);
+            return p.layout == ESC_NCHW ? launch_dense_fp32_t<__nv_bfloat16, esc::kNCHW>(p, x, w_dense, dk, out, st, dependent)
+                                        : launch_dense_fp32_t<__nv_bfloat16, esc::kNHWC>(p, x, w_dense, dk, out, st, dependent);
+        }
         if (p.dtype == ESC_F32)
             rc = p.layout == ESC_NCHW ? launch_dense_generic_t<float, esc::kNCHW>(p, x, w_dense, dk, out, st, dependent)
                                       : launch_dense_generic_t<float, esc::kNHWC>(p, x, w_dense, dk, out, st, dependent);
