@@ -260,7 +260,7 @@ int launch_copy(const Problem& p, const void* x, void* out, cudaStream_t st) {
 // The identity channels as a copy job for extra blocks of a stencil launch (blocks == 0: nothing to copy).
 esc::CopyJob make_copy_job(const Problem& p, const void* x, void* out, long long first_block, int threads) {
     esc::CopyJob j = {};
-    if (p.Ca == p.C) return j;
+    if (p.Ca == p.C || p.skip_copy) return j;
     const long long es = (long long)p.es(), HW = (long long)p.H * p.W;
     long long rows, row_b, stride_b, off_b;
     if (p.layout == ESC_NCHW) { rows = p.B; row_b = (p.C - p.Ca) * HW * es; stride_b = p.C * HW * es; off_b = p.Ca * HW * es; }
@@ -386,7 +386,7 @@ int launch_stencil(const Problem& p0, const void* x, const void* w_large0, const
             if (rn != esc::tma::kNotApplicable) return rn;
         }
     }
-    if (p.skip_copy) return ESC_ERR_UNSUPPORTED;           // only the tensor-core kernel can leave the identity channels out
+    if (p.skip_copy && p.dtype != ESC_F32) return ESC_ERR_UNSUPPORTED;   // of the kernels below only the generic one (all there is for fp32) can leave the identity channels out
     p.K = p0.K; w_large = w_large0;
     if (g_engine_policy == ESC_ENGINE_TENSOR) return launch_generic(p, x, w_large, dk, out, st, dependent);
     int tile_w = g_tile_policy;
@@ -816,11 +816,26 @@ int dense_add_const_t(const Problem& p, void* gx, const BackwardWs& w, cudaStrea
     return ESC_OK;
 }
 
+// ---- Conv_fuse on the FP32 pipe: att | idt are the two parts of its input, kTrans: the matrix is read transposed ----
+template <typename T, bool kTrans>
+int launch_fuse_fp32(const Problem& p, const void* att, const void* idt, const void* w, const void* bias, const void* residual,
+                     void* out, cudaStream_t st) {
+    esc::fuse::f32::Params<T> fp;
+    fp.att = static_cast<const T*>(att); fp.idt = static_cast<const T*>(idt); fp.w = static_cast<const T*>(w);
+    fp.bias = static_cast<const T*>(bias); fp.residual = static_cast<const T*>(residual); fp.out = static_cast<T*>(out);
+    fp.HW = (long long)p.H * p.W; fp.pixels = fp.HW * p.B; fp.B = p.B; fp.Ca = p.Ca; fp.vec = fp.HW % 4 == 0;
+    ESC_CUDA(p.layout == ESC_NCHW ? (esc::fuse::f32::launch<T, esc::kNCHW, kTrans>(p.C, fp, st))
+                                  : (esc::fuse::f32::launch<T, esc::kNHWC, kTrans>(p.C, fp, st)));
+    ++g_last_launches;
+    return ESC_OK;
+}
+
 // ---- backward pass of Conv_fuse -------------------------------------------------------------------------------
 struct FuseBackwardWs {
     void* wt;                        // W_fuse transposed, element type of the tensors
     float* part;                     // [blocks][C * C + C]
-    int passes, blocks;
+    int passes, blocks;              // tensor-core kernels
+    int passes32, blocks32;          // wgrad_fp32
     size_t bytes;
 };
 FuseBackwardWs carve_fuse_backward(void* ws, int C, long long pixels) {
@@ -829,28 +844,30 @@ FuseBackwardWs carve_fuse_backward(void* ws, int C, long long pixels) {
     const long long runs = (pixels + esc::fuse::bwd::kThreads - 1) / esc::fuse::bwd::kThreads, cap = sms_or_nominal();
     w.passes = (int)std::max(2LL, (runs + cap - 1) / cap);
     w.blocks = (int)((runs + w.passes - 1) / w.passes);
+    // wgrad_fp32: two blocks per SM
+    const long long runs32 = (pixels + esc::fuse::f32::kWPx - 1) / esc::fuse::f32::kWPx;
+    w.passes32 = (int)std::max(2LL, (runs32 + 2 * cap - 1) / (2 * cap));
+    w.blocks32 = (int)((runs32 + w.passes32 - 1) / w.passes32);
     char* base = static_cast<char*>(ws);
     size_t off = 0;
     w.wt = base + off;                              off += round_up((size_t)C * C * 4, 256);
-    w.part = reinterpret_cast<float*>(base + off);  off += round_up((size_t)w.blocks * ((size_t)C * C + C) * 4, 256);
+    w.part = reinterpret_cast<float*>(base + off);  off += round_up((size_t)std::max(w.blocks, w.blocks32) * ((size_t)C * C + C) * 4, 256);
     w.bytes = off;
     return w;
 }
 
 template <typename T, int LAYOUT, int C>
 int fuse_wgrad_c(const void* cat, const void* go, long long HW, long long pixels, const FuseBackwardWs& w, cudaStream_t st) {
-    using G = esc::fuse::bwd::Geom<C>;
-    if (G::kSmemBytes > 48 * 1024) {
-        static bool attr_set[esc::tma::kMaxDevices] = {};
-        const int dev = esc::tma::current_device();
-        if (dev < 0) return ESC_ERR_UNSUPPORTED;
-        if (!attr_set[dev]) {
-            ESC_CUDA(cudaFuncSetAttribute(esc::fuse::bwd::wgrad<T, LAYOUT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::kSmemBytes));
-            attr_set[dev] = true;
-        }
+    namespace F = esc::fuse::f32;
+    static bool attr_set[esc::tma::kMaxDevices] = {};
+    const int dev = esc::tma::current_device();
+    if (dev < 0) return ESC_ERR_UNSUPPORTED;
+    if (!attr_set[dev]) {
+        ESC_CUDA(cudaFuncSetAttribute(F::wgrad_fp32<T, LAYOUT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::WGeom<C>::kSmemBytes));
+        attr_set[dev] = true;
     }
-    esc::fuse::bwd::wgrad<T, LAYOUT, C><<<(unsigned)w.blocks, esc::fuse::bwd::kThreads, G::kSmemBytes, st>>>(
-        static_cast<const T*>(cat), static_cast<const T*>(go), HW, pixels, w.passes, w.part);
+    F::wgrad_fp32<T, LAYOUT, C><<<(unsigned)w.blocks32, F::kWThreads, F::WGeom<C>::kSmemBytes, st>>>(
+        static_cast<const T*>(cat), static_cast<const T*>(go), HW, pixels, w.passes32, w.part);
     ESC_CUDA(cudaGetLastError());
     ++g_last_launches;
     return ESC_OK;
@@ -890,7 +907,8 @@ int fuse_wgrad_mma_nchw_c(const void* cat, const void* go, long long HW, long lo
 }
 
 template <typename T, int LAYOUT>
-int fuse_wgrad_t(int C, const void* cat, const void* go, long long HW, long long pixels, const FuseBackwardWs& w, cudaStream_t st) {
+int fuse_wgrad_t(int C, const void* cat, const void* go, long long HW, long long pixels, const FuseBackwardWs& w, int* blocks, cudaStream_t st) {
+    *blocks = w.blocks;
     if (std::is_same<T, __nv_bfloat16>::value && LAYOUT == esc::kNCHW && HW % 8 == 0 && g_engine_policy != ESC_ENGINE_FP32) {
         // bf16 NCHW with whole 16-byte pieces per image: the same matrix product, operands without transposition
         switch (C) {
@@ -907,6 +925,7 @@ int fuse_wgrad_t(int C, const void* cat, const void* go, long long HW, long long
             case 64: return fuse_wgrad_mma_c<64>(cat, go, pixels, w, st);
         }
     }
+    *blocks = w.blocks32;
     switch (C) {
         case 16: return fuse_wgrad_c<T, LAYOUT, 16>(cat, go, HW, pixels, w, st);
         case 32: return fuse_wgrad_c<T, LAYOUT, 32>(cat, go, HW, pixels, w, st);
@@ -1328,6 +1347,15 @@ int esc_convattn_forward_fused(const void* x, int B, int C, int C_a, int H, int 
         ++g_last_launches;
         return ESC_OK;
     }
+    if (esc::fuse::f32::supported(C)) {
+        // The FP32-pipe 1x1 kernel.  For fp32 the identity channels are read from x and never copied; a bf16 forward may run on a
+        // kernel that always copies them, so there the whole concatenated map is in out.
+        p.skip_copy = dtype == ESC_F32;
+        rc = forward_impl(p, x, w_large, est, out, workspace, st);
+        if (rc != ESC_OK) return rc;
+        return dtype == ESC_F32 ? launch_fuse_fp32<float, false>(p, out, x, w_fuse, b_fuse, residual, out, st)
+                                : launch_fuse_fp32<__nv_bfloat16, false>(p, out, out, w_fuse, b_fuse, residual, out, st);
+    }
     rc = forward_impl(p, x, w_large, est, out, workspace, st);
     if (rc != ESC_OK) return rc;
     const size_t smem = (size_t)esc::fuse::kGenPix * C * sizeof(float);
@@ -1532,25 +1560,28 @@ int esc_conv_fuse_backward(const void* cat, const void* grad_out, int B, int C, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // the weight's and the bias's gradients
     if (grad_w_fuse || grad_b_fuse) {
+        int blocks = 0;
         if (dtype == ESC_F32)
-            rc = layout == ESC_NCHW ? fuse_wgrad_t<float, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, st)
-                                    : fuse_wgrad_t<float, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, st);
+            rc = layout == ESC_NCHW ? fuse_wgrad_t<float, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, &blocks, st)
+                                    : fuse_wgrad_t<float, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, &blocks, st);
         else
-            rc = layout == ESC_NCHW ? fuse_wgrad_t<__nv_bfloat16, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, st)
-                                    : fuse_wgrad_t<__nv_bfloat16, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, st);
+            rc = layout == ESC_NCHW ? fuse_wgrad_t<__nv_bfloat16, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, &blocks, st)
+                                    : fuse_wgrad_t<__nv_bfloat16, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, &blocks, st);
         if (rc != ESC_OK) return rc;
         const int elems = C * C + C;
-        esc::fuse::bwd::sum_wgrad<<<(unsigned)((elems + 7) / 8), 256, 0, st>>>(w.part, C, w.blocks, grad_w_fuse, grad_b_fuse);
+        esc::fuse::bwd::sum_wgrad<<<(unsigned)((elems + 7) / 8), 256, 0, st>>>(w.part, C, blocks, grad_w_fuse, grad_b_fuse);
         ESC_CUDA(cudaGetLastError());
         ++g_last_launches;
     }
     // grad_cat = W_fuse^T grad_out per pixel: the forward's 1x1 kernels with the transposed matrix, no bias, no residual
-    const unsigned tb = (unsigned)((C * C + 255) / 256);
-    if (dtype == ESC_F32) esc::fuse::bwd::transpose_w<float><<<tb, 256, 0, st>>>(static_cast<const float*>(w_fuse), C, static_cast<float*>(w.wt));
-    else esc::fuse::bwd::transpose_w<__nv_bfloat16><<<tb, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(w_fuse), C, static_cast<__nv_bfloat16*>(w.wt));
-    ESC_CUDA(cudaGetLastError());
-    ++g_last_launches;
-    if (esc::fuse::fast_applies(C, 8, dtype, layout)) {
+    const bool nhwc = esc::fuse::fast_applies(C, 8, dtype, layout);
+    if (nhwc || esc::fuse::nchw::applies(C, 8, HW, dtype, layout, grad_out, grad_cat, nullptr, w.wt)) {
+        const unsigned tb = (unsigned)((C * C + 255) / 256);
+        esc::fuse::bwd::transpose_w<__nv_bfloat16><<<tb, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(w_fuse), C, static_cast<__nv_bfloat16*>(w.wt));
+        ESC_CUDA(cudaGetLastError());
+        ++g_last_launches;
+    }
+    if (nhwc) {
         esc::fuse::Params fp;
         fp.att = static_cast<const __nv_bfloat16*>(grad_out); fp.idt = static_cast<const __nv_bfloat16*>(grad_out);
         fp.w = static_cast<const __nv_bfloat16*>(w.wt); fp.bias = nullptr; fp.residual = nullptr;
@@ -1570,18 +1601,9 @@ int esc_conv_fuse_backward(const void* cat, const void* grad_out, int B, int C, 
         ++g_last_launches;
         return ESC_OK;
     }
-    // any type and layout: the generic kernel works in place on a copy of grad_out
-    ESC_CUDA(cudaMemcpyAsync(grad_cat, grad_out, p.elems() * p.es(), cudaMemcpyDeviceToDevice, st));
-    const size_t smem = (size_t)esc::fuse::kGenPix * C * sizeof(float);
-    const unsigned blocks = (unsigned)((pixels + esc::fuse::kGenPix - 1) / esc::fuse::kGenPix);
-#define ESC_FUSE_GENERIC(T, L) esc::fuse::conv_fuse_generic<T, L><<<blocks, esc::fuse::kGenThreads, smem, st>>>( \
-        static_cast<T*>(grad_cat), static_cast<const T*>(w.wt), static_cast<const T*>(nullptr), static_cast<const T*>(nullptr), B, C, H, W)
-    if (dtype == ESC_F32) { if (layout == ESC_NCHW) ESC_FUSE_GENERIC(float, esc::kNCHW); else ESC_FUSE_GENERIC(float, esc::kNHWC); }
-    else { if (layout == ESC_NCHW) ESC_FUSE_GENERIC(__nv_bfloat16, esc::kNCHW); else ESC_FUSE_GENERIC(__nv_bfloat16, esc::kNHWC); }
-#undef ESC_FUSE_GENERIC
-    ESC_CUDA(cudaGetLastError());
-    g_last_launches += 2;
-    return ESC_OK;
+    const Problem pc{B, C, C, H, W, 3, dtype, layout};
+    return dtype == ESC_F32 ? launch_fuse_fp32<float, true>(pc, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st)
+                            : launch_fuse_fp32<__nv_bfloat16, true>(pc, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st);
 }
 
 int esc_convattn_selftest_bounded_wait(void* workspace, void* stream) {
