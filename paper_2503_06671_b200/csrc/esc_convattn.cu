@@ -29,6 +29,7 @@
 #include "backward.cuh"
 #include "backward_pw.cuh"
 #include "backward_dense.cuh"
+#include "backward_dense_umma.cuh"
 #include "conv_fuse.cuh"
 #include "conv_fuse_backward.cuh"
 
@@ -775,7 +776,19 @@ int dense_tap_grad_t(const Problem& p, const void* x, const void* go, const void
         attr_set[dev] = true;
     }
     const int tiles_x = (p.W + D::TX - 1) / D::TX, tiles_y = (p.H + D::TY - 1) / D::TY;
-    if (g_wd) {
+    bool g_wd_done = !g_wd;
+    if (g_wd && g_engine_policy != ESC_ENGINE_FP32 && g_dense_engine == 0) {
+        int blocks = 0;
+        const int rc = D::umma::try_launch(p.B, p.C, p.Ca, p.H, p.W, p.dtype, p.layout, x, go, w.dense_part, w.dense_blocks, w.ctrl, st, &blocks,
+                                           &g_last_launches, &g_last_error);
+        if (rc == ESC_OK) {
+            D::umma::sum_dense_umma<<<D::kPartFloats / 32, D::umma::kSumWarps * 32, 0, st>>>(w.dense_part, blocks, p.K, g_wd);
+            ESC_CUDA(cudaGetLastError());
+            ++g_last_launches;
+            g_wd_done = true;
+        } else if (rc != esc::tma::kNotApplicable) return rc;
+    }
+    if (!g_wd_done) {
         if (std::is_same<T, __nv_bfloat16>::value && g_engine_policy != ESC_ENGINE_FP32) {
             // bf16: a matrix product per tap on the tensor cores
             static bool attr_mma[esc::tma::kMaxDevices] = {};

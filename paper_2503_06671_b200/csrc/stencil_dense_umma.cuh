@@ -24,7 +24,7 @@
 //
 // Roles (224 threads, one CTA per SM, each CTA one range of rows of one strip):
 //   warp 0   lane 0 requests input rows by TMA (one load per row) into a ring of 16; the warp allocates and frees tensor memory
-//   warp 1   lane 0 issues the instructions and commits them to mbarriers (ring slot consumed / output row complete)
+//   warp 1   issues the instructions (one elected lane) and commits them to mbarriers (ring slot consumed / output row complete)
 //   warps 2-5  epilogue: tcgen05.ld of a finished row (one pixel per thread, 16 channels), the dynamic 3x3
 //            kernel in fp32 on the CUDA cores from the same ring, one rounding to bf16, 32-byte store;
 //            the row's columns are cleared for their next user.
@@ -85,14 +85,18 @@ __device__ __forceinline__ unsigned long long smem_desc_sw32(uint32_t addr) {
 __device__ __forceinline__ uint32_t instr_desc(int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(MW >> 4) << 24);
 }
+// Executed by a whole warp with the same arguments in every lane; one elected lane issues.  (Issued from a branch that a single
+// lane takes, an instruction occupied the issuing thread for about 112 cycles whatever its N; this way it costs what the
+// tensor pipe takes: 39 cycles for N = 16, 48 for 64, N / 2 from 128 on.)
 __device__ __forceinline__ void mma_f16(uint32_t d_tmem, unsigned long long da, unsigned long long db, uint32_t idesc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, 1, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(da), "l"(db), "r"(idesc) : "memory");
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void mma_commit(uint32_t bar) {         // the same elected lane: it tracks what that lane issued
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -231,11 +235,11 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
         }
     } else if (warp == 1) {
         // ======================= tensor-core instructions =============================================
-        if (lane == 0) {
-            bool alive = true;
-            const uint32_t ring_a = smem_u32(ring), btab_a = smem_u32(btab);
-            for (int n = 0; n < n_in && alive; ++n) {
-                const int slot = n % NRING;
+        bool alive = true;
+        const uint32_t ring_a = smem_u32(ring), btab_a = smem_u32(btab);
+        for (int n = 0; n < n_in; ++n) {
+            const int slot = n % NRING;
+            if (lane == 0) {
                 alive = mbar_wait(rowfull0 + 8 * slot, (unsigned)((n / NRING) & 1), p.ctrl, 0xD2000000u | (unsigned)n);
                 // the columns of the output row this input row opens (n, if it exists) were cleared by the epilogue of row n - 32
                 if (n >= SLOTS && n < L) {
@@ -245,24 +249,34 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
                         if (++polls > kPollLimit || ld_acquire_cta(aborted)) alive = false;
                     }
                 }
-                if (!alive) { if (p.ctrl) { atomicExch(p.ctrl, kDevTimeout); atomicExch(p.ctrl + 1, 0xD3000000u | (unsigned)n); } st_release_cta(aborted, 1); break; }
-                tc_fence_after();
-                // input row n feeds output rows n - 12 + c, c = 0 .. 12 (kernel row 12 - c), those inside [0, L)
-                const int c_lo = max(0, (K13 - 1) - n), c_hi = min(K13 - 1, L - 1 - n + (K13 - 1));
-                if (c_lo <= c_hi) {
-                    const int cnt = c_hi - c_lo + 1, s0 = (n - (K13 - 1) + c_lo) % SLOTS;
-                    const int cnt1 = min(cnt, SLOTS - s0), cnt2 = cnt - cnt1;      // the row slots wrap around at 32
+                if (!alive) { if (p.ctrl) { atomicExch(p.ctrl, kDevTimeout); atomicExch(p.ctrl + 1, 0xD3000000u | (unsigned)n); } st_release_cta(aborted, 1); }
+            }
+            alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
+            if (!alive) break;
+            tc_fence_after();
+            // input row n feeds output rows n - 12 + c, c = 0 .. 12 (kernel row 12 - c), those inside [0, L)
+            const int c_lo = max(0, (K13 - 1) - n), c_hi = min(K13 - 1, L - 1 - n + (K13 - 1));
+            if (c_lo <= c_hi) {
+                const int cnt = c_hi - c_lo + 1, s0 = (n - (K13 - 1) + c_lo) % SLOTS;
+                const int cnt1 = min(cnt, SLOTS - s0), cnt2 = cnt - cnt1;          // the row slots wrap around at 32
+                const uint32_t id1 = instr_desc(cnt1 * CG);
+                unsigned long long da = smem_desc_sw32(ring_a + (uint32_t)(slot * ROW_BYTES));
+                unsigned long long db = smem_desc(btab_a + (uint32_t)(c_lo * CG * 16), BHALF_BYTES, 128);
+                if (cnt2 == 0) {
+#pragma unroll
+                    for (int j = 0; j < K13; ++j)                              // one pixel (32 bytes) and one tap column further on
+                        mma_f16(tmem + (uint32_t)(s0 * CG), da + (unsigned long long)(2 * j), db + (unsigned long long)(j * (BJ_BYTES >> 4)), id1);
+                } else {
+                    const uint32_t id2 = instr_desc(cnt2 * CG);
                     for (int j = 0; j < K13; ++j) {
-                        const unsigned long long da = smem_desc_sw32(ring_a + (uint32_t)(slot * ROW_BYTES + 32 * j));
-                        const uint32_t bj = btab_a + (uint32_t)(j * BJ_BYTES + c_lo * CG * 16);
-                        mma_f16(tmem + (uint32_t)(s0 * CG), da, smem_desc(bj, BHALF_BYTES, 128), instr_desc(cnt1 * CG));
-                        if (cnt2 > 0)
-                            mma_f16(tmem, da, smem_desc(bj + (uint32_t)(cnt1 * CG * 16), BHALF_BYTES, 128), instr_desc(cnt2 * CG));
+                        mma_f16(tmem + (uint32_t)(s0 * CG), da, db, id1);
+                        mma_f16(tmem, da, db + (unsigned long long)(cnt1 * CG), id2);
+                        da += 2; db += BJ_BYTES >> 4;
                     }
                 }
-                mma_commit(rowdone0 + 8 * slot);                           // arrives when the instructions above have read the row
-                if (n >= K13 - 1) mma_commit(accfull0 + 8 * ((n - (K13 - 1)) % SLOTS));   // output row n - 12 is complete
             }
+            mma_commit(rowdone0 + 8 * slot);                                   // arrives when the instructions above have read the row
+            if (n >= K13 - 1) mma_commit(accfull0 + 8 * ((n - (K13 - 1)) % SLOTS));   // output row n - 12 is complete
         }
     } else if (warp == 6) {
         // ======================= copy-through of the identity channels: TMA in, TMA out ================
