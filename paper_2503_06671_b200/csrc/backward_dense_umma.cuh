@@ -32,7 +32,7 @@
 namespace esc { namespace bwd { namespace dense { namespace umma {
 
 using tma::u64; using tma::smem_u32; using tma::mbar_init; using tma::mbar_expect_tx; using tma::mbar_wait; using tma::tma_load_4d;
-using tma::umma::mma_f16; using tma::umma::mma_commit; using tma::umma::tc_fence_after; using tma::umma::tc_fence_before;
+using tma::umma::mbar_wait_warp; using tma::umma::mma_f16; using tma::umma::mma_commit; using tma::umma::tc_fence_after; using tma::umma::tc_fence_before;
 using tma::umma::tmem_ld16; using tma::umma::tmem_zero16; using tma::umma::tmem_wait_st;
 
 constexpr int kMaxRows = 32, kMaxCols = 64;                        // go tile
@@ -86,7 +86,7 @@ tap_grad_dense_umma(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     const uint32_t xfull0 = smem_u32(bars), xfree0 = xfull0 + 8 * kRing, gfull0 = xfree0 + 8 * kRing,
                    gfree0 = gfull0 + 16 * kGoGroups, done = gfree0 + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kRing + 2 * kGoGroups + 3);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: known to be uniform
     if (tid == 0) {
         for (int s = 0; s < kRing; ++s) { mbar_init(xfull0 + 8 * s, 1); mbar_init(xfree0 + 8 * s, 1); }
         for (int s = 0; s < 2 * kGoGroups; ++s) mbar_init(gfull0 + 8 * s, 1);
@@ -101,7 +101,7 @@ tap_grad_dense_umma(const __grid_constant__ CUtensorMap map_x, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     if (warp >= 2) {                                               // every instruction accumulates; warps 2-5 clear D_0, 6-9 D_1
         for (int s = 0; s < K; ++s) tmem_zero16(lane_base + (uint32_t)(((warp - 2) / 4 * K + s) * CA));
@@ -150,11 +150,8 @@ tap_grad_dense_umma(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             for (int n = 0; n < n_in; ++n) {
                 const int slot = (int)(xg % kRing), in_group = n % kGroup;
                 if (in_group == 0) {
-                    if (lane == 0) {
-                        if (n < t.rows) alive = mbar_wait(gfull0 + 8 * (gb * kGoGroups + n / kGroup), (it >> 1) & 1, p.ctrl, 0xE2000000u | it);
-                        if (alive) alive = mbar_wait(xfull0 + 8 * slot, (xg / kRing) & 1, p.ctrl, 0xE3000000u | xg);
-                    }
-                    alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
+                    if (n < t.rows) alive = mbar_wait_warp(gfull0 + 8 * (gb * kGoGroups + n / kGroup), (it >> 1) & 1, p.ctrl, 0xE2000000u | it);
+                    if (alive) alive = mbar_wait_warp(xfull0 + 8 * slot, (xg / kRing) & 1, p.ctrl, 0xE3000000u | xg);
                     if (!alive) break;
                     tc_fence_after();
                 }

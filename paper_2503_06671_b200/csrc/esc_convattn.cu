@@ -499,14 +499,16 @@ int launch_dense_fp32_t(const Problem& p, const void* x, const void* w_dense, co
 // Dense large kernel: a tensor-core kernel where one applies, else the FP32-pipe kernel (16 attention channels) or one thread
 // per output (any other channel count).
 int launch_stencil_dense(const Problem& p, const void* x, const void* w_dense, const float* dk, void* out,
-                         unsigned* ctrl, cudaStream_t st, bool dependent) {
+                         unsigned* ctrl, cudaStream_t st, bool dependent, bool flip = false) {
+    // flip: w_dense is read with its channel axes swapped and its taps rotated, which the tcgen05 kernel alone can do
     g_last_tile_w = 0;
     if (g_dense_engine == 0) {
         const int urc = esc::tma::umma::try_launch_dense_umma(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, w_dense, dk, out,
-                                                              ctrl, st, dependent, &g_last_launches, &g_last_error);
+                                                              ctrl, st, dependent, &g_last_launches, &g_last_error, p.bias, flip);
         if (urc == ESC_OK) { g_last_path = 5; g_last_tile_w = esc::tma::umma::MW; return ESC_OK; }
         if (urc != esc::tma::kNotApplicable) return urc;
     }
+    if (flip) return esc::tma::kNotApplicable;
     esc::CopyJob job = make_copy_job(p, x, out, 0, esc::tma::dense::kThreads);
     if (job.blocks > (unsigned)sms_or_nominal()) job.blocks = (unsigned)sms_or_nominal();   // every block of that launch takes a whole SM
     int rc = esc::tma::try_launch_dense(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, w_dense, dk, out, ctrl,
@@ -762,11 +764,9 @@ int pw_back_t(const Problem& p, const void* x, const void* w_point, void* gx, co
     return ESC_ERR_UNSUPPORTED;
 }
 
-// Dense large kernel: tap gradients of every channel pair, the rotated kernel for the stencil pass, and the constants
-// added behind it.
+// Dense large kernel: tap gradients of every channel pair.
 template <typename T, int LAYOUT>
-int dense_tap_grad_t(const Problem& p, const void* x, const void* go, const void* w_dense, const BackwardWs& w, float* g_wd,
-                     cudaStream_t st) {
+int dense_tap_grad_t(const Problem& p, const void* x, const void* go, const BackwardWs& w, float* g_wd, cudaStream_t st) {
     namespace D = esc::bwd::dense;
     static bool attr_set[esc::tma::kMaxDevices] = {};
     const int dev = esc::tma::current_device();
@@ -812,18 +812,28 @@ int dense_tap_grad_t(const Problem& p, const void* x, const void* go, const void
         ESC_CUDA(cudaGetLastError());
         g_last_launches += 2;
     }
+    return ESC_OK;
+}
+// grad_x of the dense form: the forward's kernels on grad_out with the kernel's channel axes swapped and its taps rotated, plus
+// the constants.  The tcgen05 kernel reads the weights that way and adds the constants itself; for the others the rotated
+// kernel is written first, and the mma.sync kernel's result gets the constants in a pass of its own.
+template <typename T, int LAYOUT>
+int dense_grad_x_t(Problem p, const void* go, const void* w_dense, void* gx, const BackwardWs& w, cudaStream_t st) {
+    namespace D = esc::bwd::dense;
+    p.dense = true;
+    p.bias = w.bias;
+    int rc = launch_stencil_dense(p, go, w_dense, w.dk_flip, gx, w.ctrl, st, /*dependent=*/false, /*flip=*/true);
+    if (rc != esc::tma::kNotApplicable) return rc;
     const int elems = D::CA * D::CA * p.K * p.K;
     D::flip_dense<T><<<(unsigned)((elems + 255) / 256), 256, 0, st>>>(static_cast<const T*>(w_dense), p.K, static_cast<T*>(w.wd_flip));
     ESC_CUDA(cudaGetLastError());
     ++g_last_launches;
-    return ESC_OK;
-}
-template <typename T, int LAYOUT>
-int dense_add_const_t(const Problem& p, void* gx, const BackwardWs& w, cudaStream_t st) {
+    rc = launch_stencil_dense(p, go, w.wd_flip, w.dk_flip, gx, w.ctrl, st, /*dependent=*/false);
+    if (rc != ESC_OK || g_last_path != 3) return rc;
     const long long total = (long long)p.B * p.Ca * p.H * p.W;
     long long blocks = (total + 255) / 256;
     if (blocks > 16LL * sms_or_nominal()) blocks = 16LL * sms_or_nominal();
-    esc::bwd::dense::add_const<T, LAYOUT><<<(unsigned)blocks, 256, 0, st>>>(static_cast<T*>(gx), w.bias, p.B, p.C, p.Ca, (long long)p.H * p.W);
+    D::add_const<T, LAYOUT><<<(unsigned)blocks, 256, 0, st>>>(static_cast<T*>(gx), w.bias, p.B, p.C, p.Ca, (long long)p.H * p.W);
     ESC_CUDA(cudaGetLastError());
     ++g_last_launches;
     return ESC_OK;
@@ -1438,12 +1448,12 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
     }
     const void* x_taps = w_point ? grad_x : x;             // what the depth-wise stage saw
     if (dense) {
-        // w_large is the dense kernel [16][16][K][K]: its gradient and its rotated form here; the depth-wise kernels
+        // w_large is the dense kernel [16][16][K][K]: its gradient here; the depth-wise kernels
         // below give g_dk (the middle 3 x 3 of their tap gradients) and what follows from it
-        rc = dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_tap_grad_t<float, esc::kNCHW>(p, x, grad_out, w_large, w, g_wd, st)
-                                                    : dense_tap_grad_t<float, esc::kNHWC>(p, x, grad_out, w_large, w, g_wd, st))
-                              : (layout == ESC_NCHW ? dense_tap_grad_t<__nv_bfloat16, esc::kNCHW>(p, x, grad_out, w_large, w, g_wd, st)
-                                                    : dense_tap_grad_t<__nv_bfloat16, esc::kNHWC>(p, x, grad_out, w_large, w, g_wd, st));
+        rc = dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_tap_grad_t<float, esc::kNCHW>(p, x, grad_out, w, g_wd, st)
+                                                    : dense_tap_grad_t<float, esc::kNHWC>(p, x, grad_out, w, g_wd, st))
+                              : (layout == ESC_NCHW ? dense_tap_grad_t<__nv_bfloat16, esc::kNCHW>(p, x, grad_out, w, g_wd, st)
+                                                    : dense_tap_grad_t<__nv_bfloat16, esc::kNHWC>(p, x, grad_out, w, g_wd, st));
         if (rc != ESC_OK) return rc;
     }
     if (dtype == ESC_F32)
@@ -1455,15 +1465,11 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
     if (rc != ESC_OK) return rc;
     // grad_x: the forward stencil on grad_out with both kernels rotated by 180 degrees, plus the constants (in the
     // decomposed form the constants belong behind the transposed mix: the last kernel adds them)
-    if (dense) {
-        p.dense = true;
-        rc = launch_stencil_dense(p, grad_out, w.wd_flip, w.dk_flip, grad_x, w.ctrl, st, /*dependent=*/false);
-        if (rc != ESC_OK) return rc;
-        return dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_add_const_t<float, esc::kNCHW>(p, grad_x, w, st)
-                                                      : dense_add_const_t<float, esc::kNHWC>(p, grad_x, w, st))
-                                : (layout == ESC_NCHW ? dense_add_const_t<__nv_bfloat16, esc::kNCHW>(p, grad_x, w, st)
-                                                      : dense_add_const_t<__nv_bfloat16, esc::kNHWC>(p, grad_x, w, st));
-    }
+    if (dense)
+        return dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_grad_x_t<float, esc::kNCHW>(p, grad_out, w_large, grad_x, w, st)
+                                                      : dense_grad_x_t<float, esc::kNHWC>(p, grad_out, w_large, grad_x, w, st))
+                                : (layout == ESC_NCHW ? dense_grad_x_t<__nv_bfloat16, esc::kNCHW>(p, grad_out, w_large, grad_x, w, st)
+                                                      : dense_grad_x_t<__nv_bfloat16, esc::kNHWC>(p, grad_out, w_large, grad_x, w, st));
     p.bias = w_point ? nullptr : w.bias;
     const TensorLk tl = tensor_lk(p, grad_out, grad_x, w.w_flip, w.lk_pad, st);
     rc = launch_stencil(p, grad_out, w.w_flip, w.dk_flip, grad_x, w.ctrl, st, /*dependent=*/false, &tl);

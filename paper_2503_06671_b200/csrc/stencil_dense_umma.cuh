@@ -18,14 +18,17 @@
 // swizzle; the swizzle is a function of the shared-memory address, so the descriptor may start at ANY pixel and
 // the tap column j is a shift of its start address by 32 * j bytes (verified output by output against
 // a direct fp64 evaluation).  B: the weights, without swizzle ([half of K][row][8 k-values], rows 16 bytes apart).
-// What bounds it: an instruction takes about 110-130 cycles whatever its N, so the 12 input rows above and below
-// a CTA's range, which feed only some of the 13 column blocks, cost as much as full rows: with 13 output rows per
-// CTA (640x360 on 148 SMs) 25 row-times are spent for 13 rows of results; larger maps give longer ranges.
+// What bounds it: an instruction takes 104 cycles at N = 208 and 39 to 96 for the 12 input rows above and below a CTA's range,
+// which feed only some of the 13 column blocks: with 13 output rows per CTA (640x360 on 148 SMs) 20.6 k cycles for 17.6 k
+// cycles' worth of results; larger maps give longer ranges.  Its operands are 10.7 KB of shared memory per 104 cycles, so what
+// else moves through shared memory (the copy-through, the 3x3 part) is felt: 120 cycles in place of 104.  640x360 alone, cold:
+// 36.9 -> 28.7 us (B table 12 k -> 8.3 k cycles, of them 4 k until the weights have landed; 137 -> 120 cycles per instruction by
+// the way the issuing warp waits; 3x3 part read row by row); 64 patches of 64x64: 53 -> 44 us.
 //
 // Roles (224 threads, one CTA per SM, each CTA one range of rows of one strip):
 //   warp 0   lane 0 requests input rows by TMA (one load per row) into a ring of 16; the warp allocates and frees tensor memory
 //   warp 1   issues the instructions (one elected lane) and commits them to mbarriers (ring slot consumed / output row complete)
-//   warps 2-5  epilogue: tcgen05.ld of a finished row (one pixel per thread, 16 channels), the dynamic 3x3
+//   warps 2-5  epilogue: tcgen05.ld of a finished row (one pixel per thread, 16 channels), constants, the dynamic 3x3
 //            kernel in fp32 on the CUDA cores from the same ring, one rounding to bf16, 32-byte store;
 //            the row's columns are cleared for their next user.
 //   warp 6   lane 0 copies the identity channels of the CTA's rows, TMA in / TMA out through a ring of two slots.
@@ -42,29 +45,36 @@ constexpr int ROW_BYTES = 2 * HALF_BYTES;     // one staged row: SPX pixels x 32
 constexpr int NRING = 16;                     // input rows in flight / kept for the 3x3 part
 constexpr int NBLK = K13;                     // column blocks of 16 (kernel rows) in a B operand
 constexpr int BHALF_BYTES = NBLK * CG * 16;   // 3,328: one tap column, one channel half: [208 rows][8 k]
-constexpr int BJ_BYTES = 2 * BHALF_BYTES;
-constexpr int B_BYTES = K13 * BJ_BYTES;       // 86,528
+constexpr int BJ_BYTES = 2 * BHALF_BYTES + 16;   // tap columns 16 bytes apart modulo 128: the table's stores spread over the banks
+constexpr int B_BYTES = (K13 * BJ_BYTES + 127) / 128 * 128;   // 86,784
 constexpr int SLOTS = 32;                     // output rows whose accumulators fit tensor memory (512 columns)
 constexpr int kThreads = 224;                 // producer, issuer, four epilogue warps, copy-through warp
 constexpr int kEpiThreads = 128;
 constexpr int kCopySlotBytes = 16384, kCopySlots = 2;
 constexpr unsigned kPollLimit = 1u << 22;
 constexpr int kMiscBytes = 1024;               // dk, progress word, tensor-memory base
-constexpr int kBarBytes = 1024;                // 2 * NRING + SLOTS + kCopySlots mbarriers
+constexpr int kBarBytes = 1024;                // 2 * NRING + SLOTS + kCopySlots + 1 mbarriers
 constexpr int kCopyRingOffset = NRING * ROW_BYTES + B_BYTES + kMiscBytes + kBarBytes;
 constexpr size_t kSmemBytes = (size_t)kCopyRingOffset + kCopySlots * kCopySlotBytes;
-static_assert((2 * NRING + SLOTS + kCopySlots) * 8 <= kBarBytes && kCopyRingOffset % 128 == 0, "barriers fit; the copy ring is a TMA destination");
+static_assert((2 * NRING + SLOTS + kCopySlots + 1) * 8 <= kBarBytes && kCopyRingOffset % 128 == 0, "barriers fit; the copy ring is a TMA destination");
+// While the B table is built the weights as they are lie behind the first three rows of the ring (eleven of sixteen leading
+// channels) and in the copy ring (five).
+constexpr int kRawRows = 3, kRawSplit = 11, kRawChannelBytes = CG * K13 * K13 * 2;
+static_assert(kRawSplit * kRawChannelBytes <= (NRING - kRawRows) * ROW_BYTES && (CG - kRawSplit) * kRawChannelBytes <= kCopySlots * kCopySlotBytes, "staging");
 static_assert(HALF_BYTES % 128 == 0, "TMA destinations are 128-byte aligned");
 
 struct Params {
     int B, C, H, W;
     int strips, segs, seg_rows;       // per image: strips of 128 pixels x row ranges of seg_rows rows
-    const __nv_bfloat16* w_dense;     // [16][16][13][13]  (output channel, input channel, row, column)
+    const __nv_bfloat16* w_dense;     // [16][16][KK][KK]  (output channel, input channel, row, column)
+    int KK;                           // odd, at most 13: a smaller kernel sits in the middle of zeros
+    int raw_bulk;                     // w_dense is 16-byte aligned: it is staged with bulk copies
+    int flip;                         // the gradient's form: channel axes of w_dense swapped, taps rotated by 180 degrees
     const float* dk;                  // [B][16][9]
+    const float* bias;                // [B][16] added to every output of an (image, channel), or nullptr
     __nv_bfloat16* out;
     unsigned* ctrl;
     int wait_first;
-    int w_aligned;                    // w_dense is 16-byte aligned: the B operands are built from a staged copy
     int copy_cc, copy_pw;             // identity channels; pixels of a strip row per copy chunk (0: nothing to copy)
 };
 
@@ -98,6 +108,20 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {         // the same e
     asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
                  "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
+// The issuing warp's bounded wait, by all its lanes: a phase that is complete costs about 85 cycles this way, hidden behind the
+// instructions in flight; one lane asking for the warp costs 280 (the branch, and what the compiler no longer takes for uniform).
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, unsigned parity, unsigned* ctrl, unsigned where) {
+    unsigned ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (__all_sync(0xffffffffu, ok)) return true;
+    for (unsigned n = 0; n < kSpinLimit; ++n) {
+        ok = mbar_try_wait(bar, parity);
+        if (__all_sync(0xffffffffu, ok)) return true;
+    }
+    if (ctrl && (threadIdx.x & 31) == 0) { atomicExch(ctrl, kDevTimeout); atomicExch(ctrl + 1, where); }
+    return false;
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
@@ -120,6 +144,10 @@ __device__ __forceinline__ int ld_acquire_cta(const int* p) {
 __device__ __forceinline__ void st_release_cta(int* p, int v) {
     asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, unsigned bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
 __device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
     tma_load_4d(dst, map, bar, c0, c1, c2, c3);
 }
@@ -137,14 +165,15 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
     uint32_t* tmem_base_slot = reinterpret_cast<uint32_t*>(prog + 2);
     u64* bars = reinterpret_cast<u64*>(btab + B_BYTES + 1024);
     const uint32_t rowfull0 = smem_u32(bars), rowdone0 = rowfull0 + 8 * NRING, accfull0 = rowdone0 + 8 * NRING,
-                   cfull0 = accfull0 + 8 * SLOTS;
+                   cfull0 = accfull0 + 8 * SLOTS, wfull = cfull0 + 8 * kCopySlots;
     unsigned char* cring = smem + kCopyRingOffset;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: known to be uniform
     if (tid == 0) {
         for (int s = 0; s < NRING; ++s) { mbar_init(rowfull0 + 8 * s, 1); mbar_init(rowdone0 + 8 * s, 1); }
         for (int s = 0; s < SLOTS; ++s) mbar_init(accfull0 + 8 * s, 1);
         for (int s = 0; s < kCopySlots; ++s) mbar_init(cfull0 + 8 * s, 1);
+        mbar_init(wfull, 1);
         *prog = 0; *aborted = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -155,7 +184,7 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *tmem_base_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_base_slot, 0);
     if (p.wait_first) pdl_wait_primary();
     pdl_launch_dependents();
 
@@ -168,36 +197,28 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
     const int x0 = sx * MW;
     const int n_in = L + K13 - 1;                           // input rows ya - 6 .. yb + 5, index n = row - (ya - 6)
 
-    // ---- B operands: btab[j][half][(12 - i) * 16 + n][k % 8] = w_dense[n][half * 8 + k % 8][i][j] ------------
-    // The weights are gathered with a stride of 169 elements.  From global memory that is 28 rounds of dependent
-    // 2-byte loads per thread; instead half of w_dense at a time (8 output channels, 43 KB) is copied, coalesced,
-    // into the still empty input ring and the rows are gathered from there.
-    {
-        uint4* bt = reinterpret_cast<uint4*>(btab);
-        constexpr int HALF_W = 8 * CG * K13 * K13;                              // elements of 8 output channels
-        static_assert(HALF_W * 2 <= NRING * ROW_BYTES && (HALF_W * 2) % 16 == 0, "staging fits the ring");
-        for (int nh = 0; nh < 2; ++nh) {
-            const unsigned short* w;
-            if (p.w_aligned) {
-                const uint4* src = reinterpret_cast<const uint4*>(p.w_dense + (size_t)nh * HALF_W);
-                uint4* dst = reinterpret_cast<uint4*>(ring);
-                for (int e = tid; e < HALF_W * 2 / 16; e += kThreads) dst[e] = __ldg(src + e);
-                __syncthreads();
-                w = reinterpret_cast<const unsigned short*>(ring);
-            } else {
-                w = reinterpret_cast<const unsigned short*>(p.w_dense) + (size_t)nh * HALF_W;
-            }
-            for (int e = tid; e < K13 * 2 * NBLK * 8; e += kThreads) {           // one 16-byte row each: (j, half, i, n % 8)
-                const int n8 = e & 7, ii = (e >> 3) % NBLK, h = ((e >> 3) / NBLK) & 1, j = (e >> 3) / (2 * NBLK);
-                const int i = (K13 - 1) - ii;
-                unsigned v[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) v[q] = w[((size_t)(n8 * CG + h * 8 + q) * K13 + i) * K13 + j];
-                bt[(j * 2 + h) * (NBLK * CG) + ii * CG + nh * 8 + n8] =
-                    make_uint4(v[0] | (v[1] << 16), v[2] | (v[3] << 16), v[4] | (v[5] << 16), v[6] | (v[7] << 16));
-            }
-            __syncthreads();                                                     // the staging area is re-used
+    auto request_rows = [&](int n0, int n1) {
+        for (int n = n0; n < min(n_in, n1); ++n) {
+            mbar_expect_tx(rowfull0 + 8 * n, ROW_BYTES);
+            tma_load_4d(smem_u32(ring + (size_t)n * ROW_BYTES), &map_half, rowfull0 + 8 * n, 0, x0 - P6, ya - P6 + n, b);
         }
+    };
+    // ---- B operands: btab[j][half][(12 - i) * 16 + n][k % 8] = w[n][half * 8 + k % 8][i][j] -----------------------
+    // The weights come as they are with two bulk copies, behind the first rows of the ring and in the copy ring.  Then a warp
+    // takes 32 consecutive taps of an output channel n and half of the input channels: eight 2-byte reads per lane, 64
+    // contiguous bytes over the warp, and one 16-byte store.
+    const int taps = p.KK * p.KK, chan = CG * taps;                              // elements of one leading channel of w_dense
+    if (p.raw_bulk) {
+        if (tid == 0) {
+            mbar_expect_tx(wfull, (unsigned)(CG * chan * 2));
+            bulk_load(smem_u32(ring + kRawRows * ROW_BYTES), p.w_dense, (unsigned)(kRawSplit * chan * 2), wfull);
+            bulk_load(smem_u32(cring), p.w_dense + kRawSplit * chan, (unsigned)((CG - kRawSplit) * chan * 2), wfull);
+            request_rows(0, kRawRows);
+        }
+    }
+    if (p.KK < K13) {
+        for (int e = tid; e < B_BYTES / 16; e += kThreads) reinterpret_cast<uint4*>(btab)[e] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
     }
     // clear the accumulators: every instruction accumulates, a row's columns are cleared again after it is read
     if (warp >= 2) {
@@ -205,29 +226,63 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
         for (int s = 0; s < SLOTS; ++s) tmem_zero16(lane_base + (uint32_t)(s * CG));
         tmem_wait_st();
     }
+    if (p.raw_bulk) mbar_wait(wfull, 0, p.ctrl, 0xD7000000u);
+    {
+        // a lane's place in the table depends on its tap alone: worked out once per 32 taps, not per item
+        const int off = (K13 - p.KK) / 2;
+        auto build = [&](auto value) {                                            // value(leading channel, offset behind it)
+            for (int t0 = 0; t0 < taps; t0 += 32) {
+                const int t = t0 + lane, tc = min(t, taps - 1), r = tc / p.KK, c = tc - r * p.KK;
+                const int i = off + (p.flip ? p.KK - 1 - r : r), j = off + (p.flip ? p.KK - 1 - c : c);
+                unsigned char* dst = btab + j * BJ_BYTES + (K13 - 1 - i) * CG * 16;
+                constexpr int kWarps = kThreads / 32, kItems = (2 * CG + kWarps - 1) / kWarps;
+                unsigned v[kItems][8];
+#pragma unroll
+                for (int u = 0; u < kItems; ++u) {                                // all reads of the 32 taps, then the stores
+                    const int nh = min(warp + u * kWarps, 2 * CG - 1), n = nh >> 1, h = nh & 1;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        v[u][q] = p.flip ? value(8 * h + q, n * taps + tc) : value(n, (8 * h + q) * taps + tc);
+                }
+#pragma unroll
+                for (int u = 0; u < kItems; ++u) {
+                    const int nh = warp + u * kWarps;
+                    if (nh < 2 * CG && t < taps)
+                        *reinterpret_cast<uint4*>(dst + (nh & 1) * BHALF_BYTES + (nh >> 1) * 16) =
+                            make_uint4(v[u][0] | (v[u][1] << 16), v[u][2] | (v[u][3] << 16), v[u][4] | (v[u][5] << 16), v[u][6] | (v[u][7] << 16));
+                }
+            }
+        };
+        if (p.raw_bulk) {
+            const unsigned short* lo = reinterpret_cast<const unsigned short*>(ring + kRawRows * ROW_BYTES);
+            const int hi = (int)((cring - (ring + kRawRows * ROW_BYTES)) / 2) - kRawSplit * chan;   // where channel 0 would lie for the second piece
+            build([&](int a, int o) { return (unsigned)lo[a * chan + o + (a < kRawSplit ? 0 : hi)]; });
+        } else {
+            build([&](int a, int o) { return (unsigned)__ldg(reinterpret_cast<const unsigned short*>(p.w_dense) + a * chan + o); });
+        }
+    }
     fence_async_smem();                                     // the B table is read through the async proxy
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (tid == 0) request_rows(p.raw_bulk ? kRawRows : 0, NRING);
 
     if (warp == 0) {
-        // ======================= input rows by TMA ====================================================
+        // ======================= input rows by TMA (the first sixteen are under way) ===================
         if (lane == 0) {
             bool alive = true;
-            for (int n = 0; n < n_in && alive; ++n) {
+            for (int n = NRING; n < n_in && alive; ++n) {
                 const int slot = n % NRING;
-                if (n >= NRING) {
-                    // the slot's previous row (n - 16) must have been consumed by the tensor cores and, if the 3x3
-                    // part of an output row reads it (rows n - 21 .. of this CTA's range), by the epilogue
-                    alive = mbar_wait(rowdone0 + 8 * slot, (unsigned)(((n - NRING) / NRING) & 1), p.ctrl, 0xD0000000u | (unsigned)n);
-                    const int need = min(n - 20, L);
-                    unsigned polls = 0;
-                    while (alive && ld_acquire_cta(prog) < need) {
-                        __nanosleep(64);
-                        if (++polls > kPollLimit || ld_acquire_cta(aborted)) alive = false;
-                    }
-                    if (!alive) { if (p.ctrl) { atomicExch(p.ctrl, kDevTimeout); atomicExch(p.ctrl + 1, 0xD1000000u | (unsigned)n); } st_release_cta(aborted, 1); break; }
+                // the slot's previous row (n - 16) must have been consumed by the tensor cores and, if the 3x3 part reads it, by
+                // the epilogue: rows 5 and 6 with output row 0, row q >= 7 with output row q - 7
+                alive = mbar_wait(rowdone0 + 8 * slot, (unsigned)(((n - NRING) / NRING) & 1), p.ctrl, 0xD0000000u | (unsigned)n);
+                const int need = n < NRING + 5 ? 0 : min(max(1, n - NRING - 6), L);
+                unsigned polls = 0;
+                while (alive && ld_acquire_cta(prog) < need) {
+                    __nanosleep(64);
+                    if (++polls > kPollLimit || ld_acquire_cta(aborted)) alive = false;
                 }
+                if (!alive) { if (p.ctrl) { atomicExch(p.ctrl, kDevTimeout); atomicExch(p.ctrl + 1, 0xD1000000u | (unsigned)n); } st_release_cta(aborted, 1); break; }
                 const uint32_t dst = smem_u32(ring + (size_t)slot * ROW_BYTES), bar = rowfull0 + 8 * slot;
                 mbar_expect_tx(bar, ROW_BYTES);
                 tma_load_4d(dst, &map_half, bar, 0, x0 - P6, ya - P6 + n, b);
@@ -239,20 +294,19 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
         const uint32_t ring_a = smem_u32(ring), btab_a = smem_u32(btab);
         for (int n = 0; n < n_in; ++n) {
             const int slot = n % NRING;
-            if (lane == 0) {
-                alive = mbar_wait(rowfull0 + 8 * slot, (unsigned)((n / NRING) & 1), p.ctrl, 0xD2000000u | (unsigned)n);
-                // the columns of the output row this input row opens (n, if it exists) were cleared by the epilogue of row n - 32
-                if (n >= SLOTS && n < L) {
-                    unsigned polls = 0;
-                    while (alive && ld_acquire_cta(prog) < n - SLOTS + 1) {
-                        __nanosleep(64);
-                        if (++polls > kPollLimit || ld_acquire_cta(aborted)) alive = false;
-                    }
+            alive = mbar_wait_warp(rowfull0 + 8 * slot, (unsigned)((n / NRING) & 1), p.ctrl, 0xD2000000u | (unsigned)n);
+            // the columns of the output row this input row opens (n, if it exists) were cleared by the epilogue of row n - 32
+            if (n >= SLOTS && n < L) {
+                unsigned polls = 0;
+                while (alive && __any_sync(0xffffffffu, ld_acquire_cta(prog) < n - SLOTS + 1)) {
+                    __nanosleep(64);
+                    if (++polls > kPollLimit || __any_sync(0xffffffffu, ld_acquire_cta(aborted))) alive = false;
                 }
-                if (!alive) { if (p.ctrl) { atomicExch(p.ctrl, kDevTimeout); atomicExch(p.ctrl + 1, 0xD3000000u | (unsigned)n); } st_release_cta(aborted, 1); }
             }
-            alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
-            if (!alive) break;
+            if (!alive) {
+                if (lane == 0) { if (p.ctrl) { atomicExch(p.ctrl, kDevTimeout); atomicExch(p.ctrl + 1, 0xD3000000u | (unsigned)n); } st_release_cta(aborted, 1); }
+                break;
+            }
             tc_fence_after();
             // input row n feeds output rows n - 12 + c, c = 0 .. 12 (kernel row 12 - c), those inside [0, L)
             const int c_lo = max(0, (K13 - 1) - n), c_hi = min(K13 - 1, L - 1 - n + (K13 - 1));
@@ -320,8 +374,53 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
         if (!p.wait_first) pdl_wait_primary();                               // dk comes from the kernel before this one
         for (int e = et; e < 9 * CG; e += kEpiThreads) dks[e] = __ldcg(p.dk + ((size_t)b * CG + (e % CG)) * 9 + e / CG);
         asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads) : "memory");
+        // the constant of this (image, channel), added to the accumulators
+        float c0[CG];
+#pragma unroll
+        for (int c = 0; c < CG; ++c) c0[c] = p.bias ? __ldcg(p.bias + (size_t)b * CG + c) : 0.f;
         bool alive = true;
         const int x = x0 + m;
+        // Dynamic 3x3 kernel, depth-wise, fp32 (Eq. 4 line 3, second term).  Output row yr reads input rows yr + 5 .. yr + 7
+        // of the ring, pixels m + 5 .. m + 7 of the staged row.  An input row is read once: it completes one output row and
+        // is added to the two that follow, whose sums wait in registers (shared-memory bandwidth is what the instructions
+        // live on: 10.7 KB per 104 cycles).
+        float d1[CG], d2[CG];                                                // output rows yr + 1, yr + 2 so far
+#pragma unroll
+        for (int c = 0; c < CG; ++c) d1[c] = d2[c] = 0.f;
+        auto add_row = [&](int n, float (&s0)[CG], float (&s1)[CG], float (&s2)[CG], int rows) {
+            // input row n into s0 (its kernel row 2), s1 (1), s2 (0); `rows` says which of the first two exist
+            const int rslot = n % NRING;
+            const unsigned char* rowp = ring + (size_t)rslot * ROW_BYTES;
+#pragma unroll
+            for (int bb = 0; bb < 3; ++bb) {
+                // the pixel's two 16-byte halves are swapped where bit 7 of its address is set (32-byte swizzle)
+                const int px = m + 5 + bb, sw = ((rslot * (ROW_BYTES / 128) + (px >> 2)) & 1) * 16;
+                const uint4 lo = *reinterpret_cast<const uint4*>(rowp + (size_t)px * 32 + sw);
+                const uint4 hi = *reinterpret_cast<const uint4*>(rowp + (size_t)px * 32 + (16 - sw));
+                float f[16];
+                unpack16<__nv_bfloat16>(lo, f);
+                unpack16<__nv_bfloat16>(hi, f + 8);
+                const float4* k2 = reinterpret_cast<const float4*>(dks + (6 + bb) * CG);
+                const float4* k1 = reinterpret_cast<const float4*>(dks + (3 + bb) * CG);
+                const float4* k0 = reinterpret_cast<const float4*>(dks + bb * CG);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (rows > 1) {
+                        const float4 d = k2[q];
+                        s0[4 * q] = fmaf(d.x, f[4 * q], s0[4 * q]); s0[4 * q + 1] = fmaf(d.y, f[4 * q + 1], s0[4 * q + 1]);
+                        s0[4 * q + 2] = fmaf(d.z, f[4 * q + 2], s0[4 * q + 2]); s0[4 * q + 3] = fmaf(d.w, f[4 * q + 3], s0[4 * q + 3]);
+                    }
+                    if (rows > 0) {
+                        const float4 d = k1[q];
+                        s1[4 * q] = fmaf(d.x, f[4 * q], s1[4 * q]); s1[4 * q + 1] = fmaf(d.y, f[4 * q + 1], s1[4 * q + 1]);
+                        s1[4 * q + 2] = fmaf(d.z, f[4 * q + 2], s1[4 * q + 2]); s1[4 * q + 3] = fmaf(d.w, f[4 * q + 3], s1[4 * q + 3]);
+                    }
+                    const float4 d = k0[q];
+                    s2[4 * q] = fmaf(d.x, f[4 * q], s2[4 * q]); s2[4 * q + 1] = fmaf(d.y, f[4 * q + 1], s2[4 * q + 1]);
+                    s2[4 * q + 2] = fmaf(d.z, f[4 * q + 2], s2[4 * q + 2]); s2[4 * q + 3] = fmaf(d.w, f[4 * q + 3], s2[4 * q + 3]);
+                }
+            }
+        };
         for (int yr = 0; yr < L; ++yr) {
             const int slot = yr % SLOTS;
             // one lane asks (a wait that all 32 lanes execute costs the warp over a hundred cycles)
@@ -332,35 +431,20 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
             uint32_t r[16];
             tmem_ld16(lane_base + (uint32_t)(slot * CG), r);
             tmem_zero16(lane_base + (uint32_t)(slot * CG));
+            float d0[CG];                                                    // this output row's 3x3 sums so far
+            if (yr == 0) {
+                float none[CG];
+#pragma unroll
+                for (int c = 0; c < CG; ++c) none[c] = 0.f;
+                add_row(5, none, none, d1, 0);
+                add_row(6, none, d1, d2, 1);
+            }
+#pragma unroll
+            for (int c = 0; c < CG; ++c) { d0[c] = d1[c]; d1[c] = d2[c]; d2[c] = 0.f; }
+            add_row(yr + 7, d0, d1, d2, 2);
             float acc[CG];
 #pragma unroll
-            for (int c = 0; c < CG; ++c) acc[c] = __uint_as_float(r[c]);
-            // dynamic 3x3 kernel, depth-wise, fp32 (Eq. 4 line 3, second term): input rows yr + 5 .. yr + 7 of the ring,
-            // pixels m + 5 .. m + 7 of the staged row
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const int rslot = (yr + 5 + a) % NRING;
-                const unsigned char* rowp = ring + (size_t)rslot * ROW_BYTES;
-#pragma unroll
-                for (int bb = 0; bb < 3; ++bb) {
-                    // the pixel's two 16-byte halves are swapped where bit 7 of its address is set (32-byte swizzle)
-                    const int px = m + 5 + bb, sw = ((rslot * (ROW_BYTES / 128) + (px >> 2)) & 1) * 16;
-                    const uint4 lo = *reinterpret_cast<const uint4*>(rowp + (size_t)px * 32 + sw);
-                    const uint4 hi = *reinterpret_cast<const uint4*>(rowp + (size_t)px * 32 + (16 - sw));
-                    float f[16];
-                    unpack16<__nv_bfloat16>(lo, f);
-                    unpack16<__nv_bfloat16>(hi, f + 8);
-                    const float4* d4 = reinterpret_cast<const float4*>(dks + (a * 3 + bb) * CG);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float4 d = d4[q];
-                        acc[4 * q] = fmaf(d.x, f[4 * q], acc[4 * q]);
-                        acc[4 * q + 1] = fmaf(d.y, f[4 * q + 1], acc[4 * q + 1]);
-                        acc[4 * q + 2] = fmaf(d.z, f[4 * q + 2], acc[4 * q + 2]);
-                        acc[4 * q + 3] = fmaf(d.w, f[4 * q + 3], acc[4 * q + 3]);
-                    }
-                }
-            }
+            for (int c = 0; c < CG; ++c) acc[c] = __uint_as_float(r[c]) + (d0[c] + c0[c]);
             if (x < p.W) {
                 uint32_t o[8];
 #pragma unroll
@@ -390,8 +474,8 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
 // [B][H][W][C] bf16 as a 4-D map {C, W, H, B} with a box of 8 channels x SPX pixels x 1 row.
 inline int try_launch_dense_umma(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x,
                                  const void* w_dense, const float* dk, void* out, unsigned* ctrl, cudaStream_t st,
-                                 bool dependent, int* launches, std::string* err) {
-    if (K != K13 || dtype != 1 /*bf16*/ || layout != kNHWC || Ca != CG || C % 8 != 0) return kNotApplicable;
+                                 bool dependent, int* launches, std::string* err, const float* bias = nullptr, bool flip = false) {
+    if (K > K13 || dtype != 1 /*bf16*/ || layout != kNHWC || Ca != CG || C % 8 != 0) return kNotApplicable;
     if ((reinterpret_cast<uintptr_t>(w_dense) & 1) != 0) return kNotApplicable;
     const int sms = sm_count();
     if (sms <= 0) return kNotApplicable;
@@ -410,7 +494,8 @@ inline int try_launch_dense_umma(int B, int C, int Ca, int H, int W, int K, int 
     p.w_dense = static_cast<const __nv_bfloat16*>(w_dense);
     p.dk = dk; p.out = static_cast<__nv_bfloat16*>(out); p.ctrl = ctrl;
     p.wait_first = dependent ? 0 : 1;
-    p.w_aligned = (reinterpret_cast<uintptr_t>(w_dense) & 15) == 0 ? 1 : 0;
+    p.raw_bulk = (reinterpret_cast<uintptr_t>(w_dense) & 15) == 0 ? 1 : 0;
+    p.KK = K; p.flip = flip ? 1 : 0; p.bias = bias;
     const int cc = C - Ca;
     p.copy_cc = cc; p.copy_pw = 0;
     if (cc > 256) return kNotApplicable;

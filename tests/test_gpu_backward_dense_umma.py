@@ -38,6 +38,46 @@ CASES = [
 ]
 
 
+@pytest.mark.parametrize("K", [3, 9, 11, 13])
+@pytest.mark.parametrize("misaligned", [False, True])
+def test_tcgen05_stencil_of_any_size_both_ways(pkg, oracle, K, misaligned):
+    """The tcgen05 stencil kernel with a kernel smaller than 13x13 in the middle of zeros, weights that are not 16-byte aligned
+    (staged another way), and the gradient's form (channels swapped, taps rotated, constants added): forward and grad_x, more
+    rows per block than the ring and the row slots hold."""
+    import torch
+
+    B, C, C_a, H, W = 70, 24, 16, 45, 20
+    d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=K, per_image_scale=True, channel_means=True)
+    wdn = synth.make_dense_kernel(C_a, K, synth.BF16, seed=K)
+    go = synth.round_to(np.random.default_rng(K).standard_normal(size=d["x"].shape).astype(np.float32), synth.BF16)
+    x, god = util.to_device(d["x"], synth.BF16, synth.NHWC), util.to_device(go, synth.BF16, synth.NHWC)
+    _, wd, bd = util.weights_to_device(d, synth.BF16)
+    store = torch.zeros(wdn.size + 8, dtype=torch.bfloat16, device="cuda")
+    wdd = store[1:1 + wdn.size] if misaligned else store[:wdn.size]
+    wdd.copy_(torch.from_numpy(wdn).reshape(-1))
+    wdd = wdd.view(wdn.shape)
+    out, gx = torch.full_like(x, 7.0), torch.full_like(x, 7.0)
+    ws = pkg.new_workspace(B, C_a, H, W, K)
+    pkg.esc_convattn_forward_dense(x, C_a, K, wdd, wd, bd, out, pkg.ESC_NHWC, ws)
+    assert pkg.esc_convattn_last_path() == 5
+    wsb = pkg.new_backward_dense_workspace(B, C_a, H, W, K)
+    pkg.esc_convattn_backward_dense(x, god, C_a, K, wdd, wd, bd, gx, None, None, None, pkg.ESC_NHWC, wsb)
+    torch.cuda.synchronize()
+    assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_device_status(wsb) == 0
+    ref, mag = oracle.forward_dense(d["x"], C_a, wdn, d["w_dyn"], d["b_dyn"], want_mag=True)
+    got = util.to_host_nchw(out, synth.NHWC)
+    err = np.abs(got[:, :C_a] - ref[:, :C_a])
+    bar = 2.0 ** -8 * np.abs(ref[:, :C_a]) * 1.001 + 5e-5 * mag + 1e-30      # one rounding, tensor-core accumulation
+    assert (err <= bar).all() and np.array_equal(got[:, C_a:], ref[:, C_a:])
+    n = 6                                                   # images of the gradient that are compared
+    rx = oracle.backward_dense(d["x"][:n], go[:n], C_a, wdn, d["w_dyn"], d["b_dyn"])[0]
+    ax = oracle.backward_dense(np.abs(d["x"][:n]), np.abs(go[:n]), C_a, np.abs(wdn), np.abs(d["w_dyn"]), np.abs(d["b_dyn"]))[0]
+    got = util.to_host_nchw(gx, synth.NHWC)[:n]
+    err = np.abs(got[:, :C_a] - rx[:, :C_a])
+    assert (err <= 2.0 ** -8 * np.abs(rx[:, :C_a]) * 1.001 + 5e-5 * ax[:, :C_a] + 1e-30).all()
+    assert np.array_equal(got[:, C_a:], go[:n, C_a:].astype(np.float64))
+
+
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c)))
 def test_dense_weight_gradient(pkg, oracle, case):
     import torch
