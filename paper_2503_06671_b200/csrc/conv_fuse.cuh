@@ -323,9 +323,9 @@ inline bool applies(int C, int Ca, long long HW, int dtype, int layout, const vo
            al(residual) && al(w);
 }
 
-// `early`: the kernel may start, and read w, while the kernel before it in the stream still runs (w must then be older than that kernel)
+// The kernel may start, and read w, while the kernel before it in the stream still runs (w must be older than that kernel).
 template <int C>
-inline cudaError_t launch_c(const Params& p, cudaStream_t st, bool early) {
+inline cudaError_t launch_c(const Params& p, cudaStream_t st) {
     const size_t smem = (size_t)3 * 2 * C * kPitchN;
     static bool attr_set[tma::kMaxDevices] = {};
     const int dev = tma::current_device();
@@ -345,14 +345,14 @@ inline cudaError_t launch_c(const Params& p, cudaStream_t st, bool early) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = early ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, conv_fuse_nchw_bf16<C>, p);
 }
-inline cudaError_t launch(const Params& p, cudaStream_t st, bool early = true) {
+inline cudaError_t launch(const Params& p, cudaStream_t st) {
     switch (p.C) {
-        case 32: return launch_c<32>(p, st, early);
-        case 48: return launch_c<48>(p, st, early);
-        case 64: return launch_c<64>(p, st, early);
+        case 32: return launch_c<32>(p, st);
+        case 48: return launch_c<48>(p, st);
+        case 64: return launch_c<64>(p, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -397,7 +397,7 @@ inline bool fast_applies(int C, int Ca, int dtype, int layout) {
 }
 
 template <int C>
-inline cudaError_t launch_fast_c(const Params& p, cudaStream_t st, bool early) {
+inline cudaError_t launch_fast_c(const Params& p, cudaStream_t st) {
     constexpr int PITCH = C * 2 + 16;
     const size_t smem = (size_t)(2 * Stages<C>::N * kPix + (C <= 64 ? 0 : C)) * PITCH;   // stages of (cat, residual); w_fuse where it is not in registers
     static bool attr_set[tma::kMaxDevices] = {};
@@ -418,17 +418,17 @@ inline cudaError_t launch_fast_c(const Params& p, cudaStream_t st, bool early) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = early ? 1 : 0;
+    cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, conv_fuse_nhwc_bf16<C>, p);
 }
 
-inline cudaError_t launch_fast(const Params& p, cudaStream_t st, bool early = true) {
+inline cudaError_t launch_fast(const Params& p, cudaStream_t st) {
     switch (p.C) {
-        case 32: return launch_fast_c<32>(p, st, early);
-        case 48: return launch_fast_c<48>(p, st, early);
-        case 64: return launch_fast_c<64>(p, st, early);
-        case 96: return launch_fast_c<96>(p, st, early);
-        case 128: return launch_fast_c<128>(p, st, early);
+        case 32: return launch_fast_c<32>(p, st);
+        case 48: return launch_fast_c<48>(p, st);
+        case 64: return launch_fast_c<64>(p, st);
+        case 96: return launch_fast_c<96>(p, st);
+        case 128: return launch_fast_c<128>(p, st);
         default: return cudaErrorInvalidValue;
     }
 }

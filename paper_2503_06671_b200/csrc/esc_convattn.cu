@@ -855,7 +855,6 @@ int launch_fuse_fp32(const Problem& p, const void* att, const void* idt, const v
 
 // ---- backward pass of Conv_fuse -------------------------------------------------------------------------------
 struct FuseBackwardWs {
-    void* wt;                        // W_fuse transposed, element type of the tensors
     float* part;                     // [blocks][C * C + C]
     int passes, blocks;              // tensor-core kernels
     int passes32, blocks32;          // wgrad_fp32
@@ -873,7 +872,6 @@ FuseBackwardWs carve_fuse_backward(void* ws, int C, long long pixels) {
     w.blocks32 = (int)((runs32 + w.passes32 - 1) / w.passes32);
     char* base = static_cast<char*>(ws);
     size_t off = 0;
-    w.wt = base + off;                              off += round_up((size_t)C * C * 4, 256);
     w.part = reinterpret_cast<float*>(base + off);  off += round_up((size_t)std::max(w.blocks, w.blocks32) * ((size_t)C * C + C) * 4, 256);
     w.bytes = off;
     return w;
@@ -895,65 +893,43 @@ int fuse_wgrad_c(const void* cat, const void* go, long long HW, long long pixels
     ++g_last_launches;
     return ESC_OK;
 }
-template <int C>
-int fuse_wgrad_mma_c(const void* cat, const void* go, long long pixels, const FuseBackwardWs& w, cudaStream_t st) {
-    namespace M = esc::fuse::bwd::mma;
-    static bool attr_set[esc::tma::kMaxDevices] = {};
-    const int dev = esc::tma::current_device();
-    if (dev < 0) return ESC_ERR_UNSUPPORTED;
-    if (!attr_set[dev]) {
-        ESC_CUDA(cudaFuncSetAttribute(M::wgrad_bf16_nhwc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::MGeom<C>::kSmemBytes));
-        attr_set[dev] = true;
-    }
-    M::wgrad_bf16_nhwc<C><<<(unsigned)w.blocks, esc::fuse::bwd::kThreads, M::MGeom<C>::kSmemBytes, st>>>(
-        static_cast<const __nv_bfloat16*>(cat), static_cast<const __nv_bfloat16*>(go), pixels, w.passes, w.part);
-    ESC_CUDA(cudaGetLastError());
-    ++g_last_launches;
-    return ESC_OK;
-}
-
-template <int C>
-int fuse_wgrad_mma_nchw_c(const void* cat, const void* go, long long HW, long long pixels, const FuseBackwardWs& w, cudaStream_t st) {
-    namespace M = esc::fuse::bwd::mma;
-    static bool attr_set[esc::tma::kMaxDevices] = {};
-    const int dev = esc::tma::current_device();
-    if (dev < 0) return ESC_ERR_UNSUPPORTED;
-    if (!attr_set[dev]) {
-        ESC_CUDA(cudaFuncSetAttribute(M::wgrad_bf16_nchw<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::NGeom<C>::kSmemBytes));
-        attr_set[dev] = true;
-    }
-    M::wgrad_bf16_nchw<C><<<(unsigned)w.blocks, esc::fuse::bwd::kThreads, M::NGeom<C>::kSmemBytes, st>>>(
-        static_cast<const __nv_bfloat16*>(cat), static_cast<const __nv_bfloat16*>(go), HW, pixels, w.passes, w.part);
-    ESC_CUDA(cudaGetLastError());
-    ++g_last_launches;
-    return ESC_OK;
-}
-
 template <typename T, int LAYOUT>
-int fuse_wgrad_t(int C, const void* cat, const void* go, long long HW, long long pixels, const FuseBackwardWs& w, int* blocks, cudaStream_t st) {
-    *blocks = w.blocks;
-    if (std::is_same<T, __nv_bfloat16>::value && LAYOUT == esc::kNCHW && HW % 8 == 0 && g_engine_policy != ESC_ENGINE_FP32) {
-        // bf16 NCHW with whole 16-byte pieces per image: the same matrix product, operands without transposition
-        switch (C) {
-            case 32: return fuse_wgrad_mma_nchw_c<32>(cat, go, HW, pixels, w, st);
-            case 48: return fuse_wgrad_mma_nchw_c<48>(cat, go, HW, pixels, w, st);
-            case 64: return fuse_wgrad_mma_nchw_c<64>(cat, go, HW, pixels, w, st);
-        }
-    }
-    if (std::is_same<T, __nv_bfloat16>::value && LAYOUT == esc::kNHWC && g_engine_policy != ESC_ENGINE_FP32) {
-        // bf16 NHWC: one matrix product over the pixels on the tensor cores
-        switch (C) {
-            case 32: return fuse_wgrad_mma_c<32>(cat, go, pixels, w, st);
-            case 48: return fuse_wgrad_mma_c<48>(cat, go, pixels, w, st);
-            case 64: return fuse_wgrad_mma_c<64>(cat, go, pixels, w, st);
-        }
-    }
-    *blocks = w.blocks32;
+int fuse_wgrad_t(int C, const void* cat, const void* go, long long HW, long long pixels, const FuseBackwardWs& w, cudaStream_t st) {
     switch (C) {
         case 16: return fuse_wgrad_c<T, LAYOUT, 16>(cat, go, HW, pixels, w, st);
         case 32: return fuse_wgrad_c<T, LAYOUT, 32>(cat, go, HW, pixels, w, st);
         case 48: return fuse_wgrad_c<T, LAYOUT, 48>(cat, go, HW, pixels, w, st);
         case 64: return fuse_wgrad_c<T, LAYOUT, 64>(cat, go, HW, pixels, w, st);
+    }
+    return ESC_ERR_UNSUPPORTED;
+}
+
+// All three gradients in one pass on the tensor cores; `sums`: whether g_W or g_b is wanted.
+template <int LAYOUT, int C>
+int fuse_backward_mma_c(const void* cat, const void* go, const void* w_fuse, void* g_cat, long long HW, long long pixels,
+                        const FuseBackwardWs& w, bool sums, cudaStream_t st) {
+    namespace M = esc::fuse::bwd::mma;
+    static bool attr_set[esc::tma::kMaxDevices] = {};
+    const int dev = esc::tma::current_device();
+    if (dev < 0) return ESC_ERR_UNSUPPORTED;
+    if (!attr_set[dev]) {
+        ESC_CUDA(cudaFuncSetAttribute(M::fuse_backward_bf16<LAYOUT, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::MGeom<LAYOUT, C>::kSmemBytes));
+        attr_set[dev] = true;
+    }
+    M::fuse_backward_bf16<LAYOUT, C><<<(unsigned)w.blocks, esc::fuse::bwd::kThreads, M::MGeom<LAYOUT, C>::kSmemBytes, st>>>(
+        static_cast<const __nv_bfloat16*>(cat), static_cast<const __nv_bfloat16*>(go), static_cast<const __nv_bfloat16*>(w_fuse),
+        static_cast<__nv_bfloat16*>(g_cat), HW, pixels, w.passes, sums ? w.part : nullptr);
+    ESC_CUDA(cudaGetLastError());
+    ++g_last_launches;
+    return ESC_OK;
+}
+template <int LAYOUT>
+int fuse_backward_mma_t(int C, const void* cat, const void* go, const void* w_fuse, void* g_cat, long long HW, long long pixels,
+                        const FuseBackwardWs& w, bool sums, cudaStream_t st) {
+    switch (C) {
+        case 32: return fuse_backward_mma_c<LAYOUT, 32>(cat, go, w_fuse, g_cat, HW, pixels, w, sums, st);
+        case 48: return fuse_backward_mma_c<LAYOUT, 48>(cat, go, w_fuse, g_cat, HW, pixels, w, sums, st);
+        case 64: return fuse_backward_mma_c<LAYOUT, 64>(cat, go, w_fuse, g_cat, HW, pixels, w, sums, st);
     }
     return ESC_ERR_UNSUPPORTED;
 }
@@ -1577,52 +1553,32 @@ int esc_conv_fuse_backward(const void* cat, const void* grad_out, int B, int C, 
     const FuseBackwardWs w = carve_fuse_backward(workspace, C, pixels);
     if (workspace_bytes_ < w.bytes) return ESC_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the weight's and the bias's gradients
-    if (grad_w_fuse || grad_b_fuse) {
-        int blocks = 0;
-        if (dtype == ESC_F32)
-            rc = layout == ESC_NCHW ? fuse_wgrad_t<float, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, &blocks, st)
-                                    : fuse_wgrad_t<float, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, &blocks, st);
-        else
-            rc = layout == ESC_NCHW ? fuse_wgrad_t<__nv_bfloat16, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, &blocks, st)
-                                    : fuse_wgrad_t<__nv_bfloat16, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, &blocks, st);
-        if (rc != ESC_OK) return rc;
-        const int elems = C * C + C;
-        esc::fuse::bwd::sum_wgrad<<<(unsigned)((elems + 7) / 8), 256, 0, st>>>(w.part, C, blocks, grad_w_fuse, grad_b_fuse);
-        ESC_CUDA(cudaGetLastError());
-        ++g_last_launches;
+    const bool sums = grad_w_fuse || grad_b_fuse;
+    int blocks = w.blocks32;
+    if (esc::fuse::bwd::mma::applies(C, HW, dtype, layout, w_fuse) && g_engine_policy != ESC_ENGINE_FP32) {
+        blocks = w.blocks;
+        rc = layout == ESC_NCHW ? fuse_backward_mma_t<esc::kNCHW>(C, cat, grad_out, w_fuse, grad_cat, HW, pixels, w, sums, st)
+                                : fuse_backward_mma_t<esc::kNHWC>(C, cat, grad_out, w_fuse, grad_cat, HW, pixels, w, sums, st);
+    } else {
+        if (sums) {
+            if (dtype == ESC_F32)
+                rc = layout == ESC_NCHW ? fuse_wgrad_t<float, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, st)
+                                        : fuse_wgrad_t<float, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, st);
+            else
+                rc = layout == ESC_NCHW ? fuse_wgrad_t<__nv_bfloat16, esc::kNCHW>(C, cat, grad_out, HW, pixels, w, st)
+                                        : fuse_wgrad_t<__nv_bfloat16, esc::kNHWC>(C, cat, grad_out, HW, pixels, w, st);
+            if (rc != ESC_OK) return rc;
+        }
+        // grad_cat = W_fuse^T grad_out per pixel: the 1x1 kernel with the matrix read transposed, no bias, no residual
+        rc = dtype == ESC_F32 ? launch_fuse_fp32<float, true>(p, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st)
+                              : launch_fuse_fp32<__nv_bfloat16, true>(p, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st);
     }
-    // grad_cat = W_fuse^T grad_out per pixel: the forward's 1x1 kernels with the transposed matrix, no bias, no residual
-    const bool nhwc = esc::fuse::fast_applies(C, 8, dtype, layout);
-    if (nhwc || esc::fuse::nchw::applies(C, 8, HW, dtype, layout, grad_out, grad_cat, nullptr, w.wt)) {
-        const unsigned tb = (unsigned)((C * C + 255) / 256);
-        esc::fuse::bwd::transpose_w<__nv_bfloat16><<<tb, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(w_fuse), C, static_cast<__nv_bfloat16*>(w.wt));
-        ESC_CUDA(cudaGetLastError());
-        ++g_last_launches;
-    }
-    if (nhwc) {
-        esc::fuse::Params fp;
-        fp.att = static_cast<const __nv_bfloat16*>(grad_out); fp.idt = static_cast<const __nv_bfloat16*>(grad_out);
-        fp.w = static_cast<const __nv_bfloat16*>(w.wt); fp.bias = nullptr; fp.residual = nullptr;
-        fp.out = static_cast<__nv_bfloat16*>(grad_cat);
-        fp.pixels = pixels; fp.C = C; fp.Ca = 8;
-        ESC_CUDA(esc::fuse::launch_fast(fp, st, /*early=*/false));   // its matrix was written by the kernel before it
-        ++g_last_launches;
-        return ESC_OK;
-    }
-    if (esc::fuse::nchw::applies(C, 8, HW, dtype, layout, grad_out, grad_cat, nullptr, w.wt)) {
-        esc::fuse::nchw::Params fp;
-        fp.att = static_cast<const __nv_bfloat16*>(grad_out); fp.idt = static_cast<const __nv_bfloat16*>(grad_out);
-        fp.w = static_cast<const __nv_bfloat16*>(w.wt); fp.bias = nullptr; fp.residual = nullptr;
-        fp.out = static_cast<__nv_bfloat16*>(grad_cat);
-        fp.HW = HW; fp.B = B; fp.C = C; fp.Ca = 8;
-        ESC_CUDA(esc::fuse::nchw::launch(fp, st, /*early=*/false));
-        ++g_last_launches;
-        return ESC_OK;
-    }
-    const Problem pc{B, C, C, H, W, 3, dtype, layout};
-    return dtype == ESC_F32 ? launch_fuse_fp32<float, true>(pc, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st)
-                            : launch_fuse_fp32<__nv_bfloat16, true>(pc, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st);
+    if (rc != ESC_OK || !sums) return rc;
+    const int elems = C * C + C;
+    esc::fuse::bwd::sum_wgrad<<<(unsigned)((elems + 31) / 32), 256, 0, st>>>(w.part, C, blocks, grad_w_fuse, grad_b_fuse);
+    ESC_CUDA(cudaGetLastError());
+    ++g_last_launches;
+    return ESC_OK;
 }
 
 int esc_convattn_selftest_bounded_wait(void* workspace, void* stream) {
