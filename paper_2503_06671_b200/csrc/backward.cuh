@@ -3,11 +3,11 @@
 //
 //   g_tap[b,c,i,j] = sum_{y,x} go[b,c,y,x] * x~[b,c,y+i-6,x+j-6]      per-image tap gradient  (kernel tap_grad)
 //   g_lk = sum_b g_tap;   g_dk = central 3x3 of g_tap;   g_b = sum_b g_dk;   g_W[o,k] = sum_b g_dk[b,o] g[b,k]
-//   g_g[b,k] = sum_o W[o,k] g_dk[b,o]                                                        (kernel finish)
+//   g_g[b,k] = sum_o W[o,k] g_dk[b,o]                                          (estimator_image, estimator_weights)
 //   g_x[b,c] = go[b,c] (*) flip(Wm[b,c]) + g_g[b,c] / (H W)   (c < C_a),   g_x[b,c] = go[b,c]  (c >= C_a)
 //
 // The last line is the forward stencil applied to go with both kernels rotated by 180 degrees and a
-// per-(image, channel) constant added, so it runs on the forward kernels; `finish` prepares the rotated
+// per-(image, channel) constant added, so it runs on the forward kernels; `estimator_image` prepares the rotated
 // kernels and the constants for it.  Every reduction is done in a fixed order: results are reproducible.
 #pragma once
 #include "common.cuh"
@@ -251,11 +251,13 @@ sum_tiles(const float* __restrict__ part, int tiles, float* __restrict__ gtap)  
     __shared__ float acc[kSumGroups][192];
     const size_t bc = blockIdx.x;
     const int t = threadIdx.x % 192, grp = threadIdx.x / 192;
+    pdl_launch_dependents();
+    pdl_wait_primary();
     if (t <= TAPS) {
         const float* p = part + bc * tiles * kSlot + t;
         float s = 0.f;
 #pragma unroll 8
-        for (int k = grp; k < tiles; k += kSumGroups) s += p[(size_t)k * kSlot];
+        for (int k = grp; k < tiles; k += kSumGroups) s += __ldcg(p + (size_t)k * kSlot);
         acc[grp][t] = s;
     }
     __syncthreads();
@@ -267,86 +269,10 @@ sum_tiles(const float* __restrict__ part, int tiles, float* __restrict__ gtap)  
     }
 }
 
-// ---- kernel 2b: everything small; every output element is independent, a few blocks share them ------------
-// From g_tap [B][Ca][169 + sum x]: g_lk, g_b, g_W (fp32 outputs), and for the stencil pass that follows the
-// kernels rotated by 180 degrees -- w_flip (element type T), dk_flip [B][Ca][9] -- and the constants
-// bias[b][c] = g_g[b,c] / (H W).  g[b,k] = sum x / (H W) and dk = b_dyn + W g are recomputed here.
-constexpr int kFinishRoles = 6, kFinishBlocks = 32 * kFinishRoles;
-template <typename T>
-__global__ void __launch_bounds__(256)
-finish(const float* __restrict__ gtap, int B, int Ca, int H, int W, int KK, const T* __restrict__ w_large,
-       const T* __restrict__ w_dyn, const T* __restrict__ b_dyn, float* __restrict__ g_lk, float* __restrict__ g_w,
-       float* __restrict__ g_b, T* __restrict__ w_flip, float* __restrict__ dk_flip, float* __restrict__ bias)
-{
-    // Six independent jobs; each takes a sixth of the grid, so that their chains of dependent loads run side by side
-    // instead of one after the other in every thread.
-    const int per_role = gridDim.x / kFinishRoles, role = blockIdx.x / per_role;
-    const int tid = (blockIdx.x % per_role) * blockDim.x + threadIdx.x, nth = per_role * blockDim.x;
-    const float inv_hw = 1.0f / ((float)H * (float)W);
-    auto gdk = [&](int b, int o) {                        // o = c*9 + i*3 + j -> central 3x3 of the tap gradient
-        const int c = o / 9, i = (o % 9) / 3, j = o % 3;
-        return gtap[((size_t)b * Ca + c) * kSlot + (i + P - 1) * K + (j + P - 1)];
-    };
-    auto gmean = [&](int b, int k) { return gtap[((size_t)b * Ca + k) * kSlot + TAPS] * inv_hw; };
-    // A large kernel of size KK < 13 sits in the middle of the 13 x 13 taps whose gradients gtap holds.
-    const int off = (K - KK) / 2, taps = KK * KK;
-    if (role == 0 && g_lk)
-        for (int e = tid; e < Ca * taps; e += nth) {
-            const int c = e / taps, t = (e % taps) / KK + off, u = (e % taps) % KK + off;
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s += gtap[((size_t)b * Ca + c) * kSlot + t * K + u];
-            g_lk[e] = s;
-        }
-    if (role == 1 && g_b)
-        for (int o = tid; o < 9 * Ca; o += nth) {
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s += gdk(b, o);
-            g_b[o] = s;
-        }
-    if (role == 2 && g_w)
-        for (int e = tid; e < 9 * Ca * Ca; e += nth) {
-            const int o = e / Ca, k = e % Ca;
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s = fmaf(gdk(b, o), gmean(b, k), s);
-            g_w[e] = s;
-        }
-    if (role == 3)
-    for (int e = tid; e < Ca * taps; e += nth) {
-        const int c = e / taps, t = e % taps;
-        w_flip[(size_t)c * taps + (taps - 1 - t)] = w_large[e];
-    }
-    if (role == 4)
-    for (int e = tid; e < B * Ca * 9; e += nth) {
-        const int b = e / (9 * Ca), o = e % (9 * Ca), c = o / 9, t = o % 9;
-        float s = Elem<T>::to_f32(b_dyn[o]);
-#pragma unroll 8
-        for (int k = 0; k < Ca; ++k) s = fmaf(Elem<T>::to_f32(w_dyn[(size_t)o * Ca + k]), gmean(b, k), s);
-        dk_flip[((size_t)b * Ca + c) * 9 + (8 - t)] = s;
-    }
-    if (role == 5) {
-        // bias[b][k] = sum_o W[o][k] g_dk[b][o] / (H W): a warp per element, lane = channel c (nine taps each, all loads
-        // independent), then a fixed butterfly over the lanes
-        const int lane = threadIdx.x & 31, wid = tid >> 5, nw = nth >> 5;
-        for (int e = wid; e < B * Ca; e += nw) {
-            const int b = e / Ca, k = e % Ca;
-            float s = 0.f;
-            for (int c = lane; c < Ca; c += 32) {
-                const float* gt = gtap + ((size_t)b * Ca + c) * kSlot + (P - 1) * K + (P - 1);
-#pragma unroll
-                for (int ij = 0; ij < 9; ++ij)
-                    s = fmaf(Elem<T>::to_f32(w_dyn[(size_t)(c * 9 + ij) * Ca + k]), gt[(ij / 3) * K + ij % 3], s);
-            }
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) bias[e] = s * inv_hw;
-        }
-    }
-}
-
-// ---- the estimator as Eq. 4 line 2 writes it: two layers with the exact GELU between them ---------------------
+// ---- the estimator's part -----------------------------------------------------------------------------------------
+// One linear layer (hidden == 0): g = pooled means, dk = b_last + W g;  g_W[o,k] = sum_b g_dk[b,o] g[b,k],  g_b = sum_b g_dk,
+//   g_g[b,k] = sum_o W[o,k] g_dk[b,o].
+// Two layers with the exact GELU between them, as Eq. 4 line 2 writes it:
 //   t = W_down g + b_down,  a = phi(t),  dk = W_up a + b_up;   phi'(t) = Phi(t) + t n(t)
 //   g_a[b,m] = sum_o W_up[o,m] g_dk[b,o],   g_t = g_a * phi'(t),   g_g[b,k] = sum_m W_down[m,k] g_t[b,m]
 //   g_b_up = sum_b g_dk,  g_W_up[o,m] = sum_b g_dk[b,o] a[b,m],  g_b_down = sum_b g_t,  g_W_down[m,k] = sum_b g_t[b,m] g[b,k]
@@ -354,116 +280,169 @@ __device__ __forceinline__ float gelu_exact_prime(float t) {
     return 0.5f * erfcf(-0.70710678118654752f * t) + t * 0.3989422804014327f * expf(-0.5f * t * t);
 }
 
-// kernel 2c: one block per image -- the estimator's forward values and the part of the chain that belongs to one
-// image: a and g_t go to the workspace for the sums over images, dk (rotated) and the GAP-path constant to the
-// stencil pass that follows.  Dynamic shared memory: (10 Ca + 3 hidden) floats.
+// Tap gradients as [B*Ca][tiles][kSlot]: tiles == 1 is sum_tiles' result.  With few tiles the kernels below add them up
+// themselves, which is a launch less (64 patches of 64x64: sum_tiles took 6.5 us).
+constexpr int kDirectTiles = 16;
+struct Taps {
+    const float* p;
+    int tiles;
+    __device__ __forceinline__ float operator()(size_t bc, int slot) const {
+        const float* q = p + bc * tiles * kSlot + slot;
+        float s = 0.f;
+#pragma unroll 4
+        for (int t = 0; t < tiles; ++t) s += __ldcg(q + (size_t)t * kSlot);
+        return s;
+    }
+};
+// Per-image values for the sums over images: g_dk [B][9 Ca], pooled means [B][Ca], activations and g_t [B][hidden].
+struct ImageValues { float *gdk, *mean, *act, *gt; };
+
+// kernel 2b: block b < B is one image: its pooled means and g_dk, the estimator's forward values and the part of the chain that
+// belongs to one image; dk (rotated) and the GAP-path constant go to the stencil pass that follows.  The blocks behind them take
+// g_lk = sum_b g_tap, 32 consecutive taps each (the lanes), images dealt to the eight warps and the warps added in order, and
+// the last kFlipBlocks the rotated LK.  Bound: latency of a few dependent phases.  Every sum that is longer than a few terms is
+// taken by a warp and nothing waits for sum_tiles where there are few tiles: 64 patches of 64x64 with two layers took 6.5 (sum_tiles)
+// + 8.3 + 22 us cold, the last one a thread per output over 64 images; 8 + 4.6 us now, overlapping their neighbours.
+constexpr int kFlipBlocks = 8, kEstThreads = 256, kEstMaxCa = 1024;
 template <typename T>
-__global__ void __launch_bounds__(256)
-mlp_image(const float* __restrict__ gtap, int Ca, int hidden, int H, int W, const T* __restrict__ w_down,
-          const T* __restrict__ b_down, const T* __restrict__ w_up, const T* __restrict__ b_up,
-          float* __restrict__ act, float* __restrict__ gt, float* __restrict__ dk_flip, float* __restrict__ bias)
+__global__ void __launch_bounds__(kEstThreads)
+estimator_image(const Taps taps, const float* __restrict__ xs_part, int chunks, int B, int Ca, int hidden, int H, int W, int KK,
+                const T* __restrict__ w_large, const T* __restrict__ w_down, const T* __restrict__ b_down,
+                const T* __restrict__ w_last, const T* __restrict__ b_last, const ImageValues iv, float* __restrict__ dk_flip,
+                float* __restrict__ bias, float* __restrict__ g_lk, T* __restrict__ w_flip)
 {
     extern __shared__ float sm[];
-    float* gm = sm;                    // [Ca] pooled means
-    float* gd = gm + Ca;               // [9 Ca] g_dk of this image
-    float* tt = gd + 9 * Ca;           // [hidden] pre-activations
-    float* aa = tt + hidden;           // [hidden] activations
+    __shared__ float red[kEstThreads];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ltaps = KK * KK;
+    pdl_launch_dependents();
+    pdl_wait_primary();
+    if (blockIdx.x >= (unsigned)B) {
+        const int job = blockIdx.x - B, lk_blocks = g_lk ? (Ca * ltaps + 31) / 32 : 0;
+        if (job < lk_blocks) {
+            const int e = job * 32 + lane, off = (K - KK) / 2;   // a smaller large kernel sits in the middle of the 13 x 13 taps
+            float s = 0.f;
+            if (e < Ca * ltaps) {
+                const int c = e / ltaps, t = (e % ltaps) / KK + off, u = (e % ltaps) % KK + off;
+#pragma unroll 4
+                for (int b = warp; b < B; b += kEstThreads / 32) s += taps((size_t)b * Ca + c, t * K + u);
+            }
+            red[tid] = s;
+            __syncthreads();
+            if (warp == 0 && e < Ca * ltaps) {
+                for (int w = 1; w < kEstThreads / 32; ++w) s += red[w * 32 + lane];
+                g_lk[e] = s;
+            }
+        } else if (w_flip) {
+            for (int e = (job - lk_blocks) * kEstThreads + tid; e < Ca * ltaps; e += kFlipBlocks * kEstThreads)
+                w_flip[(size_t)(e / ltaps) * ltaps + (ltaps - 1 - e % ltaps)] = w_large[e];
+        }
+        return;
+    }
+    const int b = blockIdx.x;
+    // [Ca] pooled means, [9 Ca] g_dk of this image: in shared memory, or where they go anyway if C_a is too large for it
+    float* aa = sm;                    // [hidden] activations
     float* gs = aa + hidden;           // [hidden] g_t
-    const int b = blockIdx.x, tid = threadIdx.x, nth = blockDim.x;
+    float* gm = Ca <= kEstMaxCa ? gs + hidden : iv.mean + (size_t)b * Ca;
+    float* gd = Ca <= kEstMaxCa ? gm + Ca : iv.gdk + (size_t)b * 9 * Ca;
     const float inv_hw = 1.0f / ((float)H * (float)W);
-    for (int k = tid; k < Ca; k += nth) gm[k] = gtap[((size_t)b * Ca + k) * kSlot + TAPS] * inv_hw;
-    for (int o = tid; o < 9 * Ca; o += nth) {
+    if (xs_part) {
+        // decomposed form: the taps saw the mixed features, the pooled means are those of x: chunks of pixels, dealt to groups of
+        // Ca threads, the groups added in order
+        const int ng = kEstThreads / Ca, k = tid % Ca, j = tid / Ca;
+        float s = 0.f;
+        if (j < ng) {
+#pragma unroll 8
+            for (int c = j; c < chunks; c += ng) s += __ldcg(xs_part + ((size_t)b * chunks + c) * Ca + k);
+        }
+        red[tid] = s;
+        __syncthreads();
+        if (tid < Ca) {
+            for (int g = 1; g < ng; ++g) s += red[g * Ca + tid];
+            gm[tid] = s * inv_hw;
+        }
+    } else {
+        for (int k = tid; k < Ca; k += kEstThreads) gm[k] = taps((size_t)b * Ca + k, TAPS) * inv_hw;
+    }
+    for (int o = tid; o < 9 * Ca; o += kEstThreads) {             // o = c*9 + i*3 + j -> the middle 3x3 of the tap gradient
         const int c = o / 9, i = (o % 9) / 3, j = o % 3;
-        gd[o] = gtap[((size_t)b * Ca + c) * kSlot + (i + P - 1) * K + (j + P - 1)];
+        const float v = taps((size_t)b * Ca + c, (i + P - 1) * K + (j + P - 1));
+        gd[o] = v;
+        iv.gdk[(size_t)b * 9 * Ca + o] = v;
     }
     __syncthreads();
-    for (int m = tid; m < hidden; m += nth) {
-        float t = Elem<T>::to_f32(b_down[m]);
-        for (int k = 0; k < Ca; ++k) t = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gm[k], t);
-        tt[m] = t;
-        aa[m] = gelu_exact(t);
-        act[(size_t)b * hidden + m] = aa[m];
+    for (int k = tid; k < Ca; k += kEstThreads) iv.mean[(size_t)b * Ca + k] = gm[k];
+    const float* vin = gm;
+    int n_in = Ca;
+    if (hidden > 0) {
+        for (int m = warp; m < hidden; m += kEstThreads / 32) {
+            float t = 0.f, g = 0.f;
+            for (int k = lane; k < Ca; k += 32) t = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gm[k], t);
+#pragma unroll 8
+            for (int o = lane; o < 9 * Ca; o += 32) g = fmaf(Elem<T>::to_f32(w_last[(size_t)o * hidden + m]), gd[o], g);
+            t = warp_sum(t) + Elem<T>::to_f32(b_down[m]);
+            g = warp_sum(g) * gelu_exact_prime(t);
+            if (lane == 0) {
+                aa[m] = gelu_exact(t);
+                gs[m] = g;
+                iv.act[(size_t)b * hidden + m] = aa[m];
+                iv.gt[(size_t)b * hidden + m] = g;
+            }
+        }
+        __syncthreads();
+        vin = aa; n_in = hidden;
     }
-    __syncthreads();
-    for (int o = tid; o < 9 * Ca; o += nth) {
-        float s = Elem<T>::to_f32(b_up[o]);
-        for (int m = 0; m < hidden; ++m) s = fmaf(Elem<T>::to_f32(w_up[(size_t)o * hidden + m]), aa[m], s);
+    for (int o = tid; o < 9 * Ca; o += kEstThreads) {
+        float s = Elem<T>::to_f32(b_last[o]);
+#pragma unroll 8
+        for (int m = 0; m < n_in; ++m) s = fmaf(Elem<T>::to_f32(w_last[(size_t)o * n_in + m]), vin[m], s);
         dk_flip[(size_t)b * Ca * 9 + (o / 9) * 9 + (8 - o % 9)] = s;
     }
-    for (int m = tid; m < hidden; m += nth) {
+    // bias[b][k] = g_g[b][k] / (H W): a warp per element
+    for (int k = warp; k < Ca; k += kEstThreads / 32) {
         float s = 0.f;
-        for (int o = 0; o < 9 * Ca; ++o) s = fmaf(Elem<T>::to_f32(w_up[(size_t)o * hidden + m]), gd[o], s);
-        s *= gelu_exact_prime(tt[m]);
-        gs[m] = s;
-        gt[(size_t)b * hidden + m] = s;
-    }
-    __syncthreads();
-    for (int k = tid; k < Ca; k += nth) {
-        float s = 0.f;
-        for (int m = 0; m < hidden; ++m) s = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gs[m], s);
-        bias[(size_t)b * Ca + k] = s * inv_hw;
+        if (hidden > 0) {
+            for (int m = lane; m < hidden; m += 32) s = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gs[m], s);
+        } else {
+#pragma unroll 8
+            for (int o = lane; o < 9 * Ca; o += 32) s = fmaf(Elem<T>::to_f32(w_last[(size_t)o * Ca + k]), gd[o], s);
+        }
+        s = warp_sum(s);
+        if (lane == 0) bias[(size_t)b * Ca + k] = s * inv_hw;
     }
 }
 
-// kernel 2d: the sums over images (fixed order) and the rotated LK; six jobs on separate blocks.
-constexpr int kMlpRoles = 6, kMlpBlocks = 32 * kMlpRoles;
-template <typename T>
-__global__ void __launch_bounds__(256)
-mlp_weights(const float* __restrict__ gtap, const float* __restrict__ act, const float* __restrict__ gt, int B, int Ca,
-            int hidden, int H, int W, int KK, const T* __restrict__ w_large, float* __restrict__ g_lk, float* __restrict__ g_wd,
-            float* __restrict__ g_bd, float* __restrict__ g_wu, float* __restrict__ g_bu, T* __restrict__ w_flip)
+// kernel 2c: the estimator's weight gradients, sums over images: 32 consecutive elements per block (the lanes), images dealt to
+// the eight warps in order, the warps added in order.  Elements: g_W_last [9 Ca][n_in], g_b_last [9 Ca], then (two layers)
+// g_W_down [hidden][Ca], g_b_down [hidden].
+__global__ void __launch_bounds__(kEstThreads)
+estimator_weights(const ImageValues iv, int B, int Ca, int hidden, float* __restrict__ g_wl, float* __restrict__ g_bl,
+                  float* __restrict__ g_wd, float* __restrict__ g_bd)
 {
-    const int per_role = gridDim.x / kMlpRoles, role = blockIdx.x / per_role;
-    const int tid = (blockIdx.x % per_role) * blockDim.x + threadIdx.x, nth = per_role * blockDim.x;
-    const float inv_hw = 1.0f / ((float)H * (float)W);
-    auto gdk = [&](int b, int o) {
-        const int c = o / 9, i = (o % 9) / 3, j = o % 3;
-        return gtap[((size_t)b * Ca + c) * kSlot + (i + P - 1) * K + (j + P - 1)];
-    };
-    const int off = (K - KK) / 2, taps = KK * KK;      // a smaller large kernel sits in the middle of the 13 x 13 taps
-    if (role == 0 && g_lk)
-        for (int e = tid; e < Ca * taps; e += nth) {
-            const int c = e / taps, t = (e % taps) / KK + off, u = (e % taps) % KK + off;
-            float s = 0.f;
+    __shared__ float red[kEstThreads];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_in = hidden > 0 ? hidden : Ca, n0 = 9 * Ca * n_in, n1 = n0 + 9 * Ca, n2 = n1 + hidden * Ca, n3 = n2 + hidden;
+    pdl_launch_dependents();
+    pdl_wait_primary();
+    const int e = blockIdx.x * 32 + lane;
+    const float *p = nullptr, *q = nullptr;
+    int sp = 0, sq = 0;
+    float* out = nullptr;
+    if (e < n0) { p = iv.gdk + e / n_in; sp = 9 * Ca; q = (hidden > 0 ? iv.act : iv.mean) + e % n_in; sq = n_in; out = g_wl ? g_wl + e : nullptr; }
+    else if (e < n1) { p = iv.gdk + (e - n0); sp = 9 * Ca; out = g_bl ? g_bl + (e - n0) : nullptr; }
+    else if (e < n2) { p = iv.gt + (e - n1) / Ca; sp = hidden; q = iv.mean + (e - n1) % Ca; sq = Ca; out = g_wd ? g_wd + (e - n1) : nullptr; }
+    else if (e < n3) { p = iv.gt + (e - n2); sp = hidden; out = g_bd ? g_bd + (e - n2) : nullptr; }
+    float s = 0.f;
+    if (out) {
 #pragma unroll 8
-            for (int b = 0; b < B; ++b) s += gtap[((size_t)b * Ca + c) * kSlot + t * K + u];
-            g_lk[e] = s;
-        }
-    if (role == 1)
-        for (int e = tid; e < Ca * taps; e += nth) {
-            const int c = e / taps, t = e % taps;
-            w_flip[(size_t)c * taps + (taps - 1 - t)] = w_large[e];
-        }
-    if (role == 2 && g_bu)
-        for (int o = tid; o < 9 * Ca; o += nth) {
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s += gdk(b, o);
-            g_bu[o] = s;
-        }
-    if (role == 3 && g_wu)
-        for (int e = tid; e < 9 * Ca * hidden; e += nth) {
-            const int o = e / hidden, m = e % hidden;
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s = fmaf(gdk(b, o), act[(size_t)b * hidden + m], s);
-            g_wu[e] = s;
-        }
-    if (role == 4 && g_bd)
-        for (int m = tid; m < hidden; m += nth) {
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s += gt[(size_t)b * hidden + m];
-            g_bd[m] = s;
-        }
-    if (role == 5 && g_wd)
-        for (int e = tid; e < hidden * Ca; e += nth) {
-            const int m = e / Ca, k = e % Ca;
-            float s = 0.f;
-#pragma unroll 8
-            for (int b = 0; b < B; ++b) s = fmaf(gt[(size_t)b * hidden + m], gtap[((size_t)b * Ca + k) * kSlot + TAPS] * inv_hw, s);
-            g_wd[e] = s;
-        }
+        for (int b = warp; b < B; b += kEstThreads / 32)
+            s = fmaf(__ldcg(p + (size_t)b * sp), q ? __ldcg(q + (size_t)b * sq) : 1.0f, s);
+    }
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (warp != 0 || !out) return;
+#pragma unroll
+    for (int w = 1; w < kEstThreads / 32; ++w) s += red[w * 32 + lane];
+    *out = s;
 }
 
 }}  // namespace esc::bwd

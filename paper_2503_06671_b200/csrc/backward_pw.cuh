@@ -133,21 +133,6 @@ mix(const T* __restrict__ x, const T* __restrict__ w_point, T* __restrict__ m, i
     }
 }
 
-// ---- sum of x_att per (image, channel) into the tap-gradient table's slot for it ------------------------------------
-// A warp per (image, channel): lanes take every 32nd chunk in order, then a fixed butterfly.
-__global__ void __launch_bounds__(256)
-sum_x(const float* __restrict__ xs_part, int BCa, int Ca, int chunks, float* __restrict__ gtap)
-{
-    const int lane = threadIdx.x & 31, e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (e >= BCa) return;
-    const int b = e / Ca, k = e % Ca;
-    float s = 0.f;
-    for (int c = lane; c < chunks; c += 32) s += xs_part[((size_t)b * chunks + c) * Ca + k];
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) gtap[(size_t)e * kSlot + TAPS] = s;
-}
-
 // ---- g_x = P^T g_m + constant, in place; per-chunk partial sums of g_P ---------------------------------------------
 // Block = (image, chunk).  Per pass a thread turns its pixel's g_m into g_x (P's rows broadcast from shared memory) and
 // stages g_m and x_att of the pass channel-major.  The outer products g_m[n] x[k] are then register-tiled: the CA x CA
@@ -274,17 +259,26 @@ back(const T* __restrict__ x, const T* __restrict__ w_point, T* __restrict__ gx,
     }
 }
 
-// ---- g_P[e] = sum over blocks of the partial sums: a warp per element, lanes over blocks in order, butterfly ---------
-__global__ void __launch_bounds__(256)
+// ---- g_P[e] = sum over blocks of the partial sums: the lanes take 32 consecutive elements, the warps every 32nd block each (in
+// order), then the warps are added in order.
+constexpr int kSumGpThreads = 1024;
+__global__ void __launch_bounds__(kSumGpThreads)
 sum_gp(const float* __restrict__ gp_part, int elems, int blocks, float* __restrict__ g_wp)
 {
-    const int lane = threadIdx.x & 31, e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (e >= elems) return;
+    __shared__ float red[kSumGpThreads];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+    pdl_wait_primary();
     float s = 0.f;
-    for (int k = lane; k < blocks; k += 32) s += gp_part[(size_t)k * elems + e];
+    if (e < elems) {
+#pragma unroll 8
+        for (int k = warp; k < blocks; k += kSumGpThreads / 32) s += __ldcg(gp_part + (size_t)k * elems + e);
+    }
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (warp != 0 || e >= elems) return;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) g_wp[e] = s;
+    for (int w = 1; w < kSumGpThreads / 32; ++w) s += red[w * 32 + lane];
+    g_wp[e] = s;
 }
 
 }}}  // namespace esc::bwd::pw

@@ -15,7 +15,7 @@
 //   warp 8     lane 0 requests both tiles by TMA (zero fill = the padding)
 //   warps 0-7  transpose both tiles into per-channel planes (as the forward kernel does), then two channels each:
 //              16 rows x 5 column blocks x 2 instructions; 169 sums and the sum of the tile's x values per channel go
-//              to the tile's slot of the workspace, which sum_tiles and finish (backward.cuh) consume.
+//              to the tile's slot of the workspace, which sum_tiles and the estimator's kernels (backward.cuh) consume.
 #pragma once
 #include "backward.cuh"
 #include "stencil_toeplitz.cuh"

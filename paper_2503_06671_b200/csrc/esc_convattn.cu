@@ -581,12 +581,12 @@ int forward_impl(const Problem& p0, const void* x, const void* w_large0, const E
 struct BackwardWs {
     unsigned* ctrl;
     float *part, *gtap, *dk_flip, *bias;
-    float *act, *gt;                 // two-layer estimator: activations and g_t, [B][kMaxHidden] each
+    esc::bwd::ImageValues iv;        // per image: g_dk [B][9 Ca], means [B][Ca], activations and g_t [B][kMaxHidden]
     void* lk_pad;                    // the rotated large kernel zero-padded to 13 x 13 for the tensor-core kernels
     void* w_flip;
     float *xs_part, *gp_part;        // decomposed form: per-chunk sums of x_att [B][chunks][Ca] and of g_P [B * chunks][Ca * Ca]
     int chunks;                      // chunks of pixels per image in those
-    bool patch_xsum;                 // the tap-gradient kernels ran on the mixed features: take the sums of x_att from xs_part
+    bool mixed;                      // the tap-gradient kernels ran on the mixed features: take the sums of x_att from xs_part
     size_t bytes;
     float* dense_part;               // dense large kernel: the blocks' tap sums [blocks][16][16][169]
     void* wd_flip;                   // the dense kernel with swapped channel axes and rotated taps
@@ -606,11 +606,13 @@ BackwardWs carve_backward(void* ws, const Problem& p) {
     w.w_flip = base + off;                          off += round_up((size_t)p.Ca * esc::bwd::TAPS * 4, 256);
     w.dk_flip = reinterpret_cast<float*>(base + off); off += round_up((size_t)p.B * p.Ca * 9 * 4, 256);
     w.bias = reinterpret_cast<float*>(base + off);  off += round_up((size_t)p.B * p.Ca * 4, 256);
-    w.act = reinterpret_cast<float*>(base + off);   off += round_up((size_t)p.B * esc::kMaxHidden * 4, 256);
-    w.gt = reinterpret_cast<float*>(base + off);    off += round_up((size_t)p.B * esc::kMaxHidden * 4, 256);
+    w.iv.gdk = reinterpret_cast<float*>(base + off);  off += round_up((size_t)p.B * p.Ca * 9 * 4, 256);
+    w.iv.mean = reinterpret_cast<float*>(base + off); off += round_up((size_t)p.B * p.Ca * 4, 256);
+    w.iv.act = reinterpret_cast<float*>(base + off);  off += round_up((size_t)p.B * esc::kMaxHidden * 4, 256);
+    w.iv.gt = reinterpret_cast<float*>(base + off);   off += round_up((size_t)p.B * esc::kMaxHidden * 4, 256);
     w.lk_pad = base + off;                          off += round_up((size_t)p.Ca * esc::bwd::TAPS * 4, 256);
     w.chunks = esc::bwd::pw::chunks_of((long long)p.H * p.W);
-    w.patch_xsum = false;
+    w.mixed = false;
     w.xs_part = reinterpret_cast<float*>(base + off); off += round_up((size_t)p.B * w.chunks * p.Ca * 4, 256);
     w.gp_part = reinterpret_cast<float*>(base + off);
     if (esc::bwd::pw::supported(p.Ca)) off += round_up((size_t)p.B * w.chunks * p.Ca * p.Ca * 4, 256);
@@ -620,6 +622,22 @@ BackwardWs carve_backward(void* ws, const Problem& p) {
     w.wd_flip = base + off;                              off += round_up((size_t)esc::bwd::dense::CA * esc::bwd::dense::CA * esc::bwd::TAPS * 4, 256);
     w.bytes_dense = off;
     return w;
+}
+
+// A kernel that may be scheduled while the one before it drains; it waits (griddepcontrol) before it touches memory.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 // Weight gradients the caller asked for (fp32, any may be null): of LK, and of the estimator's layers -- last layer
@@ -671,35 +689,30 @@ int backward_t(const Problem& p, const void* x, const void* go, const void* w_la
     }
     ESC_CUDA(cudaGetLastError());
     if (tiles_done == 0) ++g_last_launches;
-    esc::bwd::sum_tiles<<<(unsigned)(p.B * p.Ca), esc::bwd::kSumThreads, 0, st>>>(w.part, tiles_done > 0 ? tiles_done : tiles_x * tiles_y, w.gtap);
-    ESC_CUDA(cudaGetLastError());
-    if (w.patch_xsum) {
-        // decomposed form: the sums the tap-gradient kernels took are those of the mixed features; g_W wants the unmixed ones
-        const int warps = p.B * p.Ca;
-        esc::bwd::pw::sum_x<<<(unsigned)((warps + 7) / 8), 256, 0, st>>>(w.xs_part, warps, p.Ca, w.chunks, w.gtap);
-        ESC_CUDA(cudaGetLastError());
+    // the estimator's part, from the tap gradients; few tiles are added up on the way
+    const int tiles = tiles_done > 0 ? tiles_done : tiles_x * tiles_y;
+    esc::bwd::Taps taps{w.part, tiles};
+    if (tiles > esc::bwd::kDirectTiles) {
+        ESC_CUDA(launch_pdl(esc::bwd::sum_tiles, (unsigned)(p.B * p.Ca), esc::bwd::kSumThreads, 0, st, w.part, tiles, w.gtap));
+        ++g_last_launches;
+        taps = esc::bwd::Taps{w.gtap, 1};
+    }
+    const size_t smem = (size_t)((p.Ca <= esc::bwd::kEstMaxCa ? 10 * p.Ca : 0) + 2 * est.hidden) * sizeof(float);
+    const int ltaps = p.Ca * p.K * p.K;
+    const long long grid = (long long)p.B + (g.g_lk ? (ltaps + 31) / 32 : 0) + (p.dense ? 0 : esc::bwd::kFlipBlocks);
+    if (grid > 0x7fffffffLL) return ESC_ERR_UNSUPPORTED;
+    ESC_CUDA(launch_pdl(esc::bwd::estimator_image<T>, (unsigned)grid, esc::bwd::kEstThreads, smem, st, taps,
+                        (const float*)(w.mixed ? w.xs_part : nullptr), w.chunks, p.B, p.Ca, est.hidden, p.H, p.W, p.K,
+                        static_cast<const T*>(w_large), static_cast<const T*>(est.w_down), static_cast<const T*>(est.b_down),
+                        static_cast<const T*>(est.w_last), static_cast<const T*>(est.b_last), w.iv, w.dk_flip, w.bias, g.g_lk,
+                        p.dense ? (T*)nullptr : static_cast<T*>(w.w_flip)));
+    ++g_last_launches;
+    if (g.g_w_last || g.g_b_last || g.g_w_down || g.g_b_down) {
+        const int elems = 9 * p.Ca * (est.hidden > 0 ? est.hidden : p.Ca) + 9 * p.Ca + est.hidden * p.Ca + est.hidden;
+        ESC_CUDA(launch_pdl(esc::bwd::estimator_weights, (unsigned)((elems + 31) / 32), esc::bwd::kEstThreads, 0, st, w.iv, p.B, p.Ca,
+                            est.hidden, g.g_w_last, g.g_b_last, g.g_w_down, g.g_b_down));
         ++g_last_launches;
     }
-    if (est.hidden == 0) {
-        esc::bwd::finish<T><<<esc::bwd::kFinishBlocks, 256, 0, st>>>(w.gtap, p.B, p.Ca, p.H, p.W, p.K, static_cast<const T*>(w_large),
-                                                static_cast<const T*>(est.w_last), static_cast<const T*>(est.b_last), g.g_lk,
-                                                g.g_w_last, g.g_b_last, static_cast<T*>(w.w_flip), w.dk_flip, w.bias);
-        ESC_CUDA(cudaGetLastError());
-        g_last_launches += 2;
-        return ESC_OK;
-    }
-    // two-layer estimator: what belongs to one image, then the sums over images
-    const size_t smem = (size_t)(10 * p.Ca + 3 * est.hidden) * sizeof(float);
-    if (smem > 48 * 1024) return ESC_ERR_UNSUPPORTED;
-    esc::bwd::mlp_image<T><<<(unsigned)p.B, 256, smem, st>>>(w.gtap, p.Ca, est.hidden, p.H, p.W, static_cast<const T*>(est.w_down),
-                                                             static_cast<const T*>(est.b_down), static_cast<const T*>(est.w_last),
-                                                             static_cast<const T*>(est.b_last), w.act, w.gt, w.dk_flip, w.bias);
-    ESC_CUDA(cudaGetLastError());
-    esc::bwd::mlp_weights<T><<<esc::bwd::kMlpBlocks, 256, 0, st>>>(w.gtap, w.act, w.gt, p.B, p.Ca, est.hidden, p.H, p.W, p.K,
-                                                                  static_cast<const T*>(w_large), g.g_lk, g.g_w_down, g.g_b_down,
-                                                                  g.g_w_last, g.g_b_last, static_cast<T*>(w.w_flip));
-    ESC_CUDA(cudaGetLastError());
-    g_last_launches += 3;
     return ESC_OK;
 }
 
@@ -747,8 +760,8 @@ int pw_back_ca(const Problem& p, const void* x, const void* w_point, void* gx, c
     ++g_last_launches;
     if (g_wp) {
         const int elems = CA * CA;
-        esc::bwd::pw::sum_gp<<<(unsigned)((elems + 7) / 8), 256, 0, st>>>(w.gp_part, elems, (int)blocks, g_wp);
-        ESC_CUDA(cudaGetLastError());
+        ESC_CUDA(launch_pdl(esc::bwd::pw::sum_gp, (unsigned)((elems + 31) / 32), esc::bwd::pw::kSumGpThreads, 0, st, (const float*)w.gp_part,
+                            elems, (int)blocks, g_wp));
         ++g_last_launches;
     }
     return ESC_OK;
@@ -822,7 +835,8 @@ int dense_grad_x_t(Problem p, const void* go, const void* w_dense, void* gx, con
     namespace D = esc::bwd::dense;
     p.dense = true;
     p.bias = w.bias;
-    int rc = launch_stencil_dense(p, go, w_dense, w.dk_flip, gx, w.ctrl, st, /*dependent=*/false, /*flip=*/true);
+    // dependent: grad_out and the weights are older than the estimator's kernels, which alone it has to wait for
+    int rc = launch_stencil_dense(p, go, w_dense, w.dk_flip, gx, w.ctrl, st, /*dependent=*/true, /*flip=*/true);
     if (rc != esc::tma::kNotApplicable) return rc;
     const int elems = D::CA * D::CA * p.K * p.K;
     D::flip_dense<T><<<(unsigned)((elems + 255) / 256), 256, 0, st>>>(static_cast<const T*>(w_dense), p.K, static_cast<T*>(w.wd_flip));
@@ -1420,7 +1434,7 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
                               : (layout == ESC_NCHW ? pw_mix_t<__nv_bfloat16, esc::kNCHW>(p, x, w_point, grad_x, w, st)
                                                     : pw_mix_t<__nv_bfloat16, esc::kNHWC>(p, x, w_point, grad_x, w, st));
         if (rc != ESC_OK) return rc;
-        w.patch_xsum = true;
+        w.mixed = true;
     }
     const void* x_taps = w_point ? grad_x : x;             // what the depth-wise stage saw
     if (dense) {
@@ -1432,6 +1446,7 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
                                                     : dense_tap_grad_t<__nv_bfloat16, esc::kNHWC>(p, x, grad_out, w, g_wd, st));
         if (rc != ESC_OK) return rc;
     }
+    p.dense = dense;
     if (dtype == ESC_F32)
         rc = layout == ESC_NCHW ? backward_t<float, esc::kNCHW>(p, x_taps, grad_out, w_large, est, w, g, st)
                                 : backward_t<float, esc::kNHWC>(p, x_taps, grad_out, w_large, est, w, g, st);
