@@ -355,7 +355,7 @@ TensorLk tensor_lk(const Problem& p, const void* x, const void* out, const void*
     TensorLk t{w_large, p.K};
     if (p.dense || p.dtype != ESC_BF16 || p.K >= esc::tma::K13 || !pad || g_engine_policy == ESC_ENGINE_FP32 || g_tile_policy != 0) return t;
     if (!esc::tma::toep::applies(p.C, p.Ca, esc::tma::K13, p.dtype, p.layout) &&
-        !esc::tma::toepn::applies(p.C, p.Ca, p.H, p.W, esc::tma::K13, p.dtype, p.layout, x, out))
+        !esc::tma::toepn::takes(p.B, p.C, p.Ca, p.H, p.W, esc::tma::K13, p.dtype, p.layout, x, out))
         return t;
     pad_large_kernel<__nv_bfloat16><<<(p.Ca * 169 + 255) / 256, 256, 0, st>>>(static_cast<const __nv_bfloat16*>(w_large), p.Ca, p.K,
                                                                             static_cast<__nv_bfloat16*>(pad));
@@ -568,7 +568,7 @@ int forward_impl(const Problem& p0, const void* x, const void* w_large0, const E
         if (rc != esc::tma::kNotApplicable) { (void)cudaGetLastError(); g_last_error.clear(); }
     }
     const bool tensor_nchw = !p.dense && (!p.w_point || p.Ca == esc::tma::CG) && !p.bias && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
-                             esc::tma::toepn::applies(p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, out);
+                             esc::tma::toepn::takes(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, out);
     int rc = launch_gap(p0, x, est, w, w.dk, st, tensor_stencil_follows(p) || tensor_nchw);
     if (rc != ESC_OK) return rc;
     if (p0.dense) return launch_stencil_dense(p0, x, w_large0, w.dk, out, w.ctrl, st, /*dependent=*/true);
@@ -1347,7 +1347,7 @@ int esc_convattn_forward_fused(const void* x, int B, int C, int C_a, int H, int 
     // The same on NCHW tensors: the NCHW tensor-core stencil without its copy of the identity planes, then the NCHW 1x1 kernel.
     if (K == esc::tma::K13 && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
         esc::fuse::nchw::applies(C, C_a, (long long)H * W, dtype, layout, x, out, residual, w_fuse) &&
-        esc::tma::toepn::applies(C, C_a, H, W, K, dtype, layout, x, out)) {
+        esc::tma::toepn::takes(B, C, C_a, H, W, K, dtype, layout, x, out)) {
         p.skip_copy = true;
         rc = forward_impl(p, x, w_large, est, out, workspace, st);
         if (rc != ESC_OK) return rc;

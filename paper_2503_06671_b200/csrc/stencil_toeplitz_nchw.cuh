@@ -21,6 +21,12 @@
 // kFused: stage 1 of the module (Eq. 4 line 2) inside this kernel, as in the NHWC kernel: every CTA adds up the
 // interiors of its (at most two) tiles, arrives on the image's counter, the last arrival advances the image's
 // flag, and every CTA then evaluates the estimator for the channels it works on.  Cooperative launch, bounded waits.
+// kRagged: widths that are not a multiple of 8 (rows that are not whole 16-byte pieces: no tensor map describes them).  Three
+// warps load the tiles instead of TMA -- the 12 aligned 16-byte pieces that cover a row of 88 columns, shifted into place in
+// registers, two rows per warp instruction -- and all warps together the first one; results leave as aligned 4-byte words.
+// With the point-wise mix they keep what the generic kernel keeps, a mixed map that is not rounded to bf16: the mix leaves its high
+// and its low half (together 16 bits of mantissa) in the two tile buffers, the products run over both, and a CTA has one tile
+// at a time.  The rule between this and the generic register-tiled kernel stands at `ragged_applies`, with both sides' times.
 #pragma once
 #include "stencil_toeplitz.cuh"
 
@@ -88,10 +94,64 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t (&r)[4]) {
 // taken from the unmixed values) the 16 planes are replaced, eight pixels at a time and in place, by LK^c applied across
 // them: D (16 output channels x 8 pixels) = LK^c (16 x 16) x B (16 channels x 8 pixels), B straight from the planes by
 // ldmatrix.trans, one rounding to bf16; then one block-wide barrier before the depth-wise products.
-template <bool kFused, bool kMix = false>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kRagged> struct Shape { static constexpr int threads = kRagged ? kThreads + 64 : kThreads; };
+constexpr int kLoaders = 3;                         // kRagged: warps 8, 10 and 11
+
+// One tile of 16 planes [ROWS][PP] for kRagged: warp `w` of `n` takes every n-th pair of rows, lanes 0-11 and 16-27 the twelve
+// aligned 16-byte pieces of one row each.  (C is a multiple of 8, so the tensor is whole pieces.)  Instructions bound it -- about
+// 45 per pair of rows --, hence 32-bit offsets inside the group's 16 planes.
+template <int BATCH>
+__device__ __forceinline__ void load_tile_ragged(unsigned char* planes, const Unit& un, const Params& p, int w, int n, int lane) {
+    constexpr int NPAIR = CG * ROWS / 2;
+    const int piece = lane & 15, half = lane >> 4;
+    const int x0 = un.tx * TW - XS, ya = un.ty * TH - P6, plane = p.H * p.W;
+    const long long g0 = ((long long)un.b * p.C + un.g * CG) * plane;                 // the group's first element: a multiple of 8
+    const uint4* base = reinterpret_cast<const uint4*>(p.x + g0);
+    const bool edge = x0 < 0 || x0 + PP + 8 > p.W;                                    // some column may lie outside the image
+    for (int r0 = w; r0 < NPAIR; r0 += BATCH * n) {
+        uint4 v[BATCH];
+        int e[BATCH];
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            const int row = (r0 + u * n) * 2 + half, c = row / ROWS, y = ya + row - c * ROWS;
+            e[u] = c * plane + y * p.W + x0;                                          // element of the row's first column
+            v[u] = make_uint4(0u, 0u, 0u, 0u);
+            const int xa = x0 - (e[u] & 7) + 8 * piece;                               // the piece's first column
+            if (c < CG && piece < 12 && (unsigned)y < (unsigned)p.H && xa > -8 && xa < p.W) v[u] = __ldg(base + ((e[u] >> 3) + piece));
+            if (edge && (xa < 0 || xa + 8 > p.W)) {                                   // zero what belongs to the rows above and below
+                uint32_t* w4 = reinterpret_cast<uint32_t*>(&v[u]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int a = xa + 2 * i;
+                    w4[i] &= ((unsigned)a < (unsigned)p.W ? 0x0000ffffu : 0u) | ((unsigned)(a + 1) < (unsigned)p.W ? 0xffff0000u : 0u);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) {
+            // elements sh .. sh + 7 of this piece and the next: words sh / 2 .. of the eight, then half a word on if sh is odd
+            uint32_t a[8] = {v[u].x, v[u].y, v[u].z, v[u].w, 0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a[4 + i] = __shfl_down_sync(0xffffffffu, a[i], 1, 16);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) a[i] = (e[u] & 4) ? a[i + 2] : a[i];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) a[i] = (e[u] & 2) ? a[i + 1] : a[i];
+            const unsigned bits = (e[u] & 1) * 16u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) a[i] = __funnelshift_r(a[i], a[i + 1], bits);
+            const int pr = r0 + u * n;
+            if (pr < NPAIR && piece < PP / 8)
+                *reinterpret_cast<uint4*>(planes + (pr * 2 + half) * (PP * 2) + piece * 16) = make_uint4(a[0], a[1], a[2], a[3]);
+        }
+    }
+}
+
+template <bool kFused, bool kMix = false, bool kRagged = false>
+__global__ void __launch_bounds__(Shape<kRagged>::threads, 1)
 stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Params p)
 {
+    constexpr bool kSplit = kRagged && kMix;
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char* bufs = smem;                                                    // 2 x 16 planes [ROWS][PP] bf16
     uint32_t* ptab = reinterpret_cast<uint32_t*>(smem + 2 * BUF_BYTES);            // [16][13][PT] packed tap pairs
@@ -102,7 +162,7 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
-        for (int s = 0; s < 2; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, kWarps); }
+        for (int s = 0; s < 2; ++s) { mbar_init(full0 + 8 * s, kRagged ? kLoaders : 1); mbar_init(empty0 + 8 * s, kWarps); }
         for (int s = 0; s < kCopySlots; ++s) mbar_init(cfull0 + 8 * s, 1);
         mbar_init(sumdone, kWarps);                          // one barrier per unit (the producer lane may fall behind by more
         mbar_init(sumdone + 8, kWarps);                      // than the one phase a parity wait can tell apart)
@@ -115,9 +175,42 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
     const long long first = blockIdx.x, stride = gridDim.x;
     const long long my_units = first < p.units ? (p.units - first + stride - 1) / stride : 0;
 
+    if constexpr (kRagged) {
+        unsigned seen[2] = {0u, 0u};
+        if (kFused && warp == kWarps) {                      // the flags as they stand before this CTA arrives anywhere
+            for (int k = 0; k < (int)my_units && k < 2; ++k) seen[k] = ld_acquire(p.gflag + decode(first + k * stride, p).b);
+        }
+        if (my_units > 0) load_tile_ragged<10>(bufs, decode(first, p), p, warp, Shape<true>::threads / 32, lane);
+        __syncthreads();
+        if (warp == kWarps || warp >= kWarps + 2) {
+            // ---- the loading warps
+            const int w = warp == kWarps ? 0 : warp - kWarps - 1;
+            bool alive = true;
+            for (long long k = 0; k < my_units; ++k) {
+                const int buf = kSplit ? 0 : (int)(k & 1);
+                if (k >= 1) {
+                    const unsigned parity = kSplit ? (unsigned)((k - 1) & 1) : (unsigned)(((k >> 1) - 1) & 1);
+                    if (kSplit || k >= 2) alive = __shfl_sync(0xffffffffu, alive && (lane != 0 || mbar_wait(empty0 + 8 * buf, parity, p.ctrl, 0xB8000000u)), 0);
+                    if (alive) load_tile_ragged<8>(bufs + buf * BUF_BYTES, decode(first + k * stride, p), p, w, kLoaders, lane);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(full0 + 8 * buf);
+            }
+            if (kFused && w == 0 && lane == 0) {
+                for (int k = 0; k < (int)my_units && k < 2; ++k) {
+                    const Unit un = decode(first + k * stride, p);
+                    if (alive) alive = mbar_wait(sumdone + 8 * k, 0u, p.ctrl, 0xB9000000u);
+                    unsigned old;
+                    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(p.garr + un.b), "r"((unsigned)(p.upi - 1)) : "memory");
+                    if (old == (unsigned)(p.upi - 1)) st_release(p.gflag + un.b, seen[k] + 1u);
+                }
+            }
+            return;
+        }
+    }
     if (warp >= kWarps) {
         if (lane != 0) return;
-        if (warp == kWarps) {
+        if (!kRagged && warp == kWarps) {
             // ---- tile producer: buffer k & 1 is free again once every warp has stored the results of unit k - 2
             bool alive = true;
             unsigned seen[2] = {0u, 0u};
@@ -286,7 +379,7 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
 
     for (long long k = 0; k < my_units; ++k) {
         const Unit un = decode(first + k * stride, p);
-        const int bufi = (int)(k & 1);
+        const int bufi = kSplit ? 0 : (int)(k & 1);
         unsigned char* planes = bufs + bufi * BUF_BYTES;
         const uint32_t planes_a = smem_u32(planes);
 
@@ -310,12 +403,12 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
         }
 
         // ---- the tile has landed: it is the 16 planes -------------------------------------------------------
-        if (alive) alive = mbar_wait(full0 + 8 * bufi, (unsigned)((k >> 1) & 1), p.ctrl, 0xA8000000u);
+        if (alive) alive = mbar_wait(full0 + 8 * bufi, (unsigned)((kSplit ? k : k >> 1) & 1), p.ctrl, 0xA8000000u);
         if (kFused && k == 0) {
             // both of this CTA's tiles are added up now, at the start, so that every image's flag advances long before
             // any CTA needs dk
             tile_sum(first, planes, 0);
-            if (my_units > 1) {
+            if (!kSplit && my_units > 1) {                   // (kSplit: one unit per CTA in the one-launch form)
                 if (alive) alive = mbar_wait(full0 + 8, 0u, p.ctrl, 0xA9000000u);
                 tile_sum(first + stride, bufs + BUF_BYTES, 1);
             }
@@ -346,6 +439,11 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
                         const __nv_bfloat162 lo = __floats2bfloat162_rn(d[0], d[1]), hi = __floats2bfloat162_rn(d[2], d[3]);
                         *reinterpret_cast<__nv_bfloat162*>(px + (size_t)g * PLANE) = lo;
                         *reinterpret_cast<__nv_bfloat162*>(px + (size_t)(g + 8) * PLANE) = hi;
+                        if constexpr (kSplit) {              // what the rounding left, into the other buffer
+                            const float2 a = __bfloat1622float2(lo), b2 = __bfloat1622float2(hi);
+                            *reinterpret_cast<__nv_bfloat162*>(px + BUF_BYTES + (size_t)g * PLANE) = __floats2bfloat162_rn(d[0] - a.x, d[1] - a.y);
+                            *reinterpret_cast<__nv_bfloat162*>(px + BUF_BYTES + (size_t)(g + 8) * PLANE) = __floats2bfloat162_rn(d[2] - b2.x, d[3] - b2.y);
+                        }
                     }
                 }
             }
@@ -357,7 +455,7 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
         float dkv[9];
 
         auto mma_all = [&](float (&a4)[NB][NA][4], const int c) {
-            const uint32_t b_lane = planes_a + (uint32_t)c * PLANE + (uint32_t)((((mi >> 1) * 8 + mr) * PP + (mi & 1) * 8) * 2);
+            uint32_t b_lane = planes_a + (uint32_t)c * PLANE + (uint32_t)((((mi >> 1) * 8 + mr) * PP + (mi & 1) * 8) * 2);
             const uint32_t* pt = ptab + c * (K13 * PT);
 #pragma unroll
             for (int q = 0; q < NB; ++q)
@@ -365,6 +463,8 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
                 for (int r = 0; r < NA; ++r)
 #pragma unroll
                     for (int v = 0; v < 4; ++v) a4[q][r][v] = 0.f;
+#pragma unroll 1
+            for (int half = 0; half < (kSplit ? 2 : 1); ++half, b_lane += BUF_BYTES)         // kSplit: the low halves too
 #pragma unroll
             for (int i = 0; i < K13; ++i) {
                 const uint32_t pa = pt[i * PT + ia], pb = pt[i * PT + ib], pc = pt[i * PT + ic];
@@ -413,6 +513,13 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
                             in[a][0] = __uint_as_float(u << 16);
                             in[a][1] = __uint_as_float(u & 0xffff0000u);
                             in[a][2] = __uint_as_float((w1 >> sh) << 16);
+                            if constexpr (kSplit) {
+                                const uint32_t l0 = plane32[BUF_BYTES / 4 + (y + 5 + a) * (PP / 2) + wi], l1 = plane32[BUF_BYTES / 4 + (y + 5 + a) * (PP / 2) + wi + 1];
+                                const uint32_t l = __funnelshift_r(l0, l1, sh);
+                                in[a][0] += __uint_as_float(l << 16);
+                                in[a][1] += __uint_as_float(l & 0xffff0000u);
+                                in[a][2] += __uint_as_float((l1 >> sh) << 16);
+                            }
                         }
                         float s0 = bias, s1 = bias;
 #pragma unroll
@@ -442,7 +549,28 @@ stencil_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_att, const Pa
                     }
             __syncwarp();
             const int px = un.tx * TW + 2 * lane, y0 = un.ty * TH;
-            if (px < p.W) {                                  // W is even: a pair of pixels is inside or outside together
+            if constexpr (kRagged) {
+                // a row starts at any element: at an even one its pairs leave as they lie in the plane, at an odd one as the
+                // pairs (2l - 1, 2l), the first and the last element alone
+                const int x0 = un.tx * TW, cols = min(TW, p.W - x0), plane_px = p.H * p.W;
+                const size_t chan = ((size_t)un.b * p.C + un.g * CG + c) * plane_px;
+                __nv_bfloat16* base = p.out + chan;
+                const int par = (int)(chan & 1), o0 = y0 * p.W + x0;
+                const uint32_t* src = reinterpret_cast<const uint32_t*>(plane) + lane;
+#pragma unroll 4
+                for (int r = 0; r < TH; ++r) {
+                    const uint32_t u = src[r * (PP / 2)], prev = __shfl_up_sync(0xffffffffu, u, 1);
+                    const int off = o0 + r * p.W, odd = (off + par) & 1, e = 2 * lane - odd;      // first element of this lane's word
+                    if (y0 + r < p.H) {
+                        __nv_bfloat16* dst = base + off + e;
+                        const uint32_t w = odd ? __funnelshift_r(prev, u, 16) : u;
+                        if (e >= 0 && e + 1 < cols) *reinterpret_cast<uint32_t*>(dst) = w;
+                        else if (e < 0) *reinterpret_cast<unsigned short*>(dst + 1) = (unsigned short)(w >> 16);
+                        else if (e < cols) *reinterpret_cast<unsigned short*>(dst) = (unsigned short)w;
+                        if (odd && lane == 31 && cols == TW) *reinterpret_cast<unsigned short*>(dst + 2) = (unsigned short)(u >> 16);
+                    }
+                }
+            } else if (px < p.W) {                                  // W is even: a pair of pixels is inside or outside together
                 __nv_bfloat16* dst = p.out + (((size_t)un.b * p.C + un.g * CG + c) * p.H + y0) * p.W + px;
                 const uint32_t* src = reinterpret_cast<const uint32_t*>(plane) + lane;
 #pragma unroll
@@ -491,7 +619,19 @@ inline bool applies(int C, int Ca, int H, int W, int K, int dtype, int layout, c
            (reinterpret_cast<uintptr_t>(x) & 15u) == 0 && (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
 }
 
-template <bool kFused, bool kMix = false>
+// Widths that are not a multiple of 8: the same kernel with its own loads and stores, from so many units on that it is faster than
+// the generic register-tiled kernel, whose blocks are smaller and which mixes a pixel once per output channel.  Measured, bf16,
+// whole forward, generic / this kernel: 64x65 (8 units) 22.7 / 23.4 us plain; 5 x (61x61) (20 units) 18.8 / 23.5; 2 x (33x257) (30
+// units) 21.3 / 23.5, decomposed 32.3 / 35.7; 180x322 (72 units) 25.8 / 23.5, decomposed 54.8 / 35.7; 240x427 (105 units)
+// 38.1 / 23.3, decomposed 71.6 / 37.6; 359x639 (240 units) 64.5 / 41.7, decomposed 145 / 70; 1079x1917, C_a = 32, 951 / 442.
+constexpr long long kRaggedUnits = 48;
+inline bool ragged_applies(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x, const void* out) {
+    return K == K13 && dtype == 1 /*bf16*/ && layout == kNCHW && Ca % CG == 0 && C >= Ca && C % 8 == 0 && W % 8 != 0 &&
+           (long long)CG * H * W < 0x7fff0000LL && units_of(B, Ca, H, W) >= kRaggedUnits && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 &&
+           (reinterpret_cast<uintptr_t>(out) & 15u) == 0;
+}
+
+template <bool kFused, bool kMix = false, bool kRagged = false>
 inline int launch(int B, int C, int Ca, int H, int W, const void* x, const void* w_large, const float* dk, const float* bias, void* out,
                   unsigned* ctrl, cudaStream_t st, bool dependent, int* launches, std::string* err, const toep::Fused* fu,
                   const void* w_point = nullptr, bool skip_copy = false) {
@@ -506,7 +646,7 @@ inline int launch(int B, int C, int Ca, int H, int W, const void* x, const void*
     if (kMix && (Ca != CG || !w_point || (reinterpret_cast<uintptr_t>(w_point) & 3u) != 0)) return kNotApplicable;   // one group, 4-byte loads
     p.dk = dk; p.bias = bias; p.out = static_cast<__nv_bfloat16*>(out); p.ctrl = ctrl;
     p.wait_first = dependent ? 0 : 1;
-    p.copy_bytes = skip_copy ? 0 : (long long)(C - Ca) * H * W * 2;   // a multiple of 16: W is a multiple of 8; skip_copy: consumed elsewhere (fused 1x1)
+    p.copy_bytes = skip_copy ? 0 : (long long)(C - Ca) * H * W * 2;   // a multiple of 16: W is (or C and Ca are) a multiple of 8; skip_copy: consumed elsewhere (fused 1x1)
     p.w_last = p.b_last = p.w_down = p.b_down = nullptr; p.hidden = 0; p.gpart = nullptr; p.garr = p.gflag = nullptr;
     p.upi = p.groups * p.tiles_x * p.tiles_y;
     if (kFused) {
@@ -514,8 +654,8 @@ inline int launch(int B, int C, int Ca, int H, int W, const void* x, const void*
         p.w_down = static_cast<const __nv_bfloat16*>(fu->w_down); p.b_down = static_cast<const __nv_bfloat16*>(fu->b_down);
         p.hidden = fu->hidden; p.gpart = fu->gpart; p.garr = fu->garr; p.gflag = fu->gflag;
     }
-    CUtensorMap m_att;
-    if (!make_map_nchw(&m_att, x, B, C, H, W)) return kNotApplicable;
+    CUtensorMap m_att = {};
+    if (!kRagged && !make_map_nchw(&m_att, x, B, C, H, W)) return kNotApplicable;
     static_assert((2 * BUF_BYTES + PTAB_BYTES + FUSED_SMEM_FLOATS * 4) % 128 == 0, "the copy ring is a bulk-copy destination");
     const size_t smem = (size_t)2 * BUF_BYTES + PTAB_BYTES + FUSED_SMEM_FLOATS * 4 + (size_t)kCopySlots * kCopySlotBytes + 128;  // 128: the mbarriers
     static_assert((size_t)2 * BUF_BYTES + PTAB_BYTES + FUSED_SMEM_FLOATS * 4 + (size_t)kCopySlots * kCopySlotBytes + 128 <= 227 * 1024, "shared memory");
@@ -523,14 +663,14 @@ inline int launch(int B, int C, int Ca, int H, int W, const void* x, const void*
     const int dev = current_device();
     if (dev < 0) return kNotApplicable;
     if (!attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(stencil_toeplitz_nchw_bf16<kFused, kMix>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaError_t e = cudaFuncSetAttribute(stencil_toeplitz_nchw_bf16<kFused, kMix, kRagged>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) { (void)cudaGetLastError(); return kNotApplicable; }
         attr_set[dev] = true;
     }
     const long long grid = p.units < sm_count() ? p.units : sm_count();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(Shape<kRagged>::threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -540,8 +680,8 @@ inline int launch(int B, int C, int Ca, int H, int W, const void* x, const void*
     attr[1].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = kFused ? 2 : 1;
-    if (kFused && (grid > sm_count() || p.units > 2 * grid)) return kNotApplicable;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, stencil_toeplitz_nchw_bf16<kFused, kMix>, m_att, p);
+    if (kFused && (grid > sm_count() || p.units > (kRagged && kMix ? 1 : 2) * grid)) return kNotApplicable;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, stencil_toeplitz_nchw_bf16<kFused, kMix, kRagged>, m_att, p);
     if (e != cudaSuccess) {
         char buf[256];
         snprintf(buf, sizeof buf, "stencil_toeplitz_nchw_bf16 launch: %s (%s)", cudaGetErrorName(e), cudaGetErrorString(e));
@@ -552,11 +692,23 @@ inline int launch(int B, int C, int Ca, int H, int W, const void* x, const void*
     return 0;
 }
 
+// Whether this kernel takes the problem, with TMA or with loads of its own.
+inline bool takes(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x, const void* out) {
+    return applies(C, Ca, H, W, K, dtype, layout, x, out) || ragged_applies(B, C, Ca, H, W, K, dtype, layout, x, out);
+}
+
 // Launches the NCHW tensor-core stencil if the problem fits it: 0 on success, kNotApplicable otherwise, or an ESC_ERR_* code.
 inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x, const void* w_large,
                       const float* dk, const float* bias, void* out, unsigned* ctrl, cudaStream_t st, bool dependent,
                       int* launches, std::string* err, const void* w_point = nullptr, bool skip_copy = false) {
-    if (!applies(C, Ca, H, W, K, dtype, layout, x, out) || sm_count() <= 0) return kNotApplicable;
+    if (sm_count() <= 0) return kNotApplicable;
+    if (ragged_applies(B, C, Ca, H, W, K, dtype, layout, x, out)) {
+        if (w_point)
+            return bias ? kNotApplicable
+                        : launch<false, true, true>(B, C, Ca, H, W, x, w_large, dk, bias, out, ctrl, st, dependent, launches, err, nullptr, w_point, skip_copy);
+        return launch<false, false, true>(B, C, Ca, H, W, x, w_large, dk, bias, out, ctrl, st, dependent, launches, err, nullptr, nullptr, skip_copy);
+    }
+    if (!applies(C, Ca, H, W, K, dtype, layout, x, out)) return kNotApplicable;
     if (w_point)
         return bias ? kNotApplicable
                     : launch<false, true>(B, C, Ca, H, W, x, w_large, dk, bias, out, ctrl, st, dependent, launches, err, nullptr, w_point, skip_copy);
@@ -564,7 +716,7 @@ inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int 
 }
 
 inline bool fused_applies(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, int hidden, const void* x, const void* out) {
-    if (!applies(C, Ca, H, W, K, dtype, layout, x, out) || sm_count() <= 0) return false;
+    if (!takes(B, C, Ca, H, W, K, dtype, layout, x, out) || sm_count() <= 0) return false;
     if (Ca > kFusedMaxCa || hidden > kMaxHidden) return false;
     return units_of(B, Ca, H, W) <= 2LL * sm_count();
 }
@@ -574,6 +726,9 @@ inline int try_launch_fused(int B, int C, int Ca, int H, int W, int K, int dtype
                             const toep::Fused& fu, void* out, unsigned* ctrl, cudaStream_t st, int* launches, std::string* err,
                             const void* w_point = nullptr, bool skip_copy = false) {
     if (!fused_applies(B, C, Ca, H, W, K, dtype, layout, fu.hidden, x, out)) return kNotApplicable;
+    if (ragged_applies(B, C, Ca, H, W, K, dtype, layout, x, out))
+        return w_point ? launch<true, true, true>(B, C, Ca, H, W, x, w_large, nullptr, nullptr, out, ctrl, st, false, launches, err, &fu, w_point, skip_copy)
+                       : launch<true, false, true>(B, C, Ca, H, W, x, w_large, nullptr, nullptr, out, ctrl, st, false, launches, err, &fu, nullptr, skip_copy);
     if (w_point)
         return launch<true, true>(B, C, Ca, H, W, x, w_large, nullptr, nullptr, out, ctrl, st, /*dependent=*/false, launches, err, &fu, w_point, skip_copy);
     return launch<true>(B, C, Ca, H, W, x, w_large, nullptr, nullptr, out, ctrl, st, /*dependent=*/false, launches, err, &fu, nullptr, skip_copy);
