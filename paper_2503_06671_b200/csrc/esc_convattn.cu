@@ -25,6 +25,7 @@
 #include "stencil_dense.cuh"
 #include "stencil_dense_umma.cuh"
 #include "stencil_dense_fp32.cuh"
+#include "dense_nchw.cuh"
 #include <type_traits>
 #include "backward.cuh"
 #include "backward_pw.cuh"
@@ -105,6 +106,7 @@ struct Workspace {
     float* partial;
     float* unit_sums;
     void* lk_pad;                    // [Ca][13][13] elements: a smaller large kernel zero-padded for the tensor-core kernels
+    void* packed;                    // C_a = 16: [B][H][W][16] bf16, the attention channels of an NCHW map for the dense form
 };
 
 bool is_large_map(int B, long long HW) { return (long double)B * HW >= 1.5e6L; }
@@ -146,6 +148,7 @@ size_t workspace_bytes(int B, int Ca, long long HW) {
     off += round_up((size_t)B * S * Ca * 4, 256);
     off += round_up((size_t)esc::tma::toep::kMaxFusedUnits * sms_or_nominal() * 16 * 4, 256);   // unit sums of the one-launch form
     off += round_up((size_t)Ca * 169 * 4, 256);            // padded large kernel
+    off += round_up(esc::dense16::packed_bytes(B, Ca, HW), 256);
     return off;
 }
 
@@ -163,6 +166,8 @@ Workspace carve(void* ws, int B, int Ca, long long HW) {
     w.unit_sums = reinterpret_cast<float*>(p);
     p += round_up((size_t)esc::tma::toep::kMaxFusedUnits * sms_or_nominal() * 16 * 4, 256);
     w.lk_pad = p;
+    p += round_up((size_t)Ca * 169 * 4, 256);
+    w.packed = p;
     return w;
 }
 
@@ -496,6 +501,31 @@ int launch_dense_fp32_t(const Problem& p, const void* x, const void* w_dense, co
     return launch_dense_fp32_k<T, LAYOUT, 17>(p, x, w_dense, dk, out, st, dependent);
 }
 
+// bf16 NCHW, dense form: the attention channels packed pixel by pixel, the identity planes copied (out may be null: packing only).
+int launch_pack16(const Problem& p, const void* x, void* packed, void* out, cudaStream_t st) {
+    const long long HW = (long long)p.H * p.W, pixels = (long long)p.B * HW;
+    long long blocks = (pixels + esc::dense16::kThreads - 1) / esc::dense16::kThreads;
+    if (blocks > 8LL * sms_or_nominal()) blocks = 8LL * sms_or_nominal();
+    esc::CopyJob job = {};
+    if (out) job = make_copy_job(p, x, out, blocks, esc::dense16::kThreads);
+    esc::dense16::pack16<<<(unsigned)(blocks + job.blocks), esc::dense16::kThreads, 0, st>>>(
+        static_cast<const __nv_bfloat16*>(x), static_cast<__nv_bfloat16*>(packed), p.C, HW, pixels, (unsigned)blocks, job);
+    ESC_CUDA(cudaGetLastError());
+    ++g_last_launches;
+    return ESC_OK;
+}
+bool wants_packing(const Problem& p) {
+    return g_dense_engine == 0 && esc::dense16::nchw_wants_packing(p.B, p.Ca, p.H, p.W, p.K, p.dtype, p.layout);
+}
+// The tcgen05 kernel on a packed map, results into the NCHW tensor `out`.
+int launch_umma_packed(const Problem& p, const void* packed, const void* w_dense, const float* dk, void* out, unsigned* ctrl,
+                       cudaStream_t st, bool dependent, bool flip) {
+    const int rc = esc::tma::umma::try_launch_dense_umma(p.B, esc::dense16::CA, p.Ca, p.H, p.W, p.K, p.dtype, ESC_NHWC, packed, w_dense, dk, out,
+                                                         ctrl, st, dependent, &g_last_launches, &g_last_error, p.bias, flip, p.C, true);
+    if (rc == ESC_OK) { g_last_path = 5; g_last_tile_w = esc::tma::umma::MW; }
+    return rc;
+}
+
 // Dense large kernel: a tensor-core kernel where one applies, else the FP32-pipe kernel (16 attention channels) or one thread
 // per output (any other channel count).
 int launch_stencil_dense(const Problem& p, const void* x, const void* w_dense, const float* dk, void* out,
@@ -569,8 +599,14 @@ int forward_impl(const Problem& p0, const void* x, const void* w_large0, const E
     }
     const bool tensor_nchw = !p.dense && (!p.w_point || p.Ca == esc::tma::CG) && !p.bias && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
                              esc::tma::toepn::takes(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, out);
-    int rc = launch_gap(p0, x, est, w, w.dk, st, tensor_stencil_follows(p) || tensor_nchw);
+    const bool packed = p0.dense && wants_packing(p0);
+    int rc = packed ? launch_pack16(p0, x, w.packed, out, st) : ESC_OK;
+    if (rc == ESC_OK) rc = launch_gap(p0, x, est, w, w.dk, st, tensor_stencil_follows(p) || tensor_nchw);
     if (rc != ESC_OK) return rc;
+    if (packed) {
+        rc = launch_umma_packed(p0, w.packed, w_large0, w.dk, out, w.ctrl, st, /*dependent=*/true, /*flip=*/false);
+        if (rc != esc::tma::kNotApplicable) return rc;
+    }
     if (p0.dense) return launch_stencil_dense(p0, x, w_large0, w.dk, out, w.ctrl, st, /*dependent=*/true);
     return launch_stencil(p0, x, w_large0, w.dk, out, w.ctrl, st, /*dependent=*/true, &tl);
 }
@@ -590,8 +626,9 @@ struct BackwardWs {
     size_t bytes;
     float* dense_part;               // dense large kernel: the blocks' tap sums [blocks][16][16][169]
     void* wd_flip;                   // the dense kernel with swapped channel axes and rotated taps
+    void *x_packed, *go_packed;      // bf16 NCHW tensors: the attention channels of x and grad_out, [B][H][W][16]
     int dense_blocks;
-    size_t bytes_dense;              // bytes with those two behind the rest
+    size_t bytes_dense;              // bytes with those behind the rest
 };
 BackwardWs carve_backward(void* ws, const Problem& p) {
     // sized for whichever tiling of the tap-gradient kernels has more tiles (32x32, or 64x16 on the tensor cores)
@@ -620,6 +657,9 @@ BackwardWs carve_backward(void* ws, const Problem& p) {
     w.dense_blocks = sms_or_nominal();
     w.dense_part = reinterpret_cast<float*>(base + off); off += round_up((size_t)w.dense_blocks * esc::bwd::dense::kPartFloats * 4, 256);
     w.wd_flip = base + off;                              off += round_up((size_t)esc::bwd::dense::CA * esc::bwd::dense::CA * esc::bwd::TAPS * 4, 256);
+    const size_t pk = round_up(esc::dense16::packed_bytes(p.B, p.Ca, (long long)p.H * p.W), 256);
+    w.x_packed = base + off;  off += pk;
+    w.go_packed = base + off; off += pk;
     w.bytes_dense = off;
     return w;
 }
@@ -831,10 +871,14 @@ int dense_tap_grad_t(const Problem& p, const void* x, const void* go, const Back
 // the constants.  The tcgen05 kernel reads the weights that way and adds the constants itself; for the others the rotated
 // kernel is written first, and the mma.sync kernel's result gets the constants in a pass of its own.
 template <typename T, int LAYOUT>
-int dense_grad_x_t(Problem p, const void* go, const void* w_dense, void* gx, const BackwardWs& w, cudaStream_t st) {
+int dense_grad_x_t(Problem p, const void* go, const void* w_dense, void* gx, const BackwardWs& w, bool packed, cudaStream_t st) {
     namespace D = esc::bwd::dense;
     p.dense = true;
     p.bias = w.bias;
+    if (packed) {                                            // go_packed is there, and gx has its identity planes
+        const int rp = launch_umma_packed(p, w.go_packed, w_dense, w.dk_flip, gx, w.ctrl, st, /*dependent=*/true, /*flip=*/true);
+        if (rp != esc::tma::kNotApplicable) return rp;
+    }
     // dependent: grad_out and the weights are older than the estimator's kernels, which alone it has to wait for
     int rc = launch_stencil_dense(p, go, w_dense, w.dk_flip, gx, w.ctrl, st, /*dependent=*/true, /*flip=*/true);
     if (rc != esc::tma::kNotApplicable) return rc;
@@ -1256,7 +1300,14 @@ int esc_convattn_stencil_dense(const void* x, int B, int C, int C_a, int H, int 
     if (workspace) {
         rc = check_workspace(p, workspace, workspace_bytes_);
         if (rc != ESC_OK) return rc;
-        ctrl = carve(workspace, B, C_a, (long long)H * W).ctrl;
+        const Workspace w = carve(workspace, B, C_a, (long long)H * W);
+        ctrl = w.ctrl;
+        if (wants_packing(p)) {
+            cudaStream_t st = static_cast<cudaStream_t>(stream);
+            rc = launch_pack16(p, x, w.packed, out, st);
+            if (rc == ESC_OK) rc = launch_umma_packed(p, w.packed, w_dense, dk, out, ctrl, st, /*dependent=*/false, /*flip=*/false);
+            if (rc != esc::tma::kNotApplicable) return rc;
+        }
     }
     return launch_stencil_dense(p, x, w_dense, dk, out, ctrl, static_cast<cudaStream_t>(stream), /*dependent=*/false);
 }
@@ -1437,9 +1488,23 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
         w.mixed = true;
     }
     const void* x_taps = w_point ? grad_x : x;             // what the depth-wise stage saw
+    bool packed = false;
     if (dense) {
         // w_large is the dense kernel [16][16][K][K]: its gradient here; the depth-wise kernels
         // below give g_dk (the middle 3 x 3 of their tap gradients) and what follows from it
+        packed = wants_packing(p) && g_engine_policy != ESC_ENGINE_FP32;
+        if (packed) {
+            // bf16 NCHW: everything that follows reads the packed attention channels, as NHWC tensors of 16 channels
+            rc = launch_pack16(p, x, w.x_packed, nullptr, st);
+            if (rc == ESC_OK) rc = launch_pack16(p, grad_out, w.go_packed, grad_x, st);
+            if (rc != ESC_OK) return rc;
+            Problem q = p;
+            q.C = esc::dense16::CA; q.layout = ESC_NHWC; q.dense = true;
+            rc = dense_tap_grad_t<__nv_bfloat16, esc::kNHWC>(q, w.x_packed, w.go_packed, w, g_wd, st);
+            if (rc == ESC_OK) rc = backward_t<__nv_bfloat16, esc::kNHWC>(q, w.x_packed, w.go_packed, w_large, est, w, g, st);
+            if (rc != ESC_OK) return rc;
+            return dense_grad_x_t<__nv_bfloat16, esc::kNCHW>(p, grad_out, w_large, grad_x, w, true, st);
+        }
         rc = dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_tap_grad_t<float, esc::kNCHW>(p, x, grad_out, w, g_wd, st)
                                                     : dense_tap_grad_t<float, esc::kNHWC>(p, x, grad_out, w, g_wd, st))
                               : (layout == ESC_NCHW ? dense_tap_grad_t<__nv_bfloat16, esc::kNCHW>(p, x, grad_out, w, g_wd, st)
@@ -1457,10 +1522,10 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
     // grad_x: the forward stencil on grad_out with both kernels rotated by 180 degrees, plus the constants (in the
     // decomposed form the constants belong behind the transposed mix: the last kernel adds them)
     if (dense)
-        return dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_grad_x_t<float, esc::kNCHW>(p, grad_out, w_large, grad_x, w, st)
-                                                      : dense_grad_x_t<float, esc::kNHWC>(p, grad_out, w_large, grad_x, w, st))
-                                : (layout == ESC_NCHW ? dense_grad_x_t<__nv_bfloat16, esc::kNCHW>(p, grad_out, w_large, grad_x, w, st)
-                                                      : dense_grad_x_t<__nv_bfloat16, esc::kNHWC>(p, grad_out, w_large, grad_x, w, st));
+        return dtype == ESC_F32 ? (layout == ESC_NCHW ? dense_grad_x_t<float, esc::kNCHW>(p, grad_out, w_large, grad_x, w, packed, st)
+                                                      : dense_grad_x_t<float, esc::kNHWC>(p, grad_out, w_large, grad_x, w, packed, st))
+                                : (layout == ESC_NCHW ? dense_grad_x_t<__nv_bfloat16, esc::kNCHW>(p, grad_out, w_large, grad_x, w, packed, st)
+                                                      : dense_grad_x_t<__nv_bfloat16, esc::kNHWC>(p, grad_out, w_large, grad_x, w, packed, st));
     p.bias = w_point ? nullptr : w.bias;
     const TensorLk tl = tensor_lk(p, grad_out, grad_x, w.w_flip, w.lk_pad, st);
     rc = launch_stencil(p, grad_out, w.w_flip, w.dk_flip, grad_x, w.ctrl, st, /*dependent=*/false, &tl);

@@ -73,6 +73,8 @@ struct Params {
     const float* dk;                  // [B][16][9]
     const float* bias;                // [B][16] added to every output of an (image, channel), or nullptr
     __nv_bfloat16* out;
+    int out_c;                        // channels of out; its layout: NHWC, or NCHW (x then is the packed map of 16 channels)
+    int out_nchw;
     unsigned* ctrl;
     int wait_first;
     int copy_cc, copy_pw;             // identity channels; pixels of a strip row per copy chunk (0: nothing to copy)
@@ -445,14 +447,19 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
             float acc[CG];
 #pragma unroll
             for (int c = 0; c < CG; ++c) acc[c] = __uint_as_float(r[c]) + (d0[c] + c0[c]);
-            if (x < p.W) {
+            if (x < p.W && p.out_nchw) {                                      // 64 contiguous bytes of a plane per warp and store
+                const size_t plane = (size_t)p.H * p.W;
+                __nv_bfloat16* dst = p.out + (size_t)b * p.out_c * plane + (size_t)(ya + yr) * p.W + x;
+#pragma unroll
+                for (int c = 0; c < CG; ++c) dst[c * plane] = __float2bfloat16_rn(acc[c]);
+            } else if (x < p.W) {
                 uint32_t o[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const __nv_bfloat162 h2 = __floats2bfloat162_rn(acc[2 * q], acc[2 * q + 1]);
                     o[q] = *reinterpret_cast<const uint32_t*>(&h2);
                 }
-                uint4* dst = reinterpret_cast<uint4*>(p.out + (((size_t)b * p.H + ya + yr) * p.W + x) * p.C);
+                uint4* dst = reinterpret_cast<uint4*>(p.out + (((size_t)b * p.H + ya + yr) * p.W + x) * p.out_c);
                 dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
                 dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
             }
@@ -474,7 +481,8 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
 // [B][H][W][C] bf16 as a 4-D map {C, W, H, B} with a box of 8 channels x SPX pixels x 1 row.
 inline int try_launch_dense_umma(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x,
                                  const void* w_dense, const float* dk, void* out, unsigned* ctrl, cudaStream_t st,
-                                 bool dependent, int* launches, std::string* err, const float* bias = nullptr, bool flip = false) {
+                                 bool dependent, int* launches, std::string* err, const float* bias = nullptr, bool flip = false,
+                                 int out_c = 0, bool out_nchw = false) {
     if (K > K13 || dtype != 1 /*bf16*/ || layout != kNHWC || Ca != CG || C % 8 != 0) return kNotApplicable;
     if ((reinterpret_cast<uintptr_t>(w_dense) & 1) != 0) return kNotApplicable;
     const int sms = sm_count();
@@ -493,6 +501,7 @@ inline int try_launch_dense_umma(int B, int C, int Ca, int H, int W, int K, int 
     if (ctas > 0x3fffffffLL) return kNotApplicable;
     p.w_dense = static_cast<const __nv_bfloat16*>(w_dense);
     p.dk = dk; p.out = static_cast<__nv_bfloat16*>(out); p.ctrl = ctrl;
+    p.out_c = out_c > 0 ? out_c : C; p.out_nchw = out_nchw ? 1 : 0;
     p.wait_first = dependent ? 0 : 1;
     p.raw_bulk = (reinterpret_cast<uintptr_t>(w_dense) & 15) == 0 ? 1 : 0;
     p.KK = K; p.flip = flip ? 1 : 0; p.bias = bias;
