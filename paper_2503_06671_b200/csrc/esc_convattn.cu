@@ -119,9 +119,9 @@ int sms_or_nominal() {
 }
 
 // Grid policy of the GAP kernel.  Narrow: at most one block per SM, which is what fits beside a CTA of the
-// FP32 stencil kernel (58 k registers).  Wide: three blocks per SM -- for maps so large that the stencil
-// kernel takes many waves and the GAP kernel runs ahead of it rather than beside it, and for batches in
-// front of the tensor-core stencil kernel, whose CTAs need every image's dk early (measured on 64 patches
+// FP32 stencil kernel (58 k registers).  Wide: three blocks per SM (two larger ones in launch_gap_t) -- for maps
+// so large that the stencil kernel takes many waves and the GAP kernel runs ahead of it rather than beside it, and for
+// batches in front of the tensor-core stencil kernel, whose CTAs need every image's dk early (measured on 64 patches
 // of 64x64: 35.5 us per forward against 37.8; a single 640x360 map: 37.4 against 36.2, so single images
 // keep the narrow grid).
 bool wide_gap(int B, long long HW, bool tensor_stencil) {
@@ -185,15 +185,12 @@ struct Estimator {
     int hidden;
 };
 
-template <typename T, int LAYOUT>
-int launch_gap_t(const Problem& p, const void* x, const Estimator& est,
-                 const Workspace& w, float* dk_out, cudaStream_t st, bool wide) {
-    const int S = slabs_for(p.B, (long long)p.H * p.W, wide);
-    const int sms = sms_or_nominal();
+template <typename T, int LAYOUT, int kThreads>
+int launch_gap_n(const Problem& p, const void* x, const Estimator& est, const Workspace& w, float* dk_out, cudaStream_t st, int S,
+                 long long cap) {
     const long long items = (long long)p.B * S;
-    const long long cap = wide ? 3LL * sms : sms;
     const unsigned grid = (unsigned)(items < cap ? items : cap);
-    const size_t scratch = (size_t)esc::gap_scratch_floats(LAYOUT, p.C, p.Ca, esc::Elem<T>::kVec);
+    const size_t scratch = (size_t)esc::gap_scratch_floats(LAYOUT, p.C, p.Ca, esc::Elem<T>::kVec, kThreads);
     const size_t smem = (scratch + p.Ca) * sizeof(float);
     if (smem > 48 * 1024) return ESC_ERR_UNSUPPORTED;
     // Same shared-memory carve-out as the stencil kernel: an SM changes its L1/shared split only
@@ -202,17 +199,31 @@ int launch_gap_t(const Problem& p, const void* x, const Estimator& est,
     const int dev = esc::tma::current_device();
     if (dev < 0) return ESC_ERR_UNSUPPORTED;
     if (!carveout_set[dev]) {
-        ESC_CUDA(cudaFuncSetAttribute(esc::gap_dynkernel<T, LAYOUT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+        ESC_CUDA(cudaFuncSetAttribute(esc::gap_dynkernel<T, LAYOUT, kThreads>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                       cudaSharedmemCarveoutMaxShared));
         carveout_set[dev] = true;
     }
-    esc::gap_dynkernel<T, LAYOUT><<<grid, esc::kGapThreads, smem, st>>>(
+    esc::gap_dynkernel<T, LAYOUT, kThreads><<<grid, kThreads, smem, st>>>(
         static_cast<const T*>(x), p.B, p.C, p.Ca, p.H, p.W, S, static_cast<const T*>(est.w_last),
         static_cast<const T*>(est.b_last), static_cast<const T*>(est.w_down), static_cast<const T*>(est.b_down),
         est.hidden, w.partial, w.arrivals, dk_out);
     ESC_CUDA(cudaGetLastError());
     ++g_last_launches;
     return ESC_OK;
+}
+template <typename T, int LAYOUT>
+int launch_gap_t(const Problem& p, const void* x, const Estimator& est,
+                 const Workspace& w, float* dk_out, cudaStream_t st, bool wide) {
+    const long long HW = (long long)p.H * p.W, sms = sms_or_nominal();
+    const int S = slabs_for(p.B, HW, wide);
+    // Large maps: bound by DRAM and by how many bytes are in flight, so two blocks of 512 threads on each SM instead of three of 128,
+    // as long as their scratch fits (C_a up to 720).  1920x1080 bf16 NHWC, 32 of 64 channels (265 MB of whole lines): 65 -> 58 us.
+    const int smem_large = (esc::gap_scratch_floats(LAYOUT, p.C, p.Ca, esc::Elem<T>::kVec, esc::kGapThreadsLarge) + p.Ca) * 4;
+    if (is_large_map(p.B, HW) && smem_large <= 48 * 1024) {
+        const long long s2 = 2 * sms / p.B < 1 ? 1 : 2 * sms / p.B;
+        return launch_gap_n<T, LAYOUT, esc::kGapThreadsLarge>(p, x, est, w, dk_out, st, S < s2 ? S : (int)s2, 2 * sms);
+    }
+    return launch_gap_n<T, LAYOUT, esc::kGapThreads>(p, x, est, w, dk_out, st, S, wide ? 3 * sms : sms);
 }
 
 int launch_gap(const Problem& p, const void* x, const Estimator& est,
