@@ -296,46 +296,57 @@ esc::CopyJob make_copy_job(const Problem& p, const void* x, void* out, long long
     return j;
 }
 
-template <typename T, int LAYOUT>
-int launch_generic_t(const Problem& p, const void* x, const void* w_large, const float* dk, void* out,
-                     cudaStream_t st, bool dependent) {
-    const bool regtile = p.K == esc::kRtK;             // the paper's kernel size: a patch of outputs per thread
-    // small launches: smaller tiles, more blocks, so that every SM has several
-    auto blocks_of = [&](int tx, int ty) { return (long long)p.B * p.Ca * ((p.W + tx - 1) / tx) * ((p.H + ty - 1) / ty); };
-    const bool small = regtile && blocks_of(esc::kRtTX, esc::kRtTY) < 4LL * sms_or_nominal();
-    const bool tiny = small && blocks_of(esc::RtSmall::TX, esc::RtSmall::TY) < 2LL * sms_or_nominal();
-    const int TX = regtile ? (tiny ? esc::RtTiny::TX : small ? esc::RtSmall::TX : esc::kRtTX) : esc::kGenTX;
-    const int TY = regtile ? (tiny ? esc::RtTiny::TY : small ? esc::RtSmall::TY : esc::kRtTY) : esc::kGenTY;
-    const int tiles_x = (p.W + TX - 1) / TX, tiles_y = (p.H + TY - 1) / TY;
-    const long long blocks = (long long)p.B * p.Ca * tiles_x * tiles_y;
-    const esc::CopyJob job = make_copy_job(p, x, out, blocks, regtile ? esc::kRtThreads : esc::kGenTX * esc::kGenTY);
+template <typename T, int LAYOUT, int KT, class G, int CB, int PER_SM>
+int launch_regtile(const Problem& p, const void* x, const void* w_large, const float* dk, void* out, cudaStream_t st, bool dependent) {
+    using L = esc::RtLayout<G, KT, CB>;
+    const int tiles_x = (p.W + G::TX - 1) / G::TX, tiles_y = (p.H + G::TY - 1) / G::TY;
+    const long long blocks = (long long)p.B * (p.Ca / CB) * tiles_x * tiles_y;
+    const esc::CopyJob job = make_copy_job(p, x, out, blocks, L::Threads);
     if (blocks + job.blocks > 0x7fffffffLL) return ESC_ERR_UNSUPPORTED;
+    const int smem = L::bytes(p.Ca, p.w_point != nullptr);
+    static bool attr_set[esc::tma::kMaxDevices] = {};
+    const int dev = esc::tma::current_device();
+    if (dev < 0) return ESC_ERR_UNSUPPORTED;
+    if (!attr_set[dev]) {
+        ESC_CUDA(cudaFuncSetAttribute(esc::stencil_regtile<T, LAYOUT, KT, G, CB, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        attr_set[dev] = true;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(blocks + job.blocks));   // the copy blocks come last
-    cfg.blockDim = regtile ? dim3(esc::kRtThreads) : dim3(esc::kGenTX, esc::kGenTY);
+    cfg.blockDim = dim3(L::Threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = dependent ? 1 : 0;
-    if (regtile && tiny)
-        ESC_CUDA(cudaLaunchKernelEx(&cfg, esc::stencil_k13_regtile<T, LAYOUT, esc::RtTiny>, static_cast<const T*>(x),
-                                    static_cast<T*>(out), p.C, p.Ca, p.H, p.W, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk,
-                                    tiles_x, tiles_y, job, p.bias));
-    else if (regtile && small)
-        ESC_CUDA(cudaLaunchKernelEx(&cfg, esc::stencil_k13_regtile<T, LAYOUT, esc::RtSmall>, static_cast<const T*>(x),
-                                    static_cast<T*>(out), p.C, p.Ca, p.H, p.W, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk,
-                                    tiles_x, tiles_y, job, p.bias));
-    else if (regtile)
-        ESC_CUDA(cudaLaunchKernelEx(&cfg, esc::stencil_k13_regtile<T, LAYOUT, esc::RtLarge>, static_cast<const T*>(x),
-                                    static_cast<T*>(out), p.C, p.Ca, p.H, p.W, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk,
-                                    tiles_x, tiles_y, job, p.bias));
-    else
-        ESC_CUDA(cudaLaunchKernelEx(&cfg, esc::stencil_generic<T, LAYOUT>, static_cast<const T*>(x), static_cast<T*>(out),
-                                    p.C, p.Ca, p.H, p.W, p.K, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk, tiles_x, tiles_y, job, p.bias));
+    ESC_CUDA(cudaLaunchKernelEx(&cfg, esc::stencil_regtile<T, LAYOUT, KT, G, CB, PER_SM>, static_cast<const T*>(x), static_cast<T*>(out), p.C, p.Ca, p.H,
+                                p.W, p.K, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk, tiles_x, tiles_y, job, p.bias));
     ++g_last_launches;
     return ESC_OK;
+}
+template <typename T, int LAYOUT, int KT>
+int launch_regtile_k(const Problem& p, const void* x, const void* w_large, const float* dk, void* out, cudaStream_t st, bool dependent) {
+    auto fewer = [&](int cb, long long per_sm) {           // blocks of the larger geometry
+        using G = esc::RtSmall;
+        return (long long)p.B * (p.Ca / cb) * ((p.W + G::TX - 1) / G::TX) * ((p.H + G::TY - 1) / G::TY) < per_sm * sms_or_nominal();
+    };
+    // four channels per block: whole groups of four, their pixels' loads aligned, and the point-wise filter within shared memory
+    const bool four = p.Ca % 4 == 0 && (LAYOUT == esc::kNHWC ? p.C % 4 == 0 : p.w_point != nullptr) && (!p.w_point || p.Ca <= 1024);
+    if (four) {
+        if (fewer(4, 1)) return launch_regtile<T, LAYOUT, KT, esc::RtTiny, 4, 2>(p, x, w_large, dk, out, st, dependent);
+        return launch_regtile<T, LAYOUT, KT, esc::RtSmall, 4, 2>(p, x, w_large, dk, out, st, dependent);
+    }
+    if (fewer(1, 2)) return launch_regtile<T, LAYOUT, KT, esc::RtTiny, 1, 6>(p, x, w_large, dk, out, st, dependent);
+    if (fewer(1, 6)) return launch_regtile<T, LAYOUT, KT, esc::RtSmall, 1, 6>(p, x, w_large, dk, out, st, dependent);
+    return launch_regtile<T, LAYOUT, KT, esc::RtSmall, 1, 8>(p, x, w_large, dk, out, st, dependent);
+}
+template <typename T, int LAYOUT>
+int launch_generic_t(const Problem& p, const void* x, const void* w_large, const float* dk, void* out, cudaStream_t st, bool dependent) {
+    if (p.K <= 9) return launch_regtile_k<T, LAYOUT, 9>(p, x, w_large, dk, out, st, dependent);
+    if (p.K <= 13) return launch_regtile_k<T, LAYOUT, 13>(p, x, w_large, dk, out, st, dependent);
+    return launch_regtile_k<T, LAYOUT, 17>(p, x, w_large, dk, out, st, dependent);
 }
 
 int launch_generic(const Problem& p, const void* x, const void* w_large, const float* dk, void* out,
