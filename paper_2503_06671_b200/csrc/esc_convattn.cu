@@ -414,7 +414,7 @@ int launch_stencil(const Problem& p0, const void* x, const void* w_large0, const
             if (rn != esc::tma::kNotApplicable) return rn;
         }
     }
-    if (p.skip_copy && p.dtype != ESC_F32) return ESC_ERR_UNSUPPORTED;   // of the kernels below only the generic one (all there is for fp32) can leave the identity channels out
+    if (p.skip_copy && p.dtype != ESC_F32 && p.layout == ESC_NHWC) return ESC_ERR_UNSUPPORTED;   // of the kernels below only the generic one (all there is for fp32 and NCHW) can leave the identity channels out
     p.K = p0.K; w_large = w_large0;
     if (g_engine_policy == ESC_ENGINE_TENSOR) return launch_generic(p, x, w_large, dk, out, st, dependent);
     int tile_w = g_tile_policy;
@@ -1056,10 +1056,18 @@ int static_scratch_address(unsigned** out) {
 // ---- host-buffer path ---------------------------------------------------------------------
 struct HostPath {
     int dev = -1;
-    cudaStream_t st = nullptr;
+    cudaStream_t st = nullptr, compute = nullptr, down = nullptr;   // st: uploads, and the order of the slot's calls
+    cudaEvent_t ev = nullptr;
     void *x = nullptr, *out = nullptr, *wts = nullptr, *ws = nullptr;
     size_t xbytes = 0, wbytes = 0, wsbytes = 0;
 };
+// NCHW keeps the identity channels of an image in one contiguous piece, which neither kernel needs: it is uploaded behind the attention
+// channels and goes back, chunk by chunk, while the next chunk comes in and the kernels run.  (NHWC interleaves them with the
+// attention channels pixel by pixel; strided copies of the two parts take longer than the overlap gains: 96 of every 128 bytes
+// 0.60 ms and 32 of 128 0.44 ms against 0.52 ms for the whole map of 640x360x64 bf16.)  From 1 MB of identity channels on;
+// chunks of 4 MB, about 80 us each.  Blocking call, bf16: 640x360x64 1115 -> 890 us (1 MB chunks 1330, 16 MB 1220), 352x352x48
+// 614 -> 390, 120x96x64 (1.1 MB) 106 -> 95; fp32 640x360x64 2328 -> 1640.
+constexpr size_t kHostOverlapBytes = 1 << 20, kHostChunkBytes = 4 << 20;
 constexpr int kHostSlots = 2;
 std::mutex g_host_mu;
 HostPath g_host[kHostSlots];
@@ -1725,11 +1733,17 @@ int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C,
             if (h.st) cudaStreamSynchronize(h.st);
             cudaFree(h.x); cudaFree(h.out); cudaFree(h.wts); cudaFree(h.ws);
             if (h.st) cudaStreamDestroy(h.st);
+            if (h.compute) cudaStreamDestroy(h.compute);
+            if (h.down) cudaStreamDestroy(h.down);
+            if (h.ev) cudaEventDestroy(h.ev);
             ESC_CUDA(cudaSetDevice(dev));
         }
         h = HostPath();
         h.dev = dev;
         ESC_CUDA(cudaStreamCreateWithFlags(&h.st, cudaStreamNonBlocking));
+        ESC_CUDA(cudaStreamCreateWithFlags(&h.compute, cudaStreamNonBlocking));
+        ESC_CUDA(cudaStreamCreateWithFlags(&h.down, cudaStreamNonBlocking));
+        ESC_CUDA(cudaEventCreateWithFlags(&h.ev, cudaEventDisableTiming));
     }
     const size_t es = p.es(), xbytes = p.elems() * es;
     const size_t n_wl = (size_t)C_a * K * K, n_wd = (size_t)9 * C_a * C_a, n_bd = (size_t)9 * C_a;
@@ -1756,14 +1770,48 @@ int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C,
         h.wsbytes = wsbytes;
     }
     char* wts = static_cast<char*>(h.wts);
-    ESC_CUDA(cudaMemcpyAsync(h.x, x_host, xbytes, cudaMemcpyHostToDevice, h.st));
+    const size_t image = xbytes / B, att = (size_t)C_a * H * W * es, identity = image - att;
+    const bool overlap = layout == ESC_NCHW && identity * B >= kHostOverlapBytes;
+    if (overlap) ESC_CUDA(cudaMemcpy2DAsync(h.x, image, x_host, image, att, B, cudaMemcpyHostToDevice, h.st));
+    else ESC_CUDA(cudaMemcpyAsync(h.x, x_host, xbytes, cudaMemcpyHostToDevice, h.st));
     ESC_CUDA(cudaMemcpyAsync(wts, w_large_host, n_wl * es, cudaMemcpyHostToDevice, h.st));
     ESC_CUDA(cudaMemcpyAsync(wts + off_wd, w_dyn_host, n_wd * es, cudaMemcpyHostToDevice, h.st));
     ESC_CUDA(cudaMemcpyAsync(wts + off_bd, b_dyn_host, n_bd * es, cudaMemcpyHostToDevice, h.st));
-    rc = forward_impl(p, h.x, wts, Estimator{wts + off_wd, wts + off_bd, nullptr, nullptr, 0}, h.out, h.ws, h.st);
-    if (rc != ESC_OK) return rc;
-    ESC_CUDA(cudaMemcpyAsync(out_host, h.out, xbytes, cudaMemcpyDeviceToHost, h.st));
-    return ESC_OK;
+    const Estimator est{wts + off_wd, wts + off_bd, nullptr, nullptr, 0};
+    if (!overlap) {
+        rc = forward_impl(p, h.x, wts, est, h.out, h.ws, h.st);
+        if (rc != ESC_OK) return rc;
+        ESC_CUDA(cudaMemcpyAsync(out_host, h.out, xbytes, cudaMemcpyDeviceToHost, h.st));
+        return ESC_OK;
+    }
+    // `to` goes on only when what `from` has been given so far is done
+    auto follow = [&](cudaStream_t to, cudaStream_t from) -> int {
+        ESC_CUDA(cudaEventRecord(h.ev, from));
+        ESC_CUDA(cudaStreamWaitEvent(to, h.ev, 0));
+        return ESC_OK;
+    };
+    auto enqueue = [&]() -> int {
+        int r = follow(h.compute, h.st);
+        if (r != ESC_OK) return r;
+        Problem pa = p;
+        pa.skip_copy = true;
+        r = forward_impl(pa, h.x, wts, est, h.out, h.ws, h.compute);
+        if (r != ESC_OK) return r;
+        ESC_CUDA(cudaMemcpy2DAsync(out_host, image, h.out, image, att, B, cudaMemcpyDeviceToHost, h.compute));
+        for (int b = 0; b < B; ++b)
+            for (size_t at = att; at < image; at += kHostChunkBytes) {
+                const size_t off = (size_t)b * image + at, n = image - at < kHostChunkBytes ? image - at : kHostChunkBytes;
+                ESC_CUDA(cudaMemcpyAsync(static_cast<char*>(h.x) + off, static_cast<const char*>(x_host) + off, n, cudaMemcpyHostToDevice, h.st));
+                r = follow(h.down, h.st);
+                if (r != ESC_OK) return r;
+                ESC_CUDA(cudaMemcpyAsync(static_cast<char*>(out_host) + off, static_cast<char*>(h.x) + off, n, cudaMemcpyDeviceToHost, h.down));
+            }
+        return ESC_OK;
+    };
+    rc = enqueue();
+    // the slot's stream ends behind the other two, also after an error: who waits for it waits for all
+    const int r1 = follow(h.st, h.compute), r2 = follow(h.st, h.down);
+    return rc != ESC_OK ? rc : r1 != ESC_OK ? r1 : r2;
 }
 
 int esc_convattn_forward_host_wait(int slot) {
