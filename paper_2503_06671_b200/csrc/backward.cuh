@@ -17,27 +17,87 @@
 namespace esc { namespace bwd {
 
 constexpr int K = 13, P = 6, TAPS = K * K;
-constexpr int TX = 64, TY = 64, OX = 8, OY = 4;           // tile of go per block, patch of go per thread
+constexpr int TX = 64, TY = 64;                           // tile of go per block
 constexpr int XP = TX + K - 1;                            // 76 floats per staged x row (a multiple of 4)
 constexpr int XR = TY + K - 1;                            // 76 staged x rows
-constexpr int kThreads = (TX / OX) * (TY / OY);           // 128
+constexpr int kThreads = 128;
 constexpr int kSlot = 176;                                // floats per (image, channel, tile): 169 taps, sum of x, padding
 static_assert(XP % 4 == 0 && TAPS + 1 <= kSlot, "layout");
 
 // ---- kernel 1: per-tile partial tap gradients and partial sums of x ---------------------------------------
-// Block = (image b, attention channel c, 64x64 tile).  The x halo tile (zeros outside the image) and the go
-// tile (zeros outside) are staged in shared memory as fp32; a thread keeps its 4x8 patch of go in registers
-// and, for every kernel row i, reads the four x rows its patch meets (five 16-byte reads each) and forms the
-// 13 partial sums of that row: 416 FMAs per 20 reads.  The 13 sums are then added over the block in a fixed
-// order (shuffle butterfly inside a warp, warps in order).
-template <typename T, int LAYOUT>
-__global__ void __launch_bounds__(kThreads)
+// Block = (image b, attention channel c, 64x64 tile), 128 threads or, with the kernel rows shared among them, four times 128.  The x halo tile (zeros outside the
+// image) and the go tile (zeros outside) are staged in shared memory as fp32; a thread keeps its patch of 8 rows x 4 columns of go in
+// registers (the eight lanes of a 16-byte read phase then sit side by side, free of bank conflicts) and, for every kernel row i, reads
+// the eight x rows its patch meets (four 16-byte reads each) and forms the 13 partial sums of that row: 416 FMAs per 32 reads.  The 13
+// sums are then added over the block in a fixed order: inside a warp by halving -- at each step a lane passes on the half of the values
+// that it does not keep, 16 shuffles where a butterfly per value takes 65 --, then warps in order.
+// Small launches share the kernel rows: one block of four warps an SM is a chain of latencies.  (The NHWC form below shares them among up
+// to four blocks, `row_shares`, which each stage the tile; here that gave 16.7 us for 21.8.)  8 images of 64x64,
+// 16 channels, fp32: 21.8 -> 12.5 us; whole backward of the module, NHWC, 93 -> 77 us, 40 of 48x48 173 -> 148 (NCHW 142 -> 131).
+constexpr int kPY = 8, kPX = 4;                           // a thread's patch of go
+// Sums of s[0 .. 15] over the warp: lane l holds that of value reduce_index(l).
+__device__ __forceinline__ float reduce16(float (&s)[16], int lane) {
+#pragma unroll
+    for (int h = 8, m = 16; h >= 1; h >>= 1, m >>= 1) {
+        const bool up = lane & m;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+            const float send = up ? s[k] : s[k + h], keep = up ? s[k + h] : s[k];
+            s[k] = keep + __shfl_xor_sync(0xffffffffu, send, m);
+        }
+    }
+    return s[0] + __shfl_xor_sync(0xffffffffu, s[0], 1);
+}
+__device__ __forceinline__ int reduce_index(int lane) { return lane >> 1; }
+// The 13 sums of kernel row i over a thread's patch g; xr: the patch's first x row and column for i = 0.
+template <int PITCH>
+__device__ __forceinline__ void row_sums(const float* xr, int i, const float (&g)[kPY][kPX], float (&s)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) s[j] = 0.f;
+#pragma unroll
+    for (int a = 0; a < kPY; ++a) {
+        float in[kPX + K - 1];                            // x row a + i of the patch, 16 columns
+        const float4* xv = reinterpret_cast<const float4*>(xr + (a + i) * PITCH);
+#pragma unroll
+        for (int v = 0; v < (kPX + K - 1) / 4; ++v) {
+            const float4 q = xv[v];
+            in[4 * v] = q.x; in[4 * v + 1] = q.y; in[4 * v + 2] = q.z; in[4 * v + 3] = q.w;
+        }
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+#pragma unroll
+            for (int o = 0; o < kPX; ++o) s[j] = fmaf(g[a][o], in[o + j], s[j]);
+    }
+}
+// A thread's patch of go, and the sum of x over it.
+template <int PITCH, int GPITCH>
+__device__ __forceinline__ float load_patch(const float* xr, const float* gr, float (&g)[kPY][kPX]) {
+    float sx = 0.f;
+#pragma unroll
+    for (int a = 0; a < kPY; ++a) {
+        const float4 q = *reinterpret_cast<const float4*>(gr + a * GPITCH);
+        g[a][0] = q.x; g[a][1] = q.y; g[a][2] = q.z; g[a][3] = q.w;
+        const float4* xv = reinterpret_cast<const float4*>(xr + (a + P) * PITCH + P - 2);   // 16-byte aligned: P - 2 = 4
+        const float4 u0 = xv[0], u1 = xv[1];              // the patch's own pixels are floats 2..5 of these
+        sx += (u0.z + u0.w) + (u1.x + u1.y);
+    }
+    return sx;
+}
+// Blocks that share a tile's kernel rows: as many as it takes to have `per_sm` blocks on every SM, at most four.
+inline int row_shares(long long blocks, int per_sm, int sms) {
+    const long long n = ((long long)per_sm * sms) / (blocks > 0 ? blocks : 1);
+    return n < 1 ? 1 : n > 4 ? 4 : (int)n;
+}
+
+template <typename T, int LAYOUT, int SHARES>
+__global__ void __launch_bounds__(kThreads * SHARES)
 tap_grad(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H, int W, int tiles_x, int tiles_y,
          float* __restrict__ part)      // [B][Ca][tiles][kSlot]
 {
     __shared__ __align__(16) float xt[XR * XP];
     __shared__ __align__(16) float gt[TY * TX];
-    __shared__ float red[kThreads / 32][16];
+    __shared__ float red[K][kThreads / 32][16];
+    __shared__ float redx[kThreads / 32];
 
     long long bid = blockIdx.x;
     const int tiles = tiles_x * tiles_y;
@@ -45,81 +105,61 @@ tap_grad(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H
     const int c = (int)(bid % Ca);
     const int b = (int)(bid / Ca);
     const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int N = kThreads * SHARES;
+    const int all = threadIdx.x, tid = all % kThreads, share = all / kThreads, lane = tid & 31, warp = tid >> 5;
     const int y0 = ty * TY, x0 = tx * TX;
+    const int i0 = K * share / SHARES, i1 = K * (share + 1) / SHARES;        // these 128 threads' kernel rows
 
-    for (int t = tid; t < XR * XP; t += kThreads) {
-        const int r = t / XP, q = t % XP;
-        const int y = y0 - P + r, xx = x0 - P + q;
-        xt[t] = (y >= 0 && y < H && xx >= 0 && xx < W) ? Elem<T>::to_f32(x[elem_index<LAYOUT>(b, c, y, xx, C, H, W)]) : 0.f;
+    constexpr int U = 8;                                  // loads of a thread in flight
+    for (int t0 = all; t0 < XR * XP; t0 += U * N) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = t0 + u * N, r = t / XP, q = t % XP, y = y0 - P + r, xx = x0 - P + q;
+            v[u] = (t < XR * XP && y >= 0 && y < H && xx >= 0 && xx < W) ? Elem<T>::to_f32(x[elem_index<LAYOUT>(b, c, y, xx, C, H, W)]) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (t0 + u * N < XR * XP) xt[t0 + u * N] = v[u];
     }
-    for (int t = tid; t < TY * TX; t += kThreads) {
-        const int r = t / TX, q = t % TX;
-        const int y = y0 + r, xx = x0 + q;
-        gt[t] = (y < H && xx < W) ? Elem<T>::to_f32(go[elem_index<LAYOUT>(b, c, y, xx, C, H, W)]) : 0.f;
+    for (int t0 = all; t0 < TY * TX; t0 += U * N) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int t = t0 + u * N, y = y0 + t / TX, xx = x0 + t % TX;
+            v[u] = (y < H && xx < W) ? Elem<T>::to_f32(go[elem_index<LAYOUT>(b, c, y, xx, C, H, W)]) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) gt[t0 + u * N] = v[u];
     }
+    static_assert(TY * TX % (U * N) == 0 && (TX / kPX) * (TY / kPY) == kThreads, "whole rounds; one patch per thread");
     __syncthreads();
 
-    const int lx = tid % (TX / OX), ly = tid / (TX / OX);
-    float g[OY][OX];
-    float sx = 0.f;                                       // sum of x over the patch (for the GAP of this image)
-#pragma unroll
-    for (int a = 0; a < OY; ++a) {
-        const float4* gr = reinterpret_cast<const float4*>(gt + (ly * OY + a) * TX + lx * OX);
-        const float4 q0 = gr[0], q1 = gr[1];
-        g[a][0] = q0.x; g[a][1] = q0.y; g[a][2] = q0.z; g[a][3] = q0.w;
-        g[a][4] = q1.x; g[a][5] = q1.y; g[a][6] = q1.z; g[a][7] = q1.w;
-        const float4* xr = reinterpret_cast<const float4*>(xt + (ly * OY + a + P) * XP + lx * OX + P - 2);   // 16-byte aligned: P - 2 = 4
-        // the patch's own pixels sit at columns lx*OX + P .. +7: floats 2..9 of the three reads from column lx*OX + 4
-        const float4 u0 = xr[0], u1 = xr[1], u2 = xr[2];
-        sx += (u0.z + u0.w) + (u1.x + u1.y + u1.z + u1.w) + (u2.x + u2.y);
-    }
-    float* slot = part + (((size_t)b * Ca + c) * tiles + tile) * kSlot;
-
+    const int lx = tid % (TX / kPX), ly = tid / (TX / kPX);
+    const float* xr = xt + ly * kPY * XP + lx * kPX;
+    float g[kPY][kPX];
+    float sx = load_patch<XP, TX>(xr, gt + ly * kPY * TX + lx * kPX, g);      // sum of x over the patch (for the GAP of this image)
 #pragma unroll 1
-    for (int i = 0; i < K; ++i) {
-        float s[K];
-#pragma unroll
-        for (int j = 0; j < K; ++j) s[j] = 0.f;
-#pragma unroll
-        for (int a = 0; a < OY; ++a) {
-            float in[OX + K - 1];                         // x row (ly*OY + a + i), columns lx*OX .. lx*OX + 19
-            const float4* xr = reinterpret_cast<const float4*>(xt + (ly * OY + a + i) * XP + lx * OX);
-#pragma unroll
-            for (int v = 0; v < (OX + K - 1) / 4; ++v) {
-                const float4 q = xr[v];
-                in[4 * v] = q.x; in[4 * v + 1] = q.y; in[4 * v + 2] = q.z; in[4 * v + 3] = q.w;
-            }
-#pragma unroll
-            for (int j = 0; j < K; ++j)
-#pragma unroll
-                for (int o = 0; o < OX; ++o) s[j] = fmaf(g[a][o], in[o + j], s[j]);
-        }
-        // block sum of the 13 values, fixed order
-#pragma unroll
-        for (int j = 0; j < K; ++j)
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
-        if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < K; ++j) red[warp][j] = s[j];
-        }
-        __syncthreads();
-        if (tid < K) {
-            float t = 0.f;
-#pragma unroll
-            for (int w = 0; w < kThreads / 32; ++w) t += red[w][tid];
-            slot[i * K + tid] = t;
-        }
-        __syncthreads();
+    for (int i = i0; i < i1; ++i) {
+        float s[16];
+        row_sums<XP>(xr, i, g, s);
+        const float t = reduce16(s, lane);
+        if ((lane & 1) == 0) red[i][warp][reduce_index(lane)] = t;
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
-    if (lane == 0) red[warp][0] = sx;
+    if (lane == 0 && share == 0) redx[warp] = sx;
     __syncthreads();
-    if (tid == 0) {
+    float* slot = part + (((size_t)b * Ca + c) * tiles + tile) * kSlot;
+    for (int e = all; e < TAPS; e += N) {
         float t = 0.f;
-        for (int w = 0; w < kThreads / 32; ++w) t += red[w][0];
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w) t += red[e / K][w][e % K];
+        slot[e] = t;
+    }
+    if (all == 0) {
+        float t = 0.f;
+        for (int w = 0; w < kThreads / 32; ++w) t += redx[w];
         slot[TAPS] = t;
     }
 }
@@ -189,56 +229,24 @@ tap_grad_nhwc8(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca,
     }
     __syncthreads();
 
-    const float* xc = xt + warp * (XR * XP);              // this warp's channel
-    const float* gc = gt + warp * (TY * TX);
-    // A lane's patch is 8 rows x 4 columns here: the eight lanes that share a 16-byte read phase then sit
-    // side by side (16 bytes apart, 128 contiguous bytes) and the reads are free of bank conflicts.
-    constexpr int PY = 8, PX = 4;
-    static_assert((TX / PX) * (TY / PY) == 32, "one warp covers a channel's tile");
-    const int lx = lane % (TX / PX), ly = lane / (TX / PX);
-    float g[PY][PX];
-    float sx = 0.f;
-#pragma unroll
-    for (int a = 0; a < PY; ++a) {
-        const float4 q0 = *reinterpret_cast<const float4*>(gc + (ly * PY + a) * TX + lx * PX);
-        g[a][0] = q0.x; g[a][1] = q0.y; g[a][2] = q0.z; g[a][3] = q0.w;
-        const float4* xr = reinterpret_cast<const float4*>(xc + (ly * PY + a + P) * XP + lx * PX + P - 2);
-        const float4 u0 = xr[0], u1 = xr[1];              // the patch's own pixels are floats 2..5 of these
-        sx += (u0.z + u0.w) + (u1.x + u1.y);
-    }
+    constexpr int TXP = TX / kPX;
+    static_assert(TXP * (TY / kPY) == 32, "one warp covers a channel's tile");
+    const int lx = lane % TXP, ly = lane / TXP;
+    const float* xr = xt + warp * (XR * XP) + ly * kPY * XP + lx * kPX;       // this warp's channel
+    float g[kPY][kPX];
+    float sx = load_patch<XP, TX>(xr, gt + warp * (TY * TX) + ly * kPY * TX + lx * kPX, g);
     float* slot = part + (((size_t)b * Ca + oct * CH + warp) * tiles + tile) * kSlot;
-
+    const int i0 = K * (int)blockIdx.y / (int)gridDim.y, i1 = K * ((int)blockIdx.y + 1) / (int)gridDim.y;   // this block's kernel rows
 #pragma unroll 1
-    for (int i = 0; i < K; ++i) {
-        float s[K];
-#pragma unroll
-        for (int j = 0; j < K; ++j) s[j] = 0.f;
-#pragma unroll
-        for (int a = 0; a < PY; ++a) {
-            float in[PX + K - 1];                         // 16 floats: four 16-byte reads
-            const float4* xr = reinterpret_cast<const float4*>(xc + (ly * PY + a + i) * XP + lx * PX);
-#pragma unroll
-            for (int v = 0; v < (PX + K - 1) / 4; ++v) {
-                const float4 q = xr[v];
-                in[4 * v] = q.x; in[4 * v + 1] = q.y; in[4 * v + 2] = q.z; in[4 * v + 3] = q.w;
-            }
-#pragma unroll
-            for (int j = 0; j < K; ++j)
-#pragma unroll
-                for (int o = 0; o < PX; ++o) s[j] = fmaf(g[a][o], in[o + j], s[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < K; ++j)
-#pragma unroll
-            for (int o = 16; o >= 1; o >>= 1) s[j] += __shfl_xor_sync(0xffffffffu, s[j], o);
-        // after the butterfly every lane holds all 13 sums: lane j writes the j-th
-#pragma unroll
-        for (int j = 0; j < K; ++j)
-            if (lane == j) slot[i * K + j] = s[j];
+    for (int i = i0; i < i1; ++i) {
+        float s[16];
+        row_sums<XP>(xr, i, g, s);
+        const float t = reduce16(s, lane);
+        if ((lane & 1) == 0 && reduce_index(lane) < K) slot[i * K + reduce_index(lane)] = t;
     }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) sx += __shfl_xor_sync(0xffffffffu, sx, o);
-    if (lane == 0) slot[TAPS] = sx;
+    if (lane == 0 && blockIdx.y == 0) slot[TAPS] = sx;
 }
 
 // ---- kernel 2a: add the tiles of one (image, channel) in a fixed order -----------------------------------------

@@ -743,11 +743,17 @@ int backward_t(const Problem& p, const void* x, const void* go, const void* w_la
                                           (int)esc::bwd::n8::kSmemBytes));
             attr_set[dev] = true;
         }
-        esc::bwd::tap_grad_nhwc8<T><<<(unsigned)blocks, esc::bwd::n8::kThreads, esc::bwd::n8::kSmemBytes, st>>>(
+        const dim3 grid8((unsigned)blocks, (unsigned)esc::bwd::row_shares(blocks, 2, sms_or_nominal()));
+        esc::bwd::tap_grad_nhwc8<T><<<grid8, esc::bwd::n8::kThreads, esc::bwd::n8::kSmemBytes, st>>>(
             static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
     } else {
-        esc::bwd::tap_grad<T, LAYOUT><<<(unsigned)blocks, esc::bwd::kThreads, 0, st>>>(
-            static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
+        // fewer than two blocks an SM: four times the threads
+        if (blocks < 2LL * sms_or_nominal())
+            esc::bwd::tap_grad<T, LAYOUT, 4><<<(unsigned)blocks, 4 * esc::bwd::kThreads, 0, st>>>(
+                static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
+        else
+            esc::bwd::tap_grad<T, LAYOUT, 1><<<(unsigned)blocks, esc::bwd::kThreads, 0, st>>>(
+                static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
     }
     ESC_CUDA(cudaGetLastError());
     if (tiles_done == 0) ++g_last_launches;
