@@ -92,6 +92,7 @@ inline int row_shares(long long blocks, int per_sm, int sms) {
 template <typename T, int LAYOUT, int SHARES>
 __global__ void __launch_bounds__(kThreads * SHARES)
 tap_grad(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H, int W, int tiles_x, int tiles_y,
+         int ia, int ib,                // the kernel rows wanted: all, or 5 to 7 where nobody asks for g_lk
          float* __restrict__ part)      // [B][Ca][tiles][kSlot]
 {
     __shared__ __align__(16) float xt[XR * XP];
@@ -108,7 +109,7 @@ tap_grad(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H
     constexpr int N = kThreads * SHARES;
     const int all = threadIdx.x, tid = all % kThreads, share = all / kThreads, lane = tid & 31, warp = tid >> 5;
     const int y0 = ty * TY, x0 = tx * TX;
-    const int i0 = K * share / SHARES, i1 = K * (share + 1) / SHARES;        // these 128 threads' kernel rows
+    const int i0 = ia + (ib - ia) * share / SHARES, i1 = ia + (ib - ia) * (share + 1) / SHARES;        // these 128 threads' kernel rows
 
     constexpr int U = 8;                                  // loads of a thread in flight
     for (int t0 = all; t0 < XR * XP; t0 += U * N) {
@@ -151,7 +152,7 @@ tap_grad(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H
     if (lane == 0 && share == 0) redx[warp] = sx;
     __syncthreads();
     float* slot = part + (((size_t)b * Ca + c) * tiles + tile) * kSlot;
-    for (int e = all; e < TAPS; e += N) {
+    for (int e = ia * K + all; e < ib * K; e += N) {
         float t = 0.f;
 #pragma unroll
         for (int w = 0; w < kThreads / 32; ++w) t += red[e / K][w][e % K];
@@ -180,7 +181,7 @@ static_assert(XP % 4 == 0, "16-byte reads of staged rows");
 template <typename T>
 __global__ void __launch_bounds__(n8::kThreads)
 tap_grad_nhwc8(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H, int W, int tiles_x, int tiles_y,
-               float* __restrict__ part)      // [B][Ca][tiles][kSlot]
+               int ia, int ib, float* __restrict__ part)      // [B][Ca][tiles][kSlot]
 {
     constexpr int TX = n8::TX, TY = n8::TY, CH = n8::CH, XP = n8::XP, XR = n8::XR, kThreads = n8::kThreads;
     constexpr int V = Elem<T>::kVec;                      // elements per 16-byte load: 8 (bf16) or 4 (fp32)
@@ -236,7 +237,7 @@ tap_grad_nhwc8(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca,
     float g[kPY][kPX];
     float sx = load_patch<XP, TX>(xr, gt + warp * (TY * TX) + ly * kPY * TX + lx * kPX, g);
     float* slot = part + (((size_t)b * Ca + oct * CH + warp) * tiles + tile) * kSlot;
-    const int i0 = K * (int)blockIdx.y / (int)gridDim.y, i1 = K * ((int)blockIdx.y + 1) / (int)gridDim.y;   // this block's kernel rows
+    const int i0 = ia + (ib - ia) * (int)blockIdx.y / (int)gridDim.y, i1 = ia + (ib - ia) * ((int)blockIdx.y + 1) / (int)gridDim.y;   // this block's kernel rows
 #pragma unroll 1
     for (int i = i0; i < i1; ++i) {
         float s[16];

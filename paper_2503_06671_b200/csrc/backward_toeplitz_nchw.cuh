@@ -18,7 +18,7 @@
 namespace esc { namespace bwd { namespace toepn {
 
 using tma::CG; using tma::K13; using tma::P6; using tma::u64; using tma::Unit;
-using tma::toep::ldsm_x4; using tma::toep::mma_bf16;
+using tma::toep::ldsm_x2; using tma::toep::ldsm_x4; using tma::toep::mma_bf16;
 constexpr int kWarps = 8, kThreads = kWarps * 32 + 32;
 constexpr int TH = tma::toepn::TH, TW = tma::toepn::TW, ROWS = tma::toepn::ROWS, PP = tma::toepn::PP, XS = tma::toepn::XS;
 constexpr int PLANE = tma::toepn::PLANE, XBUF = tma::toepn::BUF_BYTES;
@@ -48,6 +48,8 @@ __device__ __forceinline__ Unit decode(long long u64v, const Params& p) {
     return r;
 }
 
+// kCentre: as in the NHWC kernel, kernel rows 0 to 7 alone.
+template <bool kCentre>
 __global__ void __launch_bounds__(kThreads, 1)
 tap_grad_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_go, const Params p)
 {
@@ -142,13 +144,14 @@ tap_grad_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_x, const __g
 #pragma unroll
                 for (int ub = 0; ub < NUB; ++ub) {
                     uint32_t b[4];
-                    ldsm_x4(b_lane + (uint32_t)(16 * ub * 2), b);
+                    if (kCentre) ldsm_x2(b_lane + (uint32_t)(16 * ub * 2), b[0], b[1]);
+                    else ldsm_x4(b_lane + (uint32_t)(16 * ub * 2), b);
                     uint32_t a0 = __funnelshift_r(gr[8 * ub], gr[8 * ub + 1], sh);
                     uint32_t a2 = __funnelshift_r(gr[8 * ub + 4], gr[8 * ub + 5], sh);
                     if (ub == 0) { a0 &= m_a0_first; a2 &= m_a2_first; }
                     if (ub == NUB - 1) { a0 &= m_a0_last; a2 &= m_a2_last; }
                     mma_bf16(d0, a0, a_prev, a2, a0, b[0], b[1]);
-                    mma_bf16(d1, a0, a_prev, a2, a0, b[2], b[3]);
+                    if (!kCentre) mma_bf16(d1, a0, a_prev, a2, a0, b[2], b[3]);
                     a_prev = a2;
                 }
             }
@@ -159,8 +162,8 @@ tap_grad_toeplitz_nchw_bf16(const __grid_constant__ CUtensorMap map_x, const __g
                     const int i0 = 2 * t, i1 = 8 + 2 * t;
                     slot[i0 * K13 + j] = d0[2 * h];
                     slot[(i0 + 1) * K13 + j] = d0[2 * h + 1];
-                    if (i1 < K13) slot[i1 * K13 + j] = d1[2 * h];
-                    if (i1 + 1 < K13) slot[(i1 + 1) * K13 + j] = d1[2 * h + 1];
+                    if (!kCentre && i1 < K13) slot[i1 * K13 + j] = d1[2 * h];
+                    if (!kCentre && i1 + 1 < K13) slot[(i1 + 1) * K13 + j] = d1[2 * h + 1];
                 }
             }
         }
@@ -182,7 +185,8 @@ inline int make_map_go(CUtensorMap* m, const void* base, int B, int C, int H, in
 }
 
 // 0 on success, tma::kNotApplicable where the kernel does not take the problem, else an ESC_ERR_* code.
-inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x, const void* go,
+template <bool kCentre>
+inline int launch(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x, const void* go,
                       float* part, unsigned* ctrl, cudaStream_t st, int* launches, std::string* err) {
     if (!tma::toepn::applies(C, Ca, H, W, K, dtype, layout, x, go) || tma::sm_count() <= 0) return tma::kNotApplicable;
     Params p;
@@ -198,12 +202,12 @@ inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int 
     const int dev = tma::current_device();
     if (dev < 0) return tma::kNotApplicable;
     if (!attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(tap_grad_toeplitz_nchw_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+        cudaError_t e = cudaFuncSetAttribute(tap_grad_toeplitz_nchw_bf16<kCentre>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (e != cudaSuccess) { (void)cudaGetLastError(); return tma::kNotApplicable; }
         attr_set[dev] = true;
     }
     const long long grid = p.units < tma::sm_count() ? p.units : tma::sm_count();
-    tap_grad_toeplitz_nchw_bf16<<<(unsigned)grid, kThreads, kSmemBytes, st>>>(m_x, m_go, p);
+    tap_grad_toeplitz_nchw_bf16<kCentre><<<(unsigned)grid, kThreads, kSmemBytes, st>>>(m_x, m_go, p);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         char buf[256];
@@ -213,6 +217,11 @@ inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int 
     }
     ++*launches;
     return 0;
+}
+inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int layout, const void* x, const void* go,
+                      float* part, unsigned* ctrl, cudaStream_t st, int* launches, std::string* err, bool centre_only) {
+    return centre_only ? launch<true>(B, C, Ca, H, W, K, dtype, layout, x, go, part, ctrl, st, launches, err)
+                       : launch<false>(B, C, Ca, H, W, K, dtype, layout, x, go, part, ctrl, st, launches, err);
 }
 
 }}}  // namespace esc::bwd::toepn

@@ -716,12 +716,12 @@ int backward_t(const Problem& p, const void* x, const void* go, const void* w_la
     int tiles_done = 0;
     if (g_engine_policy != ESC_ENGINE_FP32) {
         const int rt = esc::bwd::toep::try_launch(p.B, p.C, p.Ca, p.H, p.W, esc::bwd::K, p.dtype, p.layout, x, go, w.part, w.ctrl, st,
-                                                  &g_last_launches, &g_last_error);
+                                                  &g_last_launches, &g_last_error, /*centre_only=*/!g.g_lk);
         if (rt == ESC_OK) tiles_done = esc::bwd::toep::tiles_of(p.H, p.W);
         else if (rt != esc::tma::kNotApplicable) return rt;
         if (tiles_done == 0) {                               // the same on NCHW tensors
             const int rn = esc::bwd::toepn::try_launch(p.B, p.C, p.Ca, p.H, p.W, esc::bwd::K, p.dtype, p.layout, x, go, w.part, w.ctrl, st,
-                                                       &g_last_launches, &g_last_error);
+                                                       &g_last_launches, &g_last_error, /*centre_only=*/!g.g_lk);
             if (rn == ESC_OK) tiles_done = esc::bwd::toep::tiles_of(p.H, p.W);
             else if (rn != esc::tma::kNotApplicable) return rn;
         }
@@ -732,6 +732,7 @@ int backward_t(const Problem& p, const void* x, const void* go, const void* w_la
     const int tiles_x = (p.W + TXs - 1) / TXs, tiles_y = (p.H + TYs - 1) / TYs;
     const long long blocks = (long long)p.B * (oct ? p.Ca / 8 : p.Ca) * tiles_x * tiles_y;
     if (blocks > 0x7fffffffLL) return ESC_ERR_UNSUPPORTED;
+    const int ia = g.g_lk ? 0 : esc::bwd::P - 1, ib = g.g_lk ? esc::bwd::K : esc::bwd::P + 2;   // without g_lk only the middle is read
     if (tiles_done > 0) {
         // done above
     } else if (oct) {
@@ -745,15 +746,15 @@ int backward_t(const Problem& p, const void* x, const void* go, const void* w_la
         }
         const dim3 grid8((unsigned)blocks, (unsigned)esc::bwd::row_shares(blocks, 2, sms_or_nominal()));
         esc::bwd::tap_grad_nhwc8<T><<<grid8, esc::bwd::n8::kThreads, esc::bwd::n8::kSmemBytes, st>>>(
-            static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
+            static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, ia, ib, w.part);
     } else {
         // fewer than two blocks an SM: four times the threads
         if (blocks < 2LL * sms_or_nominal())
             esc::bwd::tap_grad<T, LAYOUT, 4><<<(unsigned)blocks, 4 * esc::bwd::kThreads, 0, st>>>(
-                static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
+                static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, ia, ib, w.part);
         else
             esc::bwd::tap_grad<T, LAYOUT, 1><<<(unsigned)blocks, esc::bwd::kThreads, 0, st>>>(
-                static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, w.part);
+                static_cast<const T*>(x), static_cast<const T*>(go), p.C, p.Ca, p.H, p.W, tiles_x, tiles_y, ia, ib, w.part);
     }
     ESC_CUDA(cudaGetLastError());
     if (tiles_done == 0) ++g_last_launches;

@@ -48,3 +48,26 @@ def test_tap_gradients(case, layout):
     assert bool(((g_bd - gdk.sum(0)).abs() <= 1e-5 * mdk.sum(0)).all())
     mean, amean = x[:, :C_a].double().mean((2, 3)), x[:, :C_a].double().abs().mean((2, 3))
     assert bool(((g_wd - gdk.T @ mean).abs() <= 2e-5 * (mdk.T @ amean)).all())
+
+
+@pytest.mark.parametrize("layout", [synth.NCHW, synth.NHWC], ids=["nchw", "nhwc"])
+@pytest.mark.parametrize("dtype", [synth.F32, synth.BF16], ids=["fp32", "bf16"])
+def test_without_the_large_kernels_gradient(dtype, layout):
+    """Without g_lk only the middle kernel rows are formed: the other gradients keep their bits."""
+    import torch
+
+    import paper_2503_06671_b200 as pkg
+
+    B, C, C_a, H, W, K = 3, 32, 16, 37, 136, 13
+    g = torch.Generator(device="cuda").manual_seed(7)
+    dt = torch.bfloat16 if dtype == synth.BF16 else torch.float32
+    x, go = (torch.randn((B, C, H, W) if layout == synth.NCHW else (B, H, W, C), generator=g, device="cuda").to(dt) for _ in range(2))
+    wl, wd, bd = (torch.randn(s, generator=g, device="cuda").to(dt) / 13 for s in ((C_a, K, K), (9 * C_a, C_a), (9 * C_a,)))
+    res = []
+    for lk in (torch.zeros((C_a, K, K), device="cuda"), None):
+        gx, g_wd, g_bd = torch.empty_like(x), torch.zeros(wd.shape, device="cuda"), torch.zeros(bd.shape, device="cuda")
+        ws = pkg.new_backward_workspace(B, C_a, H, W, K)
+        pkg.esc_convattn_backward(x, go, C_a, K, wl, wd, bd, gx, lk, g_wd, g_bd, pkg.ESC_NHWC if layout == synth.NHWC else pkg.ESC_NCHW, ws)
+        torch.cuda.synchronize()
+        res.append((gx, g_wd, g_bd))
+    assert all(torch.equal(a, b) for a, b in zip(*res))
