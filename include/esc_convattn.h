@@ -162,8 +162,9 @@ int esc_convattn_stencil(const void* x, int B, int C, int C_a, int H, int W, int
 
 /*
  * End-to-end convenience call on HOST buffers: copies x and the weights to the device,
- * runs the forward pass, copies out back and synchronises.  Device buffers and a private
- * stream are kept by the library between calls.  Host buffers should be pinned for full
+ * runs the forward pass, copies out back and synchronises.  Device buffers and private
+ * streams are kept by the library between calls.  On NCHW tensors the identity channels travel
+ * beside the kernels: their upload, and their way back, overlap the rest.  Host buffers should be pinned for full
  * copy bandwidth but need not be.
  */
 int esc_convattn_forward_host(const void* x_host, int B, int C, int C_a, int H, int W, int K,
@@ -396,15 +397,17 @@ int esc_convattn_last_path(void);
 /* Which arithmetic units evaluate the depth-wise large-kernel stage of Eq. 4 line 3 on bf16 tensors (and the tap
  * gradients of the backward pass), for later calls on this thread.  ESC_ENGINE_AUTO (default): the tensor-core
  * kernels where they apply -- odd K up to 13 (a smaller kernel is zero-padded to 13 x 13 in the workspace), C_a a
- * multiple of 16; NHWC with C a multiple of 8 (also with the point-wise LK^c when C_a = 16), or NCHW with W a
- * multiple of 8 and 16-byte aligned tensors -- else the FP32 kernels.
+ * multiple of 16; NHWC with C a multiple of 8 (also with the point-wise LK^c when C_a = 16), or NCHW with 16-byte aligned
+ * tensors and W a multiple of 8 (forward: any W from 48 tiles of 64 x 16 pixels and 16 channels on, C a multiple
+ * of 8) -- else the FP32 kernels.
  * ESC_ENGINE_FP32: never the tensor-core kernel.  ESC_ENGINE_TENSOR: the tensor-core kernel or, where
  * it does not apply, the guarded generic kernel.  Both engines multiply exactly (bf16 x bf16 in fp32) and
  * accumulate in fp32; they differ in the order of the 169 additions, i.e. by fp32 rounding before
  * the single rounding of the result to bf16.  In the tensor-core kernel one instruction sums 16
  * horizontally adjacent inputs, three of which may lie outside an output's 13-tap window with weight
  * zero: a non-finite attention input therefore turns outputs up to 15 pixels beyond its window into
- * NaN (finite data are unaffected).  Returns ESC_ERR_UNSUPPORTED for any other value. */
+ * NaN (finite data are unaffected); likewise where a kernel size lies in the zeros of the next one built (the generic
+ * kernel: 9, 13, 17).  Returns ESC_ERR_UNSUPPORTED for any other value. */
 enum { ESC_ENGINE_AUTO = 0, ESC_ENGINE_FP32 = 1, ESC_ENGINE_TENSOR = 2 };
 int esc_convattn_set_stencil_engine(int engine);
 
@@ -420,9 +423,9 @@ int esc_convattn_set_stencil_engine(int engine);
 int esc_convattn_set_fused_stage1(int on);
 
 /* Which kernel evaluates the dense large kernel of Section 3.2 (esc_convattn_forward_dense / _stencil_dense /
- * ESC_LK_DENSE) on NHWC bf16 tensors with 16 attention channels and K = 13, for later calls on this thread:
- * 0 (default) = the tcgen05 kernel (accumulators in tensor memory, one instruction per input row and tap column
- * with all 13 kernel rows stacked in N), 1 = the warp-level mma.sync kernel.  Both multiply exactly and accumulate
+ * ESC_LK_DENSE) on NHWC bf16 tensors with 16 attention channels, for later calls on this thread:
+ * 0 (default) = the tcgen05 kernel (odd K up to 13; also NCHW tensors, through the workspace, from 4,096 pixels on;
+ * accumulators in tensor memory, one instruction per input row and tap column with all 13 kernel rows stacked in N), 1 = the warp-level mma.sync kernel (K = 13, NHWC).  Both multiply exactly and accumulate
  * in fp32; they differ in the order of the additions.  esc_convattn_last_path() reports 5 and 3.  Returns
  * ESC_ERR_UNSUPPORTED for any other value.  For tests and comparisons. */
 int esc_convattn_set_dense_engine(int engine);
