@@ -66,6 +66,7 @@ conv_fuse_fp32(const Params<T> p)
 #pragma unroll
     for (int n = 0; n < 8; ++n) bs[n] = p.bias ? Elem<T>::to_f32(p.bias[n0 + n]) : 0.f;
     pdl_wait_primary();                                            // the tensors come from the kernel before this one
+    pdl_launch_dependents();
 
     // NCHW: tiles of one image; NHWC: of the flat list of pixels
     const long long per_img = LAYOUT == kNCHW ? (p.HW + kTilePx - 1) / kTilePx : 0;

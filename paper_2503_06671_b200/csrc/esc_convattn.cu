@@ -1692,7 +1692,7 @@ int esc_conv_fuse_backward(const void* cat, const void* grad_out, int B, int C, 
     }
     if (rc != ESC_OK || !sums) return rc;
     const int elems = C * C + C;
-    esc::fuse::bwd::sum_wgrad<<<(unsigned)((elems + 31) / 32), 256, 0, st>>>(w.part, C, blocks, grad_w_fuse, grad_b_fuse);
+    ESC_CUDA(launch_pdl(esc::fuse::bwd::sum_wgrad, (unsigned)((elems + 31) / 32), esc::fuse::bwd::kSumWarps * 32, 0, st, w.part, C, blocks, grad_w_fuse, grad_b_fuse));
     ESC_CUDA(cudaGetLastError());
     ++g_last_launches;
     return ESC_OK;
