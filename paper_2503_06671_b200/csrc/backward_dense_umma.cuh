@@ -32,6 +32,7 @@
 namespace esc { namespace bwd { namespace dense { namespace umma {
 
 using tma::u64; using tma::smem_u32; using tma::mbar_init; using tma::mbar_expect_tx; using tma::mbar_wait; using tma::tma_load_4d;
+using tma::mbar_arrive;
 using tma::umma::mbar_wait_warp; using tma::umma::mma_f16; using tma::umma::mma_commit; using tma::umma::tc_fence_after; using tma::umma::tc_fence_before;
 using tma::umma::tmem_ld16; using tma::umma::tmem_zero16; using tma::umma::tmem_wait_st;
 
@@ -124,6 +125,8 @@ tap_grad_dense_umma(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                 if (!alive) break;
                 const int go_bytes = kGroup * p.strip_w * 32, go_groups = (t.rows + kGroup - 1) / kGroup;
                 const int groups = (t.rows + K - 1 + kGroup - 1) / kGroup;
+                // every barrier of the go tile completes one phase per use of the tile, which is what the issuer's parity counts
+                for (int g = go_groups; g < kGoGroups; ++g) mbar_arrive(gfull0 + 8 * (gb * kGoGroups + g));
                 for (int g = 0; g < groups && alive; ++g, ++xg) {
                     if (g < go_groups) {
                         const uint32_t bar = gfull0 + 8 * (gb * kGoGroups + g);

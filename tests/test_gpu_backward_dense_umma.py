@@ -33,8 +33,17 @@ CASES = [
     (3, 16, 40, 49, 9),        # K = 9: the middle of the sums
     (1, 16, 30, 130, 3),
     (40, 16, 96, 70, 13),      # 240 units: one or two per block, some of two images; both go tiles are used
-    (7, 16, 400, 64, 13),      # seven rows of many units: the ring wraps several times inside a block
-    (300, 16, 21, 19, 13),     # two or three small images per block: go tiles re-used
+    (7, 16, 400, 64, 13),      # 119 units of 24 rows, one per block: nine groups of input rows, one more than the ring holds
+    (300, 16, 21, 19, 13),     # two or three small images per block, all of the same number of rows: go tiles re-used
+]
+
+# Three or more units per block, and the last segment of an image has fewer groups of four rows than the others: a go tile is used
+# again after one that filled only part of it.
+REUSE = [
+    # B, C, H, W, K             segments of rows (groups of four)
+    (64, 16, 73, 73, 13),      # 25, 25, 23 (7, 7, 6), two strips
+    (4, 24, 361, 640, 13),     # eleven of 31 and one of 20 (8 and 5), ten strips
+    (150, 16, 73, 50, 9),      # 25, 25, 23, one strip
 ]
 
 
@@ -80,6 +89,16 @@ def test_tcgen05_stencil_of_any_size_both_ways(pkg, oracle, K, misaligned):
 
 @pytest.mark.parametrize("case", CASES, ids=lambda c: "x".join(map(str, c)))
 def test_dense_weight_gradient(pkg, oracle, case):
+    _dense_weight_gradient(pkg, oracle, case, synth.NHWC)
+
+
+@pytest.mark.parametrize("layout", [synth.NHWC, synth.NCHW])        # NCHW: the same kernel on packed tensors
+@pytest.mark.parametrize("case", REUSE, ids=lambda c: "x".join(map(str, c)))
+def test_dense_weight_gradient_unequal_segments(pkg, oracle, case, layout):
+    _dense_weight_gradient(pkg, oracle, case, layout)
+
+
+def _dense_weight_gradient(pkg, oracle, case, layout):
     import torch
 
     B, C, H, W, K = case
@@ -88,14 +107,14 @@ def test_dense_weight_gradient(pkg, oracle, case):
     d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=seed, per_image_scale=True, channel_means=True)
     wdn = synth.make_dense_kernel(C_a, K, synth.BF16, seed=seed)
     go = synth.round_to(np.random.default_rng(seed).standard_normal(size=d["x"].shape).astype(np.float32), synth.BF16)
-    x, god = util.to_device(d["x"], synth.BF16, synth.NHWC), util.to_device(go, synth.BF16, synth.NHWC)
+    x, god = util.to_device(d["x"], synth.BF16, layout), util.to_device(go, synth.BF16, layout)
     _, wd, bd = util.weights_to_device(d, synth.BF16)
     wdd = torch.from_numpy(wdn).to("cuda", torch.bfloat16)
     ws = pkg.new_backward_dense_workspace(B, C_a, H, W, K)
     got = []
     for _ in range(2):                                     # twice, bit for bit: fixed order of every sum
         g = torch.full((C_a, C_a, K, K), float("nan"), device="cuda")
-        pkg.esc_convattn_backward_dense(x, god, C_a, K, wdd, wd, bd, torch.empty_like(x), g, None, None, pkg.ESC_NHWC, ws)
+        pkg.esc_convattn_backward_dense(x, god, C_a, K, wdd, wd, bd, torch.empty_like(x), g, None, None, util.layout_code(layout), ws)
         torch.cuda.synchronize()
         assert pkg.esc_convattn_device_status(ws) == 0
         got.append(g.cpu().numpy())
