@@ -342,28 +342,28 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
             const int per_row = MW / p.copy_pw, chunks = L * per_row;
             const unsigned bytes = (unsigned)(p.copy_cc * p.copy_pw * 2);
             auto coords = [&](int ch, int& cx, int& cy) { cy = ya + ch / per_row; cx = x0 + (ch % per_row) * p.copy_pw; };
-            auto issue = [&](int ch) {
+            auto issue = [&](int ch, int n) {                               // the n-th chunk that is copied
                 int cx, cy; coords(ch, cx, cy);
-                const int slot = ch % kCopySlots;
+                const int slot = n % kCopySlots;
                 mbar_expect_tx(cfull0 + 8 * slot, bytes);
                 tma_load_4d(smem_u32(cring + slot * kCopySlotBytes), &map_cin, cfull0 + 8 * slot, CG, cx, cy, b);
             };
-            // chunks wholly outside the image (right of W) are skipped by both cursors alike
+            // chunks wholly outside the image (right of W) are skipped, so slots and phases go by the count of those that are not
             auto inside = [&](int ch) { int cx, cy; coords(ch, cx, cy); return cx < p.W; };
             int next = 0;
             while (next < chunks && !inside(next)) ++next;
-            if (next < chunks) issue(next);
+            if (next < chunks) issue(next, 0);
             int cur = next;
-            while (cur < chunks) {
+            for (int n = 0; cur < chunks; ++n) {
                 int nx = cur + 1;
                 while (nx < chunks && !inside(nx)) ++nx;
                 if (nx < chunks) {
                     bulk_wait_read<0>();                                    // the store that last used the other slot has read it
-                    issue(nx);
+                    issue(nx, n + 1);
                 }
-                if (alive) alive = mbar_wait(cfull0 + 8 * (cur % kCopySlots), (unsigned)((cur / kCopySlots) & 1), p.ctrl, 0xD6000000u | (unsigned)cur);
+                if (alive) alive = mbar_wait(cfull0 + 8 * (n % kCopySlots), (unsigned)((n / kCopySlots) & 1), p.ctrl, 0xD6000000u | (unsigned)cur);
                 int cx, cy; coords(cur, cx, cy);
-                tma_store_4d(&map_cout, smem_u32(cring + (cur % kCopySlots) * kCopySlotBytes), CG, cx, cy, b);
+                tma_store_4d(&map_cout, smem_u32(cring + (n % kCopySlots) * kCopySlotBytes), CG, cx, cy, b);
                 bulk_commit();
                 cur = nx;
             }

@@ -97,6 +97,46 @@ def test_dense_tensor_core_kernel(pkg, oracle, shape, forward, engine):
     _check(util.to_host_nchw(out, synth.NHWC), ref, mag, synth.BF16, C_a, f"dense {shape}")
 
 
+WIDE_C = [
+    # B, C, H, W, K: more than 64 identity channels, so that a strip row of 128 pixels is copied in two (C = 96) or four (C = 192)
+    # chunks, and widths that leave some of them wholly outside the image
+    (2, 96, 40, 64, 9),        # the second chunk never exists
+    (1, 96, 75, 190, 13),      # nor in the second strip
+    (2, 192, 30, 100, 13),     # all four partly inside
+    (1, 192, 61, 190, 5),      # two of four in the second strip
+    (1, 192, 33, 30, 13),      # one of four
+]
+
+
+@pytest.mark.parametrize("shape", WIDE_C, ids=lambda s: "x".join(map(str, s)))
+def test_many_identity_channels(pkg, oracle, shape):
+    """The tcgen05 kernel's copy of the identity channels, bit for bit, forward and gradient."""
+    import torch
+
+    B, C, H, W, K = shape
+    C_a = 16
+    d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=sum(shape), channel_means=True)
+    wd = synth.make_dense_kernel(C_a, K, synth.BF16, seed=sum(shape))
+    x = util.to_device(d["x"], synth.BF16, synth.NHWC)
+    _, wdyn, bdyn = util.weights_to_device(d, synth.BF16)
+    wd_d = torch.from_numpy(wd).to("cuda", torch.bfloat16)
+    out, gx = torch.full_like(x, 7.0), torch.full_like(x, 7.0)
+    ws, wsb = pkg.new_workspace(B, C_a, H, W, K), pkg.new_backward_dense_workspace(B, C_a, H, W, K)
+    go = torch.randn(x.shape, device="cuda").to(x.dtype)
+    for _ in range(3):
+        pkg.esc_convattn_forward_dense(x, C_a, K, wd_d, wdyn, bdyn, out, pkg.ESC_NHWC, ws)
+        assert pkg.esc_convattn_last_path() == 5
+        pkg.esc_convattn_backward_dense(x, go, C_a, K, wd_d, wdyn, bdyn, gx, None, None, None, pkg.ESC_NHWC, wsb)
+        assert pkg.esc_convattn_last_path() == 5
+        torch.cuda.synchronize()
+        assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_device_status(wsb) == 0
+        assert torch.equal(out[..., C_a:], x[..., C_a:]) and torch.equal(gx[..., C_a:], go[..., C_a:])
+        out.fill_(7.0), gx.fill_(7.0)
+    pkg.esc_convattn_forward_dense(x, C_a, K, wd_d, wdyn, bdyn, out, pkg.ESC_NHWC, ws)
+    ref, mag = oracle.forward_dense(d["x"], C_a, wd, d["w_dyn"], d["b_dyn"], want_mag=True)
+    _check(util.to_host_nchw(out, synth.NHWC), ref, mag, synth.BF16, C_a, f"dense {shape}")
+
+
 GENERIC_SHAPES = [
     # B, C, C_a, H, W, K
     (2, 24, 16, 19, 23, 13),
