@@ -201,8 +201,10 @@ conv_fuse_fp32(const Params<T> p)
     }
 }
 
+// first: no kernel of the same call stands in front of this one.  Then w may come from the kernel that does, and this one, which reads
+// w before it waits, must not start before that has finished.
 template <typename T, int LAYOUT, int C, bool kTrans>
-inline cudaError_t launch_c(const Params<T>& p, cudaStream_t st) {
+inline cudaError_t launch_c(const Params<T>& p, cudaStream_t st, bool first) {
     using G = CGeom<C>;
     auto* fn = conv_fuse_fp32<T, LAYOUT, C, kTrans>;
     static bool attr_set[tma::kMaxDevices] = {};
@@ -224,16 +226,16 @@ inline cudaError_t launch_c(const Params<T>& p, cudaStream_t st) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = first ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, fn, p);
 }
 template <typename T, int LAYOUT, bool kTrans>
-inline cudaError_t launch(int C, const Params<T>& p, cudaStream_t st) {
+inline cudaError_t launch(int C, const Params<T>& p, cudaStream_t st, bool first) {
     switch (C) {
-        case 16: return launch_c<T, LAYOUT, 16, kTrans>(p, st);
-        case 32: return launch_c<T, LAYOUT, 32, kTrans>(p, st);
-        case 48: return launch_c<T, LAYOUT, 48, kTrans>(p, st);
-        case 64: return launch_c<T, LAYOUT, 64, kTrans>(p, st);
+        case 16: return launch_c<T, LAYOUT, 16, kTrans>(p, st, first);
+        case 32: return launch_c<T, LAYOUT, 32, kTrans>(p, st, first);
+        case 48: return launch_c<T, LAYOUT, 48, kTrans>(p, st, first);
+        case 64: return launch_c<T, LAYOUT, 64, kTrans>(p, st, first);
         default: return cudaErrorInvalidValue;
     }
 }

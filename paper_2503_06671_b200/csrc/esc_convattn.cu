@@ -926,16 +926,17 @@ int dense_grad_x_t(Problem p, const void* go, const void* w_dense, void* gx, con
     return ESC_OK;
 }
 
-// ---- Conv_fuse on the FP32 pipe: att | idt are the two parts of its input, kTrans: the matrix is read transposed ----
+// ---- Conv_fuse on the FP32 pipe: att | idt are the two parts of its input, kTrans: the matrix is read transposed; first: this
+// is the call's first kernel ----
 template <typename T, bool kTrans>
 int launch_fuse_fp32(const Problem& p, const void* att, const void* idt, const void* w, const void* bias, const void* residual,
-                     void* out, cudaStream_t st) {
+                     void* out, cudaStream_t st, bool first = false) {
     esc::fuse::f32::Params<T> fp;
     fp.att = static_cast<const T*>(att); fp.idt = static_cast<const T*>(idt); fp.w = static_cast<const T*>(w);
     fp.bias = static_cast<const T*>(bias); fp.residual = static_cast<const T*>(residual); fp.out = static_cast<T*>(out);
     fp.HW = (long long)p.H * p.W; fp.pixels = fp.HW * p.B; fp.B = p.B; fp.Ca = p.Ca; fp.vec = fp.HW % 4 == 0;
-    ESC_CUDA(p.layout == ESC_NCHW ? (esc::fuse::f32::launch<T, esc::kNCHW, kTrans>(p.C, fp, st))
-                                  : (esc::fuse::f32::launch<T, esc::kNHWC, kTrans>(p.C, fp, st)));
+    ESC_CUDA(p.layout == ESC_NCHW ? (esc::fuse::f32::launch<T, esc::kNCHW, kTrans>(p.C, fp, st, first))
+                                  : (esc::fuse::f32::launch<T, esc::kNHWC, kTrans>(p.C, fp, st, first)));
     ++g_last_launches;
     return ESC_OK;
 }
@@ -1687,8 +1688,8 @@ int esc_conv_fuse_backward(const void* cat, const void* grad_out, int B, int C, 
             if (rc != ESC_OK) return rc;
         }
         // grad_cat = W_fuse^T grad_out per pixel: the 1x1 kernel with the matrix read transposed, no bias, no residual
-        rc = dtype == ESC_F32 ? launch_fuse_fp32<float, true>(p, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st)
-                              : launch_fuse_fp32<__nv_bfloat16, true>(p, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st);
+        rc = dtype == ESC_F32 ? launch_fuse_fp32<float, true>(p, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st, /*first=*/!sums)
+                              : launch_fuse_fp32<__nv_bfloat16, true>(p, grad_out, grad_out, w_fuse, nullptr, nullptr, grad_cat, st, !sums);
     }
     if (rc != ESC_OK || !sums) return rc;
     const int elems = C * C + C;

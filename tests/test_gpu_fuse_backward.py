@@ -99,3 +99,36 @@ def test_fuse_backward_optional_outputs_and_rejections(pkg, oracle):
     assert pkg.esc_conv_fuse_backward_workspace_bytes(1, 40, 8, 8) == 0
     with pytest.raises(pkg.EscError):
         pkg.esc_conv_fuse_backward(x40, x40.clone(), torch.zeros((40, 40), device="cuda", dtype=torch.bfloat16), torch.zeros_like(x40), None, None, lc)
+
+
+@pytest.mark.parametrize("layout", LAYOUTS)
+@pytest.mark.parametrize("dtype,C", [(synth.F32, 48), (synth.BF16, 16)])
+def test_matrix_written_by_the_kernel_in_front(pkg, dtype, C, layout):
+    """Without weight gradients the call is one kernel, and the one in front of it may write w_fuse.  Here that is stage 1, which
+    lets its dependents start long before it writes: with w_dyn = 0 its dk is b_dyn, bit for bit, and b_dyn is the matrix."""
+    import torch
+
+    tdt, H, W = util.torch_dtype(dtype), 33, 47
+    w = torch.from_numpy(synth.make_fuse(C, dtype, seed=3)["w_fuse"]).to("cuda", tdt).contiguous()
+    words = w.view(-1).view(torch.float32)
+    C_a = -(-words.numel() // 9)
+    b_dyn = torch.zeros(9 * C_a, device="cuda")
+    b_dyn[:words.numel()] = words
+    x = torch.randn(1, C_a, 400, 400, device="cuda")
+    w_dyn = torch.zeros(9 * C_a, C_a, device="cuda")
+    dk = torch.zeros(1, C_a, 3, 3, device="cuda")
+    w_made = dk.view(-1)[:words.numel()].view(tdt).view(C, C)
+    shape = (2, H, W, C) if layout == synth.NHWC else (2, C, H, W)
+    cat, go = (torch.randn(shape, device="cuda").to(tdt) for _ in range(2))
+    got, want = torch.empty_like(go), torch.empty_like(go)
+    ws1 = pkg.new_workspace(1, C_a, 400, 400, 3)
+    ws2 = torch.empty(pkg.esc_conv_fuse_backward_workspace_bytes(2, C, H, W), dtype=torch.uint8, device="cuda")
+    pkg.esc_conv_fuse_backward(cat, go, w, want, None, None, util.layout_code(layout), ws2)
+    for _ in range(20):
+        dk.zero_()
+        torch.cuda.synchronize()
+        pkg.esc_convattn_dynkernel(x, C_a, w_dyn, b_dyn, dk, pkg.ESC_NCHW, ws1)
+        pkg.esc_conv_fuse_backward(cat, go, w_made, got, None, None, util.layout_code(layout), ws2)
+        torch.cuda.synchronize()
+        assert torch.equal(w_made, w)
+        assert torch.equal(got, want)
