@@ -93,9 +93,9 @@ int check_tensors(const Problem& p, const void* x, const void* out) {
 }
 
 // ---- workspace layout -------------------------------------------------------------------
-//   [ctrl words: header + B arrival counters + B launch flags][pad to 256][dk: B*Ca*9 floats][pad]
+//   [ctrl words: header + arrival counters + launch flags, see ctrl_images][pad to 256][dk: B*Ca*9 floats][pad]
 //   [partials: B*S*Ca floats][pad][per-unit sums of the one-launch form: kMaxFusedUnits * SMs * 16 floats][pad]
-//   [large kernel padded to 13 x 13]
+//   [large kernel padded to 13 x 13, bf16]                        (the last two only where a tensor-core kernel can run: C_a % 16 == 0)
 size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 struct Workspace {
@@ -105,7 +105,7 @@ struct Workspace {
     float* dk;
     float* partial;
     float* unit_sums;
-    void* lk_pad;                    // [Ca][13][13] elements: a smaller large kernel zero-padded for the tensor-core kernels
+    void* lk_pad;                    // [Ca][13][13] bf16: a smaller large kernel zero-padded for the tensor-core kernels
     void* packed;                    // C_a = 16: [B][H][W][16] bf16, the attention channels of an NCHW map for the dense form
 };
 
@@ -141,34 +141,46 @@ int slabs_for(int B, long long HW, bool wide) {
     return (int)s;
 }
 
-size_t workspace_bytes(int B, int Ca, long long HW) {
-    const int S = slabs_for(B, HW, true);                   // room for either grid policy
-    size_t off = round_up((size_t)(esc::kCtrlHeaderWords + 2 * (size_t)B) * 4, 256);
-    off += round_up((size_t)B * Ca * 9 * 4, 256);
-    off += round_up((size_t)B * S * Ca * 4, 256);
-    off += round_up((size_t)esc::tma::toep::kMaxFusedUnits * sms_or_nominal() * 16 * 4, 256);   // unit sums of the one-launch form
-    off += round_up((size_t)Ca * 169 * 4, 256);            // padded large kernel
-    off += round_up(esc::dense16::packed_bytes(B, Ca, HW), 256);
+// A buffer is zeroed once and then serves calls of any shape, in any order.  The arrival counters must be zero between calls, so
+// nothing but counters may lie where another shape has them: they and the flags (whose value at rest does not matter) have a place
+// for kCtrlImages images that no shape puts anything else on.  Beyond that many images the counters are cleared by every call.
+constexpr int kCtrlImages = 640;
+int ctrl_images(int B) { return B > kCtrlImages ? B : kCtrlImages; }
+
+// Fills `w` for a workspace at `ws` (null: only the size is wanted) and returns its size.
+size_t carve(void* ws, int B, int Ca, long long HW, Workspace& w) {
+    char* base = static_cast<char*>(ws);
+    const int n = ctrl_images(B);
+    const bool tensor = Ca % esc::tma::CG == 0;
+    size_t off = round_up((size_t)(esc::kCtrlHeaderWords + 2 * (size_t)n) * 4, 256);
+    auto take = [&](size_t bytes) {
+        char* p = base + off;
+        off += round_up(bytes, 256);
+        return p;
+    };
+    w.ctrl = reinterpret_cast<unsigned*>(base);
+    w.arrivals = w.ctrl + esc::kCtrlHeaderWords;
+    w.flags = w.arrivals + n;
+    w.dk = reinterpret_cast<float*>(take((size_t)B * Ca * 9 * 4));
+    w.partial = reinterpret_cast<float*>(take((size_t)B * slabs_for(B, HW, true) * Ca * 4));   // room for either grid policy
+    w.unit_sums = reinterpret_cast<float*>(take(tensor ? (size_t)esc::tma::toep::kMaxFusedUnits * sms_or_nominal() * 16 * 4 : 0));
+    w.lk_pad = take(tensor ? (size_t)Ca * 169 * 2 : 0);
+    w.packed = take(esc::dense16::packed_bytes(B, Ca, HW));
     return off;
 }
-
 Workspace carve(void* ws, int B, int Ca, long long HW) {
     Workspace w;
-    char* p = static_cast<char*>(ws);
-    w.ctrl = reinterpret_cast<unsigned*>(p);
-    w.arrivals = w.ctrl + esc::kCtrlHeaderWords;
-    w.flags = w.arrivals + B;
-    p += round_up((size_t)(esc::kCtrlHeaderWords + 2 * (size_t)B) * 4, 256);
-    w.dk = reinterpret_cast<float*>(p);
-    p += round_up((size_t)B * Ca * 9 * 4, 256);
-    w.partial = reinterpret_cast<float*>(p);
-    p += round_up((size_t)B * slabs_for(B, HW, true) * Ca * 4, 256);
-    w.unit_sums = reinterpret_cast<float*>(p);
-    p += round_up((size_t)esc::tma::toep::kMaxFusedUnits * sms_or_nominal() * 16 * 4, 256);
-    w.lk_pad = p;
-    p += round_up((size_t)Ca * 169 * 4, 256);
-    w.packed = p;
+    carve(ws, B, Ca, HW, w);
     return w;
+}
+size_t workspace_bytes(int B, int Ca, long long HW) {
+    Workspace w;
+    return carve(nullptr, B, Ca, HW, w);
+}
+// In front of a kernel that counts arrivals.
+int clear_counters(const Workspace& w, int B, cudaStream_t st) {
+    if (B > kCtrlImages) ESC_CUDA(cudaMemsetAsync(w.arrivals, 0, (size_t)B * sizeof(unsigned), st));
+    return ESC_OK;
 }
 
 int check_workspace(const Problem& p, const void* ws, size_t bytes) {
@@ -592,6 +604,8 @@ int launch_stencil_dense(const Problem& p, const void* x, const void* w_dense, c
 int forward_impl(const Problem& p0, const void* x, const void* w_large0, const Estimator& est,
                  void* out, void* ws, cudaStream_t st) {
     const Workspace w = carve(ws, p0.B, p0.Ca, (long long)p0.H * p0.W);
+    int rc = clear_counters(w, p0.B, st);
+    if (rc != ESC_OK) return rc;
     // what the tensor-core kernels see: a smaller large kernel zero-padded to 13 x 13 (launched first, so that the GAP
     // kernel stays the stencil kernel's immediate predecessor)
     const TensorLk tl = tensor_lk(p0, x, out, w_large0, w.lk_pad, st);
@@ -602,8 +616,8 @@ int forward_impl(const Problem& p0, const void* x, const void* w_large0, const E
     if (g_fuse_stage1 && tensor_stencil_follows(p)) {
         const esc::tma::toep::Fused fu{est.w_last, est.b_last, est.w_down, est.b_down, est.hidden, w.unit_sums, w.arrivals, w.flags};
         int tw = 0;
-        const int rc = esc::tma::toep::try_launch_fused(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, w_large, fu, out,
-                                                        w.ctrl, st, &g_last_launches, &g_last_error, &tw, p.skip_copy, p.w_point);
+        rc = esc::tma::toep::try_launch_fused(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, w_large, fu, out,
+                                              w.ctrl, st, &g_last_launches, &g_last_error, &tw, p.skip_copy, p.w_point);
         if (rc == ESC_OK) { g_last_path = 4; g_last_tile_w = tw; return ESC_OK; }
         if (rc != esc::tma::kNotApplicable) {
             // a cooperative launch can be refused (SMs held by another context): fall back to two kernels
@@ -614,15 +628,15 @@ int forward_impl(const Problem& p0, const void* x, const void* w_large0, const E
     if (g_fuse_stage1 && !p.dense && (!p.w_point || p.Ca == esc::tma::CG) && !p.bias && g_engine_policy != ESC_ENGINE_FP32 &&
         g_tile_policy == 0) {
         const esc::tma::toep::Fused fu{est.w_last, est.b_last, est.w_down, est.b_down, est.hidden, w.unit_sums, w.arrivals, w.flags};
-        const int rc = esc::tma::toepn::try_launch_fused(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, w_large, fu, out, w.ctrl, st,
-                                                         &g_last_launches, &g_last_error, p.w_point, p.skip_copy);
+        rc = esc::tma::toepn::try_launch_fused(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, w_large, fu, out, w.ctrl, st,
+                                               &g_last_launches, &g_last_error, p.w_point, p.skip_copy);
         if (rc == ESC_OK) { g_last_path = 6; g_last_tile_w = esc::tma::toepn::TW; return ESC_OK; }
         if (rc != esc::tma::kNotApplicable) { (void)cudaGetLastError(); g_last_error.clear(); }
     }
     const bool tensor_nchw = !p.dense && (!p.w_point || p.Ca == esc::tma::CG) && !p.bias && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
                              esc::tma::toepn::takes(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, out);
     const bool packed = p0.dense && wants_packing(p0);
-    int rc = packed ? launch_pack16(p0, x, w.packed, out, st) : ESC_OK;
+    rc = packed ? launch_pack16(p0, x, w.packed, out, st) : ESC_OK;
     if (rc == ESC_OK) rc = launch_gap(p0, x, est, w, w.dk, st, tensor_stencil_follows(p) || tensor_nchw);
     if (rc != ESC_OK) return rc;
     if (packed) {
@@ -1181,8 +1195,10 @@ int esc_convattn_dynkernel(const void* x, int B, int C, int C_a, int H, int W, c
     if (!aligned(x, 16) || !aligned(dk_out, 4) || !aligned(w_dyn, p.es()) || !aligned(b_dyn, p.es())) return ESC_ERR_ALIGN;
     rc = check_workspace(p, workspace, workspace_bytes_);
     if (rc != ESC_OK) return rc;
-    return launch_gap(p, x, Estimator{w_dyn, b_dyn, nullptr, nullptr, 0}, carve(workspace, B, C_a, (long long)H * W), dk_out,
-                      static_cast<cudaStream_t>(stream));
+    const Workspace w = carve(workspace, B, C_a, (long long)H * W);
+    rc = clear_counters(w, B, static_cast<cudaStream_t>(stream));
+    if (rc != ESC_OK) return rc;
+    return launch_gap(p, x, Estimator{w_dyn, b_dyn, nullptr, nullptr, 0}, w, dk_out, static_cast<cudaStream_t>(stream));
 }
 
 int esc_convattn_forward_mlp(const void* x, int B, int C, int C_a, int H, int W, int K, const void* w_large,
@@ -1221,7 +1237,10 @@ int esc_convattn_dynkernel_mlp(const void* x, int B, int C, int C_a, int H, int 
     if (!aligned(x, 16) || !aligned(dk_out, 4)) return ESC_ERR_ALIGN;
     rc = check_workspace(p, workspace, workspace_bytes_);
     if (rc != ESC_OK) return rc;
-    return launch_gap(p, x, est, carve(workspace, B, C_a, (long long)H * W), dk_out, static_cast<cudaStream_t>(stream));
+    const Workspace w = carve(workspace, B, C_a, (long long)H * W);
+    rc = clear_counters(w, B, static_cast<cudaStream_t>(stream));
+    if (rc != ESC_OK) return rc;
+    return launch_gap(p, x, est, w, dk_out, static_cast<cudaStream_t>(stream));
 }
 
 int esc_convattn_dynkernel_static(const void* x, int B, int C, int C_a, int H, int W, const void* w_dyn,
