@@ -458,6 +458,7 @@ int get_scratch(size_t need, cudaStream_t st, void** out) {
         const size_t cap = round_up(need, 1 << 20);
         ESC_CUDA(cudaMalloc(&s.ptr, cap));
         ESC_CUDA(cudaMemset(s.ptr, 0, cap));
+        ESC_CUDA(cudaStreamSynchronize(cudaStreamLegacy));   // st may be a stream that does not wait for that one
         s.bytes = cap;
     }
     *out = s.ptr;
@@ -1793,7 +1794,7 @@ int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C,
     if (h.wsbytes < wsbytes) {
         cudaFree(h.ws); h.ws = nullptr; h.wsbytes = 0;
         ESC_CUDA(cudaMalloc(&h.ws, wsbytes));
-        ESC_CUDA(cudaMemset(h.ws, 0, wsbytes));
+        ESC_CUDA(cudaMemsetAsync(h.ws, 0, wsbytes, h.st));
         h.wsbytes = wsbytes;
     }
     char* wts = static_cast<char*>(h.wts);

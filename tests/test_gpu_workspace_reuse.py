@@ -70,3 +70,27 @@ def test_shapes_in_turn(case):
             else:
                 got = call(x, shared)
             assert torch.equal(got, want), (B, H, W)
+
+
+def test_first_use_while_the_default_stream_is_busy():
+    """Scratch that the library allocates on a stream's first call is zero before the kernels count in it, also on a stream that does
+    not wait for the default one."""
+    import torch
+
+    import paper_2503_06671_b200 as pkg
+
+    B, H, W = 1, 640, 360
+    x = torch.randn(B, C, H, W, device="cuda")
+    ws = [torch.randn(s, device="cuda") * 0.1 for s in ((C_A, K, K), (9 * C_A, C_A), (9 * C_A,))]
+    want, got = torch.empty_like(x), torch.empty_like(x)
+    pkg.esc_convattn_forward_ex(x, C_A, K, *ws, want, pkg.ESC_NCHW, pkg.new_workspace(B, C_A, H, W, K))
+    torch.cuda.synchronize()
+    used = [torch.full((1 << 20,), -1, dtype=torch.int32, device="cuda") for _ in range(48)]     # what the driver hands out next
+    torch.cuda.synchronize()
+    del used
+    torch.cuda.empty_cache()
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(200_000_000)                          # about 0.1 s on the default stream
+    pkg.esc_convattn_forward(x, C_A, K, *ws, got, stream=side)
+    side.synchronize()
+    assert torch.equal(got, want)
