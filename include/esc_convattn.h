@@ -83,8 +83,10 @@ int esc_convattn_forward_ex(const void* x, int B, int C, int C_a, int H, int W, 
                             void* out, int dtype, int layout,
                             void* workspace, size_t workspace_bytes, void* stream);
 
-/* Bytes of scratch needed by the calls that take a workspace (dk, GAP partial sums,
- * arrival counters, status word).  Returns 0 for invalid arguments. */
+/* Bytes of scratch for the calls that take a workspace (dk, GAP partial sums, arrival counters,
+ * status word).  With C_a = 16 and K <= 13 this includes 32 bytes per pixel that only the dense large
+ * kernel on bf16 NCHW tensors uses (a packed copy of its input); every call accepts a workspace without
+ * them, and that form then runs on the FP32 pipe.  Returns 0 for invalid arguments. */
 size_t esc_convattn_workspace_bytes(int B, int C_a, int H, int W, int K);
 
 /* Zero a fresh workspace (enqueued on `stream`).  Needed once per allocation; the kernels
@@ -329,7 +331,8 @@ int esc_convattn_backward_pw(const void* x, const void* grad_out, int B, int C, 
  *   grad_x, grad_w_dyn, grad_b_dyn as in esc_convattn_backward (grad_x's large-kernel term sums over the output channels).
  * C_a must be 16 (ESC_ERR_UNSUPPORTED otherwise); K odd, 3 .. 13.  The workspace is one of
  * esc_convattn_backward_dense_workspace_bytes(...) bytes (larger than the depth-wise one: every block of the tap-gradient
- * kernel keeps 16 x 16 x 169 sums there), 256-byte aligned, zeroed once with esc_convattn_workspace_init().  Same
+ * kernel keeps 16 x 16 x 169 sums there), 256-byte aligned, zeroed once with esc_convattn_workspace_init().  Its last 64
+ * bytes per pixel serve bf16 NCHW tensors alone (packed copies of x and grad_out) and may be missing, as in the forward.  Same
  * restrictions and error codes as esc_convattn_backward.  All device memory; asynchronous on `stream`.
  */
 size_t esc_convattn_backward_dense_workspace_bytes(int B, int C_a, int H, int W, int K);

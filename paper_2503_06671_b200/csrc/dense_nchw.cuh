@@ -33,14 +33,15 @@ pack16(const __nv_bfloat16* __restrict__ x, __nv_bfloat16* __restrict__ packed, 
     }
 }
 
-inline size_t packed_bytes(int B, int Ca, long long HW) { return Ca == CA ? (size_t)B * HW * CA * 2 : 0; }
+constexpr int kMaxK = 13;                           // the tcgen05 kernel's
+inline size_t packed_bytes(int B, int Ca, long long HW, int K) { return Ca == CA && K <= kMaxK ? (size_t)B * HW * CA * 2 : 0; }
 
 // bf16 NCHW, K <= 13: tcgen05 behind a packing pass from so many pixels on that it is the faster way.  Measured, forward, K = 13,
 // FP32 pipe / packed: 64x64 30.5 / 27 us, 90x90 45.6 / 26.7, 427x240 213 / 29.4, 640x360 430 / 39; 48x48 (K = 9) 22.9 / 25.
 // Backward, the old kernels / packed: 17 x (96x96) 759 / 129 us, 640x360 1,530 / 156.
 constexpr long long kPackPixels = 4096;
 inline bool nchw_wants_packing(int B, int Ca, int H, int W, int K, int dtype, int layout) {
-    return dtype == 1 /*bf16*/ && layout == kNCHW && Ca == CA && K <= 13 && (long long)B * H * W >= kPackPixels;
+    return dtype == 1 /*bf16*/ && layout == kNCHW && Ca == CA && K <= kMaxK && (long long)B * H * W >= kPackPixels;
 }
 
 }}  // namespace esc::dense16

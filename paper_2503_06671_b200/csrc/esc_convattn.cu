@@ -65,6 +65,7 @@ struct Problem {
     bool dense = false;              // w_large is the dense kernel [Ca][Ca][K][K] of Section 3.2
     const float* bias = nullptr;     // [B][Ca] constant per (image, channel) added to the attention outputs (backward pass)
     bool skip_copy = false;          // the identity channels are not written (the fused 1x1 convolution reads them from x)
+    bool pack_room = false;          // the caller's workspace has room for the packed map(s)
     size_t es() const { return elem_size(dtype); }
     size_t elems() const { return (size_t)B * C * H * W; }
 };
@@ -147,7 +148,8 @@ int slabs_for(int B, long long HW, bool wide) {
 constexpr int kCtrlImages = 640;
 int ctrl_images(int B) { return B > kCtrlImages ? B : kCtrlImages; }
 
-// Fills `w` for a workspace at `ws` (null: only the size is wanted) and returns its size.
+// Fills `w` for a workspace at `ws` (null: only the size is wanted) and returns the size that every call needs.  The packed map
+// lies behind that: only the dense form on bf16 NCHW tensors has a use for it, and does without where there is no room.
 size_t carve(void* ws, int B, int Ca, long long HW, Workspace& w) {
     char* base = static_cast<char*>(ws);
     const int n = ctrl_images(B);
@@ -165,7 +167,7 @@ size_t carve(void* ws, int B, int Ca, long long HW, Workspace& w) {
     w.partial = reinterpret_cast<float*>(take((size_t)B * slabs_for(B, HW, true) * Ca * 4));   // room for either grid policy
     w.unit_sums = reinterpret_cast<float*>(take(tensor ? (size_t)esc::tma::toep::kMaxFusedUnits * sms_or_nominal() * 16 * 4 : 0));
     w.lk_pad = take(tensor ? (size_t)Ca * 169 * 2 : 0);
-    w.packed = take(esc::dense16::packed_bytes(B, Ca, HW));
+    w.packed = base + off;
     return off;
 }
 Workspace carve(void* ws, int B, int Ca, long long HW) {
@@ -176,6 +178,9 @@ Workspace carve(void* ws, int B, int Ca, long long HW) {
 size_t workspace_bytes(int B, int Ca, long long HW) {
     Workspace w;
     return carve(nullptr, B, Ca, HW, w);
+}
+size_t workspace_bytes_packed(int B, int Ca, long long HW, int K) {
+    return workspace_bytes(B, Ca, HW) + round_up(esc::dense16::packed_bytes(B, Ca, HW, K), 256);
 }
 // In front of a kernel that counts arrivals.
 int clear_counters(const Workspace& w, int B, cudaStream_t st) {
@@ -550,7 +555,7 @@ int launch_pack16(const Problem& p, const void* x, void* packed, void* out, cuda
     return ESC_OK;
 }
 bool wants_packing(const Problem& p) {
-    return g_dense_engine == 0 && esc::dense16::nchw_wants_packing(p.B, p.Ca, p.H, p.W, p.K, p.dtype, p.layout);
+    return p.pack_room && g_dense_engine == 0 && esc::dense16::nchw_wants_packing(p.B, p.Ca, p.H, p.W, p.K, p.dtype, p.layout);
 }
 // The tcgen05 kernel on a packed map, results into the NCHW tensor `out`.
 int launch_umma_packed(const Problem& p, const void* packed, const void* w_dense, const float* dk, void* out, unsigned* ctrl,
@@ -665,7 +670,8 @@ struct BackwardWs {
     void* wd_flip;                   // the dense kernel with swapped channel axes and rotated taps
     void *x_packed, *go_packed;      // bf16 NCHW tensors: the attention channels of x and grad_out, [B][H][W][16]
     int dense_blocks;
-    size_t bytes_dense;              // bytes with those behind the rest
+    size_t bytes_dense;              // bytes with the first two behind the rest: what the dense form needs
+    size_t bytes_packed;             // bytes with all of them
 };
 BackwardWs carve_backward(void* ws, const Problem& p) {
     // sized for whichever tiling of the tap-gradient kernels has more tiles (32x32, or 64x16 on the tensor cores)
@@ -694,10 +700,11 @@ BackwardWs carve_backward(void* ws, const Problem& p) {
     w.dense_blocks = sms_or_nominal();
     w.dense_part = reinterpret_cast<float*>(base + off); off += round_up((size_t)w.dense_blocks * esc::bwd::dense::kPartFloats * 4, 256);
     w.wd_flip = base + off;                              off += round_up((size_t)esc::bwd::dense::CA * esc::bwd::dense::CA * esc::bwd::TAPS * 4, 256);
-    const size_t pk = round_up(esc::dense16::packed_bytes(p.B, p.Ca, (long long)p.H * p.W), 256);
+    w.bytes_dense = off;
+    const size_t pk = round_up(esc::dense16::packed_bytes(p.B, p.Ca, (long long)p.H * p.W, p.K), 256);
     w.x_packed = base + off;  off += pk;
     w.go_packed = base + off; off += pk;
-    w.bytes_dense = off;
+    w.bytes_packed = off;
     return w;
 }
 
@@ -1143,7 +1150,7 @@ const char* esc_status_string(int s) {
 
 size_t esc_convattn_workspace_bytes(int B, int C_a, int H, int W, int K) {
     if (B <= 0 || C_a <= 0 || H <= 0 || W <= 0 || K < 3 || (K & 1) == 0 || K > ESC_MAX_K) return 0;
-    return workspace_bytes(B, C_a, (long long)H * W);
+    return workspace_bytes_packed(B, C_a, (long long)H * W, K);
 }
 
 int esc_convattn_workspace_init(void* workspace, size_t workspace_bytes_, void* stream) {
@@ -1360,6 +1367,7 @@ int esc_convattn_stencil_dense(const void* x, int B, int C, int C_a, int H, int 
         if (rc != ESC_OK) return rc;
         const Workspace w = carve(workspace, B, C_a, (long long)H * W);
         ctrl = w.ctrl;
+        p.pack_room = workspace_bytes_ >= workspace_bytes_packed(B, C_a, (long long)H * W, K);
         if (wants_packing(p)) {
             cudaStream_t st = static_cast<cudaStream_t>(stream);
             rc = launch_pack16(p, x, w.packed, out, st);
@@ -1384,6 +1392,7 @@ int esc_convattn_forward_dense(const void* x, int B, int C, int C_a, int H, int 
     rc = check_workspace(p, workspace, workspace_bytes_);
     if (rc != ESC_OK) return rc;
     p.dense = true;
+    p.pack_room = workspace_bytes_ >= workspace_bytes_packed(B, C_a, (long long)H * W, K);
     return forward_impl(p, x, w_dense, Estimator{w_dyn, b_dyn, nullptr, nullptr, 0}, out, workspace,
                         static_cast<cudaStream_t>(stream));
 }
@@ -1410,6 +1419,7 @@ int esc_convattn_forward_variant(const void* x, int B, int C, int C_a, int H, in
     if (rc != ESC_OK) return rc;
     if (large_kernel == ESC_LK_DECOMPOSED) p.w_point = w_point;
     p.dense = large_kernel == ESC_LK_DENSE;
+    p.pack_room = workspace_bytes_ >= workspace_bytes_packed(B, C_a, (long long)H * W, K);
     return forward_impl(p, x, w_large, est, out, workspace, static_cast<cudaStream_t>(stream));
 }
 
@@ -1534,6 +1544,7 @@ int backward_entry(const void* x, const void* grad_out, int B, int C, int C_a, i
     if (g_wd && !aligned(g_wd, 4)) return ESC_ERR_ALIGN;
     BackwardWs w = carve_backward(workspace, p);
     if (workspace_bytes_ < (dense ? w.bytes_dense : w.bytes)) return ESC_ERR_WORKSPACE;
+    p.pack_room = dense && workspace_bytes_ >= w.bytes_packed;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (w_point) {
         // decomposed form (Eq. 5): the mixed features go into grad_x's attention channels, where the tap-gradient kernels
@@ -1630,7 +1641,7 @@ int esc_convattn_backward_pw(const void* x, const void* grad_out, int B, int C, 
 size_t esc_convattn_backward_dense_workspace_bytes(int B, int C_a, int H, int W, int K) {
     if (B <= 0 || C_a != esc::bwd::dense::CA || H <= 0 || W <= 0 || K < 3 || K > esc::bwd::K || (K & 1) == 0) return 0;
     const Problem p{B, C_a, C_a, H, W, K, ESC_F32, ESC_NCHW};
-    return carve_backward(nullptr, p).bytes_dense;
+    return carve_backward(nullptr, p).bytes_packed;
 }
 
 int esc_convattn_backward_dense(const void* x, const void* grad_out, int B, int C, int C_a, int H, int W, int K,

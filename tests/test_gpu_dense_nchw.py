@@ -85,3 +85,47 @@ def test_dense_nchw(pkg, oracle, case):
     for name, got, r, s in zip(("w_dense", "w_dyn", "b_dyn"), g, ref[1:], mag[1:]):
         err = np.abs(got.cpu().numpy().astype(np.float64) - r)
         assert (err <= 1e-5 * s + 1e-30).all(), f"grad {name}: worst {(err / np.maximum(s, 1e-30)).max():.3e} of its scale"
+
+
+def test_workspace_without_room_for_packed_maps(pkg):
+    """The packed maps are the last part of a workspace (32 bytes per pixel forward, 64 backward) and may be missing: the same calls
+    then run on the kernels that need none, forward, stage alone and gradients.  One byte less is refused."""
+    import torch
+
+    B, C, C_a, H, W, K = 2, 24, 16, 50, 60, 13
+    d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=5, channel_means=True)
+    x, god = (util.to_device(a, synth.BF16, synth.NCHW) for a in (d["x"], synth.round_to(d["x"][::-1].copy(), synth.BF16)))
+    _, wd, bd = util.weights_to_device(d, synth.BF16)
+    wdd = torch.from_numpy(synth.make_dense_kernel(C_a, K, synth.BF16, seed=5)).to("cuda", torch.bfloat16)
+    dk = torch.rand(B, C_a, 3, 3, device="cuda") - 0.5
+    part = -(-B * H * W * 32 // 256) * 256
+    res = {}
+    for room in (True, False):
+        ws, wsb = pkg.new_workspace(B, C_a, H, W, K), pkg.new_backward_dense_workspace(B, C_a, H, W, K)
+        if not room:
+            ws, wsb = ws[:ws.numel() - part], wsb[:wsb.numel() - 2 * part]
+        o = [torch.full_like(x, 7.0) for _ in range(3)]
+        g = [torch.full(s, float("nan"), device="cuda") for s in ((C_a, C_a, K, K), (9 * C_a, C_a), (9 * C_a,))]
+        paths = []
+        pkg.esc_convattn_forward_dense(x, C_a, K, wdd, wd, bd, o[0], pkg.ESC_NCHW, ws)
+        paths.append(pkg.esc_convattn_last_path())
+        pkg.esc_convattn_stencil_dense(x, C_a, K, wdd, dk, o[1], pkg.ESC_NCHW, ws)
+        paths.append(pkg.esc_convattn_last_path())
+        pkg.esc_convattn_backward_dense(x, god, C_a, K, wdd, wd, bd, o[2], *g, pkg.ESC_NCHW, wsb)
+        paths.append(pkg.esc_convattn_last_path())
+        torch.cuda.synchronize()
+        assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_device_status(wsb) == 0
+        assert paths == [5 if room else 1] * 3
+        res[room] = o + g
+        if not room:
+            with pytest.raises(pkg.EscError):
+                pkg.esc_convattn_forward_dense(x, C_a, K, wdd, wd, bd, o[0], pkg.ESC_NCHW, ws[:-1])
+            with pytest.raises(pkg.EscError):
+                pkg.esc_convattn_backward_dense(x, god, C_a, K, wdd, wd, bd, o[2], *g, pkg.ESC_NCHW, wsb[:-1])
+    # maps: fp32 sums in another order (5e-5 of magnitudes of about 10), one rounding each: at most one bf16 step apart; weight gradients:
+    # 1e-5 of the scale on either side
+    for a, b in zip(res[True][:3], res[False][:3]):
+        diff, size = (a.float() - b.float()).abs(), b.float().abs()
+        assert bool((diff <= 2.0 ** -7 * size + 1e-3).all()) and torch.equal(a[:, C_a:], b[:, C_a:])
+    for a, b in zip(res[True][3:], res[False][3:]):
+        assert float((a - b).abs().max()) <= 2e-5 * float(b.abs().max())
