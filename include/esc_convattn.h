@@ -165,9 +165,9 @@ int esc_convattn_stencil(const void* x, int B, int C, int C_a, int H, int W, int
 /*
  * End-to-end convenience call on HOST buffers: copies x and the weights to the device,
  * runs the forward pass, copies out back and synchronises.  Device buffers and private
- * streams are kept by the library between calls.  On NCHW tensors the identity channels travel
- * beside the kernels: their upload, and their way back, overlap the rest.  Host buffers should be pinned for full
- * copy bandwidth but need not be.
+ * streams are kept by the library between calls.  On NCHW tensors in pinned memory the identity channels
+ * travel beside the kernels: their upload, and their way back, overlap the rest.  Host buffers should be
+ * pinned for full copy bandwidth but need not be.
  */
 int esc_convattn_forward_host(const void* x_host, int B, int C, int C_a, int H, int W, int K,
                               const void* w_large_host, const void* w_dyn_host,
@@ -181,7 +181,8 @@ int esc_convattn_forward_host(const void* x_host, int B, int C, int C_a, int H, 
  * submit(i % 2) for step i, then wait((i - 1) % 2) -- the upload of one step overlaps the download
  * of the step before.  The host buffers must be pinned (page-locked) for the copies to be
  * asynchronous and must stay valid and untouched until the matching wait returns; two steps in
- * flight need two out_host buffers.  esc_convattn_forward_host is submit(0) followed by wait(0).
+ * flight need two out_host buffers.  esc_convattn_forward_host is submit(0) followed by wait(0)
+ * with the copies cut up as it says.
  * ESC_ERR_UNSUPPORTED for a slot other than 0 or 1.
  */
 int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C, int C_a, int H, int W, int K,

@@ -1091,16 +1091,33 @@ struct HostPath {
     void *x = nullptr, *out = nullptr, *wts = nullptr, *ws = nullptr;
     size_t xbytes = 0, wbytes = 0, wsbytes = 0;
 };
-// NCHW keeps the identity channels of an image in one contiguous piece, which neither kernel needs: it is uploaded behind the attention
-// channels and goes back, chunk by chunk, while the next chunk comes in and the kernels run.  (NHWC interleaves them with the
-// attention channels pixel by pixel; strided copies of the two parts take longer than the overlap gains: 96 of every 128 bytes
-// 0.60 ms and 32 of 128 0.44 ms against 0.52 ms for the whole map of 640x360x64 bf16.)  From 1 MB of identity channels on;
-// chunks of 4 MB, about 80 us each.  Blocking call, bf16: 640x360x64 1115 -> 890 us (1 MB chunks 1330, 16 MB 1220), 352x352x48
-// 614 -> 390, 120x96x64 (1.1 MB) 106 -> 95; fp32 640x360x64 2328 -> 1640.
-constexpr size_t kHostOverlapBytes = 1 << 20, kHostChunkBytes = 4 << 20;
+// NCHW keeps the identity channels of an image in one contiguous piece, which neither kernel needs: in a call that waits for its result
+// they are uploaded behind the attention channels and go back, piece by piece, while the next piece comes in and the kernels run.
+// (NHWC interleaves them with the attention channels pixel by pixel; strided copies of the two parts take longer than the overlap
+// gains: 96 of every 128 bytes 0.60 ms and 32 of 128 0.44 ms against 0.52 ms for the whole map of 640x360x64 bf16.)
+// Pieces of 4 MB, about 80 us each: part of an image, or several images as rows of one 2D copy.  From 1 MB of identity channels on, and
+// 16 KB of them an image: shorter rows lose more than the overlap gains.  Blocking call, whole map up and down / overlapped, bf16:
+// 640x360x64 1110 -> 870 us (1 MB pieces 1330), 320x180x64 315 -> 272; 64 x (64x64x64) 1260 -> 940 (a piece per image: 1390),
+// 40 x (48x48x48) 369 -> 310, 800 x (16x16x64) 1100 -> 900, 800 x (16x16x24), rows of 4 KB, 527 -> 573; fp32 640x360x64 2210 -> 1570.
+// Not between submit and wait: there the other slot's step fills both directions of the link, and pieces only add copies (640x360x64
+// bf16, two slots 687 -> 780, 64 x (64x64x64) 775 -> 1335); nor for pageable buffers, whose copies hold up the submitting thread.
+constexpr size_t kHostOverlapBytes = 1 << 20, kHostChunkBytes = 4 << 20, kHostMinRow = 16 << 10;
+constexpr size_t kHostMaxPitch = 0x7fffffff;               // of a 2D copy
 constexpr int kHostSlots = 2;
 std::mutex g_host_mu;
 HostPath g_host[kHostSlots];
+
+// Whether parts of `out` may travel while parts of `x` are still to come: both pinned, and not the same memory.
+bool host_buffers_allow(const void* x, const void* out, size_t bytes) {
+    const char *a = static_cast<const char*>(x), *b = static_cast<const char*>(out);
+    if (a < b + bytes && b < a + bytes) return false;
+    for (const void* q : {x, out}) {
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, q) != cudaSuccess) { (void)cudaGetLastError(); return false; }
+        if (at.type != cudaMemoryTypeHost) return false;
+    }
+    return true;
+}
 
 }  // namespace
 
@@ -1753,9 +1770,10 @@ int esc_convattn_device_status(void* workspace, void* stream) {
     return (int)word[0];
 }
 
-int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C, int C_a, int H, int W, int K,
-                                     const void* w_large_host, const void* w_dyn_host, const void* b_dyn_host,
-                                     void* out_host, int dtype, int layout) {
+namespace {
+// alone: the caller waits for this step before it submits another
+int host_submit(int slot, const void* x_host, int B, int C, int C_a, int H, int W, int K, const void* w_large_host, const void* w_dyn_host,
+                const void* b_dyn_host, void* out_host, int dtype, int layout, bool alone) {
     g_last_launches = 0;
     if (slot < 0 || slot >= kHostSlots) return ESC_ERR_UNSUPPORTED;
     const Problem p{B, C, C_a, H, W, K, dtype, layout};
@@ -1810,7 +1828,8 @@ int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C,
     }
     char* wts = static_cast<char*>(h.wts);
     const size_t image = xbytes / B, att = (size_t)C_a * H * W * es, identity = image - att;
-    const bool overlap = layout == ESC_NCHW && identity * B >= kHostOverlapBytes;
+    const bool overlap = alone && layout == ESC_NCHW && identity * B >= kHostOverlapBytes && identity >= kHostMinRow && image <= kHostMaxPitch &&
+                         host_buffers_allow(x_host, out_host, xbytes);
     if (overlap) ESC_CUDA(cudaMemcpy2DAsync(h.x, image, x_host, image, att, B, cudaMemcpyHostToDevice, h.st));
     else ESC_CUDA(cudaMemcpyAsync(h.x, x_host, xbytes, cudaMemcpyHostToDevice, h.st));
     ESC_CUDA(cudaMemcpyAsync(wts, w_large_host, n_wl * es, cudaMemcpyHostToDevice, h.st));
@@ -1837,13 +1856,17 @@ int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C,
         r = forward_impl(pa, h.x, wts, est, h.out, h.ws, h.compute);
         if (r != ESC_OK) return r;
         ESC_CUDA(cudaMemcpy2DAsync(out_host, image, h.out, image, att, B, cudaMemcpyDeviceToHost, h.compute));
-        for (int b = 0; b < B; ++b)
-            for (size_t at = att; at < image; at += kHostChunkBytes) {
-                const size_t off = (size_t)b * image + at, n = image - at < kHostChunkBytes ? image - at : kHostChunkBytes;
-                ESC_CUDA(cudaMemcpyAsync(static_cast<char*>(h.x) + off, static_cast<const char*>(x_host) + off, n, cudaMemcpyHostToDevice, h.st));
+        // pieces of about kHostChunkBytes: part of an image's identity channels, or those of several images
+        const size_t cols = identity < kHostChunkBytes ? identity : kHostChunkBytes;
+        const int rows = (int)std::min((size_t)B, kHostChunkBytes / cols);
+        for (int b = 0; b < B; b += rows)
+            for (size_t at = att; at < image; at += cols) {
+                const size_t off = (size_t)b * image + at, n = std::min(cols, image - at);
+                const int nb = std::min(rows, B - b);
+                ESC_CUDA(cudaMemcpy2DAsync(static_cast<char*>(h.x) + off, image, static_cast<const char*>(x_host) + off, image, n, nb, cudaMemcpyHostToDevice, h.st));
                 r = follow(h.down, h.st);
                 if (r != ESC_OK) return r;
-                ESC_CUDA(cudaMemcpyAsync(static_cast<char*>(out_host) + off, static_cast<char*>(h.x) + off, n, cudaMemcpyDeviceToHost, h.down));
+                ESC_CUDA(cudaMemcpy2DAsync(static_cast<char*>(out_host) + off, image, static_cast<char*>(h.x) + off, image, n, nb, cudaMemcpyDeviceToHost, h.down));
             }
         return ESC_OK;
     };
@@ -1851,6 +1874,13 @@ int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C,
     // the slot's stream ends behind the other two, also after an error: who waits for it waits for all
     const int r1 = follow(h.st, h.compute), r2 = follow(h.st, h.down);
     return rc != ESC_OK ? rc : r1 != ESC_OK ? r1 : r2;
+}
+}  // namespace
+
+int esc_convattn_forward_host_submit(int slot, const void* x_host, int B, int C, int C_a, int H, int W, int K,
+                                     const void* w_large_host, const void* w_dyn_host, const void* b_dyn_host,
+                                     void* out_host, int dtype, int layout) {
+    return host_submit(slot, x_host, B, C, C_a, H, W, K, w_large_host, w_dyn_host, b_dyn_host, out_host, dtype, layout, /*alone=*/false);
 }
 
 int esc_convattn_forward_host_wait(int slot) {
@@ -1868,8 +1898,7 @@ int esc_convattn_forward_host_wait(int slot) {
 int esc_convattn_forward_host(const void* x_host, int B, int C, int C_a, int H, int W, int K,
                               const void* w_large_host, const void* w_dyn_host, const void* b_dyn_host,
                               void* out_host, int dtype, int layout) {
-    int rc = esc_convattn_forward_host_submit(0, x_host, B, C, C_a, H, W, K, w_large_host, w_dyn_host, b_dyn_host,
-                                              out_host, dtype, layout);
+    const int rc = host_submit(0, x_host, B, C, C_a, H, W, K, w_large_host, w_dyn_host, b_dyn_host, out_host, dtype, layout, /*alone=*/true);
     if (rc != ESC_OK) return rc;
     return esc_convattn_forward_host_wait(0);
 }

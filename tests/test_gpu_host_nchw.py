@@ -51,3 +51,42 @@ def test_equals_device_entry(case):
     got.fill_(7.0)
     pkg.esc_convattn_forward_host(x, C_a, K, *w, got, pkg.ESC_NCHW)
     assert torch.equal(got, want)
+
+
+# Batches whose images are smaller than a piece (several images a piece, the last piece with fewer), larger ones, and what must not
+# overlap: pageable buffers, and an output that shares memory with the input.
+MANY = [
+    # B, C, C_a, H, W, K, dtype
+    (23, 64, 16, 64, 64, 13, synth.BF16),      # ten images a piece: 10, 10, 3
+    (40, 48, 16, 47, 53, 13, synth.BF16),      # images of 239 KB, odd planes
+    (7, 24, 16, 64, 300, 9, synth.F32),        # 614 KB of identity channels an image: six and one
+    (3, 64, 16, 210, 333, 13, synth.BF16),     # two pieces an image
+]
+
+
+@pytest.mark.parametrize("where", ["pinned", "pageable", "in_place", "shifted"])
+@pytest.mark.parametrize("case", MANY, ids=lambda c: "x".join(map(str, c)))
+def test_batches_and_buffers(case, where):
+    import torch
+
+    import paper_2503_06671_b200 as pkg
+
+    B, C, C_a, H, W, K, dtype = case
+    x, w = _setup(case, 11)
+    want = torch.empty_like(x, device="cuda")
+    pkg.esc_convattn_forward_ex(x.cuda(), C_a, K, *[t.cuda() for t in w], want, pkg.ESC_NCHW, pkg.new_workspace(B, C_a, H, W, K))
+    want = want.cpu()
+    n = x.numel()
+    for _ in range(3):
+        if where == "pinned":
+            xi, got = x, torch.full_like(x, 7.0).pin_memory()
+        elif where == "pageable":
+            xi, got = x.clone(), torch.full_like(x, 7.0)
+            assert not xi.is_pinned() and not got.is_pinned()
+        else:                                                  # the input is read as a whole before anything comes back
+            shift = 0 if where == "in_place" else C_a * H * W
+            buf = torch.zeros(n + shift, dtype=x.dtype).pin_memory()
+            xi, got = buf[shift:].view(x.shape), buf[:n].view(x.shape)
+            xi.copy_(x)
+        pkg.esc_convattn_forward_host(xi, C_a, K, *w, got, pkg.ESC_NCHW)
+        assert torch.equal(got, want)
