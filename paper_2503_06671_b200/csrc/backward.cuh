@@ -251,30 +251,48 @@ tap_grad_nhwc8(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca,
 }
 
 // ---- kernel 2a: add the tiles of one (image, channel) in a fixed order -----------------------------------------
-// Block = (image, channel); kSumGroups groups of 192 threads take every kSumGroups-th tile each (eight loads in
-// flight, added in order), then the groups' sums are added in group order.
+// Block = (image, channel); kSumGroups groups of 192 threads take every kSumGroups-th tile each (sixteen loads in
+// flight, added in order), then the groups' sums are added in group order.  In the decomposed form the sums of x that came with the
+// taps are those of the mixed features: the threads that have no tap add up the chunks' sums of x in their place.
 constexpr int kSumGroups = 4, kSumThreads = 192 * kSumGroups;
 __global__ void __launch_bounds__(kSumThreads)
-sum_tiles(const float* __restrict__ part, int tiles, float* __restrict__ gtap)   // gtap [B*Ca][kSlot]
+sum_tiles(const float* __restrict__ part, int tiles, const float* __restrict__ xs_part, int chunks, int Ca,
+          float* __restrict__ gtap)                              // gtap [B*Ca][kSlot]
 {
-    __shared__ float acc[kSumGroups][192];
+    constexpr int kSpare = 192 - (TAPS + 1), kX = kSpare * kSumGroups;
+    static_assert(kX > 64 && kX <= 96, "one warp adds the threads' sums of x");
+    __shared__ float acc[kSumGroups][192], xacc[96];
+    auto sum = [](const float* p, int n, size_t pitch, int first, int step) {      // p[first], p[first + step], ..: sixteen in flight
+        float s = 0.f;
+        for (int k0 = first; k0 < n; k0 += 16 * step) {
+            float v[16];
+#pragma unroll
+            for (int u = 0; u < 16; ++u) v[u] = k0 + u * step < n ? __ldcg(p + (size_t)(k0 + u * step) * pitch) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 16; ++u) s += v[u];
+        }
+        return s;
+    };
     const size_t bc = blockIdx.x;
     const int t = threadIdx.x % 192, grp = threadIdx.x / 192;
     pdl_launch_dependents();
     pdl_wait_primary();
     if (t <= TAPS) {
-        const float* p = part + bc * tiles * kSlot + t;
-        float s = 0.f;
-#pragma unroll 8
-        for (int k = grp; k < tiles; k += kSumGroups) s += __ldcg(p + (size_t)k * kSlot);
-        acc[grp][t] = s;
+        acc[grp][t] = sum(part + bc * tiles * kSlot + t, tiles, kSlot, grp, kSumGroups);
+    } else if (xs_part) {
+        const int x = grp * kSpare + t - (TAPS + 1);
+        xacc[x] = sum(xs_part + (bc / Ca) * chunks * Ca + bc % Ca, chunks, Ca, x, kX);
     }
     __syncthreads();
     if (grp == 0 && t <= TAPS) {
         float s = acc[0][t];
 #pragma unroll
         for (int q = 1; q < kSumGroups; ++q) s += acc[q][t];
-        gtap[bc * kSlot + t] = s;
+        if (t < TAPS || !xs_part) gtap[bc * kSlot + t] = s;
+    }
+    if (xs_part && grp == 1 && t < 32) {
+        const float s = warp_sum(xacc[t] + xacc[t + 32] + (t + 64 < kX ? xacc[t + 64] : 0.f));
+        if (t == 0) gtap[bc * kSlot + TAPS] = s;
     }
 }
 
@@ -295,128 +313,182 @@ constexpr int kDirectTiles = 16;
 struct Taps {
     const float* p;
     int tiles;
-    __device__ __forceinline__ float operator()(size_t bc, int slot) const {
+    template <bool kAll>                                         // all loads in flight, not four
+    __device__ __forceinline__ float get(size_t bc, int slot) const {
         const float* q = p + bc * tiles * kSlot + slot;
         float s = 0.f;
+        if constexpr (kAll) {
+            float v[kDirectTiles];
+#pragma unroll
+            for (int t = 0; t < kDirectTiles; ++t) v[t] = t < tiles ? __ldcg(q + (size_t)t * kSlot) : 0.f;
+#pragma unroll
+            for (int t = 0; t < kDirectTiles; ++t) s += v[t];
+        } else {
 #pragma unroll 4
-        for (int t = 0; t < tiles; ++t) s += __ldcg(q + (size_t)t * kSlot);
+            for (int t = 0; t < tiles; ++t) s += __ldcg(q + (size_t)t * kSlot);
+        }
         return s;
     }
 };
 // Per-image values for the sums over images: g_dk [B][9 Ca], pooled means [B][Ca], activations and g_t [B][hidden].
 struct ImageValues { float *gdk, *mean, *act, *gt; };
 
-// kernel 2b: block b < B is one image: its pooled means and g_dk, the estimator's forward values and the part of the chain that
-// belongs to one image; dk (rotated) and the GAP-path constant go to the stencil pass that follows.  The blocks behind them take
-// g_lk = sum_b g_tap, 32 consecutive taps each (the lanes), images dealt to the eight warps and the warps added in order, and
-// the last kFlipBlocks the rotated LK.  Bound: latency of a few dependent phases.  Every sum that is longer than a few terms is
-// taken by a warp and nothing waits for sum_tiles where there are few tiles: 64 patches of 64x64 with two layers took 6.5 (sum_tiles)
-// + 8.3 + 22 us cold, the last one a thread per output over 64 images; 8 + 4.6 us now, overlapping their neighbours.
+// kernel 2b.  An image is one block, or two where there are few images: its pooled means and g_dk, the estimator's forward values and the
+// part of the chain that belongs to one image; dk (rotated) and the GAP-path constant go to the stencil pass that follows -- of two blocks
+// the first writes dk and the second the constant.  The blocks behind them take g_lk = sum_b g_tap, 32 consecutive taps each (the
+// lanes), images dealt to the eight warps and the warps added in order, the kFlipBlocks behind those the rotated LK, and where there are
+// few images (kFew) the last ones the estimator's weight gradients, 256 elements each, from means and g_dk of their own.
+// Bound: latency of a few dependent phases.  Every sum that is longer than a few terms is taken by a warp and nothing waits for sum_tiles
+// where there are few tiles: 64 patches of 64x64 with two layers took 6.5 (sum_tiles) + 8.3 + 22 us cold, the last one a thread per
+// output over 64 images; 8 + 4.6 us now, overlapping their neighbours.
 constexpr int kFlipBlocks = 8, kEstThreads = 256, kEstMaxCa = 1024;
-template <typename T>
+// Few images: two blocks an image, and blocks of weight gradients that work out means, g_dk and the hidden layer of all images for
+// themselves instead of a launch behind this one.  Measured, whole backward pass, bf16 NHWC, as a launch of its own / here: one layer,
+// 640x360 57.7 / 54.5 us, 4 x (96x96) 30.3 / 28.6, 8 x (64x64) 29.1 / 28.7, 16 x (64x64) 29.7 / 30.2; two layers, h = 8, 640x360
+// 59.9 / 56.0, 2 x (96x96) 30.9 / 29.9, 4 x (64x64) 29.9 / 31.2, 8 x (64x64) 30.6 / 35.6.  Not where the means are sums over chunks
+// (decomposed, up to 16 tiles an image), image after image, from three images on: 2 x (96x96) 43.0 / 42.2, 8 x (64x64) 42.8 / 45.3; nor
+// in front of the dense form's stencil, which works ahead of dk and so hides the other launch: 64x64 42.6 / 43.4.
+inline bool few_images(int B, int Ca, int hidden, bool dense, bool chunk_means) {
+    return !dense && B <= kEstThreads / 32 && B * hidden <= 16 && (!chunk_means || B <= 2) && B * Ca <= kEstMaxCa;
+}
+struct EstimatorGrads { float *w_last, *b_last, *w_down, *b_down; };
+template <typename T, bool kFew>
 __global__ void __launch_bounds__(kEstThreads)
 estimator_image(const Taps taps, const float* __restrict__ xs_part, int chunks, int B, int Ca, int hidden, int H, int W, int KK,
                 const T* __restrict__ w_large, const T* __restrict__ w_down, const T* __restrict__ b_down,
                 const T* __restrict__ w_last, const T* __restrict__ b_last, const ImageValues iv, float* __restrict__ dk_flip,
-                float* __restrict__ bias, float* __restrict__ g_lk, T* __restrict__ w_flip)
+                float* __restrict__ bias, float* __restrict__ g_lk, T* __restrict__ w_flip, const EstimatorGrads eg)
 {
     extern __shared__ float sm[];
     __shared__ float red[kEstThreads];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, ltaps = KK * KK;
-    pdl_launch_dependents();
+    const int image_blocks = kFew ? 2 * B : B, lk_blocks = g_lk ? (Ca * ltaps + 31) / 32 : 0, flip_blocks = w_flip ? kFlipBlocks : 0;
+    const int job = (int)blockIdx.x - image_blocks;
+    // The stencil that follows few images gains nothing from an early start, its blocks only take the SMs' registers from these (640x360,
+    // 105 blocks: 62.9 us for the whole pass with it, 56.9 without).
+    if (!kFew) pdl_launch_dependents();
     pdl_wait_primary();
-    if (blockIdx.x >= (unsigned)B) {
-        const int job = blockIdx.x - B, lk_blocks = g_lk ? (Ca * ltaps + 31) / 32 : 0;
-        if (job < lk_blocks) {
-            const int e = job * 32 + lane, off = (K - KK) / 2;   // a smaller large kernel sits in the middle of the 13 x 13 taps
-            float s = 0.f;
-            if (e < Ca * ltaps) {
-                const int c = e / ltaps, t = (e % ltaps) / KK + off, u = (e % ltaps) % KK + off;
-#pragma unroll 4
-                for (int b = warp; b < B; b += kEstThreads / 32) s += taps((size_t)b * Ca + c, t * K + u);
-            }
-            red[tid] = s;
-            __syncthreads();
-            if (warp == 0 && e < Ca * ltaps) {
-                for (int w = 1; w < kEstThreads / 32; ++w) s += red[w * 32 + lane];
-                g_lk[e] = s;
-            }
-        } else if (w_flip) {
-            for (int e = (job - lk_blocks) * kEstThreads + tid; e < Ca * ltaps; e += kFlipBlocks * kEstThreads)
-                w_flip[(size_t)(e / ltaps) * ltaps + (ltaps - 1 - e % ltaps)] = w_large[e];
-        }
-        return;
-    }
-    const int b = blockIdx.x;
-    // [Ca] pooled means, [9 Ca] g_dk of this image: in shared memory, or where they go anyway if C_a is too large for it
-    float* aa = sm;                    // [hidden] activations
-    float* gs = aa + hidden;           // [hidden] g_t
-    float* gm = Ca <= kEstMaxCa ? gs + hidden : iv.mean + (size_t)b * Ca;
-    float* gd = Ca <= kEstMaxCa ? gm + Ca : iv.gdk + (size_t)b * 9 * Ca;
-    const float inv_hw = 1.0f / ((float)H * (float)W);
-    if (xs_part) {
-        // decomposed form: the taps saw the mixed features, the pooled means are those of x: chunks of pixels, dealt to groups of
-        // Ca threads, the groups added in order
-        const int ng = kEstThreads / Ca, k = tid % Ca, j = tid / Ca;
+    if (job >= 0 && job < lk_blocks) {
+        const int e = job * 32 + lane, off = (K - KK) / 2;       // a smaller large kernel sits in the middle of the 13 x 13 taps
         float s = 0.f;
-        if (j < ng) {
-#pragma unroll 8
-            for (int c = j; c < chunks; c += ng) s += __ldcg(xs_part + ((size_t)b * chunks + c) * Ca + k);
+        if (e < Ca * ltaps) {
+            const int c = e / ltaps, t = (e % ltaps) / KK + off, u = (e % ltaps) % KK + off;
+#pragma unroll 4
+            for (int b = warp; b < B; b += kEstThreads / 32) s += taps.template get<kFew>((size_t)b * Ca + c, t * K + u);
         }
         red[tid] = s;
         __syncthreads();
-        if (tid < Ca) {
-            for (int g = 1; g < ng; ++g) s += red[g * Ca + tid];
-            gm[tid] = s * inv_hw;
+        if (warp == 0 && e < Ca * ltaps) {
+            for (int w = 1; w < kEstThreads / 32; ++w) s += red[w * 32 + lane];
+            g_lk[e] = s;
         }
-    } else {
-        for (int k = tid; k < Ca; k += kEstThreads) gm[k] = taps((size_t)b * Ca + k, TAPS) * inv_hw;
+        return;
     }
-    for (int o = tid; o < 9 * Ca; o += kEstThreads) {             // o = c*9 + i*3 + j -> the middle 3x3 of the tap gradient
-        const int c = o / 9, i = (o % 9) / 3, j = o % 3;
-        const float v = taps((size_t)b * Ca + c, (i + P - 1) * K + (j + P - 1));
-        gd[o] = v;
-        iv.gdk[(size_t)b * 9 * Ca + o] = v;
+    if (job >= lk_blocks && job < lk_blocks + flip_blocks) {
+        for (int e = (job - lk_blocks) * kEstThreads + tid; e < Ca * ltaps; e += kFlipBlocks * kEstThreads)
+            w_flip[(size_t)(e / ltaps) * ltaps + (ltaps - 1 - e % ltaps)] = w_large[e];
+        return;
     }
-    __syncthreads();
-    for (int k = tid; k < Ca; k += kEstThreads) iv.mean[(size_t)b * Ca + k] = gm[k];
-    const float* vin = gm;
-    int n_in = Ca;
-    if (hidden > 0) {
-        for (int m = warp; m < hidden; m += kEstThreads / 32) {
-            float t = 0.f, g = 0.f;
-            for (int k = lane; k < Ca; k += 32) t = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gm[k], t);
+    const float inv_hw = 1.0f / ((float)H * (float)W);
+    // values of images b0 .. b0 + n - 1: pooled means gm [n][Ca], g_dk gd [n][9 Ca], activations aa and g_t gs [n][hidden]
+    auto images = [&](int b0, int images_n, float* gm, float* gd, float* aa, float* gs) {
+        const int n = kFew ? images_n : 1;
+        if (xs_part) {
+            // decomposed form: the taps saw the mixed features, the pooled means are those of x: chunks of pixels, dealt to groups of
+            // Ca threads, the groups added in order
+            const int ng = kEstThreads / Ca, k = tid % Ca, j = tid / Ca;
+            for (int b = 0; b < n; ++b) {
+                float s = 0.f;
+                if (j < ng) {
 #pragma unroll 8
-            for (int o = lane; o < 9 * Ca; o += 32) g = fmaf(Elem<T>::to_f32(w_last[(size_t)o * hidden + m]), gd[o], g);
-            t = warp_sum(t) + Elem<T>::to_f32(b_down[m]);
-            g = warp_sum(g) * gelu_exact_prime(t);
-            if (lane == 0) {
-                aa[m] = gelu_exact(t);
-                gs[m] = g;
-                iv.act[(size_t)b * hidden + m] = aa[m];
-                iv.gt[(size_t)b * hidden + m] = g;
+                    for (int c = j; c < chunks; c += ng) s += __ldcg(xs_part + ((size_t)(b0 + b) * chunks + c) * Ca + k);
+                }
+                if (b) __syncthreads();
+                red[tid] = s;
+                __syncthreads();
+                if (tid < Ca) {
+                    for (int g = 1; g < ng; ++g) s += red[g * Ca + tid];
+                    gm[b * Ca + tid] = s * inv_hw;
+                }
             }
+        } else {
+            for (int k = tid; k < n * Ca; k += kEstThreads) gm[k] = taps.template get<kFew>((size_t)b0 * Ca + k, TAPS) * inv_hw;
+        }
+        for (int o = tid; o < n * 9 * Ca; o += kEstThreads) {     // o = c*9 + i*3 + j -> the middle 3x3 of the tap gradient
+            const int c = o / 9, i = (o % 9) / 3, j = o % 3;
+            const float v = taps.template get<kFew>((size_t)b0 * Ca + c, (i + P - 1) * K + (j + P - 1));
+            gd[o] = v;
+            if (!kFew) iv.gdk[(size_t)b0 * 9 * Ca + o] = v;       // iv: for estimator_weights
         }
         __syncthreads();
-        vin = aa; n_in = hidden;
-    }
-    for (int o = tid; o < 9 * Ca; o += kEstThreads) {
-        float s = Elem<T>::to_f32(b_last[o]);
-#pragma unroll 8
-        for (int m = 0; m < n_in; ++m) s = fmaf(Elem<T>::to_f32(w_last[(size_t)o * n_in + m]), vin[m], s);
-        dk_flip[(size_t)b * Ca * 9 + (o / 9) * 9 + (8 - o % 9)] = s;
-    }
-    // bias[b][k] = g_g[b][k] / (H W): a warp per element
-    for (int k = warp; k < Ca; k += kEstThreads / 32) {
-        float s = 0.f;
+        if (!kFew)
+            for (int k = tid; k < n * Ca; k += kEstThreads) iv.mean[(size_t)b0 * Ca + k] = gm[k];
         if (hidden > 0) {
-            for (int m = lane; m < hidden; m += 32) s = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gs[m], s);
-        } else {
+            for (int bm = warp; bm < n * hidden; bm += kEstThreads / 32) {
+                const int b = kFew ? bm / hidden : 0, m = bm - b * hidden;            // one image where not few
+                float t = 0.f, g = 0.f;
+                for (int k = lane; k < Ca; k += 32) t = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gm[b * Ca + k], t);
 #pragma unroll 8
-            for (int o = lane; o < 9 * Ca; o += 32) s = fmaf(Elem<T>::to_f32(w_last[(size_t)o * Ca + k]), gd[o], s);
+                for (int o = lane; o < 9 * Ca; o += 32) g = fmaf(Elem<T>::to_f32(w_last[(size_t)o * hidden + m]), gd[b * 9 * Ca + o], g);
+                t = warp_sum(t) + Elem<T>::to_f32(b_down[m]);
+                g = warp_sum(g) * gelu_exact_prime(t);
+                if (lane == 0) {
+                    aa[bm] = gelu_exact(t);
+                    gs[bm] = g;
+                    if (!kFew) { iv.act[(size_t)b0 * hidden + bm] = aa[bm]; iv.gt[(size_t)b0 * hidden + bm] = g; }
+                }
+            }
+            __syncthreads();
         }
-        s = warp_sum(s);
-        if (lane == 0) bias[(size_t)b * Ca + k] = s * inv_hw;
+    };
+    const int n_in = hidden > 0 ? hidden : Ca;
+    if (kFew && job >= 0) {
+        // weight gradients of few images: elements as in estimator_weights, images in order
+        float *aa = sm, *gs = aa + B * hidden, *gm = gs + B * hidden, *gd = gm + B * Ca;
+        const int n0 = 9 * Ca * n_in, n1 = n0 + 9 * Ca, n2 = n1 + hidden * Ca, n3 = n2 + hidden;
+        const int e = (job - lk_blocks - flip_blocks) * kEstThreads + tid;
+        images(0, B, gm, gd, aa, gs);
+        const float *p = nullptr, *q = nullptr;
+        int sp = 0, sq = 0;
+        float* out = nullptr;
+        if (e < n0) { p = gd + e / n_in; sp = 9 * Ca; q = (hidden > 0 ? aa : gm) + e % n_in; sq = n_in; out = eg.w_last ? eg.w_last + e : nullptr; }
+        else if (e < n1) { p = gd + (e - n0); sp = 9 * Ca; out = eg.b_last ? eg.b_last + (e - n0) : nullptr; }
+        else if (e < n2) { p = gs + (e - n1) / Ca; sp = hidden; q = gm + (e - n1) % Ca; sq = Ca; out = eg.w_down ? eg.w_down + (e - n1) : nullptr; }
+        else if (e < n3) { p = gs + (e - n2); sp = hidden; out = eg.b_down ? eg.b_down + (e - n2) : nullptr; }
+        if (!out) return;
+        float s = 0.f;                                           // as estimator_weights adds up one image per warp: the same bits
+        for (int b = 0; b < B; ++b) s = __fadd_rn(s, q ? __fmul_rn(p[b * sp], q[b * sq]) : p[b * sp]);
+        *out = s;
+        return;
+    }
+    const int b = kFew ? blockIdx.x / 2 : blockIdx.x, part = kFew ? 1 + (blockIdx.x & 1) : 3;     // bit 0: dk, bit 1: the constant
+    float *aa = sm, *gs = aa + hidden;
+    // in shared memory, or where they go anyway if C_a is too large for it
+    float* gm = Ca <= kEstMaxCa ? gs + hidden : iv.mean + (size_t)b * Ca;
+    float* gd = Ca <= kEstMaxCa ? gm + Ca : iv.gdk + (size_t)b * 9 * Ca;
+    images(b, 1, gm, gd, aa, gs);
+    if (part & 1) {
+        const float* vin = hidden > 0 ? aa : gm;
+        for (int o = tid; o < 9 * Ca; o += kEstThreads) {
+            float s = Elem<T>::to_f32(b_last[o]);
+#pragma unroll 8
+            for (int m = 0; m < n_in; ++m) s = fmaf(Elem<T>::to_f32(w_last[(size_t)o * n_in + m]), vin[m], s);
+            dk_flip[(size_t)b * Ca * 9 + (o / 9) * 9 + (8 - o % 9)] = s;
+        }
+    }
+    if (part & 2) {
+        // bias[b][k] = g_g[b][k] / (H W): a warp per element
+        for (int k = warp; k < Ca; k += kEstThreads / 32) {
+            float s = 0.f;
+            if (hidden > 0) {
+                for (int m = lane; m < hidden; m += 32) s = fmaf(Elem<T>::to_f32(w_down[(size_t)m * Ca + k]), gs[m], s);
+            } else {
+#pragma unroll 8
+                for (int o = lane; o < 9 * Ca; o += 32) s = fmaf(Elem<T>::to_f32(w_last[(size_t)o * Ca + k]), gd[o], s);
+            }
+            s = warp_sum(s);
+            if (lane == 0) bias[(size_t)b * Ca + k] = s * inv_hw;
+        }
     }
 }
 

@@ -783,23 +783,30 @@ int backward_t(const Problem& p, const void* x, const void* go, const void* w_la
     // the estimator's part, from the tap gradients; few tiles are added up on the way
     const int tiles = tiles_done > 0 ? tiles_done : tiles_x * tiles_y;
     esc::bwd::Taps taps{w.part, tiles};
+    const float* xs_part = w.mixed ? w.xs_part : nullptr;
     if (tiles > esc::bwd::kDirectTiles) {
-        ESC_CUDA(launch_pdl(esc::bwd::sum_tiles, (unsigned)(p.B * p.Ca), esc::bwd::kSumThreads, 0, st, w.part, tiles, w.gtap));
+        ESC_CUDA(launch_pdl(esc::bwd::sum_tiles, (unsigned)(p.B * p.Ca), esc::bwd::kSumThreads, 0, st, w.part, tiles, xs_part, w.chunks, p.Ca,
+                            w.gtap));
         ++g_last_launches;
         taps = esc::bwd::Taps{w.gtap, 1};
+        xs_part = nullptr;                                   // the sums of x are in their place in gtap
     }
-    const size_t smem = (size_t)((p.Ca <= esc::bwd::kEstMaxCa ? 10 * p.Ca : 0) + 2 * est.hidden) * sizeof(float);
     const int ltaps = p.Ca * p.K * p.K;
-    const long long grid = (long long)p.B + (g.g_lk ? (ltaps + 31) / 32 : 0) + (p.dense ? 0 : esc::bwd::kFlipBlocks);
+    const bool weights = g.g_w_last || g.g_b_last || g.g_w_down || g.g_b_down;
+    const int elems = weights ? 9 * p.Ca * (est.hidden > 0 ? est.hidden : p.Ca) + 9 * p.Ca + est.hidden * p.Ca + est.hidden : 0;
+    const bool few = esc::bwd::few_images(p.B, p.Ca, est.hidden, p.dense, xs_part != nullptr);
+    const size_t smem = (size_t)((p.Ca <= esc::bwd::kEstMaxCa ? 10 * p.Ca : 0) + 2 * est.hidden) * sizeof(float) * (few ? p.B : 1);
+    const long long grid = (long long)p.B * (few ? 2 : 1) + (g.g_lk ? (ltaps + 31) / 32 : 0) + (p.dense ? 0 : esc::bwd::kFlipBlocks) +
+                           (few ? (elems + esc::bwd::kEstThreads - 1) / esc::bwd::kEstThreads : 0);
     if (grid > 0x7fffffffLL) return ESC_ERR_UNSUPPORTED;
-    ESC_CUDA(launch_pdl(esc::bwd::estimator_image<T>, (unsigned)grid, esc::bwd::kEstThreads, smem, st, taps,
-                        (const float*)(w.mixed ? w.xs_part : nullptr), w.chunks, p.B, p.Ca, est.hidden, p.H, p.W, p.K,
+    ESC_CUDA(launch_pdl(few ? esc::bwd::estimator_image<T, true> : esc::bwd::estimator_image<T, false>, (unsigned)grid, esc::bwd::kEstThreads,
+                        smem, st, taps, xs_part, w.chunks, p.B, p.Ca, est.hidden, p.H, p.W, p.K,
                         static_cast<const T*>(w_large), static_cast<const T*>(est.w_down), static_cast<const T*>(est.b_down),
                         static_cast<const T*>(est.w_last), static_cast<const T*>(est.b_last), w.iv, w.dk_flip, w.bias, g.g_lk,
-                        p.dense ? (T*)nullptr : static_cast<T*>(w.w_flip)));
+                        p.dense ? (T*)nullptr : static_cast<T*>(w.w_flip),
+                        esc::bwd::EstimatorGrads{g.g_w_last, g.g_b_last, g.g_w_down, g.g_b_down}));
     ++g_last_launches;
-    if (g.g_w_last || g.g_b_last || g.g_w_down || g.g_b_down) {
-        const int elems = 9 * p.Ca * (est.hidden > 0 ? est.hidden : p.Ca) + 9 * p.Ca + est.hidden * p.Ca + est.hidden;
+    if (weights && !few) {
         ESC_CUDA(launch_pdl(esc::bwd::estimator_weights, (unsigned)((elems + 31) / 32), esc::bwd::kEstThreads, 0, st, w.iv, p.B, p.Ca,
                             est.hidden, g.g_w_last, g.g_b_last, g.g_w_down, g.g_b_down));
         ++g_last_launches;

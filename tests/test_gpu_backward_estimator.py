@@ -33,6 +33,13 @@ CASES = [
     (33, 24, 5, 12, 10, 0, synth.F32, synth.NCHW),        # 45 estimator outputs
     (17, 16, 3, 9, 10, 128, synth.F32, synth.NHWC),       # the widest hidden layer
     (2, 1100, 1100, 5, 6, 0, synth.F32, synth.NCHW),      # more channels than shared memory has room for
+    # few images, whose weight gradients come from the same kernel: the most of them, with one and two layers, the most channels, and
+    # the next count, whose do not
+    (8, 16, 16, 200, 40, 0, synth.BF16, synth.NHWC),      # 13 tiles an image, added up on the way
+    (2, 16, 16, 280, 24, 8, synth.BF16, synth.NCHW),      # 18, by sum_tiles
+    (4, 256, 256, 6, 7, 0, synth.F32, synth.NCHW),
+    (1, 24, 5, 12, 10, 16, synth.F32, synth.NHWC),
+    (1, 24, 5, 12, 10, 17, synth.F32, synth.NHWC),
 ]
 
 

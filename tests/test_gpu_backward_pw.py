@@ -84,6 +84,8 @@ SHAPES = [
     (1, 48, 32, 37, 88, 13),     # C_a = 32: two channel groups, four (n, k) pairs per thread
     (2, 16, 16, 20, 65, 13),     # nothing but attention channels
     (1, 12, 4, 33, 35, 5),       # C_a = 4, K = 5, rows that are not 16-byte multiples
+    (9, 16, 16, 100, 150, 13),   # 21 tiles an image: the sums of x are added up beside the taps; many images
+    (2, 24, 8, 130, 170, 13),    # the same on the FP32 kernels, few images
 ]
 
 
