@@ -410,8 +410,8 @@ int esc_convattn_last_path(void);
  * the single rounding of the result to bf16.  In the tensor-core kernel one instruction sums 16
  * horizontally adjacent inputs, three of which may lie outside an output's 13-tap window with weight
  * zero: a non-finite attention input therefore turns outputs up to 15 pixels beyond its window into
- * NaN (finite data are unaffected); likewise where a kernel size lies in the zeros of the next one built (the generic
- * kernel: 9, 13, 17).  Returns ESC_ERR_UNSUPPORTED for any other value. */
+ * NaN, and (13 - K) / 2 more, up and down too, where a smaller kernel is padded to 13 x 13 (finite data are unaffected).  The
+ * generic kernel and those of the dense form keep it inside its window.  Returns ESC_ERR_UNSUPPORTED for any other value. */
 enum { ESC_ENGINE_AUTO = 0, ESC_ENGINE_FP32 = 1, ESC_ENGINE_TENSOR = 2 };
 int esc_convattn_set_stencil_engine(int engine);
 

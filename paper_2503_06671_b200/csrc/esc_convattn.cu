@@ -339,7 +339,7 @@ int launch_regtile(const Problem& p, const void* x, const void* w_large, const f
     cfg.attrs = attr;
     cfg.numAttrs = dependent ? 1 : 0;
     ESC_CUDA(cudaLaunchKernelEx(&cfg, esc::stencil_regtile<T, LAYOUT, KT, G, CB, PER_SM>, static_cast<const T*>(x), static_cast<T*>(out), p.C, p.Ca, p.H,
-                                p.W, p.K, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk, tiles_x, tiles_y, job, p.bias));
+                                p.W, static_cast<const T*>(w_large), static_cast<const T*>(p.w_point), dk, tiles_x, tiles_y, job, p.bias));
     ++g_last_launches;
     return ESC_OK;
 }
@@ -361,9 +361,17 @@ int launch_regtile_k(const Problem& p, const void* x, const void* w_large, const
 }
 template <typename T, int LAYOUT>
 int launch_generic_t(const Problem& p, const void* x, const void* w_large, const float* dk, void* out, cudaStream_t st, bool dependent) {
-    if (p.K <= 9) return launch_regtile_k<T, LAYOUT, 9>(p, x, w_large, dk, out, st, dependent);
-    if (p.K <= 13) return launch_regtile_k<T, LAYOUT, 13>(p, x, w_large, dk, out, st, dependent);
-    return launch_regtile_k<T, LAYOUT, 17>(p, x, w_large, dk, out, st, dependent);
+    switch (p.K) {
+        case 3: return launch_regtile_k<T, LAYOUT, 3>(p, x, w_large, dk, out, st, dependent);
+        case 5: return launch_regtile_k<T, LAYOUT, 5>(p, x, w_large, dk, out, st, dependent);
+        case 7: return launch_regtile_k<T, LAYOUT, 7>(p, x, w_large, dk, out, st, dependent);
+        case 9: return launch_regtile_k<T, LAYOUT, 9>(p, x, w_large, dk, out, st, dependent);
+        case 11: return launch_regtile_k<T, LAYOUT, 11>(p, x, w_large, dk, out, st, dependent);
+        case 13: return launch_regtile_k<T, LAYOUT, 13>(p, x, w_large, dk, out, st, dependent);
+        case 15: return launch_regtile_k<T, LAYOUT, 15>(p, x, w_large, dk, out, st, dependent);
+        case 17: return launch_regtile_k<T, LAYOUT, 17>(p, x, w_large, dk, out, st, dependent);
+    }
+    return ESC_ERR_UNSUPPORTED;
 }
 
 int launch_generic(const Problem& p, const void* x, const void* w_large, const float* dk, void* out,
@@ -529,16 +537,23 @@ int launch_dense_fp32_k(const Problem& p, const void* x, const void* w_dense, co
     cfg.attrs = attr;
     cfg.numAttrs = n;
     ESC_CUDA(cudaLaunchKernelEx(&cfg, D::stencil_dense_fp32<T, LAYOUT, K>, static_cast<const T*>(x), static_cast<T*>(out), p.C, p.H, p.W,
-                                p.K, static_cast<const T*>(w_dense), dk, p.bias, tiles_x, tiles_y, split, job));
+                                static_cast<const T*>(w_dense), dk, p.bias, tiles_x, tiles_y, split, job));
     ++g_last_launches;
     return ESC_OK;
 }
-// Compiled for the sizes the paper compares (9, 13, 17); any other odd K is the next larger one with zeros around it.
 template <typename T, int LAYOUT>
 int launch_dense_fp32_t(const Problem& p, const void* x, const void* w_dense, const float* dk, void* out, cudaStream_t st, bool dependent) {
-    if (p.K <= 9) return launch_dense_fp32_k<T, LAYOUT, 9>(p, x, w_dense, dk, out, st, dependent);
-    if (p.K <= 13) return launch_dense_fp32_k<T, LAYOUT, 13>(p, x, w_dense, dk, out, st, dependent);
-    return launch_dense_fp32_k<T, LAYOUT, 17>(p, x, w_dense, dk, out, st, dependent);
+    switch (p.K) {
+        case 3: return launch_dense_fp32_k<T, LAYOUT, 3>(p, x, w_dense, dk, out, st, dependent);
+        case 5: return launch_dense_fp32_k<T, LAYOUT, 5>(p, x, w_dense, dk, out, st, dependent);
+        case 7: return launch_dense_fp32_k<T, LAYOUT, 7>(p, x, w_dense, dk, out, st, dependent);
+        case 9: return launch_dense_fp32_k<T, LAYOUT, 9>(p, x, w_dense, dk, out, st, dependent);
+        case 11: return launch_dense_fp32_k<T, LAYOUT, 11>(p, x, w_dense, dk, out, st, dependent);
+        case 13: return launch_dense_fp32_k<T, LAYOUT, 13>(p, x, w_dense, dk, out, st, dependent);
+        case 15: return launch_dense_fp32_k<T, LAYOUT, 15>(p, x, w_dense, dk, out, st, dependent);
+        case 17: return launch_dense_fp32_k<T, LAYOUT, 17>(p, x, w_dense, dk, out, st, dependent);
+    }
+    return ESC_ERR_UNSUPPORTED;
 }
 
 // bf16 NCHW, dense form: the attention channels packed pixel by pixel, the identity planes copied (out may be null: packing only).

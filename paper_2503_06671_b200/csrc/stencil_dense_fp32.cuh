@@ -43,17 +43,16 @@ template <int K> struct Geo {
     static constexpr int kStage = kTile + K * K * kWPitch;
     static constexpr int kRed = kAcc * kThreads;                      // the accumulators of a block, for the cluster's sum
     static constexpr size_t smem_bytes(int split) { return sizeof(float) * (size_t)(split > 1 && kRed > 2 * kStage ? kRed : 2 * kStage); }
-    static_assert(Pitch >= 2 * Cols && Pitch % 16 == 4 && kTile % 4 == 0 && Cols <= 96 && Rows % 4 == 0, "16-byte rows, distinct banks; staging");
+    static_assert(Pitch >= 2 * Cols && Pitch % 16 == 4 && kTile % 4 == 0 && Cols <= 96, "16-byte rows, distinct banks; staging");
 };
 
 __device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
 
-// KK is the caller's kernel size, K >= KK the compiled one: a smaller kernel sits in the middle of zeros.
 template <typename T, int LAYOUT, int K>
 __global__ void __launch_bounds__(kThreads, 4)
-stencil_dense_fp32(const T* __restrict__ x, T* __restrict__ out, int C, int H, int W, int KK, const T* __restrict__ w_dense,
+stencil_dense_fp32(const T* __restrict__ x, T* __restrict__ out, int C, int H, int W, const T* __restrict__ w_dense,
                    const float* __restrict__ dk, const float* __restrict__ bias, int tiles_x, int tiles_y, int split, const CopyJob job)
 {
     namespace cg = cooperative_groups;
@@ -72,7 +71,7 @@ stencil_dense_fp32(const T* __restrict__ x, T* __restrict__ out, int C, int H, i
     const int ty = (int)(u % (unsigned)tiles_y);
     const int b = (int)(u / (unsigned)tiles_y);
     const int xpos = (lane & 1) + 2 * (lane >> 3), row = ((lane >> 1) & 3) + 4 * (warp >> 1);
-    const int x0 = tx * TX - P, y0 = ty * TY - P, off = (K - KK) / 2;
+    const int x0 = tx * TX - P, y0 = ty * TY - P;
 
     unsigned long long acc2[PX][NH / 2];                  // output channels 2q, 2q + 1 of this half
 #pragma unroll
@@ -106,20 +105,13 @@ stencil_dense_fp32(const T* __restrict__ x, T* __restrict__ out, int C, int H, i
         float* wm = buf + G::kTile;
 #pragma unroll 1
         for (int n = warp; n < CA; n += 4) {
-            const T* wk = w_dense + ((size_t)n * CA + k) * KK * KK;
+            const T* wk = w_dense + ((size_t)n * CA + k) * K * K;
 #pragma unroll
             for (int u = 0; u < (K * K + 31) / 32; ++u) {
                 const int t = lane + 32 * u;
                 if (t < K * K) {
-                    int e = t;
-                    bool v = true;
-                    if (off != 0) {
-                        const int i = t / K - off, j = t % K - off;
-                        v = (unsigned)i < (unsigned)KK && (unsigned)j < (unsigned)KK;
-                        e = v ? i * KK + j : 0;
-                    }
-                    if constexpr (sizeof(T) == 4) fuse::cp_async4((uint32_t)__cvta_generic_to_shared(wm + t * kWPitch + n), wk + e, v);
-                    else wm[t * kWPitch + n] = v ? Elem<T>::to_f32(wk[e]) : 0.f;
+                    if constexpr (sizeof(T) == 4) fuse::cp_async4((uint32_t)__cvta_generic_to_shared(wm + t * kWPitch + n), wk + t, true);
+                    else wm[t * kWPitch + n] = Elem<T>::to_f32(wk[t]);
                 }
             }
         }

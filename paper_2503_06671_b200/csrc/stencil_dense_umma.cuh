@@ -67,7 +67,7 @@ struct Params {
     int B, C, H, W;
     int strips, segs, seg_rows;       // per image: strips of 128 pixels x row ranges of seg_rows rows
     const __nv_bfloat16* w_dense;     // [16][16][KK][KK]  (output channel, input channel, row, column)
-    int KK;                           // odd, at most 13: a smaller kernel sits in the middle of zeros
+    int KK;                           // odd, at most 13: a smaller kernel is the middle of the table, and only that is multiplied
     int raw_bulk;                     // w_dense is 16-byte aligned: it is staged with bulk copies
     int flip;                         // the gradient's form: channel axes of w_dense swapped, taps rotated by 180 degrees
     const float* dk;                  // [B][16][9]
@@ -218,10 +218,6 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
             request_rows(0, kRawRows);
         }
     }
-    if (p.KK < K13) {
-        for (int e = tid; e < B_BYTES / 16; e += kThreads) reinterpret_cast<uint4*>(btab)[e] = make_uint4(0u, 0u, 0u, 0u);
-        __syncthreads();
-    }
     // clear the accumulators: every instruction accumulates, a row's columns are cleared again after it is read
     if (warp >= 2) {
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -294,6 +290,7 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
         // ======================= tensor-core instructions =============================================
         bool alive = true;
         const uint32_t ring_a = smem_u32(ring), btab_a = smem_u32(btab);
+        const int off = (K13 - p.KK) / 2;                                      // first tap column and kernel row of a smaller kernel
         for (int n = 0; n < n_in; ++n) {
             const int slot = n % NRING;
             alive = mbar_wait_warp(rowfull0 + 8 * slot, (unsigned)((n / NRING) & 1), p.ctrl, 0xD2000000u | (unsigned)n);
@@ -310,21 +307,21 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
                 break;
             }
             tc_fence_after();
-            // input row n feeds output rows n - 12 + c, c = 0 .. 12 (kernel row 12 - c), those inside [0, L)
-            const int c_lo = max(0, (K13 - 1) - n), c_hi = min(K13 - 1, L - 1 - n + (K13 - 1));
+            // input row n feeds output rows n - 12 + c, c = off .. 12 - off (kernel row 12 - c), those inside [0, L)
+            const int c_lo = max(off, (K13 - 1) - n), c_hi = min(K13 - 1 - off, L - 1 - n + (K13 - 1));
             if (c_lo <= c_hi) {
                 const int cnt = c_hi - c_lo + 1, s0 = (n - (K13 - 1) + c_lo) % SLOTS;
                 const int cnt1 = min(cnt, SLOTS - s0), cnt2 = cnt - cnt1;          // the row slots wrap around at 32
                 const uint32_t id1 = instr_desc(cnt1 * CG);
-                unsigned long long da = smem_desc_sw32(ring_a + (uint32_t)(slot * ROW_BYTES));
-                unsigned long long db = smem_desc(btab_a + (uint32_t)(c_lo * CG * 16), BHALF_BYTES, 128);
+                unsigned long long da = smem_desc_sw32(ring_a + (uint32_t)(slot * ROW_BYTES)) + (unsigned long long)(2 * off);
+                unsigned long long db = smem_desc(btab_a + (uint32_t)(off * BJ_BYTES + c_lo * CG * 16), BHALF_BYTES, 128);
                 if (cnt2 == 0) {
 #pragma unroll
                     for (int j = 0; j < K13; ++j)                              // one pixel (32 bytes) and one tap column further on
-                        mma_f16(tmem + (uint32_t)(s0 * CG), da + (unsigned long long)(2 * j), db + (unsigned long long)(j * (BJ_BYTES >> 4)), id1);
+                        if (j < p.KK) mma_f16(tmem + (uint32_t)(s0 * CG), da + (unsigned long long)(2 * j), db + (unsigned long long)(j * (BJ_BYTES >> 4)), id1);
                 } else {
                     const uint32_t id2 = instr_desc(cnt2 * CG);
-                    for (int j = 0; j < K13; ++j) {
+                    for (int j = 0; j < p.KK; ++j) {
                         mma_f16(tmem + (uint32_t)(s0 * CG), da, db, id1);
                         mma_f16(tmem, da, db + (unsigned long long)(cnt1 * CG), id2);
                         da += 2; db += BJ_BYTES >> 4;

@@ -52,9 +52,9 @@ __device__ __forceinline__ void run_copy_job(const CopyJob& j, unsigned rank, un
 
 // Register-tiled variant: a patch of outputs per thread.  The loop runs over the input rows that a patch touches: a row costs a few
 // 16-byte reads and is used by up to OY output rows, each with its kernel row (broadcast 16-byte reads).  It serves the fp32 cases
-// and the bf16 ones that no tensor-core or TMA kernel takes.  KT, the kernel size it is built for, is 9, 13 or 17; a smaller odd
-// kernel lies in the middle of zeros (a one-output-per-thread loop over the taps themselves, the kernel above, is three times slower:
-// 174x131 fp32, K = 17, whole forward, 48 -> 21 us).
+// and the bf16 ones that no tensor-core or TMA kernel takes.  Built for every odd kernel size KT (one in the middle of a larger one's
+// zeros would multiply inputs outside its window, and make NaN of the non-finite ones).  A thread per output in a loop over the taps
+// took 48 us where this takes 21 (174x131 fp32, K = 17, whole forward).
 // Two geometries: 64 x 32 tiles with 2 x 8 patches, and 32 x 32 tiles with 2 x 4 patches for launches that would otherwise leave most
 // SMs with one block or none (a 64x64 fp32 map: 15 us as 16 tiles of 64 x 64, 6 us as 64 of the smallest).  PER_SM blocks an SM: 8
 // (64 registers a thread) where there are as many, 6 (80 registers, fewer instructions) where there are not: 640x360 fp32, whole
@@ -74,11 +74,11 @@ using RtSmall = RtGeom<64, 32, 8, 2>;
 using RtTiny = RtGeom<32, 32, 4, 2>;
 template <class G, int KT, int CB>
 struct RtLayout {
-    static constexpr int Pitch = G::TX + KT - 1, Rows = G::TY + KT - 1;           // floats per staged row, a multiple of 4; staged rows
+    static constexpr int Pitch = (G::TX + KT + 2) / 4 * 4, Rows = G::TY + KT - 1; // floats per staged row, a multiple of 4; staged rows
     static constexpr int WRow = (KT + 3) / 4 * 4;                                 // taps per kernel row, padded
     static constexpr int Threads = CB * G::Threads;
     static constexpr int Floats = CB * (Rows * Pitch + KT * WRow);
-    static_assert(KT % 4 == 1 && G::TX * G::TY <= Rows * Pitch, "16-byte rows; the results fit in the tile's place");
+    static_assert(KT % 2 == 1 && G::TX * G::TY <= Rows * Pitch, "the results fit in the tile's place");
     static int bytes(int Ca, bool mix) { return (Floats + (mix ? CB * Ca : 0)) * 4; }
 };
 
@@ -102,7 +102,7 @@ template <> struct Vec4<__nv_bfloat16> {
 
 template <typename T, int LAYOUT, int KT, class G, int CB, int PER_SM>
 __global__ void __launch_bounds__(CB * 128, PER_SM)
-stencil_regtile(const T* __restrict__ x, T* __restrict__ out, int C, int Ca, int H, int W, int K,
+stencil_regtile(const T* __restrict__ x, T* __restrict__ out, int C, int Ca, int H, int W,
                 const T* __restrict__ w_large, const T* __restrict__ w_point, const float* __restrict__ dk,
                 int tiles_x, int tiles_y, const CopyJob job, const float* __restrict__ bias)
 {
@@ -174,8 +174,8 @@ stencil_regtile(const T* __restrict__ x, T* __restrict__ out, int C, int Ca, int
         }
     }
     for (int t = tid; t < CB * KT * WRow; t += Threads) {
-        const int i = t / WRow % KT - (KT - K) / 2, j = t % WRow - (KT - K) / 2;
-        wms[t] = (unsigned)i < (unsigned)K && (unsigned)j < (unsigned)K ? Elem<T>::to_f32(w_large[((size_t)(c0 + t / (KT * WRow)) * K + i) * K + j]) : 0.f;
+        const int i = t / WRow % KT, j = t % WRow;
+        wms[t] = j < KT ? Elem<T>::to_f32(w_large[((size_t)(c0 + t / (KT * WRow)) * KT + i) * KT + j]) : 0.f;
     }
     __syncthreads();
 
@@ -200,10 +200,11 @@ stencil_regtile(const T* __restrict__ x, T* __restrict__ out, int C, int Ca, int
             __syncthreads();
         }
         const int r = rr < kLate ? rr : rr < kRows - kLateRows ? rr + kLateRows : rr - (kRows - kLateRows) + kLate;   // input row of the patch window
-        float in[OX + KT - 1];
+        constexpr int kIn = (OX + KT + 2) / 4 * 4;         // OX + KT - 1 of them are used
+        float in[kIn];
         const float4* trow = reinterpret_cast<const float4*>(tile + (ly * OY + r) * Pitch + lx * OX);
 #pragma unroll
-        for (int v = 0; v < (OX + KT - 1) / 4; ++v) {
+        for (int v = 0; v < kIn / 4; ++v) {
             const float4 q = trow[v];
             in[4 * v] = q.x; in[4 * v + 1] = q.y; in[4 * v + 2] = q.z; in[4 * v + 3] = q.w;
         }
