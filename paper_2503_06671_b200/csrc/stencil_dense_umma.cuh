@@ -154,6 +154,9 @@ __device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap
     tma_load_4d(dst, map, bar, c0, c1, c2, c3);
 }
 
+// kSmall: K < 13.  Of its own, so that the unrolled issue loop of the full size keeps its constants (with both in one kernel 640x360
+// took 28.8 us for 28.2).
+template <bool kSmall>
 __global__ void __launch_bounds__(kThreads, 1)
 stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const __grid_constant__ CUtensorMap map_cin,
                              const __grid_constant__ CUtensorMap map_cout, const Params p)
@@ -290,7 +293,7 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
         // ======================= tensor-core instructions =============================================
         bool alive = true;
         const uint32_t ring_a = smem_u32(ring), btab_a = smem_u32(btab);
-        const int off = (K13 - p.KK) / 2;                                      // first tap column and kernel row of a smaller kernel
+        const int off = kSmall ? (K13 - p.KK) / 2 : 0;                         // first tap column and kernel row of a smaller kernel
         for (int n = 0; n < n_in; ++n) {
             const int slot = n % NRING;
             alive = mbar_wait_warp(rowfull0 + 8 * slot, (unsigned)((n / NRING) & 1), p.ctrl, 0xD2000000u | (unsigned)n);
@@ -313,17 +316,18 @@ stencil_dense_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_half, const
                 const int cnt = c_hi - c_lo + 1, s0 = (n - (K13 - 1) + c_lo) % SLOTS;
                 const int cnt1 = min(cnt, SLOTS - s0), cnt2 = cnt - cnt1;          // the row slots wrap around at 32
                 const uint32_t id1 = instr_desc(cnt1 * CG);
-                unsigned long long da = smem_desc_sw32(ring_a + (uint32_t)(slot * ROW_BYTES)) + (unsigned long long)(2 * off);
-                unsigned long long db = smem_desc(btab_a + (uint32_t)(off * BJ_BYTES + c_lo * CG * 16), BHALF_BYTES, 128);
-                if (cnt2 == 0) {
+                unsigned long long da = smem_desc_sw32(ring_a + (uint32_t)(slot * ROW_BYTES));
+                unsigned long long db = smem_desc(btab_a + (uint32_t)(c_lo * CG * 16), BHALF_BYTES, 128);
+                if (!kSmall && cnt2 == 0) {
 #pragma unroll
                     for (int j = 0; j < K13; ++j)                              // one pixel (32 bytes) and one tap column further on
-                        if (j < p.KK) mma_f16(tmem + (uint32_t)(s0 * CG), da + (unsigned long long)(2 * j), db + (unsigned long long)(j * (BJ_BYTES >> 4)), id1);
+                        mma_f16(tmem + (uint32_t)(s0 * CG), da + (unsigned long long)(2 * j), db + (unsigned long long)(j * (BJ_BYTES >> 4)), id1);
                 } else {
                     const uint32_t id2 = instr_desc(cnt2 * CG);
-                    for (int j = 0; j < p.KK; ++j) {
+                    if (kSmall) { da += 2 * off; db += off * (BJ_BYTES >> 4); }
+                    for (int j = 0; j < (kSmall ? p.KK : K13); ++j) {
                         mma_f16(tmem + (uint32_t)(s0 * CG), da, db, id1);
-                        mma_f16(tmem, da, db + (unsigned long long)(cnt1 * CG), id2);
+                        if (!kSmall || cnt2) mma_f16(tmem, da, db + (unsigned long long)(cnt1 * CG), id2);
                         da += 2; db += BJ_BYTES >> 4;
                     }
                 }
@@ -529,13 +533,15 @@ inline int try_launch_dense_umma(int B, int C, int Ca, int H, int W, int K, int 
     } else {
         m_cin = m_half; m_cout = m_half;
     }
-    static bool attr_set[kMaxDevices] = {};
+    const bool small = K < K13;
+    auto* kernel = small ? stencil_dense_umma_nhwc_bf16<true> : stencil_dense_umma_nhwc_bf16<false>;
+    static bool attr_set[2][kMaxDevices] = {};
     const int dev = current_device();
     if (dev < 0) return kNotApplicable;
-    if (!attr_set[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(stencil_dense_umma_nhwc_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
+    if (!attr_set[small][dev]) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes);
         if (e != cudaSuccess) { (void)cudaGetLastError(); return kNotApplicable; }
-        attr_set[dev] = true;
+        attr_set[small][dev] = true;
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas);
@@ -547,7 +553,7 @@ inline int try_launch_dense_umma(int B, int C, int Ca, int H, int W, int K, int 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, stencil_dense_umma_nhwc_bf16, m_half, m_cin, m_cout, p);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, m_half, m_cin, m_cout, p);
     if (e != cudaSuccess) {
         char buf[256];
         snprintf(buf, sizeof buf, "stencil_dense_umma_nhwc_bf16 launch: %s (%s)", cudaGetErrorName(e), cudaGetErrorString(e));
