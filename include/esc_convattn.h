@@ -216,9 +216,9 @@ int esc_convattn_stencil_pw(const void* x, int B, int C, int C_a, int H, int W, 
  * every attention output channel sums over all C_a attention input channels and all K*K taps; the
  * dynamic 3x3 kernel stays depth-wise.
  *   w_dense [C_a,C_a,K,K]   (output channel, input channel, row, column), device, the tensor's dtype
- * For bf16 NHWC tensors with K = 13 and C_a = 16 the first sum runs on the tensor cores (bf16 products,
- * fp32 accumulation, implicit GEMM over the TMA-staged halo tile); anything else takes a slow
- * one-thread-per-output kernel.  Other arguments as for esc_convattn_forward_ex / esc_convattn_stencil.
+ * For bf16 tensors with K <= 13 and C_a = 16 the first sum runs on the tensor cores (bf16 products, fp32
+ * accumulation; NCHW from 4,096 pixels on, through the workspace); the other cases with C_a = 16 take an FP32
+ * implicit GEMM, any other C_a a slow one-thread-per-output kernel.  Other arguments as for esc_convattn_forward_ex / esc_convattn_stencil.
  */
 int esc_convattn_forward_dense(const void* x, int B, int C, int C_a, int H, int W, int K,
                                const void* w_dense, const void* w_dyn, const void* b_dyn,

@@ -169,7 +169,7 @@ tap_grad(const T* __restrict__ x, const T* __restrict__ go, int C, int Ca, int H
 // In NHWC a block per channel would fetch every pixel's line once per channel with 2-byte loads.  Here a block
 // takes eight neighbouring channels (16 bytes of a bf16 pixel, 32 of an fp32 one) of a 32x32 tile: pixels are
 // read with 16-byte loads and spread over eight planar fp32 tiles in shared memory; warp w then works on channel
-// w on its own (8x4 patch of go per lane), so the block sum of the 13 values is one shuffle butterfly.
+// w on its own (8x4 patch of go per lane), so the sums of a row's 13 values stay inside the warp.
 namespace n8 {
 constexpr int TX = 32, TY = 32, CH = 8;
 constexpr int XP = TX + K - 1, XR = TY + K - 1;          // 44 x 44 staged x per channel (44 is a multiple of 4)

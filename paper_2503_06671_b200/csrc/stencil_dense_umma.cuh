@@ -150,9 +150,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, unsigne
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2, int c3) {
-    tma_load_4d(dst, map, bar, c0, c1, c2, c3);
-}
 
 // kSmall: K < 13.  Of its own, so that the unrolled issue loop of the full size keeps its constants (with both in one kernel 640x360
 // took 28.8 us for 28.2).

@@ -1,5 +1,5 @@
-"""The host-buffer entry on NCHW tensors, whose identity channels travel beside the kernels in chunks: equal to the device entry bit
-for bit, one and several images and chunks, both element types, odd widths, kernel sizes, two slots in turn."""
+"""The host-buffer entries on NCHW tensors, whose identity channels travel beside the kernels in pieces in the blocking call: equal to
+the device entry bit for bit, one and several images and pieces, both element types, odd widths, kernel sizes; two slots in turn."""
 import pytest
 
 from paper_2503_06671_b200 import synth
