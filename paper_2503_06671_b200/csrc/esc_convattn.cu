@@ -24,6 +24,7 @@
 #include "backward_toeplitz_nchw.cuh"
 #include "stencil_dense.cuh"
 #include "stencil_dense_umma.cuh"
+#include "stencil_dw_umma.cuh"
 #include "stencil_dense_fp32.cuh"
 #include "dense_nchw.cuh"
 #include <type_traits>
@@ -403,9 +404,17 @@ struct TensorLk {
     const void* w;
     int K;
 };
+// Whether the depth-wise stage goes to the tcgen05 kernel: bf16 NHWC without the point-wise mix, unless the caller pinned the FP32
+// kernel (by engine or by one of its tile widths), and more work than the one-launch form of the mma.sync kernel takes.  It takes
+// every odd K up to 13 as it is.
+bool dw_umma_follows(const Problem& p) {
+    return !p.dense && !p.w_point && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
+           esc::tma::dwu::applies(p.C, p.Ca, p.K, p.dtype, p.layout) &&
+           esc::tma::toep::units_of<esc::tma::toep::Shape64x16>(p.B, p.Ca, p.H, p.W) > (long long)esc::tma::toep::kMaxFusedUnits * sms_or_nominal();
+}
 TensorLk tensor_lk(const Problem& p, const void* x, const void* out, const void* w_large, void* pad, cudaStream_t st) {
     TensorLk t{w_large, p.K};
-    if (p.dense || p.dtype != ESC_BF16 || p.K >= esc::tma::K13 || !pad || g_engine_policy == ESC_ENGINE_FP32 || g_tile_policy != 0) return t;
+    if (p.dense || dw_umma_follows(p) || p.dtype != ESC_BF16 || p.K >= esc::tma::K13 || !pad || g_engine_policy == ESC_ENGINE_FP32 || g_tile_policy != 0) return t;
     if (!esc::tma::toep::applies(p.C, p.Ca, esc::tma::K13, p.dtype, p.layout) &&
         !esc::tma::toepn::takes(p.B, p.C, p.Ca, p.H, p.W, esc::tma::K13, p.dtype, p.layout, x, out))
         return t;
@@ -423,6 +432,12 @@ int launch_stencil(const Problem& p0, const void* x, const void* w_large0, const
     Problem p = p0;
     const void* w_large = w_large0;
     if (tl) { p.K = tl->K; w_large = tl->w; }
+    if (dw_umma_follows(p0)) {
+        const int rc = esc::tma::dwu::try_launch(p0.B, p0.C, p0.Ca, p0.H, p0.W, p0.K, p0.dtype, p0.layout, x, w_large0, dk, p0.bias, out, ctrl, st,
+                                                        dependent, &g_last_launches, &g_last_error, p0.skip_copy);
+        if (rc == ESC_OK) { g_last_path = 4; g_last_tile_w = esc::tma::dwu::WPX; return ESC_OK; }
+        if (rc != esc::tma::kNotApplicable) return rc;
+    }
     // Depth-wise K = 13 on NHWC bf16: the tensor-core (Toeplitz) kernel unless the caller pinned the FP32
     // kernel (by engine or by one of its tile widths) or asked for the point-wise mix, which only the
     // FP32 kernel carries.

@@ -1,0 +1,127 @@
+"""The tcgen05 depth-wise kernel (bf16 NHWC, more work than the one-launch form takes) against the oracle: windows that hold many small
+images, image rows of one to a few hundred pixels, row segments, channel groups, every kernel size's ends, the copied channels, the
+constant per (image, channel) of the backward pass, and the reach of a non-finite input."""
+import numpy as np
+import pytest
+
+from paper_2503_06671_b200 import synth
+from tests import util
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [
+    # B, C, C_a, H, W, K: more than 1,184 tiles of 64x16 x 16 channels
+    (1300, 16, 16, 3, 1, 13),        # 38 images in a window, nothing to copy
+    (300, 24, 16, 70, 7, 9),         # 20 images in a window, 8 channels copied
+    (1200, 64, 16, 5, 40, 13),       # images shorter than the kernel
+    (600, 48, 32, 20, 33, 3),        # four octets, odd width
+    (420, 64, 48, 9, 67, 11),        # six octets
+    (2, 40, 32, 300, 1001, 13),      # windows that begin in one row segment and end in the next; rows copied one by one
+    (1, 64, 16, 1213, 1030, 5),      # one image, a last window that is nearly empty
+    (1, 192, 48, 420, 1000, 7),      # chunks of 56 pixels
+]
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    import paper_2503_06671_b200 as p
+
+    p.lib()
+    return p
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: "x".join(map(str, s)))
+def test_stage_against_oracle(pkg, shape):
+    import torch
+
+    import oracle
+
+    B, C, C_a, H, W, K = shape
+    d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=sum(shape) + 1)
+    dk = np.random.default_rng(6).uniform(-0.5, 0.5, size=(B, C_a, 3, 3)).astype(np.float32)
+    x = util.to_device(d["x"], synth.BF16, synth.NHWC)
+    wl, _, _ = util.weights_to_device(d, synth.BF16)
+    n = x.numel()
+    buf = torch.full((n + 4096,), 7.0, dtype=x.dtype, device="cuda")
+    out = buf[2048:2048 + n].view(x.shape)
+    ws = pkg.new_workspace(B, C_a, H, W, K)
+    for _ in range(2):
+        pkg.esc_convattn_stencil(x, C_a, K, wl, torch.from_numpy(dk).cuda(), out, pkg.ESC_NHWC, ws)
+    torch.cuda.synchronize()
+    assert pkg.esc_convattn_device_status(ws) == 0
+    assert pkg.esc_convattn_last_path() == 4 and pkg.esc_convattn_last_tile_width() == 256
+    assert bool((buf[:2048] == 7.0).all()) and bool((buf[2048 + n:] == 7.0).all()), "write outside out"
+    ref, mag = oracle.stencil(d["x"], C_a, d["w_large"], dk, want_mag=True)
+    got = util.to_host_nchw(out, synth.NHWC)
+    util.check_attention(got[:, :C_a], ref[:, :C_a], mag, synth.BF16, f"{shape}", unit_variance=True)
+    assert np.array_equal(got[:, C_a:], ref[:, C_a:])
+
+
+def test_constant_of_the_backward_pass(pkg):
+    """grad_x is this kernel on grad_out with rotated kernels and a constant per (image, channel): 1,200 small images against the
+    same images in four calls, which take the kernel for smaller launches (each result one bf16 rounding: 2^-7 of its magnitude apart at most,
+    and fp32 sums in another order)."""
+    import torch
+
+    B, C, C_a, H, W, K = 1200, 32, 16, 9, 40, 13
+    d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=5, channel_means=True)
+    x = util.to_device(d["x"], synth.BF16, synth.NHWC)
+    wl, wd, bd = util.weights_to_device(d, synth.BF16)
+    go = torch.randn(x.shape, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda").to(x.dtype)
+
+    def run(x, go):
+        gx = torch.empty_like(x)
+        gl, gw, gb = (torch.zeros(t.shape, device="cuda") for t in (wl, wd, bd))
+        ws = pkg.new_backward_workspace(x.shape[0], C_a, H, W, K)
+        pkg.esc_convattn_backward(x, go, C_a, K, wl, wd, bd, gx, gl, gw, gb, pkg.ESC_NHWC, ws)
+        torch.cuda.synchronize()
+        assert pkg.esc_convattn_device_status(ws) == 0
+        return gx, pkg.esc_convattn_last_tile_width()
+
+    whole, width = run(x, go)
+    assert width == 256
+    for k in range(4):
+        part, width = run(x[k * 300:k * 300 + 300].contiguous(), go[k * 300:k * 300 + 300].contiguous())
+        assert width == 64
+        a, b = whole[k * 300:k * 300 + 300].float(), part.float()
+        assert torch.equal(a[..., C_a:], b[..., C_a:])
+        assert bool(((a - b).abs() <= 2.0 ** -7 * torch.maximum(a.abs(), b.abs()) + 1e-4).all())
+
+
+@pytest.mark.parametrize("K", [3, 9, 13])
+def test_reach_of_a_non_finite_input(pkg, K):
+    """Zero weights stand beside every tap, so accumulators outside the window become NaN; what is written does not."""
+    import torch
+
+    B, C, C_a, H, W = 1200, 24, 16, 16, 40
+    g = torch.Generator(device="cuda").manual_seed(K)
+
+    def rand(*shape):
+        t = torch.rand(shape, generator=g, device="cuda") + 0.25
+        return t * (torch.randint(0, 2, shape, generator=g, device="cuda") * 2 - 1)
+
+    x, w, dk = rand(B, H, W, C).bfloat16(), rand(C_a, K, K).bfloat16(), rand(B, C_a, 3, 3)
+    ws = pkg.new_workspace(B, C_a, H, W, K)
+
+    def run(x):
+        out = torch.full_like(x, 7.0)
+        pkg.esc_convattn_stencil(x, C_a, K, w, dk, out, pkg.ESC_NHWC, ws)
+        torch.cuda.synchronize()
+        assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_last_tile_width() == 256
+        return out
+
+    want, P = run(x), K // 2
+    for value, (b, c, y0, x0) in ((float("inf"), (B - 1, C_a - 1, 9, 20)), (float("nan"), (0, 1, 0, W - 1)), (float("-inf"), (7, 2, H - 1, 0))):
+        xi = x.clone()
+        xi[b, y0, x0, c] = value
+        got = run(xi)
+        reached = torch.zeros(got.shape, dtype=torch.bool, device="cuda")
+        reached[b, max(0, y0 - P):y0 + P + 1, max(0, x0 - P):x0 + P + 1, c] = True
+        assert bool((~torch.isfinite(got[reached])).all()), "an output does not see an input of its window"
+        # outputs evaluated directly beside it: fp32 sums in another order, then one bf16 rounding
+        a, b_ = got[~reached].float(), want[~reached].float()
+        assert bool(torch.isfinite(a).all()) and bool(((a - b_).abs() <= 2.0 ** -7 * torch.maximum(a.abs(), b_.abs()) + 1e-4).all())
