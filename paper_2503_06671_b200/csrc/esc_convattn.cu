@@ -405,11 +405,14 @@ struct TensorLk {
     int K;
 };
 // Whether the depth-wise stage goes to the tcgen05 kernel: bf16 NHWC without the point-wise mix, unless the caller pinned the FP32
-// kernel (by engine or by one of its tile widths), and more work than the one-launch form of the mma.sync kernel takes.  It takes
-// every odd K up to 13 as it is.
+// kernel (by engine or by one of its tile widths), at least two groups of channels, and more work than the one-launch form of the
+// mma.sync kernel takes.  (Forward, mma.sync / tcgen05, us: 1920x1080, 32 of 64 channels 324 / 269, with K = 9 327 / 273; 1280x720 163 / 125;
+// 900x500, 48 of 192 channels 215 / 141; 64 images of 160x64, 32 of 64 channels 132 / 103.  With one group, 16 of 64 channels, 1920x1080 217 / 280:
+// the copies beside it slow it down there, without identity channels it is 147 / 112.)  It takes every odd K up to 13 as it is.
 bool dw_umma_follows(const Problem& p) {
-    return !p.dense && !p.w_point && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
-           esc::tma::dwu::applies(p.C, p.Ca, p.K, p.dtype, p.layout) &&
+    return !p.dense && !p.w_point && p.Ca >= 2 * esc::tma::CG && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
+           esc::tma::dwu::applies(p.C, p.Ca, p.K, p.dtype, p.layout) && (long long)p.B * p.H * p.W <= 0x7fffffffLL &&
+           (long long)p.B * (p.W + esc::tma::dwu::GAPX) <= 0x3fffffffLL &&
            esc::tma::toep::units_of<esc::tma::toep::Shape64x16>(p.B, p.Ca, p.H, p.W) > (long long)esc::tma::toep::kMaxFusedUnits * sms_or_nominal();
 }
 TensorLk tensor_lk(const Problem& p, const void* x, const void* out, const void* w_large, void* pad, cudaStream_t st) {

@@ -561,7 +561,9 @@ inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int 
         // the pixels of all images as one axis
         const long long px = (long long)B * H * W;
         if (px > 0x7fffffffLL) return kNotApplicable;
-        p.copy_cc = cc; p.copy_pw = kCopySlotBytes / (cc * 2) < 256 ? kCopySlotBytes / (cc * 2) : 256;
+        p.copy_cc = cc;
+        p.copy_pw = WPX;                                     // a power of two: whole chunks to a window row
+        while (cc * 2 * p.copy_pw > kCopySlotBytes) p.copy_pw >>= 1;
         p.copy_chunks = (int)((px + p.copy_pw - 1) / p.copy_pw);
         p.copy_rows = W >= WPX;
         EncodeTiledFn fn = encode_fn();

@@ -1,4 +1,4 @@
-"""The tcgen05 depth-wise kernel (bf16 NHWC, more work than the one-launch form takes) against the oracle: windows that hold many small
+"""The tcgen05 depth-wise kernel (bf16 NHWC, two or more groups of 16 channels, more work than the one-launch form takes) against the oracle: windows that hold many small
 images, image rows of one to a few hundred pixels, row segments, channel groups, every kernel size's ends, the copied channels, the
 constant per (image, channel) of the backward pass, and the reach of a non-finite input."""
 import numpy as np
@@ -11,14 +11,14 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [
     # B, C, C_a, H, W, K: more than 1,184 tiles of 64x16 x 16 channels
-    (1300, 16, 16, 3, 1, 13),        # 38 images in a window, nothing to copy
-    (300, 24, 16, 70, 7, 9),         # 20 images in a window, 8 channels copied
-    (1200, 64, 16, 5, 40, 13),       # images shorter than the kernel
+    (700, 32, 32, 3, 1, 13),         # 38 images in a window, nothing to copy
+    (150, 40, 32, 70, 7, 9),         # 20 images in a window, 8 channels copied
+    (600, 64, 32, 5, 40, 13),        # images shorter than the kernel
     (600, 48, 32, 20, 33, 3),        # four octets, odd width
     (420, 64, 48, 9, 67, 11),        # six octets
     (2, 40, 32, 300, 1001, 13),      # windows that begin in one row segment and end in the next; rows copied one by one
-    (1, 64, 16, 1213, 1030, 5),      # one image, a last window that is nearly empty
-    (1, 192, 48, 420, 1000, 7),      # chunks of 56 pixels
+    (1, 64, 32, 1213, 1030, 5),      # one image, a last window that is nearly empty
+    (1, 192, 48, 420, 1000, 7),      # chunks of 32 pixels
 ]
 
 
@@ -67,7 +67,7 @@ def test_constant_of_the_backward_pass(pkg):
     and fp32 sums in another order)."""
     import torch
 
-    B, C, C_a, H, W, K = 1200, 32, 16, 9, 40, 13
+    B, C, C_a, H, W, K = 1200, 48, 32, 9, 40, 13
     d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=5, channel_means=True)
     x = util.to_device(d["x"], synth.BF16, synth.NHWC)
     wl, wd, bd = util.weights_to_device(d, synth.BF16)
@@ -97,7 +97,7 @@ def test_reach_of_a_non_finite_input(pkg, K):
     """Zero weights stand beside every tap, so accumulators outside the window become NaN; what is written does not."""
     import torch
 
-    B, C, C_a, H, W = 1200, 24, 16, 16, 40
+    B, C, C_a, H, W = 700, 40, 32, 16, 40
     g = torch.Generator(device="cuda").manual_seed(K)
 
     def rand(*shape):
