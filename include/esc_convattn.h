@@ -380,8 +380,8 @@ int esc_conv_fuse_backward(const void* cat, const void* grad_out, int B, int C, 
 
 /*
  * Self-test of the error path that every device-side wait of this library shares: launches one thread that waits, with
- * the kernels' own bounded wait, on a barrier that nothing signals.  The wait gives up after its poll limit (about one
- * second), records ESC_DEV_TIMEOUT in the status word of `workspace` (any initialised forward or backward workspace, device)
+ * the kernels' own bounded waits, for a count that nothing raises and then on a barrier that nothing signals.  Each wait gives up
+ * after its poll limit (about one second); the second, if the first one's record was right, records ESC_DEV_TIMEOUT in the status word of `workspace` (any initialised forward or backward workspace, device)
  * and the kernel returns normally: no trap, no fault, the context stays usable.  esc_convattn_device_status() then returns
  * ESC_DEV_TIMEOUT once and clears the word.  Asynchronous on `stream`.
  */

@@ -1084,12 +1084,20 @@ int fuse_backward_mma_t(int C, const void* cat, const void* go, const void* w_fu
     return ESC_ERR_UNSUPPORTED;
 }
 
-// ---- the bounded wait, run on purpose -----------------------------------------------------------------------
-// One thread waits, with the kernels' own bounded wait, on a barrier that nothing signals: the wait gives up after its
-// poll limit (about a second), records the status and the kernel returns normally.
+// ---- the bounded waits, run on purpose ----------------------------------------------------------------------
+// One thread waits, with the kernels' own bounded waits, for a count that nothing raises and then on a barrier that nothing
+// signals: each gives up after its poll limit (about a second) and records the status, and the kernel returns normally.  The first
+// one's record is checked here: without it the second wait, whose record the host reads, is left out.
 __global__ void bounded_wait_probe(unsigned* ctrl) {
     __shared__ __align__(8) unsigned long long bar;
+    __shared__ int count;
+    __shared__ unsigned status[2];
     if (threadIdx.x == 0) {
+        count = 2;
+        status[0] = status[1] = 0;
+        const bool enough = esc::tma::umma::wait_count(&count, 2, status, 0u) && status[0] == 0;
+        const bool gave_up = !esc::tma::umma::wait_count(&count, 3, status, 0x5E1F0001u) && status[0] == esc::kDevTimeout && status[1] == 0x5E1F0001u;
+        if (!enough || !gave_up) return;
         const uint32_t b = esc::tma::smem_u32(&bar);
         esc::tma::mbar_init(b, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

@@ -146,6 +146,15 @@ __device__ __forceinline__ int ld_acquire_cta(const int* p) {
 __device__ __forceinline__ void st_release_cta(int* p, int v) {
     asm volatile("st.release.cta.shared.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
 }
+// One lane's bounded wait for a count that another warp of the CTA publishes; records where it gave up, as mbar_wait does.
+__device__ __forceinline__ bool wait_count(const int* count, int need, unsigned* ctrl, unsigned where) {
+    for (unsigned polls = 0; polls < kPollLimit; ++polls) {
+        if (ld_acquire_cta(count) >= need) return true;
+        __nanosleep(200);
+    }
+    if (ctrl) { atomicExch(ctrl, kDevTimeout); atomicExch(ctrl + 1, where); }
+    return false;
+}
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, unsigned bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");

@@ -312,16 +312,21 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
             const unsigned bytes = (unsigned)(p.copy_cc * p.copy_pw * 2);
             bool alive = true;
             int loads = 0, stores = 0, pend0 = 0, pend1 = 0;
+            // A wait that gave up ends the copying: what was asked for is waited for, but not stored, and nothing more is asked for.
             auto store = [&]() {                             // the oldest load
                 const int s = stores % kCopySlots;
-                if (alive) alive = mbar_wait(cfull0 + 8 * s, (unsigned)((stores / kCopySlots) & 1), p.ctrl, 0xE5000000u);
-                tma_store_2d(&map_cout, smem_u32(cring + s * kCopySlotBytes), p.Ca, pend0);
-                bulk_commit();
+                const bool landed = mbar_wait(cfull0 + 8 * s, (unsigned)((stores / kCopySlots) & 1), p.ctrl, 0xE5000000u);
+                alive = alive && landed;
+                if (alive) {
+                    tma_store_2d(&map_cout, smem_u32(cring + s * kCopySlotBytes), p.Ca, pend0);
+                    bulk_commit();
+                }
                 pend0 = pend1;
                 ++stores;
             };
             auto copy = [&](int px) {
-                if (loads - stores == 2) { store(); bulk_wait_read<1>(); }   // the store before that one has read its slot
+                if (!alive) return;
+                if (loads - stores == 2) { store(); bulk_wait_read<1>(); if (!alive) return; }   // the store before that one has read its slot
                 const int s = loads % kCopySlots;
                 mbar_expect_tx(cfull0 + 8 * s, bytes);
                 tma_load_2d(smem_u32(cring + s * kCopySlotBytes), &map_cin, cfull0 + 8 * s, p.Ca, px);
@@ -330,15 +335,11 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
             };
             if (p.copy_rows) {
                 int o = 0;
-                for (int r = r_begin; r < r_end;) {
+                for (int r = r_begin; r < r_end && alive;) {
                     const int t = r / p.R, row0 = r - t * p.R, L = min(p.R - row0, r_end - r);
-                    for (int yr = 0; yr < L; ++yr) {
+                    for (int yr = 0; yr < L && alive; ++yr) {
                         if ((row0 + yr) % p.octets != oct) continue;
-                        unsigned polls = 0;
-                        while (alive && umma::ld_acquire_cta(progress) + 8 < o + yr) {
-                            __nanosleep(200);
-                            if (++polls > umma::kPollLimit) alive = false;
-                        }
+                        alive = umma::wait_count(progress, o + yr - 8, p.ctrl, 0xE8000000u | (unsigned)(yr & 0xffff));
                         for (int f = t * WPX; f < t * WPX + WPX;) {
                             const int piece = f / p.pitch, x = f - piece * p.pitch, end = min(t * WPX + WPX, (piece + 1) * p.pitch);
                             const int b = piece / p.S, y = (piece - b * p.S) * p.R + row0 + yr, n = min(p.W - x, end - f);
@@ -351,7 +352,7 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
                     r += L;
                 }
             } else {
-                for (int k = blockIdx.x; k < p.copy_chunks; k += gridDim.x) copy(k * p.copy_pw);
+                for (int k = blockIdx.x; k < p.copy_chunks && alive; k += gridDim.x) copy(k * p.copy_pw);
             }
             while (stores < loads) store();
             bulk_wait_all<0>();
