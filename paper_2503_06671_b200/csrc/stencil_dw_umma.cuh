@@ -21,7 +21,11 @@
 // The rows of all windows are dealt evenly to the CTAs (a CTA may end one window and begin another).
 //
 // A non-finite input makes NaN of accumulators outside its window too (zero times infinity).  The epilogue sees that -- the sum of a
-// pixel's accumulators is not finite -- and evaluates those outputs directly, so what leaves the kernel has the window of the definition.
+// pixel's accumulators is not finite -- and notes the row, unless the 3x3 part is NaN as well; behind its last row it evaluates what
+// is not finite in those rows directly, so what leaves the kernel has the window of the definition.  1920x1080, 32 of 64 channels,
+// stage alone: finite 182 us, one bad pixel 458, a map of NaN 178; a bad pixel in every 16 x 16 13.9 ms, one channel of NaN beside
+// finite ones 20 ms, 4 ms where all is infinite.  (A forward whose attention channels hold NaN or infinity has NaN in dk, hence in
+// every output of that image: 239 - 259 us.)
 //
 // Roles (512 threads, one CTA per SM):
 //   warps 0-7    epilogue: one pixel x eight channels per thread and row: tcgen05.ld, the dynamic 3x3 kernel in fp32 on the CUDA cores, one
@@ -63,10 +67,10 @@ constexpr int kLaunchRegs = 128, kEpiRegs = 200, kRestRegs = 56;   // 256 * 200 
 constexpr int kMaxImages = 40;                      // images a window can touch: 256 / 7 + 2
 constexpr int kCopySlotBytes = 16384, kCopySlots = 3;
 constexpr int kOffB = NRING * ROW_BYTES, kOffCopy = kOffB + B_BYTES, kOffDk = kOffCopy + kCopySlots * kCopySlotBytes,
-              kOffBars = kOffDk + kMaxImages * 9 * OCT * 4, kSmemBytes = kOffBars + 1024;
+              kOffTaps = kOffDk + kMaxImages * 9 * OCT * 4, kOffBars = kOffTaps + K13 * K13 * OCT * 2, kSmemBytes = kOffBars + 1024;
 constexpr int kBars = 2 * NRING + 2 * SLOTS + kCopySlots + 2;
 static_assert(SPX / 2 * 16 <= PAR_BYTES && PAR_BYTES % 128 == 64, "parity plane");
-static_assert(kOffB % 128 == 0 && kOffCopy % 128 == 0 && kOffBars % 16 == 0, "alignment");
+static_assert(kOffB % 128 == 0 && kOffCopy % 128 == 0 && kOffTaps % 16 == 0 && kOffBars % 16 == 0, "alignment");
 static_assert(kBars * 8 + 16 <= 1024 && kSmemBytes <= 227 * 1024, "shared memory");
 static_assert(DEPTH + 5 <= NRING && DEPTH == 2 * kProdWarps, "rows the epilogue needs are signalled before a slot is waited for");
 
@@ -114,20 +118,99 @@ __device__ __forceinline__ void mma_row(uint32_t d, unsigned long long da, unsig
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}"
         ::"r"(d), "l"(da), "l"(db), "r"(idesc), "n"(BQ_BYTES >> 4) : "memory");
 }
+__device__ __forceinline__ void unpack8(const uint4& v, float (&f)[OCT]) {
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { f[2 * q] = __uint_as_float(w[q] << 16); f[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u); }
+}
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 2, %0;" ::"n"(kEpiThreads) : "memory"); }
 
-// The large kernel's sum for one output, straight from the definition (only where an accumulator is not finite).
-__device__ __noinline__ float direct(const Params& p, int b, int c, int y, int x) {
-    const int P = p.K / 2;
-    float s = 0.f;
-    for (int i = 0; i < p.K; ++i)
-        for (int j = 0; j < p.K; ++j) {
-            const int yy = y + i - P, xx = x + j - P;
-            if (yy >= 0 && yy < p.H && xx >= 0 && xx < p.W)
-                s = fmaf(__bfloat162float(p.w_large[((size_t)c * p.K + i) * p.K + j]),
-                         __bfloat162float(p.x[(((size_t)b * p.H + yy) * p.W + xx) * p.C + c]), s);
+// Outputs that are not finite, straight from the definition: a warp looks at its pixels again in the rows [first, last) of the CTA's
+// windows (taps: [K * K][8] weights).  Eight lanes take a pixel: a lane sums kernel rows k and k + 8 of all channels, of which the
+// sums over the lanes leave it one, to which it adds the 3x3 part.  Of its own and behind the main loop, so that the registers it
+// takes are not missing there (called from the loop, 180 -> 245 us) and no wait of another warp runs out meanwhile.
+__device__ __noinline__ void direct(const Params& p, const uint4* taps, int oct, int r_begin, int r_end, int m2, int first, int last) {
+    const int lane = threadIdx.x & 31, k = lane & 7, P = p.K / 2;
+    first = __reduce_min_sync(0xffffffffu, first);
+    last = __reduce_max_sync(0xffffffffu, last);
+    int o = 0;
+    for (int r = r_begin; r < r_end;) {
+        const int t = r / p.R, row0 = r - t * p.R, L = min(p.R - row0, r_end - r);
+        const int f = t * WPX + m2, piece = f / p.pitch, x = f - piece * p.pitch, b = piece / p.S, y0 = (piece - b * p.S) * p.R + row0;
+        const bool valid = piece < p.pieces && x < p.W;
+        for (int yr = max(0, first - o); yr < min(L, last - o); ++yr) {
+            unsigned bad = 0;                                // channels of this lane's pixel
+            if (valid && y0 + yr < p.H) {
+                float v[OCT];
+                unpack8(*reinterpret_cast<const uint4*>(p.out + (((size_t)b * p.H + y0 + yr) * p.W + x) * p.C + oct * OCT), v);
+#pragma unroll
+                for (int n = 0; n < OCT; ++n) bad |= (fabsf(v[n]) < INFINITY ? 0u : 1u) << n;
+            }
+            for (unsigned todo = __ballot_sync(0xffffffffu, bad != 0); todo != 0;) {
+                // the next four pixels, one per group of eight lanes
+                int src = -1;
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    if (g == lane >> 3 && todo != 0) src = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                }
+                const int from = max(src, 0), py = __shfl_sync(0xffffffffu, y0, from) + yr, pxx = __shfl_sync(0xffffffffu, x, from),
+                          pb = __shfl_sync(0xffffffffu, b, from);
+                const unsigned from_bad = __shfl_sync(0xffffffffu, bad, from), pbad = src < 0 ? 0u : from_bad;
+                const __nv_bfloat16* img = p.x + (size_t)(pbad ? pb : 0) * p.H * p.W * p.C + oct * OCT;
+                float s3 = 0.f;                              // the 3x3 part of channel k, as the main loop has it
+                if (pbad >> k & 1) {
+                    const size_t bc = (size_t)pb * p.Ca + oct * OCT + k;
+                    if (p.bias) s3 = __ldcg(p.bias + bc);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        const int yy = py + i / 3 - 1, xx = pxx + i % 3 - 1;
+                        const bool in = yy >= 0 && yy < p.H && xx >= 0 && xx < p.W;
+                        s3 = fmaf(__ldcg(p.dk + bc * 9 + i), in ? __bfloat162float(img[((size_t)yy * p.W + xx) * p.C + k]) : 0.f, s3);
+                    }
+                }
+                const bool open = (pbad >> k & 1) && s3 == s3;                   // else NaN whatever the large kernel's sum
+                const bool group = (__ballot_sync(0xffffffffu, open) >> (lane & 24) & 0xffu) != 0;
+                float s[OCT] = {};
+                if (group)
+                    for (int i = k; i < p.K; i += 8) {
+                        const int yy = py + i - P;
+                        if (yy < 0 || yy >= p.H) continue;
+                        const __nv_bfloat16* row = img + (size_t)yy * p.W * p.C;
+                        uint4 v[K13];
+#pragma unroll
+                        for (int j = 0; j < K13; ++j) {
+                            const int xx = pxx + j - P;
+                            v[j] = make_uint4(0u, 0u, 0u, 0u);
+                            if (j < p.K && xx >= 0 && xx < p.W) v[j] = __ldg(reinterpret_cast<const uint4*>(row + (size_t)xx * p.C));
+                        }
+#pragma unroll
+                        for (int j = 0; j < K13; ++j) {
+                            const int xx = pxx + j - P;
+                            if (j < p.K && xx >= 0 && xx < p.W) {
+                                float fv[OCT], w[OCT];
+                                unpack8(v[j], fv);
+                                unpack8(taps[i * p.K + j], w);
+#pragma unroll
+                                for (int n = 0; n < OCT; ++n) s[n] = fmaf(w[n], fv[n], s[n]);
+                            }
+                        }
+                    }
+                // sums over the eight lanes; lane k keeps channel k
+#pragma unroll
+                for (int h = 4; h > 0; h >>= 1)
+#pragma unroll
+                    for (int n = 0; n < h; ++n) {
+                        const bool up = (lane & h) != 0;
+                        const float keep = up ? s[n + h] : s[n];
+                        s[n] = keep + __shfl_xor_sync(0xffffffffu, up ? s[n] : s[n + h], h);
+                    }
+                if (open) p.out[(((size_t)pb * p.H + py) * p.W + pxx) * p.C + oct * OCT + k] = __float2bfloat16_rn(s[0] + s3);
+            }
         }
-    return s;
+        o += L;
+        r += L;
+    }
 }
 
 __global__ void __maxnreg__(kLaunchRegs)
@@ -241,6 +324,7 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
                 const int it = bt + u * kT;
                 if (it < items) {
                     const int n = it / taps, rem = it - n * taps, i = rem / p.K + off, j = rem % p.K + off;
+                    *reinterpret_cast<unsigned short*>(smem + kOffTaps + (rem * OCT + n) * 2) = v[u];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const int tt = j + e;
@@ -251,6 +335,7 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
             }
             fence_async_smem();
             asm volatile("bar.sync 3, %0;" ::"n"(kT) : "memory");
+            asm volatile("bar.arrive 4, %0;" ::"n"(kT + kEpiThreads) : "memory");   // the epilogue may read the taps
         }
         if (warp == 12) {
             // ======================= tensor-core instructions =========================================
@@ -375,7 +460,7 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
 
         if (!p.wait_first) pdl_wait_primary();                   // dk comes from the kernel before this one
 
-        int g0 = 0, o = 0;
+        int g0 = 0, o = 0, first_bad = 0x7fffffff, last_bad = 0;                // rows with sums that are not finite
         bool alive = true;
         for (int r = r_begin; r < r_end;) {
             const int t = r / p.R, row0 = r - t * p.R, L = min(p.R - row0, r_end - r);
@@ -470,14 +555,17 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
 #pragma unroll
                     for (int q = 0; q < 8; ++q) check += __uint_as_float(a[i][q]);
                 if (!(fabsf(check) < INFINITY) && valid) {
-#pragma unroll 1
-                    for (int e = 0; e < N * 8; ++e) {
-                        if (y0 + yr + e / 8 >= p.H) break;
-                        const float v = direct(p, b, oct * OCT + e % 8, y0 + yr + e / 8, x);
+                    bool open = false;                       // not finite, and the 3x3 part does not make the result NaN anyway
 #pragma unroll
-                        for (int u = 0; u < N * 8; ++u)
-                            if (u == e) a[u / 8][u % 8] = __float_as_uint(v);
-                    }
+                    for (int i = 0; i < N; ++i)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            float lo, hi;
+                            unpack2(d0[i][q], lo, hi);
+                            open |= !(fabsf(__uint_as_float(a[i][2 * q])) < INFINITY) && lo == lo;
+                            open |= !(fabsf(__uint_as_float(a[i][2 * q + 1])) < INFINITY) && hi == hi;
+                        }
+                    if (open) { first_bad = min(first_bad, o + yr); last_bad = o + yr + N; }
                 }
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
@@ -505,6 +593,10 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
             o += L;
             r += L;
         }
+        asm volatile("bar.sync 4, %0;" ::"n"(128 + kEpiThreads) : "memory");    // the taps are in place
+        __syncwarp();
+        if (__any_sync(0xffffffffu, last_bad > 0))
+            direct(p, reinterpret_cast<const uint4*>(smem + kOffTaps), oct, r_begin, r_end, 2 * m + e, first_bad, last_bad);
     }
     umma::tc_fence_before();
     __syncthreads();
