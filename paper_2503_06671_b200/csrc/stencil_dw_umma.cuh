@@ -65,13 +65,14 @@ constexpr int SLOTS = 512 / NBC;
 constexpr int kEpiWarps = 8, kEpiThreads = kEpiWarps * 32, kProdWarps = 4, kThreads = 512;
 constexpr int kLaunchRegs = 128, kEpiRegs = 200, kRestRegs = 56;   // 256 * 200 + 256 * 56 = 512 * 128
 constexpr int kMaxImages = 40;                      // images a window can touch: 256 / 7 + 2
-constexpr int kCopySlotBytes = 16384, kCopySlots = 3;
-constexpr int kOffB = NRING * ROW_BYTES, kOffCopy = kOffB + B_BYTES, kOffDk = kOffCopy + kCopySlots * kCopySlotBytes,
-              kOffTaps = kOffDk + kMaxImages * 9 * OCT * 4, kOffBars = kOffTaps + K13 * K13 * OCT * 2, kSmemBytes = kOffBars + 1024;
+constexpr int kCopyBytes = 49152, kCopyChunkBytes = 16384, kCopySlots = 12;   // identity channels: the ring, a chunk, and chunks in the ring at most
+constexpr int kCopyLead = 24;                       // rows the copies may be ahead of the epilogue
+constexpr int kOffB = NRING * ROW_BYTES, kOffCopy = kOffB + B_BYTES, kOffDk = kOffCopy + kCopyBytes,
+              kOffTaps = kOffDk + kMaxImages * 9 * OCT * 4, kOffBars = kOffTaps + K13 * K13 * OCT * 2, kSmemBytes = kOffBars + 1152;
 constexpr int kBars = 2 * NRING + 2 * SLOTS + kCopySlots + 2;
 static_assert(SPX / 2 * 16 <= PAR_BYTES && PAR_BYTES % 128 == 64, "parity plane");
 static_assert(kOffB % 128 == 0 && kOffCopy % 128 == 0 && kOffTaps % 16 == 0 && kOffBars % 16 == 0, "alignment");
-static_assert(kBars * 8 + 16 <= 1024 && kSmemBytes <= 227 * 1024, "shared memory");
+static_assert(kBars * 8 + 8 + 4 * kCopySlots <= 1152 && kSmemBytes <= 227 * 1024, "shared memory");
 static_assert(DEPTH + 5 <= NRING && DEPTH == 2 * kProdWarps, "rows the epilogue needs are signalled before a slot is waited for");
 
 struct Params {
@@ -84,7 +85,7 @@ struct Params {
     __nv_bfloat16* out;
     unsigned* ctrl;
     int wait_first;
-    int copy_cc, copy_pw, copy_chunks, copy_rows;   // identity channels, pixels a chunk, chunks in all; copied row by row
+    int copy_cc, copy_shift, copy_slots, copy_chunks, copy_rows;   // identity channels, log2 of a chunk's pixels, chunks in the ring and in all; copied row by row
 };
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
@@ -390,33 +391,38 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
             umma::mbar_wait_warp(drained, 0, p.ctrl, 0xE4000000u);
         } else if (warp == 13 && lane == 0 && p.copy_cc != 0) {
             // ======================= copy-through of the identity channels ==============================
-            // Three slots, two loads ahead of the store.  Wide maps: the rows of the CTA's own windows, dealt among the CTAs of the
-            // same rows and other channels, not far ahead of the epilogue, so that the parts of a line reach L2 together.  A chunk
-            // that would end beyond the window's part of the row copies pixels that are copied elsewhere too.  Narrow maps: all
-            // pixels in chunks dealt in turn to the CTAs.
-            const unsigned bytes = (unsigned)(p.copy_cc * p.copy_pw * 2);
+            // Chunks of a power of two of pixels, the pixels of all images counted through, in a ring that is loaded up to one slot
+            // ahead of the store.  Wide maps: a chunk goes with the row of a window that its first pixel lies in, dealt among the CTAs
+            // of the same rows and other channels, not far ahead of the epilogue, so that the parts of a line reach L2
+            // together.  Narrow maps: the chunks dealt in turn to the CTAs.  Each chunk is copied once: with chunks cut at the ends of
+            // a window's part of a row, and whole ones copied for every part, 16 x (320x320) copied 1.75 times as much as there is
+            // (stage 191 -> 150 us, 480x500 with 64 of 96 channels 133 -> 115, 900x500 with 144 of 192 109 -> 92).  Up to 8 rows
+            // ahead 1920x1080 takes 183 us, 16 180, 24 or 32 178; chunks of 8 KB 186, of 4 KB 212.
+            const unsigned bytes = (unsigned)(p.copy_cc * 2) << p.copy_shift, slot_bytes = (bytes + 127) & ~127u;
+            int* pend = progress + 1;                        // first pixel of each slot's chunk
             bool alive = true;
-            int loads = 0, stores = 0, pend0 = 0, pend1 = 0;
+            int load_slot = 0, store_slot = 0, lag = 0;      // lag: loads that are not stored yet
+            unsigned parity = 0;
             // A wait that gave up ends the copying: what was asked for is waited for, but not stored, and nothing more is asked for.
             auto store = [&]() {                             // the oldest load
-                const int s = stores % kCopySlots;
-                const bool landed = mbar_wait(cfull0 + 8 * s, (unsigned)((stores / kCopySlots) & 1), p.ctrl, 0xE5000000u);
+                const bool landed = mbar_wait(cfull0 + 8 * store_slot, parity, p.ctrl, 0xE5000000u);
                 alive = alive && landed;
                 if (alive) {
-                    tma_store_2d(&map_cout, smem_u32(cring + s * kCopySlotBytes), p.Ca, pend0);
+                    tma_store_2d(&map_cout, smem_u32(cring) + store_slot * slot_bytes, p.Ca, pend[store_slot]);
                     bulk_commit();
                 }
-                pend0 = pend1;
-                ++stores;
+                if (++store_slot == p.copy_slots) { store_slot = 0; parity ^= 1; }
+                --lag;
             };
-            auto copy = [&](int px) {
+            auto copy = [&](unsigned chunk) {
                 if (!alive) return;
-                if (loads - stores == 2) { store(); bulk_wait_read<1>(); if (!alive) return; }   // the store before that one has read its slot
-                const int s = loads % kCopySlots;
-                mbar_expect_tx(cfull0 + 8 * s, bytes);
-                tma_load_2d(smem_u32(cring + s * kCopySlotBytes), &map_cin, cfull0 + 8 * s, p.Ca, px);
-                if (loads == stores) pend0 = px; else pend1 = px;
-                ++loads;
+                if (lag == p.copy_slots - 1) { store(); bulk_wait_read<1>(); if (!alive) return; }   // the store before that one has read its slot
+                const int px = (int)(chunk << p.copy_shift);
+                mbar_expect_tx(cfull0 + 8 * load_slot, bytes);
+                tma_load_2d(smem_u32(cring) + load_slot * slot_bytes, &map_cin, cfull0 + 8 * load_slot, p.Ca, px);
+                pend[load_slot] = px;
+                if (++load_slot == p.copy_slots) load_slot = 0;
+                ++lag;
             };
             if (p.copy_rows) {
                 int o = 0;
@@ -424,12 +430,14 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
                     const int t = r / p.R, row0 = r - t * p.R, L = min(p.R - row0, r_end - r);
                     for (int yr = 0; yr < L && alive; ++yr) {
                         if ((row0 + yr) % p.octets != oct) continue;
-                        alive = umma::wait_count(progress, o + yr - 8, p.ctrl, 0xE8000000u | (unsigned)(yr & 0xffff));
+                        alive = umma::wait_count(progress, o + yr - kCopyLead, p.ctrl, 0xE8000000u | (unsigned)(yr & 0xffff));
                         for (int f = t * WPX; f < t * WPX + WPX;) {
                             const int piece = f / p.pitch, x = f - piece * p.pitch, end = min(t * WPX + WPX, (piece + 1) * p.pitch);
                             const int b = piece / p.S, y = (piece - b * p.S) * p.R + row0 + yr, n = min(p.W - x, end - f);
-                            if (piece < p.pieces && y < p.H)
-                                for (int i = 0; i < n; i += p.copy_pw) copy((b * p.H + y) * p.W + x + max(0, min(i, n - p.copy_pw)));
+                            if (piece < p.pieces && y < p.H && n > 0) {
+                                const unsigned px = (unsigned)((b * p.H + y) * p.W + x), up = (1u << p.copy_shift) - 1;
+                                for (unsigned k = (px + up) >> p.copy_shift; k < (px + (unsigned)n + up) >> p.copy_shift; ++k) copy(k);
+                            }
                             f = end;
                         }
                     }
@@ -437,9 +445,9 @@ stencil_dw_umma_nhwc_bf16(const __grid_constant__ CUtensorMap map_cin, const __g
                     r += L;
                 }
             } else {
-                for (int k = blockIdx.x; k < p.copy_chunks && alive; k += gridDim.x) copy(k * p.copy_pw);
+                for (unsigned k = blockIdx.x; k < (unsigned)p.copy_chunks && alive; k += gridDim.x) copy(k);
             }
-            while (stores < loads) store();
+            while (lag > 0) store();
             bulk_wait_all<0>();
         }
         __syncwarp();
@@ -656,14 +664,16 @@ inline int try_launch(int B, int C, int Ca, int H, int W, int K, int dtype, int 
         const long long px = (long long)B * H * W;
         if (px > 0x7fffffffLL) return kNotApplicable;
         p.copy_cc = cc;
-        p.copy_pw = WPX;                                     // a power of two: whole chunks to a window row
-        while (cc * 2 * p.copy_pw > kCopySlotBytes) p.copy_pw >>= 1;
-        p.copy_chunks = (int)((px + p.copy_pw - 1) / p.copy_pw);
+        p.copy_shift = 8;
+        while (p.copy_shift > 0 && cc * 2 << p.copy_shift > kCopyChunkBytes) --p.copy_shift;
+        const int slot_bytes = ((cc * 2 << p.copy_shift) + 127) & ~127;
+        p.copy_slots = std::min(kCopySlots, kCopyBytes / slot_bytes);
+        p.copy_chunks = (int)((px + (1 << p.copy_shift) - 1) >> p.copy_shift);
         p.copy_rows = W >= WPX;
         EncodeTiledFn fn = encode_fn();
         if (!fn) return kNotApplicable;
         const cuuint64_t dims[2] = {(cuuint64_t)C, (cuuint64_t)px}, strides[1] = {(cuuint64_t)C * 2};
-        const cuuint32_t box[2] = {(cuuint32_t)cc, (cuuint32_t)p.copy_pw}, estr[2] = {1, 1};
+        const cuuint32_t box[2] = {(cuuint32_t)cc, 1u << p.copy_shift}, estr[2] = {1, 1};
         const void* base[2] = {x, out};
         for (int i = 0; i < 2; ++i)
             if (fn(i ? &m_cout : &m_cin, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base[i]), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,

@@ -219,3 +219,30 @@ def test_time_does_not_hang_on_the_data(pkg):
     x[..., :C_a] = float("nan")
     everywhere = time()
     assert one < 4 * finite and everywhere < 2 * finite, (finite, one, everywhere)
+
+
+def test_time_does_not_hang_on_the_width(pkg):
+    """The identity channels are copied once whatever part of an image row a window takes: a pixel of 320-pixel rows costs about what
+    one of 1,920-pixel rows does (1.06 times; 1.35 times when every part of a row was copied in whole chunks)."""
+    import torch
+
+    C, C_a, K = 64, 32, 13
+    g = torch.Generator(device="cuda").manual_seed(2)
+    w = torch.randn((C_a, K, K), generator=g, device="cuda").bfloat16()
+    sides = []
+    for B, H, W in ((16, 320, 320), (1, 1080, 1920)):
+        x = torch.randn((B, H, W, C), generator=g, device="cuda").bfloat16()
+        sides.append((x, torch.randn((B, C_a, 3, 3), generator=g, device="cuda"), torch.empty_like(x), pkg.new_workspace(B, C_a, H, W, K), B * H * W))
+    best = [float("inf")] * 2
+    for _ in range(8):
+        for s, (x, dk, out, ws, pixels) in enumerate(sides):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            pkg.esc_convattn_stencil(x, C_a, K, w, dk, out, pkg.ESC_NHWC, ws)
+            a.record()
+            for _ in range(4):
+                pkg.esc_convattn_stencil(x, C_a, K, w, dk, out, pkg.ESC_NHWC, ws)
+            b.record()
+            torch.cuda.synchronize()
+            assert pkg.esc_convattn_last_tile_width() == 256
+            best[s] = min(best[s], a.elapsed_time(b) / pixels)
+    assert best[0] < 1.2 * best[1], best
