@@ -120,14 +120,21 @@ int sms_or_nominal() {
     return v > 0 ? v : 148;
 }
 
-// Grid policy of the GAP kernel.  Narrow: at most one block per SM, which is what fits beside a CTA of the
-// FP32 stencil kernel (58 k registers).  Wide: three blocks per SM (two larger ones in launch_gap_t) -- for maps
-// so large that the stencil kernel takes many waves and the GAP kernel runs ahead of it rather than beside it, and for
-// batches in front of the tensor-core stencil kernel, whose CTAs need every image's dk early (measured on 64 patches
+// Grid of the GAP kernel.  Narrow: at most one block per SM, which is what fits beside a CTA of the
+// FP32 stencil kernel (58 k registers).  Wide: three blocks per SM, for batches in front of the Toeplitz stencil kernels, whose
+// CTAs need every image's dk early (measured on 64 patches
 // of 64x64: 35.5 us per forward against 37.8; a single 640x360 map: 37.4 against 36.2, so single images
-// keep the narrow grid).
-bool wide_gap(int B, long long HW, bool tensor_stencil) {
-    return (tensor_stencil && B > 1) || is_large_map(B, HW);
+// keep the narrow grid).  Large: two blocks of 512 threads per SM, for maps so large that the stencil kernel takes many waves and
+// the GAP kernel runs ahead of it rather than beside it.
+// In front of the tcgen05 depth-wise kernel nothing runs beside it either (that kernel's CTA takes all registers of an SM): large,
+// whatever K and B are, up to 64 attention channels.  Forward, us, narrow / wide / large: 1280x720, 32 of 64 channels 131 / 130 / 124; 900x500,
+// 48 of 192 119 / 121 / 115; 64 x (96x96), 32 of 64, K = 9 109 / 105 / 103; 300 x (40x40) 108 / 90 / 91.  Beyond that many channels the
+// estimators behind the pooling count for more, and the fewer slabs there are the sooner the first image's can start: 16 x (96x96), 128 of
+// 256 172 / 243 / 277; 128 x (40x40), 96 of 128 134 / 185 / 189; 4 x (300x300), 128 262 / 305 / 303; 500x500, 128 of 256 223 / 232 / 220.
+enum class GapGrid { Narrow, Wide, Large };
+GapGrid gap_grid(int B, int Ca, long long HW, bool toeplitz, bool dw_umma) {
+    if (is_large_map(B, HW) || (dw_umma && Ca <= 64)) return GapGrid::Large;
+    return toeplitz && !dw_umma && B > 1 ? GapGrid::Wide : GapGrid::Narrow;
 }
 
 int slabs_for(int B, long long HW, bool wide) {
@@ -231,13 +238,14 @@ int launch_gap_n(const Problem& p, const void* x, const Estimator& est, const Wo
 }
 template <typename T, int LAYOUT>
 int launch_gap_t(const Problem& p, const void* x, const Estimator& est,
-                 const Workspace& w, float* dk_out, cudaStream_t st, bool wide) {
+                 const Workspace& w, float* dk_out, cudaStream_t st, GapGrid grid) {
     const long long HW = (long long)p.H * p.W, sms = sms_or_nominal();
+    const bool wide = grid != GapGrid::Narrow;
     const int S = slabs_for(p.B, HW, wide);
     // Large maps: bound by DRAM and by how many bytes are in flight, so two blocks of 512 threads on each SM instead of three of 128,
     // as long as their scratch fits (C_a up to 720).  1920x1080 bf16 NHWC, 32 of 64 channels (265 MB of whole lines): 65 -> 58 us.
     const int smem_large = (esc::gap_scratch_floats(LAYOUT, p.C, p.Ca, esc::Elem<T>::kVec, esc::kGapThreadsLarge) + p.Ca) * 4;
-    if (is_large_map(p.B, HW) && smem_large <= 48 * 1024) {
+    if (grid == GapGrid::Large && smem_large <= 48 * 1024) {
         const long long s2 = 2 * sms / p.B < 1 ? 1 : 2 * sms / p.B;
         return launch_gap_n<T, LAYOUT, esc::kGapThreadsLarge>(p, x, est, w, dk_out, st, S < s2 ? S : (int)s2, 2 * sms);
     }
@@ -245,14 +253,14 @@ int launch_gap_t(const Problem& p, const void* x, const Estimator& est,
 }
 
 int launch_gap(const Problem& p, const void* x, const Estimator& est,
-               const Workspace& w, float* dk_out, cudaStream_t st, bool tensor_stencil = false) {
+               const Workspace& w, float* dk_out, cudaStream_t st, bool toeplitz = false, bool dw_umma = false) {
     if ((long long)p.B * esc::kMaxSlabs > 0x7fffffffLL) return ESC_ERR_UNSUPPORTED;
-    const bool wide = wide_gap(p.B, (long long)p.H * p.W, tensor_stencil);
+    const GapGrid grid = gap_grid(p.B, p.Ca, (long long)p.H * p.W, toeplitz, dw_umma);
     if (p.dtype == ESC_F32)
-        return p.layout == ESC_NCHW ? launch_gap_t<float, esc::kNCHW>(p, x, est, w, dk_out, st, wide)
-                                    : launch_gap_t<float, esc::kNHWC>(p, x, est, w, dk_out, st, wide);
-    return p.layout == ESC_NCHW ? launch_gap_t<__nv_bfloat16, esc::kNCHW>(p, x, est, w, dk_out, st, wide)
-                                : launch_gap_t<__nv_bfloat16, esc::kNHWC>(p, x, est, w, dk_out, st, wide);
+        return p.layout == ESC_NCHW ? launch_gap_t<float, esc::kNCHW>(p, x, est, w, dk_out, st, grid)
+                                    : launch_gap_t<float, esc::kNHWC>(p, x, est, w, dk_out, st, grid);
+    return p.layout == ESC_NCHW ? launch_gap_t<__nv_bfloat16, esc::kNCHW>(p, x, est, w, dk_out, st, grid)
+                                : launch_gap_t<__nv_bfloat16, esc::kNHWC>(p, x, est, w, dk_out, st, grid);
 }
 
 int check_estimator(const Problem& p, const Estimator& e) {
@@ -468,7 +476,7 @@ int launch_stencil(const Problem& p0, const void* x, const void* w_large0, const
     return launch_generic(p, x, w_large, dk, out, st, dependent);
 }
 
-// Whether launch_stencil will take the tensor-core kernel for this problem (same conditions).
+// Whether launch_stencil will take the Toeplitz NHWC kernel, or for K = 13 the tcgen05 one in its place (same conditions).
 bool tensor_stencil_follows(const Problem& p) {
     return !p.dense && (!p.w_point || (p.Ca == esc::tma::CG && !p.bias)) && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
            esc::tma::toep::applies(p.C, p.Ca, p.K, p.dtype, p.layout);
@@ -676,7 +684,7 @@ int forward_impl(const Problem& p0, const void* x, const void* w_large0, const E
                              esc::tma::toepn::takes(p.B, p.C, p.Ca, p.H, p.W, p.K, p.dtype, p.layout, x, out);
     const bool packed = p0.dense && wants_packing(p0);
     rc = packed ? launch_pack16(p0, x, w.packed, out, st) : ESC_OK;
-    if (rc == ESC_OK) rc = launch_gap(p0, x, est, w, w.dk, st, tensor_stencil_follows(p) || tensor_nchw);
+    if (rc == ESC_OK) rc = launch_gap(p0, x, est, w, w.dk, st, tensor_stencil_follows(p) || tensor_nchw, dw_umma_follows(p0));
     if (rc != ESC_OK) return rc;
     if (packed) {
         rc = launch_umma_packed(p0, w.packed, w_large0, w.dk, out, w.ctrl, st, /*dependent=*/true, /*flip=*/false);
@@ -1324,7 +1332,7 @@ int esc_convattn_dynkernel_static(const void* x, int B, int C, int C_a, int H, i
     if (rc != ESC_OK) return rc;
     if (!x || !w_dyn || !b_dyn || !dk_out) return ESC_ERR_NULL;
     if (!aligned(x, 16) || !aligned(dk_out, 4) || !aligned(w_dyn, p.es()) || !aligned(b_dyn, p.es())) return ESC_ERR_ALIGN;
-    const int S = slabs_for(B, (long long)H * W, wide_gap(B, (long long)H * W, false));
+    const int S = slabs_for(B, (long long)H * W, gap_grid(B, C_a, (long long)H * W, false, false) != GapGrid::Narrow);
     if (B > kStaticMaxImages || (long long)B * S * C_a > kStaticMaxPartials) {
         char buf[200];
         snprintf(buf, sizeof buf,

@@ -246,3 +246,24 @@ def test_time_does_not_hang_on_the_width(pkg):
             assert pkg.esc_convattn_last_tile_width() == 256
             best[s] = min(best[s], a.elapsed_time(b) / pixels)
     assert best[0] < 1.2 * best[1], best
+
+
+@pytest.mark.parametrize("shape", [(64, 40, 32, 64, 160), (128, 96, 96, 40, 40)], ids=lambda s: "x".join(map(str, s)))
+def test_pooling_grid_is_the_same_for_every_kernel_size(pkg, shape):
+    """The pooling kernel in front takes the grid of a batch whatever K is: the workspace (dk, partial sums) comes out bit for bit the
+    same for K = 13, 9 and 3 on the same map."""
+    import torch
+
+    B, C, C_a, H, W = shape
+    d = synth.make_inputs(B, C, C_a, H, W, 13, synth.BF16, seed=11, channel_means=True)
+    x = util.to_device(d["x"], synth.BF16, synth.NHWC)
+    wl, wd, bd = util.weights_to_device(d, synth.BF16)
+    left = []
+    for K in (13, 9, 3):
+        off = (13 - K) // 2
+        ws = pkg.new_workspace(B, C_a, H, W, K).zero_()
+        pkg.esc_convattn_forward_ex(x, C_a, K, wl[:, off:off + K, off:off + K].contiguous(), wd, bd, torch.empty_like(x), pkg.ESC_NHWC, ws)
+        torch.cuda.synchronize()
+        assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_last_tile_width() == 256
+        left.append(ws)
+    assert bool((left[0] != 0).any()) and torch.equal(left[0], left[1]) and torch.equal(left[0], left[2])
