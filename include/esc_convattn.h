@@ -412,7 +412,7 @@ int esc_convattn_last_path(void);
  * zero: a non-finite attention input therefore turns outputs up to 15 pixels beyond its window into
  * NaN, and (13 - K) / 2 more, up and down too, where a smaller kernel is padded to 13 x 13 (finite data are unaffected).  The
  * generic kernel, those of the dense form and the tcgen05 kernel (NHWC without LK^c, C_a >= 32, more than eight tiles of 64 x 16
- * pixels and 16 channels per SM) keep it inside its window.  The tcgen05 kernel evaluates finite outputs beside a non-finite input one by
+ * pixels and 16 channels per SM; from C_a = 400 on not for every C_a) keep it inside its window.  The tcgen05 kernel evaluates finite outputs beside a non-finite input one by
  * one: a few bad pixels cost a fraction of a millisecond, a map of NaN next to nothing, but many bad pixels that each leave finite
  * outputs around them up to a hundred times the usual time.  Returns ESC_ERR_UNSUPPORTED for any other value. */
 enum { ESC_ENGINE_AUTO = 0, ESC_ENGINE_FP32 = 1, ESC_ENGINE_TENSOR = 2 };

@@ -419,7 +419,7 @@ struct TensorLk {
 // the copies beside it slow it down there, without identity channels it is 147 / 112.)  It takes every odd K up to 13 as it is.
 bool dw_umma_follows(const Problem& p) {
     return !p.dense && !p.w_point && p.Ca >= 2 * esc::tma::CG && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
-           esc::tma::dwu::applies(p.C, p.Ca, p.K, p.dtype, p.layout) && (long long)p.B * p.H * p.W <= 0x7fffffffLL &&
+           esc::tma::dwu::applies(p.C, p.Ca, p.K, p.dtype, p.layout) && esc::tma::dwu::fills(p.Ca, sms_or_nominal()) && (long long)p.B * p.H * p.W <= 0x7fffffffLL &&
            (long long)p.B * (p.W + esc::tma::dwu::GAPX) <= 0x3fffffffLL &&
            esc::tma::toep::units_of<esc::tma::toep::Shape64x16>(p.B, p.Ca, p.H, p.W) > (long long)esc::tma::toep::kMaxFusedUnits * sms_or_nominal();
 }

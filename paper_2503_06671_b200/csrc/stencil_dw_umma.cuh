@@ -619,6 +619,14 @@ inline bool applies(int C, int Ca, int K, int dtype, int layout) {
     return K <= K13 && dtype == 1 /*bf16*/ && layout == kNHWC && Ca % CG == 0 && C % 8 == 0 && C - Ca <= 256;
 }
 
+// Whether the CTAs, as many groups of one for each eight channels as fit, take at least three quarters of the SMs.  Stage, us, mma.sync /
+// this kernel: 304 channels (114 of 148 SMs) 90 / 84, 352 (132) 100 / 84, 512 (128) 139 / 131, 1024 (128) 140 / 133; but 400 (100) 109 / 131,
+// 608 (76) 165 / 236, 800 (100) 110 / 134, 1200 (150 CTAs, two rounds) 166 / 259.
+inline bool fills(int Ca, int sms) {
+    const int octets = Ca / OCT, ctas = octets < sms ? sms / octets * octets : octets, rounds = (ctas + sms - 1) / sms;
+    return 4LL * ctas >= 3LL * rounds * sms;
+}
+
 // Segments per image S, rows per segment R, rows per CTA Q: the fewest rows for the CTA that has most, a new window counted as
 // five rows (its first and last twelve input rows feed only some of the columns).
 struct Plan { int S, R, T, Q, parts; };

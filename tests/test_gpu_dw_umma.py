@@ -61,6 +61,25 @@ def test_stage_against_oracle(pkg, shape):
     assert np.array_equal(got[:, C_a:], ref[:, C_a:])
 
 
+@pytest.mark.parametrize("C_a, width", [(304, 256), (400, 64)])
+def test_many_channels(pkg, oracle, C_a, width):
+    """A group of CTAs takes one for every eight channels: where those groups leave more than a quarter of the 148 SMs empty (400
+    channels: two of 50; 304: three of 38) the mma.sync kernel is the faster one and stays."""
+    import torch
+
+    B, H, W, K = 8, 100, 66, 5
+    d = synth.make_inputs(B, C_a, C_a, H, W, K, synth.BF16, seed=C_a)
+    dk = np.random.default_rng(6).uniform(-0.5, 0.5, size=(B, C_a, 3, 3)).astype(np.float32)
+    x = util.to_device(d["x"], synth.BF16, synth.NHWC)
+    wl, _, _ = util.weights_to_device(d, synth.BF16)
+    out, ws = torch.empty_like(x), pkg.new_workspace(B, C_a, H, W, K)
+    pkg.esc_convattn_stencil(x, C_a, K, wl, torch.from_numpy(dk).cuda(), out, pkg.ESC_NHWC, ws)
+    torch.cuda.synchronize()
+    assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_last_tile_width() == width
+    ref, mag = oracle.stencil(d["x"], C_a, d["w_large"], dk, want_mag=True)
+    util.check_attention(util.to_host_nchw(out, synth.NHWC), ref, mag, synth.BF16, f"C_a = {C_a}", unit_variance=True)
+
+
 def test_constant_of_the_backward_pass(pkg):
     """grad_x is this kernel on grad_out with rotated kernels and a constant per (image, channel): 1,200 small images against the
     same images in four calls, which take the kernel for smaller launches (each result one bf16 rounding: 2^-7 of its magnitude apart at most,
