@@ -42,6 +42,18 @@ MIN_SAMPLE_S = 0.1
 PATH_NAMES = {1: "generic", 2: "tma-fp32", 3: "tensor-dense-mma.sync", 4: "tensor-toeplitz", 5: "tensor-dense-tcgen05", 6: "tensor-toeplitz-nchw"}
 KERNEL_FILES = {1: "stencil_generic.cuh", 2: "stencil_tma.cuh", 3: "stencil_dense.cuh", 4: "stencil_toeplitz.cuh", 5: "stencil_dense_umma.cuh", 6: "stencil_toeplitz_nchw.cuh"}
 TOEPLITZ_DENSITY = 13.0 / 32.0               # useful share of the multiply-adds the banded-Toeplitz kernel issues
+DW_UMMA_TILE = 256                           # path 4 with this tile width is the tcgen05 depth-wise kernel of large launches
+DW_UMMA_DENSITY = 13.0 / 112.0               # its useful share: one of eight channels, 13 of 14 kernel columns
+
+
+def path_name(path, tile_w):
+    return "tensor-dw-tcgen05" if path == 4 and tile_w == DW_UMMA_TILE else PATH_NAMES.get(path, str(path))
+
+
+def kernel_source(path, tile_w):
+    return "stencil_dw_umma.cuh" if path == 4 and tile_w == DW_UMMA_TILE else KERNEL_FILES.get(path, "stencil_tma.cuh")
+
+
 PEAK_SRC = os.path.join(ROOT, "bench_fp32_peak.cu")
 PEAK_LIB = os.path.join(ROOT, "paper_2503_06671_b200", "lib", "libbench_fp32_peak.so")
 
@@ -368,7 +380,7 @@ def measure_config(pkg, torch, np, synth, wl, layout_name, steps, pk, sms, fp32_
     ms_step, ms_kernel = st_step["median_ms"], st_kernel["median_ms"]
     rec = {
         "workload": wl.name, "layout": layout_name, "storage": wl.dtype,
-        "stencil_path": PATH_NAMES.get(path, str(path)), "tile_width": tile_w, "launches_per_step": launches_per_step,
+        "stencil_path": path_name(path, tile_w), "tile_width": tile_w, "launches_per_step": launches_per_step,
         "step_us": ms_step * 1e3, "step_us_min": st_step["min_ms"] * 1e3, "step_us_max": st_step["max_ms"] * 1e3,
         "stencil_us": ms_kernel * 1e3, "stencil_us_min": st_kernel["min_ms"] * 1e3, "stencil_us_max": st_kernel["max_ms"] * 1e3,
         "samples": st_step["samples"], "replays_per_sample": st_step["replays_per_sample"],
@@ -384,7 +396,7 @@ def measure_config(pkg, torch, np, synth, wl, layout_name, steps, pk, sms, fp32_
     ctx = dict(d=d, x_host=x_host, w_host=w_host, wl_d=wl_d, wd_d=wd_d, bd_d=bd_d, xs=xs, outs=outs, ws=ws, dk=dk,
                n_rot=n_rot, lay_code=lay_code, tdt=tdt, es=es, tensor_bytes=tensor_bytes, timer=timer, step=step,
                stencil=stencil, g_step=g_step, launches_per_step=launches_per_step, stencil_launches=stencil_launches,
-               path=path, st_step=st_step, st_kernel=st_kernel, flops=flops, alg_bytes=alg_bytes,
+               path=path, tile_w=tile_w, st_step=st_step, st_kernel=st_kernel, flops=flops, alg_bytes=alg_bytes,
                peak_tflops=peak_tflops, t_alu=t_alu, t_hbm=t_hbm)
     return rec, ctx
 
@@ -463,7 +475,7 @@ def main():
     wl_d, wd_d, bd_d, tensor_bytes = c["wl_d"], c["wd_d"], c["bd_d"], c["tensor_bytes"]
 
     flops, alg_bytes, peak_tflops, t_alu, t_hbm = (c[k] for k in ("flops", "alg_bytes", "peak_tflops", "t_alu", "t_hbm"))
-    kernel_file = KERNEL_FILES.get(c["path"], "stencil_tma.cuh")
+    kernel_file = kernel_source(c["path"], c["tile_w"])
     if args.large_kernel == "dense":
         ach = flops / (ms_step * 1e-3) / 1e12
         roof = {"bound": "tensor", "achieved": ach, "peak": peak_tflops, "unit": "TFLOP/s", "frac": ach / peak_tflops,
@@ -487,8 +499,12 @@ def main():
         # the depth-wise stage runs on the tensor cores as banded-Toeplitz products: the fraction above is still
         # the one of the FP32 roofline of the method's 169 multiply-adds per output (the contract's bound); beside
         # it, what the tensor pipe was asked to do
-        issued = flops / TOEPLITZ_DENSITY
-        roof["engine"] = "tensor cores: mma.sync m16n8k16 bf16 x bf16 -> fp32, 13 of 32 issued multiply-adds useful"
+        if c["tile_w"] == DW_UMMA_TILE:
+            issued = flops / DW_UMMA_DENSITY
+            roof["engine"] = "tensor cores: tcgen05.mma M = 128, N = 208, K = 16 bf16 x bf16 -> fp32, 13 of 112 issued multiply-adds useful"
+        else:
+            issued = flops / TOEPLITZ_DENSITY
+            roof["engine"] = "tensor cores: mma.sync m16n8k16 bf16 x bf16 -> fp32, 13 of 32 issued multiply-adds useful"
         roof["tensor_side"] = {"issued_TFLOPs_whole_step": issued / (ms_step * 1e-3) / 1e12,
                                "issued_TFLOPs_stencil_stage": issued / (ms_kernel * 1e-3) / 1e12,
                                "bf16_peak_TFLOPs": pk["bf16_tflops"],
@@ -627,7 +643,7 @@ def main():
             extras["dense_large_kernel"] = {
                 "ms_per_step": ms_dense, "bound": "tensor", "achieved": fl / (ms_dense * 1e-3) / 1e12, "peak": pk["bf16_tflops"],
                 "unit": "TFLOP/s", "frac": fl / (ms_dense * 1e-3) / 1e12 / pk["bf16_tflops"],
-                "path": PATH_NAMES.get(pkg.esc_convattn_last_path(), str(pkg.esc_convattn_last_path())),
+                "path": path_name(pkg.esc_convattn_last_path(), pkg.esc_convattn_last_tile_width()),
                 "note": "whole step (GAP kernel + dense stencil kernel with copy-through)"}
 
         # ---- end to end through the host-buffer entries (copies inside the timed region) ------------

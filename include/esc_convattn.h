@@ -438,8 +438,9 @@ int esc_convattn_set_fused_stage1(int on);
 int esc_convattn_set_dense_engine(int engine);
 
 /* Width in pixels of the output tile the TMA-staged kernel used in that call (FP32 kernel: 40 = 40x40
- * tiles, 64 = 64x16 tiles, chosen by the tile count's balance over the SMs; tensor-core kernel: 64 =
- * 64x16 tiles), 0 when the generic kernel ran.  For tests and benchmarks. */
+ * tiles, 64 = 64x16 tiles, chosen by the tile count's balance over the SMs; tensor-core Toeplitz kernels: 64 =
+ * 64x16 tiles; tcgen05 kernels: 128 = strips of the dense one, 256 = windows of the depth-wise one, which tells it
+ * from the Toeplitz kernel that shares its path 4), 0 when the generic kernel ran.  For tests and benchmarks. */
 int esc_convattn_last_tile_width(void);
 
 /* Overrides the tile choice of the TMA-staged FP32 kernel for later calls on this thread (and, when

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2503_06671_b200 import synth
-from tests import util
+from tests import test_gpu_fuse, test_gpu_mlp, test_gpu_parity, util
 
 pytestmark = pytest.mark.gpu
 
@@ -78,6 +78,31 @@ def test_many_channels(pkg, oracle, C_a, width):
     assert pkg.esc_convattn_device_status(ws) == 0 and pkg.esc_convattn_last_tile_width() == width
     ref, mag = oracle.stencil(d["x"], C_a, d["w_large"], dk, want_mag=True)
     util.check_attention(util.to_host_nchw(out, synth.NHWC), ref, mag, synth.BF16, f"C_a = {C_a}", unit_variance=True)
+
+
+@pytest.mark.parametrize("shape", [(64, 64, 32, 50, 130, 13), (1, 48, 32, 700, 901, 13), (64, 64, 32, 50, 130, 9), (1, 96, 48, 500, 800, 5), (80, 112, 96, 40, 40, 11)],
+                         ids=lambda s: "x".join(map(str, s)))
+def test_forward(pkg, oracle, shape):
+    """Behind the pooling kernel and the linear estimator, as a programmatic dependent: batches and single images, K below 13, more than
+    64 channels (a smaller pooling grid)."""
+    B, C, C_a, H, W, K = shape
+    d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=sum(shape), per_image_scale=True, channel_means=True)
+    test_gpu_parity.compare_full(pkg, oracle, d, C_a, K, synth.BF16, synth.NHWC, what=f"{shape}")
+    assert pkg.esc_convattn_last_path() == 4 and pkg.esc_convattn_last_tile_width() == 256 and pkg.esc_convattn_last_launches() == 2
+
+
+@pytest.mark.parametrize("shape", [(64, 64, 32, 50, 130, 13, 8), (1, 64, 32, 700, 901, 7, 16)], ids=lambda s: "x".join(map(str, s)))
+def test_forward_two_layer_estimator(pkg, oracle, shape):
+    test_gpu_mlp.test_forward_mlp(pkg, oracle, shape, synth.BF16, synth.NHWC)
+    assert pkg.esc_convattn_last_tile_width() == 256 and pkg.esc_convattn_last_launches() == 2
+
+
+@pytest.mark.parametrize("case", [(64, 64, 32, 50, 130, 13, synth.BF16, synth.NHWC, True, "own"), (1, 48, 32, 700, 901, 13, synth.BF16, synth.NHWC, False, "x"),
+                                  (20, 192, 48, 100, 150, 13, synth.BF16, synth.NHWC, True, "own")], ids=lambda c: "x".join(map(str, c[:6])))
+def test_module(pkg, oracle, case):
+    """Forward, 1x1 convolution and residual in one call: without the identity channels (C up to 128), and with them."""
+    test_gpu_fuse.test_forward_fused(pkg, oracle, case)
+    assert pkg.esc_convattn_last_tile_width() == 256 and pkg.esc_convattn_last_launches() == 3
 
 
 def test_constant_of_the_backward_pass(pkg):

@@ -226,9 +226,9 @@ def test_mandated_entry_fp32_nchw(pkg, oracle):
 @pytest.mark.parametrize("layout", LAYOUTS)
 def test_forward_large_map_full(pkg, oracle, layout):
     """1920x1080, C_a = 32 bf16 in the launch configuration the benchmark times: every one of the 66 M
-    attention outputs against the oracle, copy-through channels bit for bit.  On 148 SMs a CTA of the
-    TMA-staged kernel walks 17 or 18 units here: the barrier phases wrap several times and the channel
-    group (hence the weight table) changes inside a walk."""
+    attention outputs against the oracle, copy-through channels bit for bit.  NHWC: the tcgen05 kernel, whose CTAs
+    walk about 236 window rows each; NCHW: the Toeplitz kernel, 27 or 28 units a CTA, whose barrier phases wrap several
+    times and whose channel group (hence the weight table) changes inside a walk."""
     wl = synth.WORKLOADS_BY_NAME["cfg5_1920x1080_ca32_bf16"]
     d = synth.make_workload(wl, channel_means=True)
     compare_full(pkg, oracle, d, wl.C_a, wl.K, wl.dtype, layout, what="cfg5 full")

@@ -63,14 +63,18 @@ def test_engines_agree_and_switch(pkg, oracle):
         assert pkg.esc_convattn_last_path() == 1
 
 
-def test_many_units_per_cta(pkg, oracle):
-    """Eight images, two channel groups, 280x400: 2,016 units of 64x16, thirteen or fourteen per CTA on 148
-    SMs, with image and channel-group changes inside every CTA's walk; all outputs compared."""
-    B, C, C_a, H, W, K = 8, 64, 32, 280, 400, 13
+@pytest.mark.parametrize("shape, tile", [((8, 64, 32, 280, 400), 256), ((8, 64, 16, 560, 400), 64), ((4, 400, 400, 100, 100), 64)],
+                         ids=lambda s: "x".join(map(str, s)) if isinstance(s, tuple) else str(s))
+def test_many_units_per_cta(pkg, oracle, shape, tile):
+    """More than eight units of 64x16 pixels and 16 channels per SM, in two launches; all outputs compared.  Eight images of one channel
+    group: 1,960 units, thirteen or fourteen per CTA on 148 SMs, with image changes inside a walk.  25 groups: 1,400 units, and the
+    group (hence the table of the kernel's rows) changes too.  Two groups, 280x400: the tcgen05 kernel (tile 256) takes such launches."""
+    B, C, C_a, H, W = shape
+    K = 13
     d = synth.make_inputs(B, C, C_a, H, W, K, synth.BF16, seed=2031, per_image_scale=True, channel_means=True)
     with engine(pkg, pkg.ESC_ENGINE_TENSOR):
-        compare_full(pkg, oracle, d, C_a, K, synth.BF16, synth.NHWC, what="many units, tensor engine")
-        assert pkg.esc_convattn_last_path() == 4
+        compare_full(pkg, oracle, d, C_a, K, synth.BF16, synth.NHWC, what=f"{shape} many units, tensor engine")
+        assert pkg.esc_convattn_last_path() == 4 and pkg.esc_convattn_last_tile_width() == tile and pkg.esc_convattn_last_launches() == 2
 
 
 def test_stencil_stage_explicit_dk_and_determinism(pkg, oracle):
