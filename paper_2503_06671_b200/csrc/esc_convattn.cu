@@ -414,9 +414,11 @@ struct TensorLk {
 };
 // Whether the depth-wise stage goes to the tcgen05 kernel: bf16 NHWC without the point-wise mix, unless the caller pinned the FP32
 // kernel (by engine or by one of its tile widths), at least two groups of channels, and more work than the one-launch form of the
-// mma.sync kernel takes.  (Forward, mma.sync / tcgen05, us: 1920x1080, 32 of 64 channels 324 / 269, with K = 9 327 / 273; 1280x720 163 / 125;
-// 900x500, 48 of 192 channels 215 / 141; 64 images of 160x64, 32 of 64 channels 132 / 103.  With one group, 16 of 64 channels, 1920x1080 217 / 280:
-// the copies beside it slow it down there, without identity channels it is 147 / 112.)  It takes every odd K up to 13 as it is.
+// mma.sync kernel takes.  (Forward, mma.sync / tcgen05, us, bursts of twenty: 1920x1080, 32 of 64 channels 325 / 237, with K = 9 329 / 265; 1280x720
+// 168 / 123; 900x500, 48 of 192 218 / 114; 64 images of 160x64, 32 of 64 136 / 105, of 96x96, 48 of 192 307 / 155; 50 of 300x22, 32 of 128
+// 169 / 69; 44 drawn sizes of two to six groups all faster, 5 to 70 %.  With one group the pooling and the copies weigh more: 1920x1080, 16 of 64 220 / 245,
+// 16 of 48 180 / 192; only without identity channels (149 / 117) or on batches of small images (128 x (96x96), K = 9 152 / 126) it wins.)
+// It takes every odd K up to 13 as it is.
 bool dw_umma_follows(const Problem& p) {
     return !p.dense && !p.w_point && p.Ca >= 2 * esc::tma::CG && g_engine_policy != ESC_ENGINE_FP32 && g_tile_policy == 0 &&
            esc::tma::dwu::applies(p.C, p.Ca, p.K, p.dtype, p.layout) && esc::tma::dwu::fills(p.Ca, sms_or_nominal()) && (long long)p.B * p.H * p.W <= 0x7fffffffLL &&

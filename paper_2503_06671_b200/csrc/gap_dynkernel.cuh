@@ -10,7 +10,7 @@
 //
 // Every image is cut into S slabs so that a single large image still spreads over the machine;
 // the B*S work items are walked by a persistent grid of small blocks (4 warps -- one per SM sub-partition --, at most one block
-// per SM; where a large map has this kernel run ahead on its own, 16 warps and two blocks).  The blocks are kept this small on purpose: the stencil kernel is launched as a
+// per SM; where this kernel runs ahead on its own, on large maps and in front of the tcgen05 depth-wise kernel, 16 warps and two blocks).  The blocks are kept this small on purpose: the stencil kernel is launched as a
 // programmatic dependent of this one and needs nearly a whole SM per block, so the two kernels
 // can only run side by side -- this one bound by DRAM, the other by the FMA pipe -- if this one
 // leaves the registers and shared memory free.  A block reduces a slab with 16-byte loads, warp

@@ -34,13 +34,15 @@
 //   warp 12      issues the instructions; warps 12-15 build B before that
 //   warp 13      copies the identity channels, TMA in / TMA out
 //
-// What bounds it: the shared-memory / L1 data pipe.  Of 1,300 cycles per input row of a window the tensor core's operands take 640
-// wavefronts (48 %), loads and stores 540 (40 %: every 16-byte pixel part of a 128-byte line is one), TMA copies most of the rest; the tensor pipe is
-// 64 % busy, DRAM 39 %.  1920x1080, C_a = 32 of 64 channels, stage alone: 184 us (162 without the identity channels) against 263 for
-// the mma.sync Toeplitz kernel; the whole forward 324 -> 270.  On the way: one output row at a time in the epilogue and waits by one lane
+// What bounds it: the shared-memory / L1 data pipe, and under sustained load the board's power.  Of 1,290 cycles per input row of a
+// window the tensor core's operands take 640 wavefronts (48 %), loads and stores 500 (39 %: every 16-byte pixel part of a 128-byte line is
+// one), TMA copies most of the rest; the tensor pipe is 63 % busy, DRAM 42 %.  1920x1080, C_a = 32 of 64 channels, stage alone, 303 k
+// cycles on random data: 183 us in bursts of twenty launches against 264 for the mma.sync Toeplitz kernel (169 against 254 without identity
+// channels), 208 against 263 back to back, where 1,000 W hold the clock at about 1.46 GHz; the whole forward 325 -> 237 and 323 -> 256.
+// On the way (bursts): one output row at a time in the epilogue and waits by one lane
 // 316; loads ahead of the arithmetic, rows by two 241 (by four 282); slots counted on and tensor memory asked for by four rows in the
 // issuing warp, identity channels beside the same rows 185 (chunks of the whole map in turn instead: 297, the parts of a line then reach
-// DRAM one by one).  No difference: copies up to 16 rows ahead, L2 prefetch sizes on the loads.
+// DRAM one by one); those copied once each and up to 24 rows ahead 178 - 183.  No difference: L2 prefetch sizes on the loads.
 #pragma once
 #include "stencil_dense_umma.cuh"
 #include "gap_dynkernel.cuh"

@@ -262,7 +262,7 @@ def test_time_does_not_hang_on_the_data(pkg):
     one = time()
     x[..., :C_a] = float("nan")
     everywhere = time()
-    assert one < 4 * finite and everywhere < 2 * finite, (finite, one, everywhere)
+    assert one < 6 * finite and everywhere < 2 * finite, (finite, one, everywhere)
 
 
 def test_time_does_not_hang_on_the_width(pkg):
@@ -289,7 +289,7 @@ def test_time_does_not_hang_on_the_width(pkg):
             torch.cuda.synchronize()
             assert pkg.esc_convattn_last_tile_width() == 256
             best[s] = min(best[s], a.elapsed_time(b) / pixels)
-    assert best[0] < 1.2 * best[1], best
+    assert best[0] < 1.25 * best[1], best
 
 
 @pytest.mark.parametrize("shape", [(64, 40, 32, 64, 160), (128, 96, 96, 40, 40)], ids=lambda s: "x".join(map(str, s)))
